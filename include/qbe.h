@@ -323,7 +323,8 @@ int qbe_arith_issue_rates(int device, void* stream, double* rates);
  *     grid size 2N and precision.  FP64: the staged kernel with 256 threads and
  *     64 KB shared-memory chunks (3 blocks per SM) or 128 threads and 32 KB
  *     chunks (6 per SM), or the staged kernel with its global loads and
- *     stores fused into the line stages (256 threads, 64 KB).  FP32-split form, 2N = 64, 96, 128: the fused
+ *     stores fused into the line stages and the radial nodes taken in pairs +-rho_m, which share
+ *     their convolutions (256 threads, 64 KB or 128 threads, 32 KB).  FP32-split form, 2N = 64, 96, 128: the fused
  *     shared-memory kernel in three thread/accumulation shapes, or the kernel
  *     whose element passes go through shared memory, and at 2N = 128 also the
  *     kernel with warp-local passes; 2N <= 32: the element-pass kernel

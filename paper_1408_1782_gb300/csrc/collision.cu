@@ -1,5 +1,8 @@
 // Size dispatch and workspace allocation of the collision operator; the
 // kernels are instantiated per fine-grid size in collision_n*.cu.
+#include <climits>
+#include <vector>
+
 #include "internal.h"
 
 namespace qbe {
@@ -77,6 +80,30 @@ const char* i3_variant_desc(int n, int prec, int variant) {
 #undef QBE_CALL
 }
 
+bool i3_paired(int n, int prec, int variant) {
+#define QBE_CALL(nn, T) i3_variant_paired<nn, T>(variant)
+  QBE_SIZE_SWITCH(QBE_CALL, false)
+#undef QBE_CALL
+}
+
+double i3_chunk_cost(int begin, int end, int M, bool paired) {
+  if (!paired) return 18.0 * (end - begin);      // 2 shifts, 16 transforms of 8 convolutions
+  double cost = 0;
+  for (int it = begin; it < end;) {
+    if ((M & 1) && it == M - 1) {
+      cost += 18.0;                              // the middle node
+      it += 1;
+    } else if ((it & 1) == 0 && it + 1 < end) {
+      cost += 20.0;                              // a pair: 2 shifts, 8 convolutions, 2 back
+      it += 2;
+    } else {
+      cost += 11.0;                              // half a pair
+      it += 1;
+    }
+  }
+  return cost;
+}
+
 // Angle chunks per cell of the I1 and I2/I4 kernels: enough (cell, chunk) blocks to fill about one
 // wave of the device (3 resident 256-thread blocks per SM), at most J/2 (the I2/I4 angle pairs).
 int per_cell_chunks(int nb, int J) {
@@ -112,8 +139,39 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   int nmc = (8 * cw.grid_i3 + nb * t.J - 1) / (nb * t.J);
   if (nmc < 1) nmc = 1;
   if (nmc > t.M) nmc = t.M;
-  cw.mch = (t.M + nmc - 1) / nmc;
-  cw.nmc = (t.M + cw.mch - 1) / cw.mch;
+  const size_t N = t.N, Q = (N - 1) * (N - 1);
+  const size_t cz = prec == 1 ? sizeof(float2) : sizeof(double2);   // complex element
+  const size_t rz = cz / 2;                                           // real element
+  bool any_paired = false;
+  for (int v = 0; v < nv; ++v) any_paired = any_paired || i3_paired(t.n, prec, v);
+  const size_t part_bytes = (2 * P + (any_paired ? 2 * Q : 0)) * cz;
+  auto set_chunks = [&](int want) {
+    cw.mch = (t.M + want - 1) / want;
+    cw.nmc = (t.M + cw.mch - 1) / cw.mch;
+  };
+  set_chunks(nmc);
+  if (i3_paired(t.n, prec, v0)) {
+    // Up to three times as many chunks where they even out the blocks' loads (unit u goes to block
+    // u mod G) within 4 GB of partials: a unit's fixed costs (its partials written and reduced, about
+    // a fiftieth of a pair's transforms) against the last, partly filled wave.
+    const int base = cw.nmc;
+    double best = 0;
+    int best_nmc = base;
+    for (int want = base; want <= 3 * base && want <= t.M; ++want) {
+      set_chunks(want);
+      const long long units = (long long)nb * t.J * cw.nmc;
+      if (want > base && (cw.nmc == base || (size_t)units * part_bytes > ((size_t)4 << 30))) continue;
+      const int G = i3_concurrency(t.n, prec, v0, cw.grid_i3, (int)(units < INT_MAX ? units : INT_MAX));
+      std::vector<double> load(G, 0.0), cost(cw.nmc);
+      for (int mc = 0; mc < cw.nmc; ++mc)
+        cost[mc] = 0.4 + i3_chunk_cost(i3_chunk_begin(mc, cw.nmc, t.M), i3_chunk_begin(mc + 1, cw.nmc, t.M), t.M, true);
+      for (long long u = 0; u < units; ++u) load[u % G] += cost[u % cw.nmc];
+      double mx = 0;
+      for (double l : load) mx = l > mx ? l : mx;
+      if (want == base || mx < 0.99 * best) { best = mx; best_nmc = cw.nmc; }
+    }
+    set_chunks(best_nmc);
+  }
   const size_t nparts = (size_t)nb * t.J * cw.nmc;
   cw.nparts_cap = nparts;
   cw.ws_slots = nb > cw.grid_i3 ? nb : cw.grid_i3;
@@ -121,10 +179,11 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   size_t ws_fields = 6 * (size_t)nb;
   if (5 * (size_t)nb * cw.nch > ws_fields) ws_fields = 5 * (size_t)nb * cw.nch;   // k_i24: 5 fields per block
   if (3 * (size_t)cw.grid_max > ws_fields) ws_fields = 3 * (size_t)cw.grid_max;
+  // the FP64 kernel that takes the nodes in pairs needs a fourth field per block; the number of blocks
+  // the scratch serves stays
+  cw.i3_fields = (any_paired && prec == 0) ? 4 : 3;
+  ws_fields = ws_fields / 3 * cw.i3_fields + ws_fields % 3;
   cw.ws_fields = ws_fields;
-  const size_t N = t.N;
-  const size_t cz = prec == 1 ? sizeof(float2) : sizeof(double2);   // complex element
-  const size_t rz = cz / 2;                                           // real element
   cudaError_t e;
 #define QBE_ALLOC(ptr, bytes) \
   if ((e = cudaMalloc((void**)&(ptr), (bytes))) != cudaSuccess) { free_collision_work(cw); return e; }
@@ -139,6 +198,8 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
     QBE_ALLOC(cw.K4part, (size_t)nb * cw.nch * 2 * P * cz);
   }
   QBE_ALLOC(cw.K3part, nparts * 2 * P * cz);
+  if (any_paired) QBE_ALLOC(cw.K3spec, nparts * 2 * Q * cz);
+  if (prec == 1) QBE_ALLOC(cw.K3sum, (size_t)nb * 2 * P * sizeof(double2));
   QBE_ALLOC(cw.ws, ws_fields * P * cz);
   QBE_ALLOC(cw.cbuf, (size_t)nb * 4 * N * N * sizeof(double));
   QBE_ALLOC(cw.wbuf, (size_t)nb * 4 * N * N * sizeof(double));
@@ -149,7 +210,7 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
 void free_collision_work(CollisionWork& cw) {
   cudaFree(cw.what); cudaFree(cw.wfine); cudaFree(cw.Dacc); cudaFree(cw.K2acc); cudaFree(cw.K4acc);
   cudaFree(cw.Dpart); cudaFree(cw.K2part); cudaFree(cw.K4part);
-  cudaFree(cw.K3part); cudaFree(cw.ws); cudaFree(cw.cbuf); cudaFree(cw.wbuf);
+  cudaFree(cw.K3part); cudaFree(cw.K3spec); cudaFree(cw.K3sum); cudaFree(cw.ws); cudaFree(cw.cbuf); cudaFree(cw.wbuf);
   cw = CollisionWork();
 }
 

@@ -52,6 +52,36 @@ __device__ __forceinline__ bool in_xi(int k) {
   return (k < N / 2) || (k > n - N / 2);
 }
 
+// Fourier-space partials are kept only on the frequencies the final projection keeps (in_xi in both
+// coordinates, n/2 - 1 per coordinate): xi_slot is the compact index, ascending in the permuted
+// position, or -1.  Position B k1 + t holds a frequency of Xi where xi_t<B>(t); its -N/2 line sits at
+// k1 = 0, t = 3 B / 4.
+template <int n>
+__host__ __device__ constexpr int xi_kept() {
+  return n / 2 - 1;
+}
+template <int n>
+__host__ __device__ constexpr int xi_slot(int pos) {
+  constexpr int B = Split<n>::B;
+  const int k1 = pos / B, t = pos % B;
+  if (!xi_t<B>(t) || pos == 3 * B / 4) return -1;
+  return k1 * (B / 2) + (t < B / 4 ? t : t - B / 2) - (pos > 3 * B / 4 ? 1 : 0);
+}
+template <int n>
+__device__ __forceinline__ void build_xi_slots(int* slot) {
+  for (int pos = threadIdx.x; pos < n; pos += blockDim.x) slot[pos] = xi_slot<n>(pos);
+  __syncthreads();
+}
+template <int n>
+__device__ __forceinline__ void build_xi_slots(int* slot, int* kept_pos) {
+  for (int pos = threadIdx.x; pos < n; pos += blockDim.x) {
+    const int k = xi_slot<n>(pos);
+    slot[pos] = k;
+    if (k >= 0) kept_pos[k] = pos;
+  }
+  __syncthreads();
+}
+
 template <class C2>
 __device__ __forceinline__ void zero_fields(C2* p, int count) {
   for (int i = threadIdx.x; i < count; i += blockDim.x) p[i] = mk2((typename RealOf<C2>::type)0, (typename RealOf<C2>::type)0);
@@ -69,6 +99,29 @@ __device__ __forceinline__ int i3_job_of(const I3Jobs<T>& jobs, int gunit) {
   int k = 0;
   while (k + 1 < jobs.njobs && gunit >= jobs.job[k + 1].unit_begin) ++k;
   return k;
+}
+
+// Node group at item `it` of a chunk that ends at it1 (items as in i3_chunk_begin): node m, with its
+// partner M-1-m where `pair` is set, and the pairs q in [q0, q1) of the first index of U_ab (w_0 + i w_1,
+// w_2 + i w_3) that the chunk covers; `next` is the item after it.
+struct I3Group {
+  int m, q0, q1, next;
+  bool pair;
+};
+__device__ __forceinline__ I3Group i3_group_at(int it, int it1, int M) {
+  I3Group g;
+  g.m = it >> 1;
+  g.pair = !((M & 1) && it == M - 1);
+  if (!g.pair) {
+    g.q0 = 0;
+    g.q1 = 2;
+    g.next = it + 1;
+  } else {
+    g.q0 = it & 1;
+    g.q1 = (g.q0 == 0 && it + 1 < it1) ? 2 : g.q0 + 1;
+    g.next = it + g.q1 - g.q0;
+  }
+  return g;
 }
 
 // --------------------------------------------------------------------------
@@ -309,7 +362,7 @@ __global__ void __launch_bounds__(NTH, MINB)
   for (int gunit = blockIdx.x; gunit < jobs.total; gunit += gridDim.x) {
     const I3Job<T>& jb = jobs.job[i3_job_of(jobs, gunit)];
     const int unit = gunit - jb.unit_begin;
-    const int J = jb.J, M = jb.M, nmc = jb.nmc, mch = jb.mch;
+    const int J = jb.J, M = jb.M, nmc = jb.nmc;
     const C2* what = jb.what;
     const T* __restrict__ psip_s = jb.psip_s;
     const C2* __restrict__ phase = jb.phase;
@@ -320,7 +373,7 @@ __global__ void __launch_bounds__(NTH, MINB)
     zero_fields(acc, 2 * P);
     const T* psp = psip_s + (size_t)j * P;
     const C2* wf = jb.wfine + (size_t)c * 2 * P;
-    const int m0 = mc * mch, m1 = min(M, m0 + mch);
+    const int m0 = i3_chunk_begin(mc, nmc, M), m1 = i3_chunk_begin(mc + 1, nmc, M);
     for (int m = m0; m < m1; ++m) {
       const C2* px = phase + ((size_t)j * M + m) * 2 * n;
       const C2* py = px + n;
@@ -401,7 +454,7 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_smem(const I3Jobs<floa
   for (int gunit = blockIdx.x; gunit < jobs.total; gunit += gridDim.x) {
     const I3Job<float>& jb = jobs.job[i3_job_of(jobs, gunit)];
     const int unit = gunit - jb.unit_begin;
-    const int J = jb.J, M = jb.M, nmc = jb.nmc, mch = jb.mch;
+    const int J = jb.J, M = jb.M, nmc = jb.nmc;
     const C2* what = jb.what;
     const float* __restrict__ psip_s = jb.psip_s;
     const C2* __restrict__ phase = jb.phase;
@@ -417,7 +470,7 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_smem(const I3Jobs<floa
       __syncthreads();
     }
     const C2* wf = jb.wfine + (size_t)c * 2 * P;
-    const int m0 = mc * mch, m1 = min(M, m0 + mch);
+    const int m0 = i3_chunk_begin(mc, nmc, M), m1 = i3_chunk_begin(mc + 1, nmc, M);
     for (int m = m0; m < m1; ++m) {
       const C2* px = phase + ((size_t)j * M + m) * 2 * n;
       const C2* py = px + n;
@@ -737,7 +790,7 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
   for (int gunit = cluster_index(); gunit < jobs.total; gunit += cluster_count()) {
     const I3Job<float>& jb = jobs.job[i3_job_of(jobs, gunit)];
     const int unit = gunit - jb.unit_begin;
-    const int J = jb.J, M = jb.M, nmc = jb.nmc, mch = jb.mch;
+    const int J = jb.J, M = jb.M, nmc = jb.nmc;
     const C2* what = jb.what;
     const C2* __restrict__ phase = jb.phase;
     const int c = unit / (J * nmc);
@@ -756,7 +809,7 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
     for (int idx = tid; idx < n * R; idx += NT) psl[idx] = psp[(idx / R) * n + r0 + idx % R];
     __syncthreads();
     const C2* wf = jb.wfine + (size_t)c * 2 * P;
-    const int m0 = mc * mch, m1 = min(M, m0 + mch);
+    const int m0 = i3_chunk_begin(mc, nmc, M), m1 = i3_chunk_begin(mc + 1, nmc, M);
     for (int m = m0; m < m1; ++m) {
       const C2* px = phase + ((size_t)j * M + m) * 2 * n;
       const C2* py = px + n;
@@ -853,16 +906,63 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
 }
 
 // --------------------------------------------------------------------------
+// Sums of the per-unit I3 partials of each cell, in FP64: the np fine-grid values (2 n^2 complex) and
+// the nq Fourier-space values (kept frequencies; nq = 0 where the launch wrote none).  A block takes
+// 256 / G points with G threads each, thread g the units u = g mod G, added in the order of g.
+// Bound by HBM (or L2, where the partials still sit there).  It was part of k_assemble, whose one
+// block per cell read a single cell's partials alone: at one cell of N = 32, J = M = 32, 1024 units,
+// 5.2 of the 5.5 ms of that kernel.
+// sum: [ncells][np], or null (FP64): in place into the cell's first unit; the Fourier-space sums are
+// always put there.
+// --------------------------------------------------------------------------
+template <class T, int G>
+__global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* part, double2* sum,
+                                                   typename Vec2Of<T>::type* spec, int nparts, int np, int nq,
+                                                   int chunks) {
+  using C2 = typename Vec2Of<T>::type;
+  constexpr int PT = 256 / G;
+  const size_t c = blockIdx.x / chunks;
+  const int i = (blockIdx.x % chunks) * PT + threadIdx.x % PT, g = threadIdx.x / PT;
+  const bool real_space = i < np;
+  C2* src = real_space ? part + c * nparts * np + i : spec + c * nparts * nq + (i - np);
+  const size_t stride = real_space ? np : nq;
+  double sx = 0, sy = 0;
+  if (i < np + nq) {
+#pragma unroll 8
+    for (int u = g; u < nparts; u += G) {
+      const C2 v = src[(size_t)u * stride];
+      sx += (double)v.x;
+      sy += (double)v.y;
+    }
+  }
+  if constexpr (G > 1) {
+    __shared__ double2 red[G][PT];
+    red[g][threadIdx.x % PT] = mk2(sx, sy);
+    __syncthreads();
+    if (g > 0) return;
+    for (int k = 1; k < G; ++k) {
+      sx += red[k][threadIdx.x].x;
+      sy += red[k][threadIdx.x].y;
+    }
+  }
+  if (i >= np + nq) return;
+  if (real_space && sum) sum[c * np + i] = mk2(sx, sy);
+  else *src = mk2((T)sx, (T)sy);
+}
+
+// --------------------------------------------------------------------------
 // Assemble C on the fine grid from D, K2, K3, K4 (Pauli formulas of Sec. 3.1),
 // then FFT, cut to Xi (without the -N/2 line), inverse FFT and sample the
-// coarse nodes.  One block per cell.  The K3 partial sums are added in FP64.
+// coarse nodes.  One block per cell.  k3: the reduced K3 pairs (FP64) of a cell, k3_stride apart;
+// spec (may be null): their Fourier-space parts, added to the spectrum of C inside the projection
+// (C_0 holds -2 pi K3_0 and C_c holds +2 pi K3raw_c; the sign of component 0 is already in spec).
 // --------------------------------------------------------------------------
 template <int n, class T>
 __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>::type* wfine,
                                                        const typename Vec2Of<T>::type* Dacc, const T* K2acc,
-                                                       const typename Vec2Of<T>::type* K4acc,
-                                                       const typename Vec2Of<T>::type* K3part, int nparts,
-                                                       typename Vec2Of<T>::type* ws,
+                                                       const typename Vec2Of<T>::type* K4acc, const double2* k3,
+                                                       size_t k3_stride, const typename Vec2Of<T>::type* spec,
+                                                       size_t spec_stride, typename Vec2Of<T>::type* ws,
                                                        const typename Vec2Of<T>::type* __restrict__ gtw,
                                                        double* cout) {
   using C2 = typename Vec2Of<T>::type;
@@ -885,23 +985,19 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
         sm, tw, [&](int ix, int iy) { return out[ix * n + iy]; }, NoMid(),
         [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
   }
-  const C2* parts = K3part + (size_t)c * nparts * 2 * P;
+  constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
+  const double2* k3c = k3 + c * k3_stride;
   const C2* wf0 = wfine + (size_t)c * 2 * P;
   const C2* wf1 = wf0 + P;
   const T* K2 = K2acc + (size_t)c * P;
   const double tp = 2.0 * kPi;
   for (int i = threadIdx.x; i < P; i += blockDim.x) {
-    double k3ax = 0, k3ay = 0, k3bx = 0, k3by = 0;
-    for (int u = 0; u < nparts; ++u) {
-      const C2 x = parts[(size_t)u * 2 * P + i];
-      const C2 y = parts[(size_t)u * 2 * P + P + i];
-      k3ax += (double)x.x; k3ay += (double)x.y; k3bx += (double)y.x; k3by += (double)y.y;
-    }
+    const double2 k3a = k3c[i], k3b = k3c[P + i];
     const double w0 = wf0[i].x, w1 = wf0[i].y, w2 = wf1[i].x, w3 = wf1[i].y;
     const double D1 = slot[i].x, D2 = slot[i].y, D3 = slot[P + i].x;
     const double K40 = slot[2 * P + i].x, K41 = -(double)slot[2 * P + i].y;   // eta_b applied
     const double K42 = -(double)slot[3 * P + i].x, K43 = -(double)slot[3 * P + i].y;
-    const double K30 = k3ax, K31 = -k3ay, K32 = -k3bx, K33 = -k3by;
+    const double K30 = k3a.x, K31 = -k3a.y, K32 = -k3b.x, K33 = -k3b.y;
     const double k2 = K2[i];
     const double C0 = tp * (k2 * (1.0 - w0) - K30 + w0 * K40 + w1 * K41 + w2 * K42 + w3 * K43);
     const double C1 = -2.0 * (D2 * w3 - D3 * w2) + tp * (-k2 * w1 - K31 + w0 * K41 + K40 * w1);
@@ -916,14 +1012,20 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
   C2* H = slot + 2 * P;
   for (int p = 0; p < 2; ++p) {
     const C2* F = B0 + (size_t)p * P;
+    const C2* Hs = spec ? spec + c * spec_stride + (size_t)p * Q : nullptr;
     row_pass<n, -1, false, 0>(
         sm, tw, [&](int ix, int iy) { return F[ix * n + iy]; }, NoMid(),
         [&](int ix, int iy, C2 v) { H[ix * n + iy] = v; });
     col_pass<n, -1, true, 1>(
         sm, tw, [&](int ix, int iy) { return H[ix * n + iy]; },
         [&](int ix, int iy, C2 v) {
-          const bool keep = in_xi<n>(freq_of_pos<n>(ix)) && in_xi<n>(freq_of_pos<n>(iy));
-          return keep ? cscale(v, invP) : zero2<T>();
+          const int sx = xi_slot<n>(ix), sy = xi_slot<n>(iy);
+          if (sx < 0 || sy < 0) return zero2<T>();
+          if (Hs) {
+            const C2 h = Hs[sx * NQ + sy];
+            v = mk2(fmaT((T)tp, h.x, v.x), fmaT((T)tp, h.y, v.y));
+          }
+          return cscale(v, invP);
         },
         [&](int ix, int iy, C2 v) { H[ix * n + iy] = v; });
     row_pass<n, 1, false, 0>(
@@ -954,8 +1056,10 @@ size_t i3_staged_smem_bytes() {
 
 // Launch variants of the I3 kernel for padded size n and transform type T: the shapes the
 // autotuner chooses among (i3_default_variant gives the one a new handle starts with).
-//   FP64 (every size): the staged kernel as (threads, chunk bytes, blocks per SM)
-//     0: (256, 64 KB, 3)   1: (128, 32 KB, 6);  k_i3_sf 2: (256, 64 KB, 3)   3: (128, 32 KB, 6)
+//   FP64 (every size): the staged kernel, node by node, as (threads, chunk bytes, blocks per SM)
+//     0: (256, 64 KB, 3)   1: (128, 32 KB, 6);  k_i3_sf, nodes in pairs, 2: (256, 64 KB, 3)
+//     3: (128, 32 KB, 6).  Variant 0 also serves the allocation-free entry point, whose static array
+//     has no room for the pairs' Fourier-space partials at the sizes it accepts.
 //   FP32, n = 64, 96, 128: 0, 1, 2: the fused shared-memory kernel in the FusedShapes<n> shapes,
 //     3: k_i3_smem (1024 threads, element passes through shared memory)
 //   FP32, n <= 32: k_i3_smem;  FP32, n > 128: the cluster kernel, 0: 1024 threads per CTA with a
@@ -1089,9 +1193,10 @@ int i3_variant_count() {
 }
 
 // The variant a new handle starts with (the fastest measured on a GB300 for this size).  FP64, I3
-// launch in ms for variants 0..3 (J = M = 32): N = 16, 128 cells 136.8 136.2 132.9 129.4;
-// N = 32, 128 cells 652.2 640.5 625.3 630.4; N = 48, 64 cells 868.4 886.2 860.3 879.5; N = 64,
-// 32 cells 752.1 760.2 732.5 742.2; N = 128, 8 cells 897.0 902.9 885.5 901.9.
+// launch in ms for variants 0..3 (J = M = 32; 0 and 1 node by node, 2 and 3 in pairs): N = 16, 128
+// cells 135.5 135.1 76.9 77.1; N = 32, 128 cells 646.9 635.0 365.3 371.5; N = 48, 64 cells 861.7 879.5
+// 486.7 499.6; N = 64, 32 cells 746.4 755.8 423.6 433.1; N = 128, 8 cells 926.8 935.8 521.0 533.0 (the
+// fused line stages node by node: 132.9, 625.3, 860.3, 732.5, 885.5 for variant 2).
 // FP32 cluster kernel (I3 launch, J = M = 32): N = 128, 32 cells 219.1 ms (variant 0), 192.4 ms
 // (variant 1); N = 96, 64 cells 217.6 and 208.9 ms.
 template <int n, class T>
@@ -1123,6 +1228,12 @@ int i3_variant_concurrency(int v, int grid, int total) {
     if (g > gmax) g = gmax;
   }
   return g < 1 ? 1 : g;
+}
+
+// Variants that take the radial nodes in pairs (Fourier-space partials beside the real-space ones).
+template <int n, class T>
+bool i3_variant_paired(int v) {
+  return std::is_same<T, double>::value && v >= 2;
 }
 
 template <int n, class T>
@@ -1193,20 +1304,20 @@ I3Job<T> i3_job(const Tables& t, const CollisionWork& cw, int ncells, int unit_b
   jb.what = (const C2*)cw.what;
   jb.wfine = (const C2*)cw.wfine;
   jb.K3part = (C2*)cw.K3part;
+  jb.K3spec = (C2*)cw.K3spec;
   jb.psip_s = tb.psip_s;
   jb.phase = tb.phase;
   jb.J = t.J;
   jb.M = t.M;
   jb.nmc = cw.nmc;
-  jb.mch = cw.mch;
   jb.unit_begin = unit_begin;
   jb.nunits = ncells * t.J * cw.nmc;
   return jb;
 }
 
 // I3 over the units of njobs simulations (same n and precision, njobs <= kMaxI3Jobs); ws must hold
-// 3 (2N)^2 complex values for each of `grid` blocks (the cluster form uses one such slot per cluster
-// of kI3Cluster blocks).
+// i3_fields (2N)^2 complex values for each of `grid` blocks (the cluster form uses one such slot per
+// cluster of kI3Cluster blocks).
 template <int n, class T>
 cudaError_t i3_group_n(const Tables* const* tabs, const CollisionWork* const* cws, const int* ncells, int njobs,
                        void* ws, int grid, cudaStream_t s, long long& launches, int max_units) {
@@ -1226,6 +1337,11 @@ cudaError_t i3_group_n(const Tables* const* tabs, const CollisionWork* const* cw
   const TabPtrs<T> tb = tab_ptrs<T>(*tabs[0]);
   int v = cws[0]->i3_variant;
   if (v < 0 || v >= i3_nvariants<n, T>()) v = 0;
+  const bool paired = i3_variant_paired<n, T>(v);
+  for (int k = 0; k < njobs; ++k) {
+    if (paired && !cws[k]->K3spec) return cudaErrorInvalidValue;
+    cws[k]->i3_paired = paired;
+  }
   const I3Launch l = i3_variant<n, T>(v);
   int g = total < grid ? total : grid;
   if constexpr (std::is_same<T, float>::value && use_i3_cluster<n>()) {
@@ -1257,11 +1373,24 @@ cudaError_t collide_post_n(const Tables& t, CollisionWork& cw, double* c, int nc
   set_smem_attributes<n, T>();
   const TabPtrs<T> tb = tab_ptrs<T>(t);
   if (tm) tm->begin(KG_ASSEMBLE, s);
-  k_assemble<n, T><<<ncells, kThreads, smem_bytes<n, T>(), s>>>((C2*)cw.wfine, (C2*)cw.Dacc, (T*)cw.K2acc,
-                                                                (C2*)cw.K4acc, (C2*)cw.K3part, t.J * cw.nmc,
-                                                                (C2*)cw.ws, tb.tw, c);
+  constexpr int np = 2 * n * n;
+  constexpr int nq = 2 * xi_kept<n>() * xi_kept<n>();
+  const int nparts = t.J * cw.nmc, nqp = cw.i3_paired ? nq : 0;
+  C2* spec = cw.i3_paired ? (C2*)cw.K3spec : nullptr;
+  // from 16 units per cell on, eight threads per point: short columns of loads, more of them in flight
+  if (nparts >= 16) {
+    const int chunks = (np + nqp + 31) / 32;
+    k_reduce_k3<T, 8><<<(unsigned)chunks * ncells, 256, 0, s>>>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, chunks);
+  } else {
+    const int chunks = (np + nqp + 255) / 256;
+    k_reduce_k3<T, 1><<<(unsigned)chunks * ncells, 256, 0, s>>>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, chunks);
+  }
+  const double2* k3 = cw.K3sum ? cw.K3sum : (const double2*)cw.K3part;
+  k_assemble<n, T><<<ncells, kThreads, smem_bytes<n, T>(), s>>>(
+      (C2*)cw.wfine, (C2*)cw.Dacc, (T*)cw.K2acc, (C2*)cw.K4acc, k3, cw.K3sum ? (size_t)np : (size_t)nparts * np, spec,
+      (size_t)nparts * nq, (C2*)cw.ws, tb.tw, c);
   if (tm) tm->end(s);
-  ++launches;
+  launches += 2;
   return cudaGetLastError();
 }
 

@@ -9,6 +9,7 @@ template int i3_variant_count<128, float>();
 template int i3_default_variant<128, float>();
 template int i3_variant_concurrency<128, float>(int, int, int);
 template const char* i3_variant_name<128, float>(int);
+template bool i3_variant_paired<128, float>(int);
 template cudaError_t collide_vjp_n<128, float>(const Tables&, CollisionWork&, VjpWork&, const double*,
                                               const double* const*, double* const*, int, int, int, cudaStream_t,
                                               long long&, KernelTimer*);

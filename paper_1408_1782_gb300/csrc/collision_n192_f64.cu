@@ -9,6 +9,7 @@ template int i3_variant_count<192, double>();
 template int i3_default_variant<192, double>();
 template int i3_variant_concurrency<192, double>(int, int, int);
 template const char* i3_variant_name<192, double>(int);
+template bool i3_variant_paired<192, double>(int);
 template cudaError_t collide_vjp_n<192, double>(const Tables&, CollisionWork&, VjpWork&, const double*,
                                               const double* const*, double* const*, int, int, int, cudaStream_t,
                                               long long&, KernelTimer*);

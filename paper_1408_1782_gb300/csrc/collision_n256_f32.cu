@@ -9,6 +9,7 @@ template int i3_variant_count<256, float>();
 template int i3_default_variant<256, float>();
 template int i3_variant_concurrency<256, float>(int, int, int);
 template const char* i3_variant_name<256, float>(int);
+template bool i3_variant_paired<256, float>(int);
 template cudaError_t collide_vjp_n<256, float>(const Tables&, CollisionWork&, VjpWork&, const double*,
                                               const double* const*, double* const*, int, int, int, cudaStream_t,
                                               long long&, KernelTimer*);

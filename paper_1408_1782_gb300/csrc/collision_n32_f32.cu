@@ -9,6 +9,7 @@ template int i3_variant_count<32, float>();
 template int i3_default_variant<32, float>();
 template int i3_variant_concurrency<32, float>(int, int, int);
 template const char* i3_variant_name<32, float>(int);
+template bool i3_variant_paired<32, float>(int);
 template cudaError_t collide_vjp_n<32, float>(const Tables&, CollisionWork&, VjpWork&, const double*,
                                               const double* const*, double* const*, int, int, int, cudaStream_t,
                                               long long&, KernelTimer*);

@@ -9,6 +9,7 @@ template int i3_variant_count<96, float>();
 template int i3_default_variant<96, float>();
 template int i3_variant_concurrency<96, float>(int, int, int);
 template const char* i3_variant_name<96, float>(int);
+template bool i3_variant_paired<96, float>(int);
 template cudaError_t collide_vjp_n<96, float>(const Tables&, CollisionWork&, VjpWork&, const double*,
                                               const double* const*, double* const*, int, int, int, cudaStream_t,
                                               long long&, KernelTimer*);

@@ -354,27 +354,6 @@ __global__ void __launch_bounds__(kThreads) k_add_chunks(const T* __restrict__ n
   }
 }
 
-// The Fourier-space partials of the I3 transpose are kept only on the frequencies the final
-// projection keeps (in_xi in both coordinates, n/2 - 1 per coordinate): slot[pos] is the compact
-// index of permuted position pos, or -1.  Every kernel that reads or writes the compact partials
-// builds the table with this same ascending loop.
-template <int n>
-__host__ __device__ constexpr int xi_kept() {
-  return n / 2 - 1;
-}
-template <int n>
-__device__ __forceinline__ void build_xi_slots(int* slot, int* kept_pos) {
-  if (threadIdx.x == 0) {
-    int cnt = 0;
-    for (int pos = 0; pos < n; ++pos) {
-      const bool keep = in_xi<n>(freq_of_pos<n>(pos));
-      slot[pos] = keep ? cnt : -1;
-      if (keep) kept_pos[cnt++] = pos;
-    }
-  }
-  __syncthreads();
-}
-
 // dst = Psi'_j(x) for the field x(i) = ld(i), i = ix * n + iy: row FFT, column convolution with the
 // angle's psi' table, row IFFT (the forward's convolution); G is the staging field.
 template <int n, class C2, class T, class LD>

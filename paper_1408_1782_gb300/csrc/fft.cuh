@@ -234,40 +234,41 @@ __device__ __forceinline__ void dft_scaled(C2 (&a)[R], const typename RealOf<C2>
   for (int i = 0; i < R; ++i) a[i] = b[i];
 }
 
-// DFT of length 16 whose inputs a[4..11] are zero -- a stage-B line of the 128-point padded grid
-// holding only band-limited (Xi) frequencies -- with the first radix-2 stage reduced to copies: its
-// butterflies pair a[r] with a[r + 8], r < 8, and one of the two is zero.
-template <int SIGN, class C2>
-__device__ __forceinline__ void dft16_xi(C2 (&a)[16]) {
-  C2 b[16];
+// Band-limited (Xi) frequencies |k| < n/4 of a line of n = A B points: in the permuted order
+// pos = B k1 + t of frequency k1 + A t they are the t below B / 4 and from 3 B / 4 on, for every k1.
+template <int B>
+__host__ __device__ constexpr bool xi_t(int t) {
+  return t < B / 4 || t >= 3 * B / 4;
+}
+
+// DFT of a stage-B line (length R = B >= 4) whose inputs vanish outside Xi, with the first radix-2
+// stage reduced to copies: its butterflies pair a[r] with a[r + R / 2], and one of the two is zero.
+template <int R, int SIGN, class C2>
+__device__ __forceinline__ void dft_xi(C2 (&a)[R]) {
+  static_assert((R & (R - 1)) == 0 && R >= 4, "power-of-two length");
+  constexpr int L2 = ilog2c(R);
+  C2 b[R];
 #pragma unroll
-  for (int g = 0; g < 16; g += 2) {
-    const int r = bitrev(g, 4);   // 0..7; bitrev(g + 1, 4) = r + 8
-    if (r < 4) {
+  for (int g = 0; g < R; g += 2) {
+    const int r = bitrev(g, L2);   // 0 .. R/2 - 1; bitrev(g + 1) = r + R / 2
+    if (r < R / 4) {
       b[g] = a[r];
       b[g + 1] = a[r];
     } else {
-      b[g] = a[r + 8];
-      b[g + 1] = mk2(-a[r + 8].x, -a[r + 8].y);
+      b[g] = a[r + R / 2];
+      b[g + 1] = mk2(-a[r + R / 2].x, -a[r + R / 2].y);
     }
   }
-  DftStage<16, SIGN, 4, C2>::run(b);
+  DftStage<R, SIGN, 4, C2>::run(b);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) a[i] = b[i];
-}
-
-// Padded grids whose stage-B lines (B = 16) hold the band-limited frequencies |k| < n/4 (Xi) at
-// t = 0..3, 12..15 only: n = A B with n / 4 = 4 A.
-template <int n>
-__host__ __device__ constexpr bool xi_prunable() {
-  return Split<n>::B == 16;
+  for (int i = 0; i < R; ++i) a[i] = b[i];
 }
 
 // FFT of nl lines of length n held in shared (or global) memory:
 // element e of line l at buf[l*ls + e*es].  tw[t2*A + k1] = exp(-2 pi i t2 k1 / n).
 // SIGN < 0: forward, natural -> permuted.  SIGN > 0: inverse, permuted -> natural.
-// XI (inverse only): the input is zero outside Xi, so where xi_prunable<n>() the first stage reads
-// the Xi values of each line only and runs dft16_xi.
+// XI (inverse only): the input is zero outside Xi, so the first stage reads the Xi values of each
+// line only and runs dft_xi.
 // Must be called by every thread of the block; ends with __syncthreads().
 template <int n, int SIGN, bool XI = false, class C2>
 __device__ __forceinline__ void fft_lines(C2* buf, int nl, int ls, int es, const C2* __restrict__ tw) {
@@ -303,10 +304,11 @@ __device__ __forceinline__ void fft_lines(C2* buf, int nl, int ls, int es, const
       const int l = task % nl, k1 = task / nl;
       C2* base = buf + l * ls + B * k1 * es;
       C2 b[B];
-      if constexpr (XI && xi_prunable<n>()) {
+      if constexpr (XI) {
 #pragma unroll
-        for (int k2 = 0; k2 < B; ++k2) b[k2] = (k2 < 4 || k2 >= 12) ? base[k2 * es] : mk2((typename RealOf<C2>::type)0, (typename RealOf<C2>::type)0);
-        dft16_xi<1>(b);
+        for (int k2 = 0; k2 < B; ++k2)
+          b[k2] = xi_t<B>(k2) ? base[k2 * es] : mk2((typename RealOf<C2>::type)0, (typename RealOf<C2>::type)0);
+        dft_xi<B, 1>(b);
       } else {
 #pragma unroll
         for (int k2 = 0; k2 < B; ++k2) b[k2] = base[k2 * es];

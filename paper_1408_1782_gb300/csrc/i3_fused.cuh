@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(NT, MINB) k_i3_fused(const I3Jobs<float> jobs,
   for (int gunit = blockIdx.x; gunit < jobs.total; gunit += gridDim.x) {
     const I3Job<float>& jb = jobs.job[i3_job_of(jobs, gunit)];
     const int unit = gunit - jb.unit_begin;
-    const int J = jb.J, M = jb.M, nmc = jb.nmc, mch = jb.mch;
+    const int J = jb.J, M = jb.M, nmc = jb.nmc;
     const C2* what = jb.what;
     const C2* __restrict__ phase = jb.phase;
     const int c = unit / (J * nmc);
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(NT, MINB) k_i3_fused(const I3Jobs<float> jobs,
       __syncthreads();
     }
     const C2* wf = jb.wfine + (size_t)c * 2 * P;
-    const int m0 = mc * mch, m1 = min(M, m0 + mch);
+    const int m0 = i3_chunk_begin(mc, nmc, M), m1 = i3_chunk_begin(mc + 1, nmc, M);
     for (int m = m0; m < m1; ++m) {
       const C2* px = phase + ((size_t)j * M + m) * 2 * n;
       const C2* py = px + n;
@@ -374,7 +374,7 @@ __device__ __forceinline__ void wl_shift(float2* G, const float2* tw, const floa
         b[t] = zero2<float>();
       }
     }
-    dft16_xi<1>(b);
+    dft_xi<B, 1>(b);
 #pragma unroll
     for (int t = 0; t < B; ++t) G[wl_addr(x, B * k1 + t)] = b[t];
   }
@@ -400,7 +400,7 @@ __device__ __forceinline__ void wl_shift(float2* G, const float2* tw, const floa
     C2 b[B];
 #pragma unroll
     for (int t = 0; t < B; ++t) b[t] = (t < 4 || t >= 12) ? G[wl_addr(B * k1 + t, y)] : zero2<float>();
-    dft16_xi<1>(b);
+    dft_xi<B, 1>(b);
 #pragma unroll
     for (int t = 0; t < B; ++t) G[wl_addr(B * k1 + t, y)] = b[t];
   }
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(kWlThreads, 1) k_i3_wl(const I3Jobs<float> job
   for (int gunit = blockIdx.x; gunit < jobs.total; gunit += gridDim.x) {
     const I3Job<float>& jb = jobs.job[i3_job_of(jobs, gunit)];
     const int unit = gunit - jb.unit_begin;
-    const int J = jb.J, M = jb.M, nmc = jb.nmc, mch = jb.mch;
+    const int J = jb.J, M = jb.M, nmc = jb.nmc;
     const C2* what = jb.what;
     const C2* __restrict__ phase = jb.phase;
     const int c = unit / (J * nmc);
@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(kWlThreads, 1) k_i3_wl(const I3Jobs<float> job
       __syncthreads();
     }
     const C2* wf = jb.wfine + (size_t)c * 2 * P;
-    const int m0 = mc * mch, m1 = min(M, m0 + mch);
+    const int m0 = i3_chunk_begin(mc, nmc, M), m1 = i3_chunk_begin(mc + 1, nmc, M);
     for (int m = m0; m < m1; ++m) {
       const C2* px = phase + ((size_t)j * M + m) * 2 * n;
       const C2* py = px + n;

@@ -1,17 +1,33 @@
 // I3 (Hu-Ying term, eq. approxH-JM) for fields larger than one block's shared memory (the FP64 form):
-// staged row and column passes over chunks of RC rows / CC lines, with every global load and store
-// of a convolution fused into a line stage.  Included by collision_kernels.cuh inside its anonymous
-// namespace.
+// the radial nodes taken in pairs +-rho_m, staged row and line passes with every global load and
+// store fused into a line stage.  Included by collision_kernels.cuh inside its anonymous namespace.
+//
+// Node pairs.  With S the shift by node m (rho_m < 0) and S* = S^-1 that of its partner M-1-m (the
+// Gauss-Legendre nodes are symmetric, with equal weights), write s_a = S w_a.  Translations commute
+// with Psi'_j and with products, so
+//   sum_a eta_a S*w_a Psi'(w_a S*w_b) = S*[ sum_a eta_a w_a Psi'(s_a w_b) ]
+// and both nodes of the pair use the same sixteen real convolutions U_ab = Psi'(w_a s_b):
+//   node m:      K3_b += sum_a eta_a s_a U_ab          (real space)
+//   node M-1-m:  K3_a += S*[ sum_b eta_b w_b U_ab ]    (Fourier space, on the kept frequencies)
+// The product of three Xi-limited fields aliases only outside Xi on the padded grid and Xi is all that
+// the final projection keeps, so the regrouping is exact up to rounding.  Per pair: 2 shifts, 8 complex
+// convolutions, 2 transforms back, against 4 shifts and 16 convolutions node by node.  The middle node
+// of an odd M (rho = 0) has no partner.
+//
+// What bounds it: FP64 issue (two lanes per clock and SM); the scratch traffic through L2 is nearly
+// free beside it.  I3 launch, J = M = 32, on a GB300, node by node -> in pairs: see i3_default_variant.
 //
 // The block's scratch field between the passes is stored transposed, G'[ky][x] (ky in the row
 // transform's permuted order), so that each pass reads and writes it with coalesced accesses
 // straight from its line stages:
-//   row pass, forward:  stage A loads w_a Sigma_p (tasks (row, t2), t2-fastest), stage B stores its
+//   row pass, forward:  stage A loads the product (tasks (row, t2), t2-fastest), stage B stores its
 //                       B spectral values of a row into B lines of G' (lanes = consecutive rows);
 //   line pass (x):      stage A loads a line of G' (contiguous in x), stage B with the psi'_j
 //                       multiplier between forward and inverse, stage A stores the line back;
 //   row pass, inverse:  stage B loads B lines of G' at its row (lanes = consecutive rows), stage A
-//                       multiplies by eta_a S_a and accumulates into the unit's partial sum.
+//                       hands its results to the accumulations.
+// The shifts run the lines and then the rows, the transforms back the rows and then the lines, both
+// with the n / 2 lines of Xi only and with the Xi values only of each spectral stage (xi_t).
 // Shared memory holds one chunk at a time; no pass copies a chunk through it without transforming.
 #pragma once
 
@@ -21,95 +37,146 @@ __global__ void __launch_bounds__(NTH, MINB)
   using C2 = typename Vec2Of<T>::type;
   constexpr int A = Split<n>::A, B = Split<n>::B, P = n * n;
   constexpr int RC = Chunk<n, sizeof(C2), CB>::RC, CC = Chunk<n, sizeof(C2), CB>::CC, LS = Chunk<n, sizeof(C2), CB>::LS;
+  constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C2* tw = reinterpret_cast<C2*>(smem_raw);   // tw[t2 A + k1]
-  C2* twT = tw + n;                           // twT[k1 B + t2] = tw[t2 A + k1] (t2-fastest lanes)
+  C2* twT = reinterpret_cast<C2*>(smem_raw);  // twT[k1 B + t2] = exp(-2 pi i t2 k1 / n) (t2-fastest lanes)
   C2* sm = twT + n;                           // one chunk: [RC][LS] rows, or [CC][LS] lines of G'
   static_assert(RC == CC, "row and line chunks share the buffer");
-  __shared__ int xcols[n];
-  __shared__ unsigned char xmask[n];
-  if (threadIdx.x == 0) {
-    int cnt = 0;
-    for (int pos = 0; pos < n; ++pos) {
-      const int k = freq_of_pos<n>(pos);
-      const bool in = (k < n / 4) || (k >= n - n / 4);
-      xmask[pos] = in ? 1 : 0;
-      if (in) xcols[cnt++] = pos;
-    }
-  }
+  __shared__ int kslot[n];
   for (int pos = threadIdx.x; pos < n; pos += NTH) twT[(pos % A) * B + pos / A] = gtw[pos];
-  load_twiddles<n>(tw, gtw);
+  build_xi_slots<n>(kslot);
   const int tid = threadIdx.x;
-  C2* slot = ws + (size_t)blockIdx.x * 3 * P;
-  C2* Sig = slot;           // [2][P]
+  C2* slot = ws + (size_t)blockIdx.x * 4 * P;
+  C2* Sig = slot;           // [2][P] shifted pairs s_0 + i s_1, s_2 + i s_3
   C2* G = slot + 2 * P;     // G'[ky][x] between the passes
+  C2* V = slot + 3 * P;     // sum_b eta_b w_b U_ab of the current pair of a
+
+  // rows of load(idx), idx = row * n + y, into lines of G' (XI: into the Xi lines only)
+  auto rows_forward = [&](auto xi, auto load) {
+    for (int r0 = 0; r0 < n; r0 += RC) {
+      for (int task = tid; task < RC * B; task += NTH) {
+        const int r = task / B, t2 = task % B;
+        C2 v[A];
+#pragma unroll
+        for (int t1 = 0; t1 < A; ++t1) v[t1] = load((r0 + r) * n + B * t1 + t2);
+        dft<A, -1>(v);
+#pragma unroll
+        for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) sm[r * LS + B * k1 + t2] = v[k1];
+      }
+      __syncthreads();
+      for (int task = tid; task < RC * A; task += NTH) {
+        const int r = task % RC, k1 = task / RC;
+        const C2* base = sm + r * LS + B * k1;
+        C2 b[B];
+#pragma unroll
+        for (int t = 0; t < B; ++t) b[t] = base[t];
+        dft<B, -1>(b);
+#pragma unroll
+        for (int t = 0; t < B; ++t)
+          if (!decltype(xi)::value || xi_t<B>(t)) G[(B * k1 + t) * n + r0 + r] = b[t];
+      }
+      __syncthreads();
+    }
+  };
+  // rows of G' back to real space, handed to epi(idx, v) (XI: only the Xi lines are non-zero)
+  auto rows_inverse = [&](auto xi, auto epi) {
+    for (int r0 = 0; r0 < n; r0 += RC) {
+      for (int task = tid; task < RC * A; task += NTH) {
+        const int r = task % RC, k1 = task / RC;
+        C2* base = sm + r * LS + B * k1;
+        C2 b[B];
+#pragma unroll
+        for (int t = 0; t < B; ++t)
+          b[t] = (!decltype(xi)::value || xi_t<B>(t)) ? G[(B * k1 + t) * n + r0 + r] : zero2<T>();
+        if constexpr (decltype(xi)::value) dft_xi<B, 1>(b);
+        else dft<B, 1>(b);
+#pragma unroll
+        for (int t = 0; t < B; ++t) base[t] = b[t];
+      }
+      __syncthreads();
+      for (int task = tid; task < RC * B; task += NTH) {
+        const int r = task / B, t2 = task % B;
+        C2 v[A];
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) v[k1] = sm[r * LS + B * k1 + t2];
+#pragma unroll
+        for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2]);
+        dft<A, 1>(v);
+#pragma unroll
+        for (int t1 = 0; t1 < A; ++t1) epi((r0 + r) * n + B * t1 + t2, v[t1]);
+      }
+      __syncthreads();
+    }
+  };
+  // the li-th of the n / 2 lines ky of Xi: its permuted position
+  auto xi_line = [&](int li) {
+    const int k1 = li / (B / 2), t = li % (B / 2);
+    return B * k1 + (t < B / 4 ? t : t + B / 2);
+  };
+
   for (int gunit = blockIdx.x; gunit < jobs.total; gunit += gridDim.x) {
     const I3Job<T>& jb = jobs.job[i3_job_of(jobs, gunit)];
     const int unit = gunit - jb.unit_begin;
-    const int J = jb.J, M = jb.M, nmc = jb.nmc, mch = jb.mch;
+    const int J = jb.J, M = jb.M, nmc = jb.nmc;
     const C2* what = jb.what;
     const C2* __restrict__ phase = jb.phase;
     const int c = unit / (J * nmc);
     const int j = (unit / nmc) % J;
     const int mc = unit % nmc;
     C2* acc = jb.K3part + (size_t)unit * 2 * P;
-    zero_fields(acc, 2 * P);
+    C2* spec = jb.K3spec + (size_t)unit * 2 * Q;
     const T* __restrict__ psp = jb.psip_s + (size_t)j * P;
     const C2* wf = jb.wfine + (size_t)c * 2 * P;
-    const int m0 = mc * mch, m1 = min(M, m0 + mch);
-    for (int m = m0; m < m1; ++m) {
-      const C2* px = phase + ((size_t)j * M + m) * 2 * n;
+    const int it1 = i3_chunk_begin(mc + 1, nmc, M);
+    bool k_first = true, s_first[2] = {true, true};
+    for (int it = i3_chunk_begin(mc, nmc, M); it < it1;) {
+      const I3Group gr = i3_group_at(it, it1, M);
+      it = gr.next;
+      const C2* px = phase + ((size_t)j * M + gr.m) * 2 * n;
       const C2* py = px + n;
-      // shifted pairs, as in k_i3 (only the Xi columns are transformed along x)
+      // shifted pairs: the Xi lines along x, then the rows
       for (int p = 0; p < 2; ++p) {
         const C2* in = what + ((size_t)c * 4 + p) * P;
-        C2* S = Sig + (size_t)p * P;
-        col_pass_list<n, 1, false, 0, CB, true>(
-            sm, tw, xcols, n / 2,
-            [&](int ix, int iy) { return xmask[ix] ? cmul(in[ix * n + iy], cmul(px[ix], py[iy])) : zero2<T>(); },
-            NoMid(), [&](int ix, int iy, C2 v) { S[ix * n + iy] = v; });
-        row_pass<n, 1, false, 0, CB, true>(
-            sm, tw, [&](int ix, int iy) { return xmask[iy] ? S[ix * n + iy] : zero2<T>(); }, NoMid(),
-            [&](int ix, int iy, C2 v) { S[ix * n + iy] = v; });
-      }
-      for (int a = 0; a < 4; ++a) {
-        const C2* wa = wf + (size_t)(a >> 1) * P;
-        const C2* Sa = Sig + (size_t)(a >> 1) * P;
-        const bool im = (a & 1) != 0;
-        const bool pos_eta = (a == 0);   // eta_a = +1 for a = 0, -1 otherwise
-        for (int p = 0; p < 2; ++p) {
-          const C2* Sp = Sig + (size_t)p * P;
-          C2* accp = acc + (size_t)p * P;
-          // ---- row pass, forward: rows r0..r0+RC into lines of G' ----
-          for (int r0 = 0; r0 < n; r0 += RC) {
-            for (int task = tid; task < RC * B; task += NTH) {
-              const int r = task / B, t2 = task % B, row = r0 + r;
-              C2 v[A];
+        for (int c0 = 0; c0 < n / 2; c0 += CC) {
+          const int nl = (n / 2 - c0) < CC ? (n / 2 - c0) : CC;
+          for (int task = tid; task < nl * A; task += NTH) {
+            const int cc = task % nl, k1 = task / nl, ky = xi_line(c0 + cc);
+            const C2 pyy = py[ky];
+            C2* base = sm + cc * LS + B * k1;
+            C2 b[B];
 #pragma unroll
-              for (int t1 = 0; t1 < A; ++t1) {
-                const int idx = row * n + B * t1 + t2;
-                const C2 z = wa[idx];
-                v[t1] = cscale(Sp[idx], im ? z.y : z.x);
-              }
-              dft<A, -1>(v);
+            for (int t = 0; t < B; ++t)
+              b[t] = xi_t<B>(t) ? cmul(in[(B * k1 + t) * n + ky], cmul(px[B * k1 + t], pyy)) : zero2<T>();
+            dft_xi<B, 1>(b);
 #pragma unroll
-              for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
-#pragma unroll
-              for (int k1 = 0; k1 < A; ++k1) sm[r * LS + B * k1 + t2] = v[k1];
-            }
-            __syncthreads();
-            for (int task = tid; task < RC * A; task += NTH) {
-              const int r = task % RC, k1 = task / RC;
-              const C2* base = sm + r * LS + B * k1;
-              C2 b[B];
-#pragma unroll
-              for (int t = 0; t < B; ++t) b[t] = base[t];
-              dft<B, -1>(b);
-#pragma unroll
-              for (int t = 0; t < B; ++t) G[(B * k1 + t) * n + r0 + r] = b[t];
-            }
-            __syncthreads();
+            for (int t = 0; t < B; ++t) base[t] = b[t];
           }
+          __syncthreads();
+          for (int task = tid; task < nl * B; task += NTH) {
+            const int cc = task / B, t2 = task % B, ky = xi_line(c0 + cc);
+            C2 v[A];
+#pragma unroll
+            for (int k1 = 0; k1 < A; ++k1) v[k1] = sm[cc * LS + B * k1 + t2];
+#pragma unroll
+            for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2]);
+            dft<A, 1>(v);
+#pragma unroll
+            for (int t1 = 0; t1 < A; ++t1) G[ky * n + B * t1 + t2] = v[t1];
+          }
+          __syncthreads();
+        }
+        C2* S = Sig + (size_t)p * P;
+        rows_inverse(std::true_type{}, [&](int idx, C2 v) { S[idx] = v; });
+      }
+      for (int q = gr.q0; q < gr.q1; ++q) {
+        const C2* wq = wf + (size_t)q * P;
+        const C2* Sq = Sig + (size_t)q * P;
+        for (int b = 0; b < 4; ++b) {
+          // U_{2q,b} + i U_{2q+1,b} = Psi'((w_2q + i w_2q+1) s_b)
+          const T* Sb = reinterpret_cast<const T*>(Sig + (size_t)(b >> 1) * P) + (b & 1);
+          rows_forward(std::false_type{}, [&](int idx) { return cscale(wq[idx], Sb[2 * idx]); });
           // ---- line pass along x: forward, psi'_j, inverse on lines c0..c0+CC of G' ----
           for (int c0 = 0; c0 < n; c0 += CC) {
             for (int task = tid; task < CC * B; task += NTH) {
@@ -127,16 +194,16 @@ __global__ void __launch_bounds__(NTH, MINB)
             for (int task = tid; task < CC * A; task += NTH) {
               const int cc = task % CC, k1 = task / CC;
               C2* base = sm + cc * LS + B * k1;
-              C2 b[B];
+              C2 z[B];
 #pragma unroll
-              for (int t = 0; t < B; ++t) b[t] = base[t];
-              dft<B, -1>(b);
+              for (int t = 0; t < B; ++t) z[t] = base[t];
+              dft<B, -1>(z);
               T sc[B];
 #pragma unroll
               for (int t = 0; t < B; ++t) sc[t] = psp[(B * k1 + t) * n + c0 + cc];
-              dft_scaled<B, 1>(b, sc);
+              dft_scaled<B, 1>(z, sc);
 #pragma unroll
-              for (int t = 0; t < B; ++t) base[t] = b[t];
+              for (int t = 0; t < B; ++t) base[t] = z[t];
             }
             __syncthreads();
             for (int task = tid; task < CC * B; task += NTH) {
@@ -152,47 +219,78 @@ __global__ void __launch_bounds__(NTH, MINB)
             }
             __syncthreads();
           }
-          // ---- row pass, inverse, accumulated with eta_a S_a ----
-          for (int r0 = 0; r0 < n; r0 += RC) {
-            for (int task = tid; task < RC * A; task += NTH) {
-              const int r = task % RC, k1 = task / RC;
-              C2* base = sm + r * LS + B * k1;
-              C2 b[B];
-#pragma unroll
-              for (int t = 0; t < B; ++t) b[t] = G[(B * k1 + t) * n + r0 + r];
-              dft<B, 1>(b);
-#pragma unroll
-              for (int t = 0; t < B; ++t) base[t] = b[t];
-            }
-            __syncthreads();
-            for (int task = tid; task < RC * B; task += NTH) {
-              const int r = task / B, t2 = task % B, row = r0 + r;
-              C2 v[A];
-#pragma unroll
-              for (int k1 = 0; k1 < A; ++k1) v[k1] = sm[r * LS + B * k1 + t2];
-#pragma unroll
-              for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2]);
-              dft<A, 1>(v);
-#pragma unroll
-              for (int t1 = 0; t1 < A; ++t1) {
-                const int idx = row * n + B * t1 + t2;
-                const C2 s = Sa[idx];
-                const T f = im ? s.y : s.x;
-                const C2 d = accp[idx];
-                accp[idx] = pos_eta ? mk2(fmaT(f, v[t1].x, d.x), fmaT(f, v[t1].y, d.y))
-                                    : mk2(fmaT(-f, v[t1].x, d.x), fmaT(-f, v[t1].y, d.y));
+          // ---- K3_b += eta_2q s_2q Re U + eta_2q+1 s_2q+1 Im U;  V_q += eta_b w_b U (x part of q = 0
+          // with the sign that C_0 has against C_1..C_3, see k_assemble) ----
+          T* Kb = reinterpret_cast<T*>(acc + (size_t)(b >> 1) * P) + (b & 1);
+          const T* wb = reinterpret_cast<const T*>(wf + (size_t)(b >> 1) * P) + (b & 1);
+          const T e0 = q == 0 ? (T)1 : (T)-1, eb = b == 0 ? (T)1 : (T)-1;
+          rows_inverse(std::false_type{}, [&](int idx, C2 v) {
+            const C2 s = Sq[idx];
+            const T k = fmaT(e0 * s.x, v.x, -s.y * v.y);
+            Kb[2 * idx] = k_first ? k : Kb[2 * idx] + k;
+            if (gr.pair) {
+              const T f = eb * wb[2 * idx], fx = -e0 * f;
+              if (b == 0) {
+                V[idx] = mk2(fx * v.x, f * v.y);
+              } else {
+                const C2 d = V[idx];
+                V[idx] = mk2(fmaT(fx, v.x, d.x), fmaT(f, v.y, d.y));
               }
             }
-            __syncthreads();
+          });
+        }
+        k_first = false;
+        if (!gr.pair) continue;
+        // ---- shifted back: rows, then the Xi lines along x, times the conjugate phase ----
+        rows_forward(std::true_type{}, [&](int idx) { return V[idx]; });
+        C2* sq = spec + (size_t)q * Q;
+        const bool first = s_first[q];
+        s_first[q] = false;
+        for (int c0 = 0; c0 < n / 2; c0 += CC) {
+          const int nl = (n / 2 - c0) < CC ? (n / 2 - c0) : CC;
+          for (int task = tid; task < nl * B; task += NTH) {
+            const int cc = task / B, t2 = task % B, ky = xi_line(c0 + cc);
+            C2 v[A];
+#pragma unroll
+            for (int t1 = 0; t1 < A; ++t1) v[t1] = G[ky * n + B * t1 + t2];
+            dft<A, -1>(v);
+#pragma unroll
+            for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
+#pragma unroll
+            for (int k1 = 0; k1 < A; ++k1) sm[cc * LS + B * k1 + t2] = v[k1];
           }
+          __syncthreads();
+          for (int task = tid; task < nl * A; task += NTH) {
+            const int cc = task % nl, k1 = task / nl, ky = xi_line(c0 + cc), sy = kslot[ky];
+            const C2* base = sm + cc * LS + B * k1;
+            C2 b[B];
+#pragma unroll
+            for (int t = 0; t < B; ++t) b[t] = base[t];
+            dft<B, -1>(b);
+            if (sy < 0) continue;
+            const C2 pyy = py[ky];
+#pragma unroll
+            for (int t = 0; t < B; ++t)
+              if (xi_t<B>(t)) {
+                const int sx = kslot[B * k1 + t];
+                if (sx >= 0) {
+                  const C2 z = cmulc(b[t], cmul(px[B * k1 + t], pyy));
+                  C2* o = sq + sx * NQ + sy;
+                  *o = first ? z : cadd(*o, z);
+                }
+              }
+          }
+          __syncthreads();
         }
       }
     }
+    for (int q = 0; q < 2; ++q)
+      if (s_first[q]) zero_fields(spec + (size_t)q * Q, Q);
   }
 }
 
 template <int n, class T, int CB>
-constexpr size_t i3_sf_smem_bytes() {   // twiddles (two orders) and one chunk of RC padded lines
+constexpr size_t i3_sf_smem_bytes() {   // twiddles and one chunk of RC padded lines
   using C2 = typename Vec2Of<T>::type;
-  return (size_t)(2 * n + Chunk<n, sizeof(C2), CB>::RC * Chunk<n, sizeof(C2), CB>::LS) * sizeof(C2);
+  return (size_t)(n + Chunk<n, sizeof(C2), CB>::RC * Chunk<n, sizeof(C2), CB>::LS) * sizeof(C2);
 }

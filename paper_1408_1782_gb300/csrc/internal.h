@@ -49,6 +49,18 @@ template <> inline TabPtrs<float> tab_ptrs<float>(const Tables& t) {
   return {t.tw_f, t.phip_f, t.Ktab_f, t.psi_f, t.psip_s_f, t.phase_f};
 }
 
+// The radial nodes of a (cell, angle) are split into nmc chunks.  They are counted in M items: items
+// 2 m and 2 m + 1 are the two halves (pairs of the first index of U_ab) of the node pair {m, M - 1 - m},
+// and with an odd M the last item is the middle node.  Chunk mc covers the items
+// [i3_chunk_begin(mc), i3_chunk_begin(mc + 1)): whole pairs while there are no more chunks than pairs
+// (a split pair computes its shifts twice).  Kernels that take node by node read an item as a node.
+__host__ __device__ inline int i3_chunk_begin(int mc, int nmc, int M) {
+  const int np = (M + 1) / 2;
+  if (nmc > np) return mc * M / nmc;
+  const int i = 2 * (mc * np / nmc);
+  return i < M ? i : M;
+}
+
 // One simulation's share of an I3 launch: the Hu-Ying kernels run a work queue over
 // the (cell, j, m-chunk) units of up to kMaxI3Jobs simulations of the same padded size
 // (passed by value as a kernel parameter).
@@ -58,9 +70,10 @@ struct I3Job {
   const typename std::conditional<sizeof(T) == 8, double2, float2>::type* what;
   const typename std::conditional<sizeof(T) == 8, double2, float2>::type* wfine;
   typename std::conditional<sizeof(T) == 8, double2, float2>::type* K3part;
+  typename std::conditional<sizeof(T) == 8, double2, float2>::type* K3spec;
   const T* psip_s;
   const typename std::conditional<sizeof(T) == 8, double2, float2>::type* phase;
-  int J, M, nmc, mch;
+  int J, M, nmc;
   int unit_begin;   // first global unit of this simulation
   int nunits;
 };
@@ -76,7 +89,7 @@ struct CollisionWork {
   int prec = 0;        // 0: FP64 transforms, 1: FP32 transforms (FP32-split form)
   int nb = 0;          // cells per batch
   int nmc = 1;         // m-chunks per (cell, j) unit of the I3 kernel
-  int mch = 1;         // m values per chunk
+  int mch = 1;         // m values per chunk (the largest)
   int grid_i3 = 0;     // persistent grid of the I3 kernel
   int grid_max = 0;    // its occupancy limit (SMs x resident blocks, the largest over the variants)
   int i3_variant = 0;  // launch variant of the I3 kernel (i3_variants)
@@ -92,8 +105,16 @@ struct CollisionWork {
   void* K2part = nullptr;
   void* K4part = nullptr;
   void* K3part = nullptr;    // [nb*J*nmc][2][n*n] fine-grid K3 pair partial sums
+  // Fourier-space partial sums of the kernels that take the nodes in pairs, kept frequencies only
+  // [nb*J*nmc][2][(n/2-1)^2]; null: the workspace serves the node-by-node kernels only
+  void* K3spec = nullptr;
+  double2* K3sum = nullptr;  // [nb][2][n*n] reduced K3 pairs (FP32 form; FP64 reduces in place)
+  // whether the last I3 launch over this workspace took the nodes in pairs (its post-processing
+  // then adds K3spec); a batch launches its first member's variant for the whole group
+  mutable bool i3_paired = false;
   void* ws = nullptr;        // per-CTA scratch
-  size_t ws_fields = 0;      // complex n*n fields of scratch per CTA slot
+  size_t ws_fields = 0;      // complex n*n fields of scratch
+  int i3_fields = 3;         // of which an I3 block (or cluster) uses this many
   int ws_slots = 0;          // number of CTA slots in ws
   double* cbuf = nullptr;    // [nb][4][N][N] staging for collide in/out
   double* wbuf = nullptr;
@@ -213,6 +234,8 @@ template <int n, class T>
 int i3_variant_concurrency(int variant, int grid, int total);
 template <int n, class T>
 const char* i3_variant_name(int variant);
+template <int n, class T>
+bool i3_variant_paired(int variant);
 // Launch variants of the I3 kernel ("tile shapes" the autotuner chooses among) for a grid and
 // precision: their number, resident blocks per SM, and a description.
 int i3_variants(int n, int prec);
@@ -220,6 +243,10 @@ int i3_default(int n, int prec);
 int i3_variant_bps(int n, int prec, int variant);
 int i3_concurrency(int n, int prec, int variant, int grid, int total);
 const char* i3_variant_desc(int n, int prec, int variant);
+bool i3_paired(int n, int prec, int variant);
+// Relative time of the items [begin, end) of a chunk (i3_chunk_begin) in a kernel that takes the nodes
+// in pairs or node by node: the 2-D transforms it runs.
+double i3_chunk_cost(int begin, int end, int M, bool paired);
 // The collision operator in parts (collision_kernels.cuh): the per-cell terms before I3, the I3
 // work queue over one or several simulations of the same padded size, the per-cell assembly.
 cudaError_t collide_pre(const Tables& t, CollisionWork& cw, const double* w, int ncells, cudaStream_t s,

@@ -380,7 +380,7 @@ int qbe_set_i3_shape(qbe_handle* h, int variant, int grid, int m_chunks) {
   if (m_chunks > cap_nmc) return fail(h, QBE_ERR_ARG, "set_i3_shape: more m-chunks than the partial sums hold");
   if (variant >= 0) h->cw.i3_variant = variant;
   if (grid > 0) {
-    const int cap = (int)(h->cw.ws_fields / 3);
+    const int cap = (int)(h->cw.ws_fields / h->cw.i3_fields);
     h->cw.grid_i3 = grid < cap ? grid : cap;
   }
   if (m_chunks > 0) {
@@ -903,9 +903,9 @@ namespace {
 // m-chunking, two waves of the group's work queue are timed on the simulations' current state
 // (the per-cell terms are computed first, so the I3 inputs are those of the state).  The launch
 // assigns unit u to block (cluster) u mod G, so its time is that of the busiest block: the sample's
-// time divided by its busiest block's m-evaluations gives the cost of one m, and the candidate's
-// time is that cost times the busiest block's m-evaluations over the whole queue (units of
-// different members carry different numbers of m).  The fastest shape is set on every member;
+// time divided by its busiest block's work (i3_chunk_cost) gives the cost of a unit of work, and the
+// candidate's time is that cost times the busiest block's work over the whole queue (units of
+// different members carry different numbers of nodes).  The fastest shape is set on every member;
 // returns its predicted launch time in ms.
 int tune_group(const std::vector<qbe_handle*>& hs, cudaStream_t s, double* best_ms, std::string& err) {
   if (hs.empty()) return QBE_ERR_ARG;
@@ -933,7 +933,7 @@ int tune_group(const std::vector<qbe_handle*>& hs, cudaStream_t s, double* best_
   }
   int nmc_top = 1;
   for (int v : nmc_max) nmc_top = v > nmc_top ? v : nmc_top;
-  const int ws_blocks = (int)(h0->cw.ws_fields / 3);
+  const int ws_blocks = (int)(h0->cw.ws_fields / h0->cw.i3_fields);
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     err = "autotune: event creation failed";
@@ -961,25 +961,26 @@ int tune_group(const std::vector<qbe_handle*>& hs, cudaStream_t s, double* best_
       if (grid < 1) grid = 1;
       for (int nmc = nmc_top; nmc >= 1 && rc == QBE_OK; nmc = (nmc == 1 ? 0 : (nmc + 1) / 2)) {
         apply(v, nmc);
-        // the queue's units in launch order, each with its number of m evaluations
-        std::vector<int> mwork;
+        // the queue's units in launch order, each with the transforms of its items
+        const bool paired = i3_paired(n, prec, v);
+        std::vector<double> mwork;
         for (size_t i = 0; i < hs.size(); ++i) {
           const CollisionWork& cw = hs[i]->cw;
           const int M = hs[i]->tab.M;
           for (long long u = 0; u < (long long)nc[i] * hs[i]->tab.J * cw.nmc; ++u) {
-            const int mc = (int)(u % cw.nmc), m0 = mc * cw.mch;
-            mwork.push_back((M - m0) < cw.mch ? (M - m0) : cw.mch);
+            const int mc = (int)(u % cw.nmc);
+            mwork.push_back(i3_chunk_cost(i3_chunk_begin(mc, cw.nmc, M), i3_chunk_begin(mc + 1, cw.nmc, M), M, paired));
           }
         }
         const long long total = (long long)mwork.size();
         const int conc_full = i3_concurrency(n, prec, v, grid, (int)(total < INT_MAX ? total : INT_MAX));
         const int sample = (int)(total < 2LL * conc_full ? total : 2LL * conc_full);
         const int conc_sample = i3_concurrency(n, prec, v, grid, sample);
-        auto busiest = [&](long long units, int conc) {   // m evaluations of the busiest block
-          std::vector<long long> load(conc, 0);
+        auto busiest = [&](long long units, int conc) {   // work of the busiest block
+          std::vector<double> load(conc, 0.0);
           for (long long u = 0; u < units; ++u) load[u % conc] += mwork[u];
-          long long mx = 0;
-          for (long long x : load) mx = x > mx ? x : mx;
+          double mx = 0;
+          for (double x : load) mx = x > mx ? x : mx;
           return mx;
         };
         long long lc = 0;
@@ -996,8 +997,8 @@ int tune_group(const std::vector<qbe_handle*>& hs, cudaStream_t s, double* best_
           rc = QBE_ERR_CUDA;
           break;
         }
-        const double per_m = ms / (double)busiest(sample, conc_sample);
-        const double pred = per_m * (double)busiest(total, conc_full);
+        const double per_unit = ms / busiest(sample, conc_sample);
+        const double pred = per_unit * busiest(total, conc_full);
         if (pred < best) { best = pred; bv = v; bgrid = grid; bnmc = nmc; }
         if (nmc == 1) break;
       }
@@ -1075,7 +1076,7 @@ int batch_capture_step(qbe_batch* b, double dt, cudaStream_t origin) {
         nc.push_back(b->sims[i]->g.Nx);
       }
       const CollisionWork& c0 = b->sims[g[0]]->cw;
-      const int cap = (int)(c0.ws_fields / 3);            // blocks the first simulation's scratch can hold
+      const int cap = (int)(c0.ws_fields / c0.i3_fields);            // blocks the first simulation's scratch can hold
       const int grid = c0.grid_i3 < cap ? c0.grid_i3 : cap;   // the group's (tuned) persistent grid
       cudaError_t e = i3_group(tabs.data(), cws.data(), nc.data(), (int)g.size(), c0.ws, grid, origin, launches);
       if (e != cudaSuccess) return QBE_ERR_CUDA;
