@@ -326,9 +326,10 @@ int qbe_arith_issue_rates(int device, void* stream, double* rates);
  *     stores fused into the line stages and the radial nodes taken in pairs +-rho_m, which share
  *     their convolutions (256 threads, 64 KB or 128 threads, 32 KB).  FP32-split form, 2N = 64, 96, 128: the fused
  *     shared-memory kernel in three thread/accumulation shapes, or the kernel
- *     whose element passes go through shared memory, and at 2N = 128 also the
- *     kernel with warp-local passes; 2N <= 32: the element-pass kernel
- *     only; 2N = 192, 256: the cluster kernel with 1024 threads per CTA, or
+ *     whose element passes go through shared memory; the kernel with node pairs
+ *     and tensor-memory exchanges as variant 0 (2N = 64, in place of the first
+ *     shape) or 4 (2N = 128), and as the only one at 2N = 32; 2N = 16: the
+ *     element-pass kernel; 2N = 192, 256: the cluster kernel with 1024 threads per CTA, or
  *     with two row tasks per thread and register accumulation;
  *   - the persistent grid (blocks; at most the variant's residency);
  *   - the number of m-chunks per (cell, angle) work unit.

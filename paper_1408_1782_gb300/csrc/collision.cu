@@ -135,8 +135,12 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   cw.i3_variant = v0;
   cw.grid_i3 = nsm * bps;
   cw.grid_max = nsm * bps_max;
-  // enough (cell, j, m-chunk) units for about 8 waves of the persistent grid
-  int nmc = (8 * cw.grid_i3 + nb * t.J - 1) / (nb * t.J);
+  // enough (cell, j, m-chunk) units for about 8 waves of the persistent grid (of its teams, where a
+  // block works on several units at a time)
+  int slots = i3_concurrency(t.n, prec, v0, cw.grid_i3, INT_MAX);
+  if (slots < cw.grid_i3) slots = cw.grid_i3;
+  const long long cj = (long long)nb * t.J, want_nmc = (8LL * slots + cj - 1) / cj;
+  int nmc = (int)(want_nmc < t.M ? want_nmc : t.M);
   if (nmc < 1) nmc = 1;
   if (nmc > t.M) nmc = t.M;
   const size_t N = t.N, Q = (N - 1) * (N - 1);
@@ -179,16 +183,19 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   size_t ws_fields = 6 * (size_t)nb;
   if (5 * (size_t)nb * cw.nch > ws_fields) ws_fields = 5 * (size_t)nb * cw.nch;   // k_i24: 5 fields per block
   if (3 * (size_t)cw.grid_max > ws_fields) ws_fields = 3 * (size_t)cw.grid_max;
-  // the FP64 kernel that takes the nodes in pairs needs a fourth field per block; the number of blocks
-  // the scratch serves stays
-  cw.i3_fields = (any_paired && prec == 0) ? 4 : 3;
-  ws_fields = ws_fields / 3 * cw.i3_fields + ws_fields % 3;
+  // A requested grid is cut to this many blocks (and a launch to the resident ones, at most grid_max).
+  cw.grid_cap = (int)(ws_fields / 3 < (size_t)INT_MAX ? ws_fields / 3 : INT_MAX);
+  // fields per block of the kernels that take the nodes in pairs: four in FP64; in FP32 two per team, of
+  // which a block has (128 / n)^2
+  cw.i3_fields = prec == 0 ? 4 : t.n == 64 ? 8 : t.n == 32 ? 32 : 3;
+  if ((size_t)cw.i3_fields * cw.grid_max > ws_fields) ws_fields = (size_t)cw.i3_fields * cw.grid_max;
   cw.ws_fields = ws_fields;
   cudaError_t e;
 #define QBE_ALLOC(ptr, bytes) \
   if ((e = cudaMalloc((void**)&(ptr), (bytes))) != cudaSuccess) { free_collision_work(cw); return e; }
   QBE_ALLOC(cw.what, (size_t)nb * 4 * P * cz);
   QBE_ALLOC(cw.wfine, (size_t)nb * 2 * P * cz);
+  if (prec == 1 && (t.n == 32 || t.n == 64 || t.n == 128)) QBE_ALLOC(cw.wplane, (size_t)nb * 4 * P * rz);
   QBE_ALLOC(cw.Dacc, (size_t)nb * 2 * P * cz);
   QBE_ALLOC(cw.K2acc, (size_t)nb * P * rz);
   QBE_ALLOC(cw.K4acc, (size_t)nb * 2 * P * cz);
@@ -208,7 +215,7 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
 }
 
 void free_collision_work(CollisionWork& cw) {
-  cudaFree(cw.what); cudaFree(cw.wfine); cudaFree(cw.Dacc); cudaFree(cw.K2acc); cudaFree(cw.K4acc);
+  cudaFree(cw.what); cudaFree(cw.wfine); cudaFree(cw.wplane); cudaFree(cw.Dacc); cudaFree(cw.K2acc); cudaFree(cw.K4acc);
   cudaFree(cw.Dpart); cudaFree(cw.K2part); cudaFree(cw.K4part);
   cudaFree(cw.K3part); cudaFree(cw.K3spec); cudaFree(cw.K3sum); cudaFree(cw.ws); cudaFree(cw.cbuf); cudaFree(cw.wbuf);
   cw = CollisionWork();

@@ -38,6 +38,7 @@
 
 #include "fft.cuh"
 #include "internal.h"
+#include "tmem.cuh"
 
 namespace qbe {
 
@@ -128,13 +129,15 @@ __device__ __forceinline__ I3Group i3_group_at(int it, int it1, int M) {
 // Prep: Xi coefficients of the four Pauli components (paired) and the
 // fine-grid interpolants.  One block per cell.
 //   what[c][0] = w0^ + i w1^, [1] = w2^ + i w3^, [2] = w1^ + i w2^, [3] = w3^
-//   wfine[c][0] = w0 + i w1, [1] = w2 + i w3  on the fine grid.
+//   wfine[c][0] = w0 + i w1, [1] = w2 + i w3  on the fine grid;
+//   wplane (may be null): the same four components as planes [c][4][n*n].
 // The coarse DFT is the fine forward FFT of the zero-interleaved samples
 // (its spectrum repeats with period N), scaled by 1/N^2 and cut to Xi.
 // --------------------------------------------------------------------------
 template <int n, class T>
 __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w, typename Vec2Of<T>::type* what,
-                                                   typename Vec2Of<T>::type* wfine, typename Vec2Of<T>::type* ws,
+                                                   typename Vec2Of<T>::type* wfine, T* wplane,
+                                                   typename Vec2Of<T>::type* ws,
                                                    const typename Vec2Of<T>::type* __restrict__ gtw) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -173,7 +176,14 @@ __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w,
         [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
     row_pass<n, 1, false, 0>(
         sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
-        [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
+        [&](int ix, int iy, C2 v) {
+          out[ix * n + iy] = v;
+          if (wplane) {
+            T* pl = wplane + ((size_t)c * 4 + 2 * p) * P + ix * n + iy;
+            pl[0] = v.x;
+            pl[P] = v.y;
+          }
+        });
   }
 }
 
@@ -541,6 +551,7 @@ constexpr size_t i3_smem_bytes() {   // twiddles, the field (padded rows), psi'_
 
 #include "i3_fused.cuh"
 #include "i3_staged_fused.cuh"
+#include "i3_tmem.cuh"
 
 // Padded sizes with the fused shared-memory FP32 kernel (whole row tasks per thread for its shapes).
 template <int n>
@@ -548,17 +559,20 @@ __host__ __device__ constexpr bool use_i3_fused() {
   return n == 64 || n == 96 || n == 128;
 }
 // Its launch shapes per size: (threads, blocks per SM, accumulation mode of k_i3_fused), and the
-// default variant (I3 launch of 128 cells, J = M = 32, on a GB300: N = 32 28.6 ms for shape 0,
-// 32.5 and 35.4 for shapes 1 and 2, 31.0 for k_i3_smem; N = 48 74.7 ms for k_i3_smem, 77.5, 81.7,
-// 108.6 for the fused shapes; N = 64 100.9 ms for shape 0, 116.3, 112.1, 124.0 for k_i3_smem).
+// default variant (I3 launch, J = M = 32, on a GB300).  N = 32, 128 cells: 13.6 ms for k_i3_tmem
+// (variant 0; 28.6 ms for the fused kernel with register accumulation that it replaces), 38.8 and 52.2
+// for shapes 1 and 2, 31.2 for k_i3_smem.  N = 48, 64 cells: 38.5 for k_i3_smem, 40.3, 42.5, 56.4 for
+// the fused shapes.  N = 64, 128 cells: 49.8 for k_i3_tmem (88.6 for the warp-local kernel, node by
+// node, that it replaces; 57.8 for that kernel in pairs), 101.0, 115.8, 111.6 for shapes 0 to 2, 122.2
+// for k_i3_smem.  N = 16, 128 cells: 3.0 for k_i3_tmem.
 template <int n> struct FusedShapes;
-template <> struct FusedShapes<64> {
-  static constexpr int T0 = 512, B0 = 2, M0 = 1, T1 = 512, B1 = 2, M1 = 2, T2 = 256, B2 = 4, M2 = 2, DEFAULT = 0;
+template <> struct FusedShapes<64> {   // variant 0: k_i3_tmem
+  static constexpr int T0 = 0, B0 = 0, M0 = 1, T1 = 512, B1 = 2, M1 = 2, T2 = 256, B2 = 4, M2 = 2, DEFAULT = 0;
 };
 template <> struct FusedShapes<96> {
   static constexpr int T0 = 768, B0 = 1, M0 = 0, T1 = 768, B1 = 1, M1 = 2, T2 = 384, B2 = 2, M2 = 2, DEFAULT = 3;
 };
-template <> struct FusedShapes<128> {   // variant 4: k_i3_wl, 88.8 ms (shape 0: 101.1 ms)
+template <> struct FusedShapes<128> {   // variant 4: k_i3_tmem
   static constexpr int T0 = 512, B0 = 1, M0 = 1, T1 = 1024, B1 = 1, M1 = 2, T2 = 1024, B2 = 1, M2 = 0, DEFAULT = 4;
 };
 
@@ -953,8 +967,8 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
 // --------------------------------------------------------------------------
 // Assemble C on the fine grid from D, K2, K3, K4 (Pauli formulas of Sec. 3.1),
 // then FFT, cut to Xi (without the -N/2 line), inverse FFT and sample the
-// coarse nodes.  One block per cell.  k3: the reduced K3 pairs (FP64) of a cell, k3_stride apart;
-// spec (may be null): their Fourier-space parts, added to the spectrum of C inside the projection
+// coarse nodes.  One block per cell.  k3: the reduced K3 of a cell (FP64), k3_stride apart; spec (null
+// after a node-by-node kernel): their Fourier-space parts, added to the spectrum of C inside the projection
 // (C_0 holds -2 pi K3_0 and C_c holds +2 pi K3raw_c; the sign of component 0 is already in spec).
 // --------------------------------------------------------------------------
 template <int n, class T>
@@ -991,8 +1005,11 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
   const C2* wf1 = wf0 + P;
   const T* K2 = K2acc + (size_t)c * P;
   const double tp = 2.0 * kPi;
+  const double* k3r = reinterpret_cast<const double*>(k3c);
   for (int i = threadIdx.x; i < P; i += blockDim.x) {
-    const double2 k3a = k3c[i], k3b = k3c[P + i];
+    // node-by-node kernels: pairs (K3_0, K3_1), (K3_2, K3_3); kernels in pairs: four planes
+    const double2 k3a = spec ? mk2(k3r[i], k3r[P + i]) : k3c[i];
+    const double2 k3b = spec ? mk2(k3r[2 * P + i], k3r[3 * P + i]) : k3c[P + i];
     const double w0 = wf0[i].x, w1 = wf0[i].y, w2 = wf1[i].x, w3 = wf1[i].y;
     const double D1 = slot[i].x, D2 = slot[i].y, D3 = slot[P + i].x;
     const double K40 = slot[2 * P + i].x, K41 = -(double)slot[2 * P + i].y;   // eta_b applied
@@ -1060,9 +1077,10 @@ size_t i3_staged_smem_bytes() {
 //     0: (256, 64 KB, 3)   1: (128, 32 KB, 6);  k_i3_sf, nodes in pairs, 2: (256, 64 KB, 3)
 //     3: (128, 32 KB, 6).  Variant 0 also serves the allocation-free entry point, whose static array
 //     has no room for the pairs' Fourier-space partials at the sizes it accepts.
-//   FP32, n = 64, 96, 128: 0, 1, 2: the fused shared-memory kernel in the FusedShapes<n> shapes,
-//     3: k_i3_smem (1024 threads, element passes through shared memory)
-//   FP32, n <= 32: k_i3_smem;  FP32, n > 128: the cluster kernel, 0: 1024 threads per CTA with a
+//   FP32, n = 64, 96, 128: 0, 1, 2: the fused shared-memory kernel in the FusedShapes<n> shapes
+//     (0 at n = 64: k_i3_tmem), 3: k_i3_smem (1024 threads, element passes through shared memory), 4
+//     (n = 128): k_i3_tmem
+//   FP32, n = 32: k_i3_tmem;  n = 16: k_i3_smem;  FP32, n > 128: the cluster kernel, 0: 1024 threads per CTA with a
 //     partial-sum update per convolution, 1: two row tasks per thread with register accumulation.
 struct I3Launch {
   const void* fn = nullptr;
@@ -1070,13 +1088,23 @@ struct I3Launch {
   size_t smem = 0;
   bool cluster = false;
   const char* name = "";
+  int teams = 1;   // units a block works on at a time
 };
+
+template <int n>
+I3Launch i3_tmem_launch() {
+  using S = TmShape<n>;
+  return {(const void*)k_i3_tmem<n>, S::NT, S::smem, false,
+          n == 128 ? "node pairs, tensor-memory exchanges, one team of 512 threads per block"
+          : n == 64 ? "node pairs, tensor-memory exchanges, four teams of 128 threads per block"
+                    : "node pairs, a warp per unit, sixteen per block", S::TEAMS};
+}
 
 template <int n, class T>
 constexpr int i3_nvariants() {
   if constexpr (std::is_same<T, float>::value) {
     if constexpr (use_i3_cluster<n>()) return 2;
-    else if constexpr (use_i3_fused<n>()) return n == kWlN ? 5 : 4;   // 128 points: + k_i3_wl
+    else if constexpr (use_i3_fused<n>()) return n == 128 ? 5 : 4;   // 128 points: + k_i3_tmem
     else return 1;
   } else {
     return 4;
@@ -1099,17 +1127,20 @@ I3Launch i3_variant(int v) {
     using S = FusedShapes<n>;
     constexpr const char* names[3] = {"fused, per-convolution partial sums", "fused, register accumulation",
                                       "fused, paired w with register accumulation"};
-    if (v == 0)
-      l = {(const void*)k_i3_fused<n, S::T0, S::B0, S::M0>, S::T0, i3_fused_smem_bytes<n>(), false, names[S::M0]};
-    else if (v == 1)
+    if (v == 0) {
+      if constexpr (n == 64) l = i3_tmem_launch<n>();
+      else l = {(const void*)k_i3_fused<n, S::T0, S::B0, S::M0>, S::T0, i3_fused_smem_bytes<n>(), false, names[S::M0]};
+    } else if (v == 1)
       l = {(const void*)k_i3_fused<n, S::T1, S::B1, S::M1>, S::T1, i3_fused_smem_bytes<n>(), false, names[S::M1]};
     else if (v == 2)
       l = {(const void*)k_i3_fused<n, S::T2, S::B2, S::M2>, S::T2, i3_fused_smem_bytes<n>(), false, names[S::M2]};
-    else if (v == 4 && n == kWlN)
-      l = {(const void*)k_i3_wl, kWlThreads, i3_wl_smem_bytes(), false,
-           "fused, warp-local passes, register accumulation"};
     else
       l = {(const void*)k_i3_smem<n>, kThreadsI3Smem, i3_smem_bytes<n>(), false, "shared-memory, 1024 threads"};
+    if constexpr (n == 128) {
+      if (v == 4) l = i3_tmem_launch<n>();
+    }
+  } else if constexpr (std::is_same<T, float>::value && n == 32) {
+    l = i3_tmem_launch<n>();
   } else if constexpr (std::is_same<T, float>::value) {
     l = {(const void*)k_i3_smem<n>, kThreadsI3Smem, i3_smem_bytes<n>(), false, "shared-memory, 1024 threads"};
   } else {
@@ -1226,6 +1257,7 @@ int i3_variant_concurrency(int v, int grid, int total) {
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const int gmax = nsm * i3_blocks_per_sm<n, T>(v);
     if (g > gmax) g = gmax;
+    g *= i3_variant<n, T>(v).teams;
   }
   return g < 1 ? 1 : g;
 }
@@ -1233,7 +1265,8 @@ int i3_variant_concurrency(int v, int grid, int total) {
 // Variants that take the radial nodes in pairs (Fourier-space partials beside the real-space ones).
 template <int n, class T>
 bool i3_variant_paired(int v) {
-  return std::is_same<T, double>::value && v >= 2;
+  if constexpr (std::is_same<T, double>::value) return v >= 2;
+  else return (n == 128 && v == 4) || ((n == 64 || n == 32) && v == 0);
 }
 
 template <int n, class T>
@@ -1288,7 +1321,7 @@ cudaError_t collide_pre_n(const Tables& t, CollisionWork& cw, const double* w, i
   auto begin = [&](int g) { if (tm) tm->begin(g, s); };
   auto end = [&]() { if (tm) tm->end(s); };
   begin(KG_PREP);
-  k_prep<n, T><<<ncells, kThreads, sm, s>>>(w, what, wfine, ws, tb.tw);
+  k_prep<n, T><<<ncells, kThreads, sm, s>>>(w, what, wfine, (T*)cw.wplane, ws, tb.tw);
   end();
   cudaError_t e = per_cell_terms<n, T>(t, cw, ws, ncells, s, launches, tm);
   if (e != cudaSuccess) return e;
@@ -1303,6 +1336,7 @@ I3Job<T> i3_job(const Tables& t, const CollisionWork& cw, int ncells, int unit_b
   I3Job<T> jb;
   jb.what = (const C2*)cw.what;
   jb.wfine = (const C2*)cw.wfine;
+  jb.wplane = (const T*)cw.wplane;
   jb.K3part = (C2*)cw.K3part;
   jb.K3spec = (C2*)cw.K3spec;
   jb.psip_s = tb.psip_s;

@@ -823,7 +823,7 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
   auto begin = [&](int g) { if (tm) tm->begin(g, s); };
   auto end = [&]() { if (tm) tm->end(s); };
   begin(KG_VJP);
-  k_prep<n, T><<<ncells, kThreads, sm, s>>>(w, what, wfine, ws, tb.tw);
+  k_prep<n, T><<<ncells, kThreads, sm, s>>>(w, what, wfine, (T*)cw.wplane, ws, tb.tw);
   ++launches;
   {
     const cudaError_t e = per_cell_terms<n, T>(t, cw, ws, ncells, s, launches, nullptr);

@@ -73,41 +73,48 @@ __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {  // a * conj(b)
 }
 __device__ __forceinline__ double2 cscale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
 
-// cos(2 pi k / 16) for integer k (mathematical constants cos(pi/8), sin(pi/8), sqrt(1/2)).
-__host__ __device__ constexpr double cos16(int k) {
-  constexpr double c1 = 0.92387953251128675613;   // cos(pi/8)
-  constexpr double s1 = 0.38268343236508977173;   // sin(pi/8)
-  constexpr double r2 = 0.70710678118654752440;   // sqrt(1/2)
-  k &= 15;
-  return k == 0 ? 1.0 : k == 1 ? c1 : k == 2 ? r2 : k == 3 ? s1 : k == 4 ? 0.0 : k == 5 ? -s1
-       : k == 6 ? -r2 : k == 7 ? -c1 : k == 8 ? -1.0 : k == 9 ? -c1 : k == 10 ? -r2 : k == 11 ? -s1
-       : k == 12 ? 0.0 : k == 13 ? s1 : k == 14 ? r2 : c1;
+// cos(2 pi k / 32) for integer k (mathematical constants cos(pi j / 16)).
+__host__ __device__ constexpr double cos32(int k) {
+  constexpr double c1 = 0.98078528040323044913;   // cos(pi/16)
+  constexpr double c2 = 0.92387953251128675613;   // cos(pi/8)
+  constexpr double c3 = 0.83146961230254523708;   // cos(3 pi/16)
+  constexpr double c4 = 0.70710678118654752440;   // cos(pi/4)
+  constexpr double c5 = 0.55557023301960222474;   // cos(5 pi/16)
+  constexpr double c6 = 0.38268343236508977173;   // cos(3 pi/8)
+  constexpr double c7 = 0.19509032201612826785;   // cos(7 pi/16)
+  k &= 31;
+  k = k > 16 ? 32 - k : k;
+  const double s = k > 8 ? -1.0 : 1.0;
+  k = k > 8 ? 16 - k : k;
+  return k == 8 ? 0.0 : s * (k == 0 ? 1.0 : k == 1 ? c1 : k == 2 ? c2 : k == 3 ? c3 : k == 4 ? c4 : k == 5 ? c5
+                             : k == 6 ? c6 : c7);
 }
-__host__ __device__ constexpr double sin16(int k) { return cos16(k - 4); }
+__host__ __device__ constexpr double sin32(int k) { return cos32(k - 8); }
 
-// x * exp(SIGN * 2 pi i k / R) for R <= 16, k a compile-time constant after unrolling.
+// x * exp(SIGN * 2 pi i k / R) for R <= 32, k a compile-time constant after unrolling.
 template <int R, int SIGN, class C2>
 __device__ __forceinline__ C2 twid(int k, C2 x) {
   using T = typename RealOf<C2>::type;
-  const int k16 = (k * (16 / R)) & 15;
-  if (k16 == 0) return x;
-  if (k16 == 8) return mk2(-x.x, -x.y);
-  if (k16 == 4) return SIGN > 0 ? mk2(-x.y, x.x) : mk2(x.y, -x.x);
-  if (k16 == 12) return SIGN > 0 ? mk2(x.y, -x.x) : mk2(-x.y, x.x);
-  const T c = (T)cos16(k16), s = (T)(SIGN * sin16(k16));
+  const int k32 = (k * (32 / R)) & 31;
+  if (k32 == 0) return x;
+  if (k32 == 16) return mk2(-x.x, -x.y);
+  if (k32 == 8) return SIGN > 0 ? mk2(-x.y, x.x) : mk2(x.y, -x.x);
+  if (k32 == 24) return SIGN > 0 ? mk2(x.y, -x.x) : mk2(-x.y, x.x);
+  const T c = (T)cos32(k32), s = (T)(SIGN * sin32(k32));
   return mk2(fmaT(x.x, c, -x.y * s), fmaT(x.x, s, x.y * c));
 }
 
 __host__ __device__ constexpr int ilog2c(int r) { return r <= 1 ? 0 : 1 + ilog2c(r / 2); }
-// Bit reversal of i within `bits` <= 4 bits (closed form so that it folds after unrolling).
+// Bit reversal of i within `bits` <= 5 bits (closed form so that it folds after unrolling).
 __host__ __device__ constexpr int bitrev(int i, int bits) {
-  return (((i & 1) << 3) | ((i & 2) << 1) | ((i & 4) >> 1) | ((i & 8) >> 3)) >> (4 - bits);
+  return (((i & 1) << 4) | ((i & 2) << 2) | (i & 4) | ((i & 8) >> 2) | ((i & 16) >> 4)) >> (5 - bits);
 }
 
 // One radix-2 decimation-in-time stage of butterfly span S on R registers.
 // Butterflies with a non-trivial twiddle w = c + i s use the cosine-factored
 // form (u +- w x) = u +- c (x + (s/c) i x): six FMAs instead of two products,
-// two FMAs and four additions (|s/c| <= tan(3 pi/8) for R <= 16).
+// two FMAs and four additions (|s/c| <= tan(3 pi/8) for R <= 16, tan(7 pi/16) for R = 32; the factor c
+// takes the ratio's size out again).
 template <int R, int SIGN, int S, class C2>
 struct DftStage {
   __device__ __forceinline__ static void run(C2 (&b)[R]) {
@@ -116,16 +123,16 @@ struct DftStage {
     for (int g = 0; g < R; g += S) {
 #pragma unroll
       for (int k = 0; k < S / 2; ++k) {
-        const int k16 = (k * (16 / S)) & 15;
+        const int k32 = (k * (32 / S)) & 31;
         const C2 u = b[g + k];
         const C2 x = b[g + k + S / 2];
-        if ((k16 & 3) == 0) {
-          const C2 t = twid<16, SIGN>(k16, x);
+        if ((k32 & 7) == 0) {
+          const C2 t = twid<32, SIGN>(k32, x);
           b[g + k] = cadd(u, t);
           b[g + k + S / 2] = csub(u, t);
         } else {
-          const T c = (T)cos16(k16);
-          const T r = (T)((SIGN * sin16(k16)) / cos16(k16));
+          const T c = (T)cos32(k32);
+          const T r = (T)((SIGN * sin32(k32)) / cos32(k32));
           const T qx = fmaT(-r, x.y, x.x);
           const T qy = fmaT(r, x.x, x.y);
           b[g + k] = mk2(fmaT(c, qx, u.x), fmaT(c, qy, u.y));
@@ -150,7 +157,7 @@ __host__ __device__ constexpr double cos12(int k) {
 }
 __host__ __device__ constexpr double sin12(int k) { return cos12(k - 3); }
 
-// In-register DFT of length R (natural order in and out): R a power of two <= 16
+// In-register DFT of length R (natural order in and out): R a power of two <= 32
 // (radix-2 decimation in time), or R = 3 * 2^q <= 12 (one radix-3 decimation-in-time
 // step on top of power-of-two sub-DFTs).
 template <int R, int SIGN, class C2, bool POW2 = ((R & (R - 1)) == 0)>

@@ -280,14 +280,13 @@ __global__ void __launch_bounds__(NT, MINB) k_i3_fused(const I3Jobs<float> jobs,
 }
 
 // --------------------------------------------------------------------------
-// The fused FP32 I3 kernel with warp-local passes (padded grid of 128 points, 512 threads, the
-// accumulation of mode 1).  In the row passes warp w owns rows [8 w, 8 w + 8), in the column passes
-// warp pair g owns columns [16 g, 16 g + 16): their stages synchronise with __syncwarp or a named
-// barrier of the pair, and the block synchronises only where the passes change ownership (rows ->
-// columns, columns -> rows), twice per convolution instead of seven times, so warps in different
-// stages overlap their shared-memory, global and arithmetic latencies.  Field layout: element
-// (x, y) at x * WL_PITCH + y + y / 16 (one pad word per 16 elements, row pitch 146 = 2 mod 16),
-// which keeps every stage's accesses free of bank conflicts under the lane mappings below.
+// Warp-local passes (padded grid of 128 points, 512 threads), used by the I3 transpose.  In the row
+// passes warp w owns rows [8 w, 8 w + 8), in the column passes warp pair g owns columns
+// [16 g, 16 g + 16): their stages synchronise with __syncwarp or a named barrier of the pair, and the
+// block synchronises only where the passes change ownership (rows -> columns, columns -> rows).  Field
+// layout: element (x, y) at x * kWlPitch + y + y / 16 (one pad word per 16 elements, row pitch
+// 146 = 2 mod 16), which keeps every stage's accesses free of bank conflicts under the lane mappings
+// below.
 // --------------------------------------------------------------------------
 constexpr int kWlN = 128, kWlThreads = 512, kWlPitch = 146;
 
@@ -418,140 +417,4 @@ __device__ __forceinline__ void wl_shift(float2* G, const float2* tw, const floa
     for (int k = 0; k < A; ++k) S[(B * k + t2) * n + y] = v[k];
   }
   __syncthreads();
-}
-
-__global__ void __launch_bounds__(kWlThreads, 1) k_i3_wl(const I3Jobs<float> jobs, float2* ws,
-                                                        const float2* __restrict__ gtw) {
-  using C2 = float2;
-  constexpr int n = kWlN, A = Split<n>::A, B = Split<n>::B, P = n * n, NT = kWlThreads;
-  constexpr int TPT = n * B / NT;   // 4 row tasks (row, t2) per thread in the fused row stages
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C2* tw = reinterpret_cast<C2*>(smem_raw);                   // tw[t2 A + k1]
-  C2* twT = tw + n;                                           // twT[k1 B + t2]
-  C2* G = twT + n;                                            // skewed field
-  float* psm = reinterpret_cast<float*>(G + n * kWlPitch);    // psi'_j of the current unit, [n][kWlPsiPitch]
-  for (int pos = threadIdx.x; pos < n; pos += blockDim.x) twT[(pos % A) * B + pos / A] = gtw[pos];
-  load_twiddles<n>(tw, gtw);
-  C2* Sig = ws + (size_t)blockIdx.x * 3 * P;   // [2][P]
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, g = w >> 1, tt = tid & 63;
-  const int t2r = lane & 15;                   // t2 of this thread's row tasks
-  // row task k of this thread: row 8 w + lane / 16 + 2 k, t2 = lane mod 16
-  auto row_of = [&](int k) { return 8 * w + (lane >> 4) + 2 * k; };
-  for (int gunit = blockIdx.x; gunit < jobs.total; gunit += gridDim.x) {
-    const I3Job<float>& jb = jobs.job[i3_job_of(jobs, gunit)];
-    const int unit = gunit - jb.unit_begin;
-    const int J = jb.J, M = jb.M, nmc = jb.nmc;
-    const C2* what = jb.what;
-    const C2* __restrict__ phase = jb.phase;
-    const int c = unit / (J * nmc);
-    const int j = (unit / nmc) % J;
-    const int mc = unit % nmc;
-    C2* acc = jb.K3part + (size_t)unit * 2 * P;
-    {
-      const float4* src = reinterpret_cast<const float4*>(jb.psip_s + (size_t)j * P);
-      for (int i4 = tid; i4 < P / 4; i4 += NT) {
-        const float4 q = src[i4];
-        float* d = psm + (4 * i4 / n) * kWlPsiPitch + (4 * i4) % n;
-        d[0] = q.x; d[1] = q.y; d[2] = q.z; d[3] = q.w;
-      }
-      __syncthreads();
-    }
-    const C2* wf = jb.wfine + (size_t)c * 2 * P;
-    const int m0 = i3_chunk_begin(mc, nmc, M), m1 = i3_chunk_begin(mc + 1, nmc, M);
-    for (int m = m0; m < m1; ++m) {
-      const C2* px = phase + ((size_t)j * M + m) * 2 * n;
-      const C2* py = px + n;
-      const bool first_m = (m == m0);
-      // shifted pairs (S complete for every thread when wl_shift returns)
-      for (int p = 0; p < 2; ++p)
-        wl_shift(G, tw, twT, what + ((size_t)c * 4 + p) * P, px, py, Sig + (size_t)p * P, w, lane, g, tt);
-      for (int p = 0; p < 2; ++p) {
-        const C2* Sp = Sig + (size_t)p * P;      // rewritten every m: plain (coherent) loads
-        C2* accp = acc + (size_t)p * P;
-        C2 racc[TPT][A];
-        for (int a = 0; a < 4; ++a) {
-          // component im of the fine pair and of the shifted pair, loaded as single floats
-          const int im = a & 1;
-          const float* __restrict__ wa = reinterpret_cast<const float*>(wf + (size_t)(a >> 1) * P) + im;
-          const float* Sa = reinterpret_cast<const float*>(Sig + (size_t)(a >> 1) * P) + im;
-          // forward rows of w_a Sigma_p (warp-local): stage A loads the product, stage B
-#pragma unroll
-          for (int k = 0; k < TPT; ++k) {
-            const int x = row_of(k);
-            C2 v[A];
-#pragma unroll
-            for (int t1 = 0; t1 < A; ++t1) {
-              const int idx = x * n + B * t1 + t2r;
-              v[t1] = cscale(Sp[idx], wa[2 * idx]);
-            }
-            dft<A, -1>(v);
-#pragma unroll
-            for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2r]);
-#pragma unroll
-            for (int k1 = 0; k1 < A; ++k1) G[wl_addr(x, B * k1 + t2r)] = v[k1];
-          }
-          __syncwarp();
-          wl_rows_stage_b<-1>(G, w, lane);
-          __syncthreads();
-          // columns (pair-local): forward stage A, stage B with psi'_j, inverse stage A
-          wl_cols_stage_a<-1>(G, tw, g, tt);
-          wl_pair_sync(g);
-          {
-            const int y = 16 * g + (tt & 15);
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-              const int k1 = (tt >> 4) + 4 * i;
-              C2 b[B];
-#pragma unroll
-              for (int t = 0; t < B; ++t) b[t] = G[wl_addr(B * k1 + t, y)];
-              dft<B, -1>(b);
-              float sc[B];
-#pragma unroll
-              for (int t = 0; t < B; ++t) sc[t] = psm[(B * k1 + t) * kWlPsiPitch + y];
-              dft_scaled<B, 1>(b, sc);
-#pragma unroll
-              for (int t = 0; t < B; ++t) G[wl_addr(B * k1 + t, y)] = b[t];
-            }
-          }
-          wl_pair_sync(g);
-          wl_cols_stage_a<1>(G, tw, g, tt);
-          __syncthreads();
-          // inverse rows (warp-local): stage B, stage A times eta_a S_a, accumulated over a
-          wl_rows_stage_b<1>(G, w, lane);
-          __syncwarp();
-          const float eta = (a == 0) ? 1.f : -1.f;
-#pragma unroll
-          for (int k = 0; k < TPT; ++k) {
-            const int x = row_of(k);
-            float f[A];
-#pragma unroll
-            for (int t1 = 0; t1 < A; ++t1) f[t1] = eta * Sa[2 * (x * n + B * t1 + t2r)];
-            C2 v[A];
-#pragma unroll
-            for (int k1 = 0; k1 < A; ++k1) v[k1] = G[wl_addr(x, B * k1 + t2r)];
-#pragma unroll
-            for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2r]);
-            dft<A, 1>(v);
-#pragma unroll
-            for (int t1 = 0; t1 < A; ++t1) {
-              if (a == 0) racc[k][t1] = mk2(f[t1] * v[t1].x, f[t1] * v[t1].y);
-              else racc[k][t1] = mk2(fmaT(f[t1], v[t1].x, racc[k][t1].x), fmaT(f[t1], v[t1].y, racc[k][t1].y));
-            }
-          }
-          __syncwarp();   // this warp's rows of G are rewritten by the next a's forward stage A
-        }
-#pragma unroll
-        for (int k = 0; k < TPT; ++k) {
-          const int x = row_of(k);
-#pragma unroll
-          for (int t1 = 0; t1 < A; ++t1) {
-            const int idx = x * n + B * t1 + t2r;
-            accp[idx] = first_m ? racc[k][t1] : cadd(accp[idx], racc[k][t1]);
-          }
-        }
-      }
-      __syncthreads();   // G and Sig are rewritten by the next m's shift transforms
-    }
-    __syncthreads();     // psm is reloaded by the next unit
-  }
 }

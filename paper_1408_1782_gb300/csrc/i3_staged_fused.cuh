@@ -221,13 +221,13 @@ __global__ void __launch_bounds__(NTH, MINB)
           }
           // ---- K3_b += eta_2q s_2q Re U + eta_2q+1 s_2q+1 Im U;  V_q += eta_b w_b U (x part of q = 0
           // with the sign that C_0 has against C_1..C_3, see k_assemble) ----
-          T* Kb = reinterpret_cast<T*>(acc + (size_t)(b >> 1) * P) + (b & 1);
+          T* Kb = reinterpret_cast<T*>(acc) + (size_t)b * P;
           const T* wb = reinterpret_cast<const T*>(wf + (size_t)(b >> 1) * P) + (b & 1);
           const T e0 = q == 0 ? (T)1 : (T)-1, eb = b == 0 ? (T)1 : (T)-1;
           rows_inverse(std::false_type{}, [&](int idx, C2 v) {
             const C2 s = Sq[idx];
             const T k = fmaT(e0 * s.x, v.x, -s.y * v.y);
-            Kb[2 * idx] = k_first ? k : Kb[2 * idx] + k;
+            Kb[idx] = k_first ? k : Kb[idx] + k;
             if (gr.pair) {
               const T f = eb * wb[2 * idx], fx = -e0 * f;
               if (b == 0) {

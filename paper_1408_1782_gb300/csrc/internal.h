@@ -69,6 +69,7 @@ template <class T>
 struct I3Job {
   const typename std::conditional<sizeof(T) == 8, double2, float2>::type* what;
   const typename std::conditional<sizeof(T) == 8, double2, float2>::type* wfine;
+  const T* wplane;
   typename std::conditional<sizeof(T) == 8, double2, float2>::type* K3part;
   typename std::conditional<sizeof(T) == 8, double2, float2>::type* K3spec;
   const T* psip_s;
@@ -97,6 +98,7 @@ struct CollisionWork {
   // buffers of the transform precision (complex = double2 or float2)
   void* what = nullptr;      // [nb][4][n*n] spectral pairs (w0+iw1, w2+iw3, w1+iw2, w3)
   void* wfine = nullptr;     // [nb][2][n*n] fine-grid fields (w0+iw1, w2+iw3)
+  void* wplane = nullptr;    // [nb][4][n*n] the same as planes (FP32, n = 32, 64, 128 only)
   void* Dacc = nullptr;      // [nb][2][n*n] spectral D (pairs (1,2), (3,-))
   void* K2acc = nullptr;     // [nb][n*n] (real)
   void* K4acc = nullptr;     // [nb][2][n*n] spectral K4 pairs (0,1), (2,3)
@@ -104,17 +106,20 @@ struct CollisionWork {
   void* Dpart = nullptr;     // their per-chunk partials [nb][nch][...] (nch > 1 only)
   void* K2part = nullptr;
   void* K4part = nullptr;
-  void* K3part = nullptr;    // [nb*J*nmc][2][n*n] fine-grid K3 pair partial sums
+  // fine-grid K3 partial sums [nb*J*nmc]: [2][n*n] pairs (0,1), (2,3) of the node-by-node kernels, four
+  // planes [4][n*n] (reals) of the kernels that take the nodes in pairs
+  void* K3part = nullptr;
   // Fourier-space partial sums of the kernels that take the nodes in pairs, kept frequencies only
   // [nb*J*nmc][2][(n/2-1)^2]; null: the workspace serves the node-by-node kernels only
   void* K3spec = nullptr;
-  double2* K3sum = nullptr;  // [nb][2][n*n] reduced K3 pairs (FP32 form; FP64 reduces in place)
+  double2* K3sum = nullptr;  // [nb][2][n*n] reduced K3 in the same order (FP32 form; FP64 reduces in place)
   // whether the last I3 launch over this workspace took the nodes in pairs (its post-processing
   // then adds K3spec); a batch launches its first member's variant for the whole group
   mutable bool i3_paired = false;
   void* ws = nullptr;        // per-CTA scratch
   size_t ws_fields = 0;      // complex n*n fields of scratch
   int i3_fields = 3;         // of which an I3 block (or cluster) uses this many
+  int grid_cap = 0;          // largest persistent grid a caller may set
   int ws_slots = 0;          // number of CTA slots in ws
   double* cbuf = nullptr;    // [nb][4][N][N] staging for collide in/out
   double* wbuf = nullptr;

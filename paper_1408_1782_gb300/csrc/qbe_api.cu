@@ -380,8 +380,7 @@ int qbe_set_i3_shape(qbe_handle* h, int variant, int grid, int m_chunks) {
   if (m_chunks > cap_nmc) return fail(h, QBE_ERR_ARG, "set_i3_shape: more m-chunks than the partial sums hold");
   if (variant >= 0) h->cw.i3_variant = variant;
   if (grid > 0) {
-    const int cap = (int)(h->cw.ws_fields / h->cw.i3_fields);
-    h->cw.grid_i3 = grid < cap ? grid : cap;
+    h->cw.grid_i3 = grid < h->cw.grid_cap ? grid : h->cw.grid_cap;
   }
   if (m_chunks > 0) {
     h->cw.mch = (h->tab.M + m_chunks - 1) / m_chunks;

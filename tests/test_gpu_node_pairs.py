@@ -78,3 +78,18 @@ def test_batch_of_members_with_different_variants(qbe, first, second):
         ref = s1.get_state()
         assert np.abs(s.get_state() - ref).max() <= 1e-12 * np.abs(ref).max()
     b.close()
+
+
+@pytest.mark.parametrize("N,J,M,ncells", [(16, 32, 8, 24), (32, 32, 8, 8), (64, 16, 3, 12)])
+def test_fp32_with_every_team_busy(qbe, N, J, M, ncells):
+    """More units than the launch works on at a time (16, 4 and 1 per block for N = 16, 32, 64), so that
+    every team of every block has several: against the FP64 form."""
+    import torch
+
+    w = torch.from_numpy(inputs.synthetic_w(N, ncells, seed=120 + N, perturb=0.05)).cuda()
+    out = []
+    for prec in (0, 1):
+        s = qbe.Solver(N, ncells, J=J, M=M, stream=torch.cuda.current_stream(), precision=prec)
+        out.append(s.collide(w).cpu().numpy())
+        s.close()
+    assert np.abs(out[1] - out[0]).max() < TOL[1] * np.abs(out[0]).max()
