@@ -330,7 +330,7 @@ int qbe_arith_issue_rates(int device, void* stream, double* rates);
  *     and tensor-memory exchanges as variant 0 (2N = 64, in place of the first
  *     shape) or 4 (2N = 128), and as the only one at 2N = 32; 2N = 16: the
  *     element-pass kernel; 2N = 192, 256: the cluster kernel with 1024 threads per CTA, or
- *     with two row tasks per thread and register accumulation;
+ *     with two row tasks per thread, node pairs and register accumulation;
  *   - the persistent grid (blocks; at most the variant's residency);
  *   - the number of m-chunks per (cell, angle) work unit.
  * qbe_i3_shape reports the current shape and the number of variants

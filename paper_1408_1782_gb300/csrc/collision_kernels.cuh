@@ -436,11 +436,10 @@ __global__ void __launch_bounds__(NTH, MINB)
 
 // --------------------------------------------------------------------------
 // I3 with the transform field resident in shared memory (FP32, n <= 128: an
-// n x (n+1) complex float field is at most 129 KB).  Same units, arithmetic
-// and accumulation order as k_i3 (the line transforms are the same code, so
-// results are bitwise identical); each convolution (row FFT, column psi'
-// convolution, row IFFT) runs entirely on chip, global memory holds only the
-// two shifted fields per block and the partial sums.
+// n x (n+1) complex float field is at most 129 KB), nodes in pairs as in k_i3_sf
+// (i3_staged_fused.cuh).  Each convolution (row FFT, column psi' convolution, row
+// IFFT) runs entirely on chip; global memory holds the two shifted fields and V_q
+// per block and the partial sums.
 // --------------------------------------------------------------------------
 constexpr int kThreadsI3Smem = 1024;
 
@@ -453,14 +452,16 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_smem(const I3Jobs<floa
   C2* G = tw + n;                       // [n][LS]
   float* psm = reinterpret_cast<float*>(G + n * (n + 1));   // psi'_j of the current unit, [n][n]
   constexpr int LS = n + 1, P = n * n;
+  constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
   constexpr int kIter = (P + kThreadsI3Smem - 1) / kThreadsI3Smem;
   __shared__ unsigned char xmask[n];
-  for (int pos = threadIdx.x; pos < n; pos += blockDim.x) {
-    const int k = freq_of_pos<n>(pos);
-    xmask[pos] = ((k < n / 4) || (k >= n - n / 4)) ? 1 : 0;
-  }
+  __shared__ int kslot[n];
+  __shared__ int kcols[n];
+  for (int pos = threadIdx.x; pos < n; pos += blockDim.x) xmask[pos] = xi_t<Split<n>::B>(pos % Split<n>::B) ? 1 : 0;
+  build_xi_slots<n>(kslot, kcols);
   load_twiddles<n>(tw, gtw);
   C2* Sig = ws + (size_t)blockIdx.x * 3 * P;   // [2][P]
+  C2* V = Sig + 2 * P;
   for (int gunit = blockIdx.x; gunit < jobs.total; gunit += gridDim.x) {
     const I3Job<float>& jb = jobs.job[i3_job_of(jobs, gunit)];
     const int unit = gunit - jb.unit_begin;
@@ -471,18 +472,21 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_smem(const I3Jobs<floa
     const int c = unit / (J * nmc);
     const int j = (unit / nmc) % J;
     const int mc = unit % nmc;
-    C2* acc = jb.K3part + (size_t)unit * 2 * P;
-    zero_fields(acc, 2 * P);
+    float* K = reinterpret_cast<float*>(jb.K3part + (size_t)unit * 2 * P);   // [4][P]
+    C2* spec = jb.K3spec + (size_t)unit * 2 * Q;
     {
       const float4* src = reinterpret_cast<const float4*>(psip_s + (size_t)j * P);
       float4* dst = reinterpret_cast<float4*>(psm);
       for (int i4 = threadIdx.x; i4 < P / 4; i4 += blockDim.x) dst[i4] = src[i4];
       __syncthreads();
     }
-    const C2* wf = jb.wfine + (size_t)c * 2 * P;
-    const int m0 = i3_chunk_begin(mc, nmc, M), m1 = i3_chunk_begin(mc + 1, nmc, M);
-    for (int m = m0; m < m1; ++m) {
-      const C2* px = phase + ((size_t)j * M + m) * 2 * n;
+    const C2* __restrict__ wf = jb.wfine + (size_t)c * 2 * P;
+    const int it1 = i3_chunk_begin(mc + 1, nmc, M);
+    bool k_first = true, s_first[2] = {true, true};
+    for (int it = i3_chunk_begin(mc, nmc, M); it < it1;) {
+      const I3Group gr = i3_group_at(it, it1, M);
+      it = gr.next;
+      const C2* px = phase + ((size_t)j * M + gr.m) * 2 * n;
       const C2* py = px + n;
       for (int p = 0; p < 2; ++p) {
         const C2* in = what + ((size_t)c * 4 + p) * P;
@@ -497,25 +501,21 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_smem(const I3Jobs<floa
         for (int idx = threadIdx.x; idx < P; idx += blockDim.x) S[idx] = G[(idx / n) * LS + idx % n];
         __syncthreads();
       }
-      for (int a = 0; a < 4; ++a) {
-        const C2* wa = wf + (size_t)(a >> 1) * P;
-        const C2* Sa = Sig + (size_t)(a >> 1) * P;
-        const bool im = (a & 1) != 0;
-        const float eta = (a == 0) ? 1.f : -1.f;
-        for (int p = 0; p < 2; ++p) {
-          const C2* __restrict__ Sp = Sig + (size_t)p * P;
-          const C2* __restrict__ wv = wa;
-          const C2* __restrict__ sa = Sa;
-          C2* __restrict__ accp = acc + (size_t)p * P;
+      for (int q = gr.q0; q < gr.q1; ++q) {
+        const C2* __restrict__ wq = wf + (size_t)q * P;
+        const C2* Sq = Sig + (size_t)q * P;
+        const float e0 = q == 0 ? 1.f : -1.f;
+        for (int b = 0; b < 4; ++b) {
+          const float* Sb = reinterpret_cast<const float*>(Sig + (size_t)(b >> 1) * P) + (b & 1);
+          const float* __restrict__ wb = reinterpret_cast<const float*>(wf + (size_t)(b >> 1) * P) + (b & 1);
+          float* Kb = K + (size_t)b * P;
+          const float eb = b == 0 ? 1.f : -1.f;
           // element loops with a compile-time trip count, unrolled so each thread keeps several
           // L2 loads in flight (one block per SM leaves few warps to hide their latency)
 #pragma unroll 8
           for (int k = 0; k < kIter; ++k) {
             const int idx = threadIdx.x + k * kThreadsI3Smem;
-            if (kIter * kThreadsI3Smem == P || idx < P) {
-              const C2 z = wv[idx];
-              G[(idx / n) * LS + idx % n] = cscale(Sp[idx], im ? z.y : z.x);
-            }
+            if (kIter * kThreadsI3Smem == P || idx < P) G[(idx / n) * LS + idx % n] = cscale(wq[idx], Sb[2 * idx]);
           }
           __syncthreads();
           fft_lines<n, -1>(G, n, LS, 1, tw);                                           // rows forward
@@ -525,17 +525,41 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_smem(const I3Jobs<floa
           for (int k = 0; k < kIter; ++k) {
             const int idx = threadIdx.x + k * kThreadsI3Smem;
             if (kIter * kThreadsI3Smem == P || idx < P) {
-              const C2 v = G[(idx / n) * LS + idx % n];
-              const C2 s2 = sa[idx];
-              const float f = eta * (im ? s2.y : s2.x);
-              const C2 d = accp[idx];
-              accp[idx] = mk2(fmaT(f, v.x, d.x), fmaT(f, v.y, d.y));
+              const C2 u = G[(idx / n) * LS + idx % n];
+              const C2 s2 = Sq[idx];
+              const float t = fmaT(e0 * s2.x, u.x, -s2.y * u.y);
+              if (k_first) Kb[idx] = t;
+              else atomicAdd(Kb + idx, t);     // no other thread adds to this point
+              const float f = eb * wb[2 * idx], fx = -e0 * f;
+              if (b == 0) {
+                V[idx] = mk2(fx * u.x, f * u.y);
+              } else {
+                const C2 d = V[idx];
+                V[idx] = mk2(fmaT(fx, u.x, d.x), fmaT(f, u.y, d.y));
+              }
             }
           }
           __syncthreads();
         }
+        k_first = false;
+        if (!gr.pair) continue;
+        for (int idx = threadIdx.x; idx < P; idx += blockDim.x) G[(idx / n) * LS + idx % n] = V[idx];
+        __syncthreads();
+        fft_lines<n, -1>(G, n, LS, 1, tw);    // rows
+        fft_lines<n, -1>(G, n, 1, LS, tw);    // columns
+        C2* dst = spec + (size_t)q * Q;
+        const bool first = s_first[q];
+        s_first[q] = false;
+        for (int e = threadIdx.x; e < Q; e += blockDim.x) {
+          const int ix = kcols[e / NQ], iy = kcols[e % NQ];
+          const C2 z = cmulc(G[ix * LS + iy], cmul(px[ix], py[iy]));
+          dst[e] = first ? z : cadd(dst[e], z);
+        }
+        __syncthreads();
       }
     }
+    for (int q = 0; q < 2; ++q)
+      if (s_first[q]) zero_fields(spec + (size_t)q * Q, Q);
   }
 }
 
@@ -561,8 +585,8 @@ __host__ __device__ constexpr bool use_i3_fused() {
 // Its launch shapes per size: (threads, blocks per SM, accumulation mode of k_i3_fused), and the
 // default variant (I3 launch, J = M = 32, on a GB300).  N = 32, 128 cells: 13.6 ms for k_i3_tmem
 // (variant 0; 28.6 ms for the fused kernel with register accumulation that it replaces), 38.8 and 52.2
-// for shapes 1 and 2, 31.2 for k_i3_smem.  N = 48, 64 cells: 38.5 for k_i3_smem, 40.3, 42.5, 56.4 for
-// the fused shapes.  N = 64, 128 cells: 49.8 for k_i3_tmem (88.6 for the warp-local kernel, node by
+// for shapes 1 and 2, 31.2 for k_i3_smem.  N = 48, 64 cells: 25.4 for k_i3_smem (38.5 node by
+// node), 39.0, 40.9, 54.1 for the fused shapes.  N = 64, 128 cells: 49.8 for k_i3_tmem (88.6 for the warp-local kernel, node by
 // node, that it replaces; 57.8 for that kernel in pairs), 101.0, 115.8, 111.6 for shapes 0 to 2, 122.2
 // for k_i3_smem.  N = 16, 128 cells: 3.0 for k_i3_tmem.
 template <int n> struct FusedShapes;
@@ -593,7 +617,7 @@ template <> struct FusedShapes<128> {   // variant 4: k_i3_tmem
 // every global access: 4 CTAs x 1024 threads 239.9 ms; 8 CTAs x 512 threads (two CTAs of
 // different clusters per SM) 255.4 ms; the staged k_i3 294.5 ms.  With the line stages reading
 // and writing the transposed field directly: 219.1 ms (1024 threads, mode 0 below), 192.4 ms
-// (512 threads, mode 1).
+// (512 threads, mode 1 node by node), 132.4 ms (mode 1, nodes in pairs).
 constexpr int kI3Cluster = 4;             // CTAs per cluster
 constexpr int kThreadsI3Cluster = 1024;   // threads per CTA of mode 0
 
@@ -656,6 +680,7 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
   constexpr int A = Split<n>::A, B = Split<n>::B;
   constexpr int TA = (R * B + NT - 1) / NT;          // row tasks (r, t2) per thread in an A stage
   constexpr int TB = (R * A + NT - 1) / NT;          // tasks (r, k1) per thread in a B stage
+  constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
   static_assert(MODE == 0 || R * B == 2 * NT, "register accumulation: two row tasks per thread");
   static_assert(n % kI3Cluster == 0 && (n / 2) % kI3Cluster == 0, "cluster split");
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -823,9 +848,14 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
     for (int idx = tid; idx < n * R; idx += NT) psl[idx] = psp[(idx / R) * n + r0 + idx % R];
     __syncthreads();
     const C2* wf = jb.wfine + (size_t)c * 2 * P;
-    const int m0 = i3_chunk_begin(mc, nmc, M), m1 = i3_chunk_begin(mc + 1, nmc, M);
-    for (int m = m0; m < m1; ++m) {
-      const C2* px = phase + ((size_t)j * M + m) * 2 * n;
+    const int it1 = i3_chunk_begin(mc + 1, nmc, M);
+    C2* spec = jb.K3spec + (size_t)unit * 2 * Q;     // MODE 1
+    bool k_first = true, s_first0 = true, s_first1 = true;
+    for (int it = i3_chunk_begin(mc, nmc, M); it < it1;) {
+      I3Group gr = {it, 0, 2, it + 1, false};        // MODE 0: an item is a node
+      if constexpr (MODE == 1) gr = i3_group_at(it, it1, M);
+      it = gr.next;
+      const C2* px = phase + ((size_t)j * M + gr.m) * 2 * n;
       const C2* py = px + n;
       cluster_sync_global();                         // the previous m's (or unit's) Sig and Gs are read
       // shifted fields, column transforms over this CTA's share of the Xi columns
@@ -882,38 +912,100 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
           }
         }
       } else {
-        const bool first_m = (m == m0);
-        for (int p = 0; p < 2; ++p) {
-          const C2* Sp = Sig + (size_t)p * P + (size_t)r0 * n;
-          C2* accp = acc + (size_t)p * P + (size_t)r0 * n;
-          C2 racc[TA][A];
-          for (int a = 0; a < 4; ++a) {
-            const C2* wa = wf + (size_t)(a >> 1) * P + (size_t)r0 * n;
-            const C2* Sa = Sig + (size_t)(a >> 1) * P + (size_t)r0 * n;
-            const bool im = (a & 1) != 0;
-            const float eta = (a == 0) ? 1.f : -1.f;
-            convolve(
-                [&](int idx) {
-                  const C2 z = wa[idx];
-                  return cscale(Sp[idx], im ? z.y : z.x);
-                },
-                [&](int i, int t1, int idx, C2 v) {
-                  const C2 sv = Sa[idx];
-                  const float f = eta * (im ? sv.y : sv.x);
-                  if (a == 0) racc[i][t1] = mk2(f * v.x, f * v.y);
-                  else racc[i][t1] = mk2(fmaT(f, v.x, racc[i][t1].x), fmaT(f, v.y, racc[i][t1].y));
-                });
+        const int xl0 = rank * XC;                   // this CTA's share of the n / 2 lines ky of Xi
+        auto xi_line = [&](int cc) { return xcols[xl0 + cc]; };
+        for (int q = gr.q0; q < gr.q1; ++q) {
+          const C2* wq = wf + (size_t)q * P + (size_t)r0 * n;
+          const C2* Sq = Sig + (size_t)q * P + (size_t)r0 * n;
+          const float e0 = q == 0 ? 1.f : -1.f;
+          C2 V[TA][A];
+          for (int b = 0; b < 4; ++b) {
+            const float* Sb = reinterpret_cast<const float*>(Sig + (size_t)(b >> 1) * P + (size_t)r0 * n) + (b & 1);
+            const float* wb = reinterpret_cast<const float*>(wf + (size_t)(b >> 1) * P + (size_t)r0 * n) + (b & 1);
+            float* Kb = reinterpret_cast<float*>(acc) + (size_t)b * P + (size_t)r0 * n;
+            const float eb = b == 0 ? 1.f : -1.f;
+            convolve([&](int idx) { return cscale(wq[idx], Sb[2 * idx]); },
+                     [&](int i, int t1, int idx, C2 v) {
+                       const C2 s = Sq[idx];
+                       const float k = fmaT(e0 * s.x, v.x, -s.y * v.y);
+                       if (k_first) Kb[idx] = k;
+                       else atomicAdd(Kb + idx, k);  // no other thread adds to this point
+                       const float f = eb * wb[2 * idx], fx = -e0 * f;
+                       if (b == 0) V[i][t1] = mk2(fx * v.x, f * v.y);
+                       else V[i][t1] = mk2(fmaT(fx, v.x, V[i][t1].x), fmaT(f, v.y, V[i][t1].y));
+                     });
           }
+          k_first = false;
+          if (!gr.pair) continue;
+          // V_q shifted back: forward rows from the registers into the Xi lines of Gs'
 #pragma unroll
           for (int i = 0; i < TA; ++i) {
             const int task = tid + i * NT, r = task / B, t2 = task % B;
+            dft<A, -1>(V[i]);
 #pragma unroll
-            for (int t1 = 0; t1 < A; ++t1) {
-              const int idx = r * n + B * t1 + t2;
-              accp[idx] = first_m ? racc[i][t1] : cadd(accp[idx], racc[i][t1]);
+            for (int k1 = 1; k1 < A; ++k1) V[i][k1] = cmul(V[i][k1], twT[k1 * B + t2]);
+#pragma unroll
+            for (int k1 = 0; k1 < A; ++k1) F[r * LS + B * k1 + t2] = V[i][k1];
+          }
+          __syncthreads();
+#pragma unroll
+          for (int i = 0; i < TB; ++i) {
+            const int task = tid + i * NT;
+            if (TB * NT == R * A || task < R * A) {
+              const int r = task % R, k1 = task / R;
+              C2 b[B];
+#pragma unroll
+              for (int t = 0; t < B; ++t) b[t] = F[r * LS + B * k1 + t];
+              dft<B, -1>(b);
+#pragma unroll
+              for (int t = 0; t < B; ++t)
+                if (xi_t<B>(t)) Gs[(size_t)(B * k1 + t) * n + r0 + r] = b[t];
             }
           }
+          cluster_sync_global();                     // the Xi lines are complete
+          // forward along x on this CTA's Xi lines, times the conjugate phase
+          for (int task = tid; task < XC * B; task += NT) {
+            const int cc = task / B, t2 = task % B, ky = xi_line(cc);
+            C2 v[A];
+#pragma unroll
+            for (int t1 = 0; t1 < A; ++t1) v[t1] = __ldcg(&Gs[(size_t)ky * n + B * t1 + t2]);
+            dft<A, -1>(v);
+#pragma unroll
+            for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
+#pragma unroll
+            for (int k1 = 0; k1 < A; ++k1) F[cc * LS + B * k1 + t2] = v[k1];
+          }
+          __syncthreads();
+          const bool first = q == 0 ? s_first0 : s_first1;
+          if (q == 0) s_first0 = false;
+          else s_first1 = false;
+          for (int task = tid; task < XC * A; task += NT) {
+            const int cc = task % XC, k1 = task / XC, ky = xi_line(cc), sy = xi_slot<n>(ky);
+            C2 b[B];
+#pragma unroll
+            for (int t = 0; t < B; ++t) b[t] = F[cc * LS + B * k1 + t];
+            dft<B, -1>(b);
+            if (sy < 0) continue;
+            const C2 pyy = py[ky];
+#pragma unroll
+            for (int t = 0; t < B; ++t)
+              if (xi_t<B>(t)) {
+                const int sx = xi_slot<n>(B * k1 + t);
+                if (sx >= 0) {
+                  const C2 z = cmulc(b[t], cmul(px[B * k1 + t], pyy));
+                  C2* o = spec + (size_t)q * Q + sx * NQ + sy;
+                  *o = first ? z : cadd(*o, z);
+                }
+              }
+          }
+          cluster_sync_global();                     // Gs is rewritten by the next convolution
         }
+      }
+    }
+    if constexpr (MODE == 1) {
+      for (int e = rank * NT + tid; e < Q; e += kI3Cluster * NT) {
+        if (s_first0) spec[e] = zero2<float>();
+        if (s_first1) spec[Q + e] = zero2<float>();
       }
     }
   }
@@ -1118,8 +1210,8 @@ I3Launch i3_variant(int v) {
     constexpr int NT1 = i3_cluster_threads<n>(1);
     if (v == 1)
       l = {(const void*)k_i3_cluster<n, NT1, 1>, NT1, i3_cluster_smem_bytes<n>(), true,
-           n == 256 ? "cluster of 4 CTAs x 512 threads, register accumulation"
-                    : "cluster of 4 CTAs x 384 threads, register accumulation"};
+           n == 256 ? "node pairs, cluster of 4 CTAs x 512 threads, register accumulation"
+                    : "node pairs, cluster of 4 CTAs x 384 threads, register accumulation"};
     else
       l = {(const void*)k_i3_cluster<n, kThreadsI3Cluster, 0>, kThreadsI3Cluster, i3_cluster_smem_bytes<n>(), true,
            "cluster of 4 CTAs x 1024 threads"};
@@ -1135,14 +1227,14 @@ I3Launch i3_variant(int v) {
     else if (v == 2)
       l = {(const void*)k_i3_fused<n, S::T2, S::B2, S::M2>, S::T2, i3_fused_smem_bytes<n>(), false, names[S::M2]};
     else
-      l = {(const void*)k_i3_smem<n>, kThreadsI3Smem, i3_smem_bytes<n>(), false, "shared-memory, 1024 threads"};
+      l = {(const void*)k_i3_smem<n>, kThreadsI3Smem, i3_smem_bytes<n>(), false, "node pairs, shared-memory, 1024 threads"};
     if constexpr (n == 128) {
       if (v == 4) l = i3_tmem_launch<n>();
     }
   } else if constexpr (std::is_same<T, float>::value && n == 32) {
     l = i3_tmem_launch<n>();
   } else if constexpr (std::is_same<T, float>::value) {
-    l = {(const void*)k_i3_smem<n>, kThreadsI3Smem, i3_smem_bytes<n>(), false, "shared-memory, 1024 threads"};
+    l = {(const void*)k_i3_smem<n>, kThreadsI3Smem, i3_smem_bytes<n>(), false, "node pairs, shared-memory, 1024 threads"};
   } else {
     if (v == 1)
       l = {(const void*)k_i3<n, T, 128, 32768, 6>, 128, i3_staged_smem_bytes<n, T, 32768>(), false,
@@ -1228,8 +1320,8 @@ int i3_variant_count() {
 // cells 135.5 135.1 76.9 77.1; N = 32, 128 cells 646.9 635.0 365.3 371.5; N = 48, 64 cells 861.7 879.5
 // 486.7 499.6; N = 64, 32 cells 746.4 755.8 423.6 433.1; N = 128, 8 cells 926.8 935.8 521.0 533.0 (the
 // fused line stages node by node: 132.9, 625.3, 860.3, 732.5, 885.5 for variant 2).
-// FP32 cluster kernel (I3 launch, J = M = 32): N = 128, 32 cells 219.1 ms (variant 0), 192.4 ms
-// (variant 1); N = 96, 64 cells 217.6 and 208.9 ms.
+// FP32 cluster kernel (I3 launch, J = M = 32): N = 128, 32 cells 216.2 ms (variant 0, node by node),
+// 132.4 ms (variant 1, in pairs; 192.4 node by node); N = 96, 64 cells 217.1 and 141.7 (208.9) ms.
 template <int n, class T>
 int i3_default_variant() {
   if constexpr (std::is_same<T, float>::value && use_i3_fused<n>()) return FusedShapes<n>::DEFAULT;
@@ -1266,7 +1358,8 @@ int i3_variant_concurrency(int v, int grid, int total) {
 template <int n, class T>
 bool i3_variant_paired(int v) {
   if constexpr (std::is_same<T, double>::value) return v >= 2;
-  else return (n == 128 && v == 4) || ((n == 64 || n == 32) && v == 0);
+  else if constexpr (n > 128) return v == 1;
+  else return n <= 32 || v == 3 || v == (n == 128 ? 4 : n == 64 ? 0 : -1);
 }
 
 template <int n, class T>
