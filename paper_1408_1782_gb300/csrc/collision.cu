@@ -326,16 +326,22 @@ cudaError_t alloc_vjp_work(const Tables& t, int nb, VjpWork& vw, int prec, int k
   vw.nb = nb;
   vw.kcap = kcap;
   vw.grid = nsm * bps;
+  // teams (units at a time) of a block of the FP32 kernels with tensor-memory exchanges
+  const bool tm = prec == 1 && (t.n == 32 || t.n == 64 || t.n == 128);
+  const int teams = tm ? (128 / t.n) * (128 / t.n) : 1;
   // about 4 waves of (cell, j, m-chunk) units
-  int nmc = (4 * vw.grid + nb * t.J - 1) / (nb * t.J);
+  const long long cj = (long long)nb * t.J, want_nmc = (4LL * vw.grid * teams + cj - 1) / cj;
+  int nmc = (int)(want_nmc < t.M ? want_nmc : t.M);
   if (nmc < 1) nmc = 1;
-  if (nmc > t.M) nmc = t.M;
   vw.mch = (t.M + nmc - 1) / nmc;
   vw.nmc = (t.M + vw.mch - 1) / vw.mch;
   const size_t nparts = (size_t)nb * t.J * vw.nmc;
-  // per-cell kernels: 7 fields per cell; I3 transpose: 7 + 2 K fields per block (staged form)
+  // per-cell kernels: 7 fields per cell; I3 transpose per block: 3 + 4 K fields (staged; the
+  // shared-memory kernel one less), 6 per team
+  const size_t per_block = tm ? (6 * (size_t)teams > 2 + 4 * (size_t)kcap ? 6 * (size_t)teams : 2 + 4 * (size_t)kcap)
+                              : 3 + 4 * (size_t)kcap;
   size_t ws_fields = 7 * (size_t)nb;
-  if ((7 + 2 * (size_t)kcap) * vw.grid > ws_fields) ws_fields = (7 + 2 * (size_t)kcap) * vw.grid;
+  if (per_block * vw.grid > ws_fields) ws_fields = per_block * vw.grid;
   // per (cell, angle chunk) block: the recomputed forward's I2/I4 kernel 5 fields, the I2/I4
   // transpose 7
   const size_t nch = (size_t)per_cell_chunks(nb, t.J);
@@ -352,6 +358,8 @@ cudaError_t alloc_vjp_work(const Tables& t, int nb, VjpWork& vw, int prec, int k
   QBE_ALLOC(vw.muK2, kc * nb * P * rz);
   QBE_ALLOC(vw.mu4, kc * nb * 2 * P * cz);
   QBE_ALLOC(vw.mu3, kc * nb * 2 * P * cz);
+  QBE_ALLOC(vw.muh, kc * nb * 2 * P * cz);
+  if (tm) QBE_ALLOC(vw.mupl, kc * nb * 4 * P * rz);
   QBE_ALLOC(vw.part_r, kc * nparts * 2 * P * cz);
   const size_t Q = (size_t)(t.n / 2 - 1) * (t.n / 2 - 1);   // kept frequencies (Fourier-space partials)
   QBE_ALLOC(vw.part_s, kc * nparts * 2 * Q * cz);
@@ -362,6 +370,7 @@ cudaError_t alloc_vjp_work(const Tables& t, int nb, VjpWork& vw, int prec, int k
 
 void free_vjp_work(VjpWork& vw) {
   cudaFree(vw.nu); cudaFree(vw.nuf); cudaFree(vw.muD); cudaFree(vw.muK2); cudaFree(vw.mu4); cudaFree(vw.mu3);
+  cudaFree(vw.muh); cudaFree(vw.mupl);
   cudaFree(vw.part_r); cudaFree(vw.part_s); cudaFree(vw.ws);
   vw = VjpWork();
 }

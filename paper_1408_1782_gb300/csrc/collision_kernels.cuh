@@ -1056,6 +1056,19 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
   else *src = mk2((T)sx, (T)sy);
 }
 
+// From 16 units per cell on, eight threads per point: short columns of loads, more of them in flight.
+template <class T>
+void reduce_partials(typename Vec2Of<T>::type* part, double2* sum, typename Vec2Of<T>::type* spec, int nparts, int np,
+                     int nq, int ncells, cudaStream_t s) {
+  if (nparts >= 16) {
+    const int chunks = (np + nq + 31) / 32;
+    k_reduce_k3<T, 8><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, nparts, np, nq, chunks);
+  } else {
+    const int chunks = (np + nq + 255) / 256;
+    k_reduce_k3<T, 1><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, nparts, np, nq, chunks);
+  }
+}
+
 // --------------------------------------------------------------------------
 // Assemble C on the fine grid from D, K2, K3, K4 (Pauli formulas of Sec. 3.1),
 // then FFT, cut to Xi (without the -N/2 line), inverse FFT and sample the
@@ -1504,14 +1517,7 @@ cudaError_t collide_post_n(const Tables& t, CollisionWork& cw, double* c, int nc
   constexpr int nq = 2 * xi_kept<n>() * xi_kept<n>();
   const int nparts = t.J * cw.nmc, nqp = cw.i3_paired ? nq : 0;
   C2* spec = cw.i3_paired ? (C2*)cw.K3spec : nullptr;
-  // from 16 units per cell on, eight threads per point: short columns of loads, more of them in flight
-  if (nparts >= 16) {
-    const int chunks = (np + nqp + 31) / 32;
-    k_reduce_k3<T, 8><<<(unsigned)chunks * ncells, 256, 0, s>>>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, chunks);
-  } else {
-    const int chunks = (np + nqp + 255) / 256;
-    k_reduce_k3<T, 1><<<(unsigned)chunks * ncells, 256, 0, s>>>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, chunks);
-  }
+  reduce_partials<T>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, ncells, s);
   const double2* k3 = cw.K3sum ? cw.K3sum : (const double2*)cw.K3part;
   k_assemble<n, T><<<ncells, kThreads, smem_bytes<n, T>(), s>>>(
       (C2*)cw.wfine, (C2*)cw.Dacc, (T*)cw.K2acc, (C2*)cw.K4acc, k3, cw.K3sum ? (size_t)np : (size_t)nparts * np, spec,

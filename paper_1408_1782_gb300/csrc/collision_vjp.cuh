@@ -39,14 +39,16 @@ __device__ __forceinline__ C2 mul_i(C2 v, typename RealOf<C2>::type s) {   // v 
 // the transpose of the pointwise Pauli assembly.  One block per cell.
 // Outputs: nu[c][2] (direct cotangent of the w pairs), nuf[c] (cotangent of
 // f = 2 w0 - 1), muD[c][2] (pairs (D1,D2),(D3,-)), muK2[c], mu4[c][2] (raw K4
-// pairs), mu3[c][2] (raw K3 pairs).
+// pairs), mu3[c][2] (raw K3 pairs), muh[c][2] (2 pi times the Xi coefficients of
+// the pairs mu_0 + i mu_1, mu_2 + i mu_3).
 // --------------------------------------------------------------------------
 template <int n, class T>
 __global__ void __launch_bounds__(kThreads) k_vjp_seed(
     const double* __restrict__ lam, const typename Vec2Of<T>::type* wfine, const typename Vec2Of<T>::type* Dacc,
     const T* K2acc, const typename Vec2Of<T>::type* K4acc, typename Vec2Of<T>::type* nu, T* nuf,
     typename Vec2Of<T>::type* muD, T* muK2, typename Vec2Of<T>::type* mu4, typename Vec2Of<T>::type* mu3,
-    typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__ gtw) {
+    typename Vec2Of<T>::type* muh, T* mupl, typename Vec2Of<T>::type* ws,
+    const typename Vec2Of<T>::type* __restrict__ gtw) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
@@ -61,6 +63,7 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
   const T invP = (T)(1.0 / (double)P);
   for (int p = 0; p < 2; ++p) {
     C2* M = MU + (size_t)p * P;
+    C2* muhp = muh + ((size_t)c * 2 + p) * P;
     row_pass<n, -1, false, 0>(
         sm, tw,
         [&](int ix, int iy) {
@@ -73,7 +76,9 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
         sm, tw, [&](int ix, int iy) { return M[ix * n + iy]; },
         [&](int ix, int iy, C2 v) {
           const bool keep = in_xi<n>(freq_of_pos<n>(ix)) && in_xi<n>(freq_of_pos<n>(iy));
-          return keep ? cscale(v, invP) : zero2<T>();
+          const C2 z = keep ? cscale(v, invP) : zero2<T>();
+          muhp[ix * n + iy] = cscale(z, (T)(2.0 * kPi));
+          return z;
         },
         [&](int ix, int iy, C2 v) { M[ix * n + iy] = v; });
     row_pass<n, 1, false, 0>(
@@ -129,6 +134,13 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
     // K3_b = eta_b raw_b, C_b has -2 pi K3_b
     mu3c[i] = mk2((T)(-tp * m0), (T)(tp * m1));
     mu3c[P + i] = mk2((T)(tp * m2), (T)(tp * m3));
+    if (mupl) {   // mu3 as planes
+      T* pl = mupl + (size_t)c * 4 * P + i;
+      pl[0] = mu3c[i].x;
+      pl[P] = mu3c[i].y;
+      pl[2 * P] = mu3c[P + i].x;
+      pl[3 * P] = mu3c[P + i].y;
+    }
   }
 }
 
@@ -354,71 +366,47 @@ __global__ void __launch_bounds__(kThreads) k_add_chunks(const T* __restrict__ n
   }
 }
 
-// dst = Psi'_j(x) for the field x(i) = ld(i), i = ix * n + iy: row FFT, column convolution with the
-// angle's psi' table, row IFFT (the forward's convolution); G is the staging field.
-template <int n, class C2, class T, class LD>
-__device__ __forceinline__ void psi_conv(C2* sm, const C2* tw, const T* __restrict__ psp, C2* G, LD ld, C2* dst) {
-  row_pass<n, -1, false, 0>(
-      sm, tw, [&](int ix, int iy) { return ld(ix * n + iy); }, NoMid(),
-      [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-  col_conv_pass<n>(
-      sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, [&](int ix, int iy) { return psp[ix * n + iy]; },
-      [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-  row_pass<n, 1, false, 0>(
-      sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
-      [&](int ix, int iy, C2 v) { dst[ix * n + iy] = v; });
-}
-
 // --------------------------------------------------------------------------
-// I3 transpose (Hu-Ying term).  K3raw_b = sum_{j,m} sum_a eta_a S(w_a) T_ab,
-// T_ab = Psi'(w_a S(w_b)), with cotangents mu_b of K3raw_b:
-//   (i)   nu_a += S^T(eta_a sum_b mu_b T_ab)
-//   (ii)  nu_a += eta_a sum_b Q_ab S(w_b),        Q_ab = Psi'(mu_b S(w_a))
-//   (iii) nu_b += S^T(sum_a eta_a w_a Q_ab)
-// (i) and (iii) are summed before one forward FFT and accumulated in Fourier
-// space with the conjugate phase; (ii) is accumulated in real space.
-// Persistent blocks over units (cell, j, m-chunk); per unit outputs a real
-// partial [2][P] and a spectral partial [2][Q] on the kept frequencies
-// (Q = (n/2 - 1)^2, see build_xi_slots).
-// Several cotangents (K of them, mu3 / part_r / part_s of cotangent k at
-// offsets k * mu_stride, k * part_stride and k * spart_stride) share the shifted fields and the
-// T transforms, which depend on the state only: per (j, m) 8 + 8 K
-// convolutions instead of 16 K.
+// I3 transpose (Hu-Ying term), nodes in pairs as in k_i3_sf (i3_staged_fused.cuh).  With s = S w,
+// U_ab = Psi'(w_a s_b), K3raw_b = sum_a eta_a s_a U_ab (node m) and K3raw_a = S*[sum_b eta_b w_b U_ab]
+// (its partner), cotangents mu_b of K3raw_b and nu = S mu:
+//   Z_ab = Psi'(eta_a mu_b s_a + eta_b nu_a w_b)                 (cotangent of w_a s_b)
+//   R_a += sum_b Z_ab s_b,  R_b += eta_b sum_a nu_a U_ab          (of w, real space)
+//   X_b  = sum_a Z_ab w_a,  X_a += eta_a sum_b mu_b U_ab          (of s, then S* X of w, Fourier space)
+// The middle node of an odd M has no partner and no nu.  With the first index in pairs q (2q, 2q + 1)
+// a pair of nodes takes 8 complex convolutions for U and 8 for Z, 4 shifts and 2 transforms back, half
+// of what its two nodes take one by one.
+// Persistent blocks over units (cell, j, m-chunk); per unit outputs a real-space partial R[4][P] (planes)
+// and a spectral partial [2][Q] on the kept frequencies (Q = (n/2 - 1)^2).
+// Several cotangents (K of them, mu3 / muh / part_r / part_s of cotangent k at offsets k * mu_stride,
+// k * part_stride and k * spart_stride) share the shifted fields and the U convolutions, which depend on
+// the state only: per pair 8 + 8 K convolutions instead of 16 K.
+// Bound by FP64 issue like k_i3_sf.
 // --------------------------------------------------------------------------
+constexpr int kVjpCB = 65536;
 template <int n, class T>
-__global__ void __launch_bounds__(kThreads, 2) k_i3_vjp(
+__global__ void __launch_bounds__(kThreads, 3) k_i3_vjp(
     const typename Vec2Of<T>::type* what, const typename Vec2Of<T>::type* wfine,
-    const typename Vec2Of<T>::type* mu3, typename Vec2Of<T>::type* part_r, typename Vec2Of<T>::type* part_s,
-    typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__ gtw,
-    const T* __restrict__ psip_s, const typename Vec2Of<T>::type* __restrict__ phase, int J, int M, int nmc, int mch,
+    const typename Vec2Of<T>::type* mu3, const typename Vec2Of<T>::type* muh, typename Vec2Of<T>::type* part_r,
+    typename Vec2Of<T>::type* part_s, typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__ gtw,
+    const T* __restrict__ psip_s, const typename Vec2Of<T>::type* __restrict__ phase, int J, int M, int nmc,
     int nunits, int K, size_t mu_stride, size_t part_stride, size_t spart_stride) {
   using C2 = typename Vec2Of<T>::type;
+  using Lines = StagedLines<n, T, kThreads, kVjpCB>;
+  constexpr int A = Split<n>::A, B = Split<n>::B, P = n * n, Q = Lines::Q;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C2* tw = reinterpret_cast<C2*>(smem_raw);
-  C2* sm = tw + n;
-  __shared__ int xcols[n];
-  __shared__ unsigned char xmask[n];
   __shared__ int kslot[n];
-  __shared__ int kcols[n];
-  constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
-  build_xi_slots<n>(kslot, kcols);
-  if (threadIdx.x == 0) {
-    int cnt = 0;
-    for (int pos = 0; pos < n; ++pos) {
-      const int k = freq_of_pos<n>(pos);
-      const bool in = (k < n / 4) || (k >= n - n / 4);
-      xmask[pos] = in ? 1 : 0;
-      if (in) xcols[cnt++] = pos;
-    }
-  }
-  load_twiddles<n>(tw, gtw);
-  constexpr int P = n * n;
-  C2* slot = ws + (size_t)blockIdx.x * (7 + 2 * K) * P;
-  C2* Sig = slot;            // [2] shifted pairs
-  C2* Tp = slot + 2 * P;     // [2] T_{a, pair}
-  C2* Qp = slot + 4 * P;     // [2] Q_{a, pair}
-  C2* G = slot + 6 * P;
-  C2* XZall = slot + 7 * P;  // [K][2] (i)+(iii) real-space terms, pairs by component
+  C2* slot = ws + (size_t)blockIdx.x * (3 + 4 * K) * P;
+  C2* Sig = slot;                                  // [2][P] shifted pairs of the state
+  C2* Nu = slot + 3 * P;                           // [K][2][P] shifted pairs of the cotangents
+  T* X = reinterpret_cast<T*>(slot + (3 + 2 * K) * (size_t)P);   // [K][4][P]
+  Lines ln;
+  ln.twT = reinterpret_cast<C2*>(smem_raw);
+  ln.sm = ln.twT + n;
+  ln.kslot = kslot;
+  ln.G = slot + 2 * P;
+  for (int pos = threadIdx.x; pos < n; pos += kThreads) ln.twT[(pos % A) * B + pos / A] = gtw[pos];
+  build_xi_slots<n>(kslot);
   for (int unit = blockIdx.x; unit < nunits; unit += gridDim.x) {
     const int c = unit / (J * nmc);
     const int j = (unit / nmc) % J;
@@ -427,141 +415,124 @@ __global__ void __launch_bounds__(kThreads, 2) k_i3_vjp(
       zero_fields(part_r + k * part_stride + (size_t)unit * 2 * P, 2 * P);
       zero_fields(part_s + k * spart_stride + (size_t)unit * 2 * Q, 2 * Q);
     }
-    const T* psp = psip_s + (size_t)j * P;
+    const T* __restrict__ psp = psip_s + (size_t)j * P;
     const C2* wf = wfine + (size_t)c * 2 * P;
-    const int m0 = mc * mch, m1 = min(M, m0 + mch);
-    for (int m = m0; m < m1; ++m) {
-      const C2* px = phase + ((size_t)j * M + m) * 2 * n;
+    const int it1 = i3_chunk_begin(mc + 1, nmc, M);
+    for (int it = i3_chunk_begin(mc, nmc, M); it < it1;) {
+      const I3Group gr = i3_group_at(it, it1, M);
+      it = gr.next;
+      const C2* px = phase + ((size_t)j * M + gr.m) * 2 * n;
       const C2* py = px + n;
-      for (int p = 0; p < 2; ++p) {
-        const C2* in = what + ((size_t)c * 4 + p) * P;
-        C2* S = Sig + (size_t)p * P;
-        col_pass_list<n, 1, false, 0, 65536, true>(
-            sm, tw, xcols, n / 2,
-            [&](int ix, int iy) { return xmask[ix] ? cmul(in[ix * n + iy], cmul(px[ix], py[iy])) : zero2<T>(); },
-            NoMid(), [&](int ix, int iy, C2 v) { S[ix * n + iy] = v; });
-        row_pass<n, 1, false, 0, 65536, true>(
-            sm, tw, [&](int ix, int iy) { return xmask[iy] ? S[ix * n + iy] : zero2<T>(); }, NoMid(),
-            [&](int ix, int iy, C2 v) { S[ix * n + iy] = v; });
+      // shifted pairs of the state, then of each cotangent (component 0 of mu3 is -2 pi mu_0)
+      for (int f = 0; f < (gr.pair ? 2 + 2 * K : 2); ++f) {
+        const int k = (f - 2) >> 1, p = f & 1;
+        const C2* in = f < 2 ? what + ((size_t)c * 4 + p) * P : muh + k * mu_stride + ((size_t)c * 2 + p) * P;
+        C2* S = f < 2 ? Sig + (size_t)p * P : Nu + ((size_t)2 * k + p) * P;
+        const T sx = (f >= 2 && p == 0) ? (T)-1 : (T)1;
+        ln.shift(in, px, py, [&](int idx, C2 v) { S[idx] = mk2(sx * v.x, v.y); });
       }
-      zero_fields(XZall, 2 * K * P);
-      for (int a = 0; a < 4; ++a) {
-        const C2* wa = wf + (size_t)(a >> 1) * P;
-        const C2* Sa = Sig + (size_t)(a >> 1) * P;
-        const bool im = (a & 1) != 0;
-        const T eta_a = (a == 0) ? (T)1 : (T)-1;
-        // T_{a, pair} = Psi'(w_a S_pair): the state's, shared by every cotangent
-        for (int p = 0; p < 2; ++p) {
-          const C2* Sp = Sig + (size_t)p * P;
-          psi_conv<n>(sm, tw, psp, G,
-                      [&](int i) {
-                        const C2 z = wa[i];
-                        return cscale(Sp[i], im ? z.y : z.x);
-                      },
-                      Tp + (size_t)p * P);
-        }
-        for (int k = 0; k < K; ++k) {
-          const C2* mu = mu3 + k * mu_stride + (size_t)c * 2 * P;
-          C2* XZ = XZall + (size_t)k * 2 * P;
-          // Q_{a, pair} = Psi'(S_a mu_pair)
-          for (int p = 0; p < 2; ++p) {
-            const C2* mup = mu + (size_t)p * P;
-            psi_conv<n>(sm, tw, psp, G,
-                        [&](int i) {
-                          const C2 sv = Sa[i];
-                          return cscale(mup[i], im ? sv.y : sv.x);
-                        },
-                        Qp + (size_t)p * P);
-          }
-          // pointwise: (i) X_a = eta_a sum_b mu_b T_ab ; (ii) Y_a = eta_a sum_b Q_ab S_b ; (iii) Z_b += eta_a w_a Q_ab
-          C2* accr_a = part_r + k * part_stride + (size_t)unit * 2 * P + (size_t)(a >> 1) * P;
-          C2* XZ_a = XZ + (size_t)(a >> 1) * P;
-          for (int i = threadIdx.x; i < P; i += blockDim.x) {
-            const C2 t0 = Tp[i], t1 = Tp[P + i], q0 = Qp[i], q1 = Qp[P + i];
-            const C2 m0v = mu[i], m1v = mu[P + i];
-            const C2 s0 = Sig[i], s1 = Sig[P + i];
-            const C2 wz = wa[i];
-            const T wv = im ? wz.y : wz.x;
-            const T X = eta_a * (m0v.x * t0.x + m0v.y * t0.y + m1v.x * t1.x + m1v.y * t1.y);
-            const T Y = eta_a * (q0.x * s0.x + q0.y * s0.y + q1.x * s1.x + q1.y * s1.y);
-            if (im) {
-              accr_a[i].y += Y;
-              XZ_a[i].y += X;
-            } else {
-              accr_a[i].x += Y;
-              XZ_a[i].x += X;
-            }
-            const T e = eta_a * wv;
-            XZ[i].x += e * q0.x;
-            XZ[i].y += e * q0.y;
-            XZ[P + i].x += e * q1.x;
-            XZ[P + i].y += e * q1.y;
-          }
-          __syncthreads();
-        }
-      }
-      // S^T: forward FFT of the XZ pairs, times the conjugate phase, accumulated in Fourier space on
-      // the kept frequencies only (column transforms of the kept columns only)
-      for (int k = 0; k < K; ++k) {
-        for (int p = 0; p < 2; ++p) {
-          const C2* src = XZall + (size_t)(2 * k + p) * P;
-          C2* dst = part_s + k * spart_stride + (size_t)unit * 2 * Q + (size_t)p * Q;
-          row_pass<n, -1, false, 0>(
-              sm, tw, [&](int ix, int iy) { return src[ix * n + iy]; }, NoMid(),
-              [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-          col_pass_list<n, -1, false, 0>(
-              sm, tw, kcols, NQ, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
-              [&](int ix, int iy, C2 v) {
-                const int sx = kslot[ix];
-                if (sx < 0) return;
-                const C2 ph = cmul(px[ix], py[iy]);
-                const C2 z = cmulc(v, ph);
-                C2* o = dst + sx * NQ + kslot[iy];
-                C2 d = *o;
-                d.x += z.x;
-                d.y += z.y;
-                *o = d;
+      zero_fields(reinterpret_cast<C2*>(X), 2 * K * P);
+      for (int q = gr.q0; q < gr.q1; ++q) {
+        const C2* wq = wf + (size_t)q * P;
+        const C2* Sq = Sig + (size_t)q * P;
+        const T e0 = q == 0 ? (T)1 : (T)-1;
+        for (int b = 0; b < 4; ++b) {
+          const T* Sb = reinterpret_cast<const T*>(Sig + (size_t)(b >> 1) * P) + (b & 1);
+          const T* wb = reinterpret_cast<const T*>(wf + (size_t)(b >> 1) * P) + (b & 1);
+          const T eb = b == 0 ? (T)1 : (T)-1;
+          const size_t mu_b = ((size_t)c * 2 + (b >> 1)) * P * 2 + (b & 1);   // of component b in the pairs of mu3
+          // U: X_q += eta_q mu_b U, R_b += eta_b nu_q . U
+          ln.convolve(
+              psp, [&](int idx) { return cscale(wq[idx], Sb[2 * idx]); },
+              [&](int idx, C2 v) {
+                for (int k = 0; k < K; ++k) {
+                  const T m = reinterpret_cast<const T*>(mu3 + k * mu_stride)[mu_b + 2 * idx];
+                  T* Xq = X + ((size_t)4 * k + 2 * q) * P + idx;
+                  Xq[0] = fmaT(e0 * m, v.x, Xq[0]);
+                  Xq[P] = fmaT(-m, v.y, Xq[P]);
+                  if (gr.pair) {
+                    const C2 nu = Nu[((size_t)2 * k + q) * P + idx];
+                    T* Rb = reinterpret_cast<T*>(part_r + k * part_stride + (size_t)unit * 2 * P) + (size_t)b * P + idx;
+                    *Rb = fmaT(eb * nu.x, v.x, fmaT(eb * nu.y, v.y, *Rb));
+                  }
+                }
               });
+          // Z per cotangent: R_q += s_b Z, X_b += w_q . Z
+          for (int k = 0; k < K; ++k) {
+            const T* mub = reinterpret_cast<const T*>(mu3 + k * mu_stride) + mu_b;
+            const C2* nuq = Nu + ((size_t)2 * k + q) * P;
+            T* Rq = reinterpret_cast<T*>(part_r + k * part_stride + (size_t)unit * 2 * P) + (size_t)2 * q * P;
+            T* Xb = X + ((size_t)4 * k + b) * P;
+            ln.convolve(
+                psp,
+                [&](int idx) {
+                  const T m = mub[2 * idx];
+                  const C2 s = Sq[idx];
+                  C2 g = mk2(e0 * m * s.x, -m * s.y);
+                  if (gr.pair) {
+                    const C2 nu = nuq[idx];
+                    const T f = eb * wb[2 * idx];
+                    g = mk2(fmaT(f, nu.x, g.x), fmaT(f, nu.y, g.y));
+                  }
+                  return g;
+                },
+                [&](int idx, C2 v) {
+                  const T s = Sb[2 * idx];
+                  const C2 wv = wq[idx];
+                  Rq[idx] = fmaT(s, v.x, Rq[idx]);
+                  Rq[P + idx] = fmaT(s, v.y, Rq[P + idx]);
+                  Xb[idx] = fmaT(wv.x, v.x, fmaT(wv.y, v.y, Xb[idx]));
+                });
+          }
         }
       }
+      for (int k = 0; k < K; ++k)
+        for (int p = 0; p < 2; ++p) {
+          const T* Xp = X + ((size_t)4 * k + 2 * p) * P;
+          ln.shift_back(px, py, part_s + k * spart_stride + (size_t)unit * 2 * Q + (size_t)p * Q, false,
+                        [&](int idx) { return mk2(Xp[idx], Xp[P + idx]); });
+        }
     }
   }
 }
 
 // --------------------------------------------------------------------------
-// I3 transpose with the transform field resident in shared memory (FP32,
-// n <= 128), the counterpart of k_i3_smem.  Each convolution's epilogue adds
-// its terms straight into the accumulators, so T_ab and Q_ab are never stored:
-//   after T_ap = Psi'(w_a S_p):  XZ_a += eta_a mu_p . T_ap           (i)
-//   after Q_ap = Psi'(S_a mu_p): part_r_a += eta_a Q_ap . S_p         (ii)
-//                                XZ_p += eta_a w_a Q_ap               (iii)
-// then S^T of XZ in Fourier space as in k_i3_vjp.
+// The same with the transform field resident in shared memory (FP32, n <= 128),
+// the counterpart of k_i3_smem: each convolution's epilogue adds its terms straight
+// into the accumulators (R in the unit's partial, X in scratch).
 // --------------------------------------------------------------------------
 template <int n>
 __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_vjp_smem(
-    const float2* what, const float2* wfine, const float2* mu3, float2* part_r, float2* part_s, float2* ws,
-    const float2* __restrict__ gtw, const float* __restrict__ psip_s, const float2* __restrict__ phase, int J, int M,
-    int nmc, int mch, int nunits, int K, size_t mu_stride, size_t part_stride, size_t spart_stride) {
+    const float2* what, const float2* wfine, const float2* mu3, const float2* muh, float2* part_r, float2* part_s,
+    float2* ws, const float2* __restrict__ gtw, const float* __restrict__ psip_s, const float2* __restrict__ phase,
+    int J, int M, int nmc, int nunits, int K, size_t mu_stride, size_t part_stride, size_t spart_stride) {
   using C2 = float2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
-  C2* G = tw + n;                       // [n][LS]
-  float* psm = reinterpret_cast<float*>(G + n * (n + 1));   // psi'_j of the current unit, [n][n]
+  C2* G = tw + n;
+  float* psm = reinterpret_cast<float*>(G + n * (n + 1));
   constexpr int LS = n + 1, P = n * n;
+  constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
   constexpr int kIter = (P + kThreadsI3Smem - 1) / kThreadsI3Smem;
   __shared__ unsigned char xmask[n];
   __shared__ int kslot[n];
   __shared__ int kcols[n];
-  constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
-  for (int pos = threadIdx.x; pos < n; pos += blockDim.x) {
-    const int k = freq_of_pos<n>(pos);
-    xmask[pos] = ((k < n / 4) || (k >= n - n / 4)) ? 1 : 0;
-  }
+  for (int pos = threadIdx.x; pos < n; pos += blockDim.x) xmask[pos] = xi_t<Split<n>::B>(pos % Split<n>::B) ? 1 : 0;
   build_xi_slots<n>(kslot, kcols);
   load_twiddles<n>(tw, gtw);
-  C2* slot = ws + (size_t)blockIdx.x * (2 + 2 * K) * P;
-  C2* Sig = slot;            // [2]
-  C2* XZall = slot + 2 * P;  // [K][2]
+  C2* slot = ws + (size_t)blockIdx.x * (2 + 4 * K) * P;
+  C2* Sig = slot;                                                 // [2][P]
+  C2* Nu = slot + 2 * P;                                          // [K][2][P]
+  float* X = reinterpret_cast<float*>(slot + (2 + 2 * K) * (size_t)P);   // [K][4][P]
+  // element loop over the field with a compile-time trip count
+  auto elements = [&](auto body) {
+#pragma unroll 4
+    for (int k = 0; k < kIter; ++k) {
+      const int idx = threadIdx.x + k * kThreadsI3Smem;
+      if (kIter * kThreadsI3Smem == P || idx < P) body(idx, G[(idx / n) * LS + idx % n]);
+    }
+    __syncthreads();
+  };
   for (int unit = blockIdx.x; unit < nunits; unit += gridDim.x) {
     const int c = unit / (J * nmc);
     const int j = (unit / nmc) % J;
@@ -576,109 +547,97 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_vjp_smem(
       for (int i4 = threadIdx.x; i4 < P / 4; i4 += blockDim.x) dst[i4] = src[i4];
       __syncthreads();
     }
-    const C2* wf = wfine + (size_t)c * 2 * P;
-    const int m0 = mc * mch, m1 = min(M, m0 + mch);
-    for (int m = m0; m < m1; ++m) {
-      const C2* px = phase + ((size_t)j * M + m) * 2 * n;
+    const C2* __restrict__ wf = wfine + (size_t)c * 2 * P;
+    auto convolve = [&]() {
+      fft_lines<n, -1>(G, n, LS, 1, tw);
+      fft_conv_lines<n>(G, n, 1, LS, tw, [&](int l, int pos) { return psm[pos * n + l]; });
+      fft_lines<n, 1>(G, n, LS, 1, tw);
+    };
+    const int it1 = i3_chunk_begin(mc + 1, nmc, M);
+    for (int it = i3_chunk_begin(mc, nmc, M); it < it1;) {
+      const I3Group gr = i3_group_at(it, it1, M);
+      it = gr.next;
+      const C2* px = phase + ((size_t)j * M + gr.m) * 2 * n;
       const C2* py = px + n;
-      for (int p = 0; p < 2; ++p) {
-        const C2* in = what + ((size_t)c * 4 + p) * P;
-        for (int idx = threadIdx.x; idx < P; idx += blockDim.x) {
+      for (int f = 0; f < (gr.pair ? 2 + 2 * K : 2); ++f) {
+        const int k = (f - 2) >> 1, p = f & 1;
+        const C2* in = f < 2 ? what + ((size_t)c * 4 + p) * P : muh + k * mu_stride + ((size_t)c * 2 + p) * P;
+        C2* S = f < 2 ? Sig + (size_t)p * P : Nu + ((size_t)2 * k + p) * P;
+        const float sx = (f >= 2 && p == 0) ? -1.f : 1.f;   // component 0 of mu3 is -2 pi mu_0
+        elements([&](int idx, C2& g) {
           const int ix = idx / n, iy = idx % n;
-          G[ix * LS + iy] = (xmask[ix] && xmask[iy]) ? cmul(in[idx], cmul(px[ix], py[iy])) : zero2<float>();
-        }
-        __syncthreads();
+          g = (xmask[ix] && xmask[iy]) ? cmul(in[idx], cmul(px[ix], py[iy])) : zero2<float>();
+        });
         fft_lines<n, 1, true>(G, n, 1, LS, tw);   // shifts: input zero outside Xi x Xi
         fft_lines<n, 1, true>(G, n, LS, 1, tw);
-        C2* S = Sig + (size_t)p * P;
-        for (int idx = threadIdx.x; idx < P; idx += blockDim.x) S[idx] = G[(idx / n) * LS + idx % n];
-        __syncthreads();
+        elements([&](int idx, C2& g) { S[idx] = mk2(sx * g.x, g.y); });
       }
-      zero_fields(XZall, 2 * K * P);
-      for (int a = 0; a < 4; ++a) {
-        const C2* wa = wf + (size_t)(a >> 1) * P;
-        const C2* Sa = Sig + (size_t)(a >> 1) * P;
-        const bool im = (a & 1) != 0;
-        const float eta_a = (a == 0) ? 1.f : -1.f;
-        for (int p = 0; p < 2; ++p) {
-          const C2* Sp = Sig + (size_t)p * P;
-          // which 0: T = Psi'(w_a S_pair), the state's, shared by every cotangent;
-          // which 1: Q = Psi'(S_a mu_pair), once per cotangent
-          for (int which = 0; which < 1 + K; ++which) {
-            const int kq = which - 1;                          // cotangent of a Q transform
-            const C2* __restrict__ src = which == 0 ? Sp : mu3 + kq * mu_stride + (size_t)c * 2 * P + (size_t)p * P;
-            const C2* __restrict__ scl = which == 0 ? wa : Sa;
-#pragma unroll 8
-            for (int k = 0; k < kIter; ++k) {
-              const int idx = threadIdx.x + k * kThreadsI3Smem;
-              if (kIter * kThreadsI3Smem == P || idx < P) {
-                const C2 z = scl[idx];
-                G[(idx / n) * LS + idx % n] = cscale(src[idx], im ? z.y : z.x);
+      zero_fields(reinterpret_cast<C2*>(X), 2 * K * P);
+      for (int q = gr.q0; q < gr.q1; ++q) {
+        const C2* __restrict__ wq = wf + (size_t)q * P;
+        const C2* Sq = Sig + (size_t)q * P;
+        const float e0 = q == 0 ? 1.f : -1.f;
+        for (int b = 0; b < 4; ++b) {
+          const float* Sb = reinterpret_cast<const float*>(Sig + (size_t)(b >> 1) * P) + (b & 1);
+          const float* __restrict__ wb = reinterpret_cast<const float*>(wf + (size_t)(b >> 1) * P) + (b & 1);
+          const float eb = b == 0 ? 1.f : -1.f;
+          const size_t mu_b = ((size_t)c * 2 + (b >> 1)) * P * 2 + (b & 1);
+          // U: X_q += eta_q mu_b U, R_b += eta_b nu_q . U
+          elements([&](int idx, C2& g) { g = cscale(wq[idx], Sb[2 * idx]); });
+          convolve();
+          for (int k = 0; k < K; ++k) {
+            const float* __restrict__ mb = reinterpret_cast<const float*>(mu3 + k * mu_stride) + mu_b;
+            const C2* nuq = Nu + ((size_t)2 * k + q) * P;
+            float* Xq = X + ((size_t)4 * k + 2 * q) * P;
+            float* Rb = reinterpret_cast<float*>(part_r + k * part_stride + (size_t)unit * 2 * P) + (size_t)b * P;
+            elements([&](int idx, C2& g) {
+              const float m = mb[2 * idx];
+              Xq[idx] = fmaf(e0 * m, g.x, Xq[idx]);
+              Xq[P + idx] = fmaf(-m, g.y, Xq[P + idx]);
+              if (gr.pair) {
+                const C2 nu = nuq[idx];
+                Rb[idx] = fmaf(eb * nu.x, g.x, fmaf(eb * nu.y, g.y, Rb[idx]));
               }
-            }
-            __syncthreads();
-            fft_lines<n, -1>(G, n, LS, 1, tw);
-            fft_conv_lines<n>(G, n, 1, LS, tw, [&](int l, int pos) { return psm[pos * n + l]; });
-            fft_lines<n, 1>(G, n, LS, 1, tw);
-            if (which == 0) {
-              // (i): X_a += eta_a mu_pair . T for every cotangent
-              for (int kc = 0; kc < K; ++kc) {
-                const C2* __restrict__ mv_ = mu3 + kc * mu_stride + (size_t)c * 2 * P + (size_t)p * P;
-                float* __restrict__ xz =
-                    reinterpret_cast<float*>(XZall + (size_t)(2 * kc + (a >> 1)) * P) + (im ? 1 : 0);
-#pragma unroll 8
-                for (int k = 0; k < kIter; ++k) {
-                  const int idx = threadIdx.x + k * kThreadsI3Smem;
-                  if (kIter * kThreadsI3Smem == P || idx < P) {
-                    const C2 g = G[(idx / n) * LS + idx % n];
-                    const C2 mv = mv_[idx];
-                    xz[2 * idx] += eta_a * (mv.x * g.x + mv.y * g.y);
-                  }
-                }
+            });
+          }
+          // Z per cotangent: R_q += s_b Z, X_b += w_q . Z
+          for (int k = 0; k < K; ++k) {
+            const float* __restrict__ mb = reinterpret_cast<const float*>(mu3 + k * mu_stride) + mu_b;
+            const C2* nuq = Nu + ((size_t)2 * k + q) * P;
+            float* Rq = reinterpret_cast<float*>(part_r + k * part_stride + (size_t)unit * 2 * P) + (size_t)2 * q * P;
+            float* Xb = X + ((size_t)4 * k + b) * P;
+            elements([&](int idx, C2& g) {
+              const float m = mb[2 * idx];
+              const C2 s = Sq[idx];
+              g = mk2(e0 * m * s.x, -m * s.y);
+              if (gr.pair) {
+                const C2 nu = nuq[idx];
+                const float f = eb * wb[2 * idx];
+                g = mk2(fmaf(f, nu.x, g.x), fmaf(f, nu.y, g.y));
               }
-            } else {
-              // (ii) into the real-space partial, (iii) into Z_pair
-              const C2* __restrict__ sp_ = Sp;
-              const C2* __restrict__ wa_ = wa;
-              float* __restrict__ ar = reinterpret_cast<float*>(part_r + kq * part_stride + (size_t)unit * 2 * P +
-                                                                (size_t)(a >> 1) * P) + (im ? 1 : 0);
-              C2* __restrict__ xzp = XZall + (size_t)(2 * kq + p) * P;
-#pragma unroll 4
-              for (int k = 0; k < kIter; ++k) {
-                const int idx = threadIdx.x + k * kThreadsI3Smem;
-                if (kIter * kThreadsI3Smem == P || idx < P) {
-                  const C2 g = G[(idx / n) * LS + idx % n];
-                  const C2 sp = sp_[idx];
-                  const C2 z = wa_[idx];
-                  ar[2 * idx] += eta_a * (g.x * sp.x + g.y * sp.y);
-                  const float e = eta_a * (im ? z.y : z.x);
-                  C2 o = xzp[idx];
-                  o.x += e * g.x;
-                  o.y += e * g.y;
-                  xzp[idx] = o;
-                }
-              }
-            }
-            __syncthreads();
+            });
+            convolve();
+            elements([&](int idx, C2& g) {
+              const float s = Sb[2 * idx];
+              const C2 wv = wq[idx];
+              Rq[idx] = fmaf(s, g.x, Rq[idx]);
+              Rq[P + idx] = fmaf(s, g.y, Rq[P + idx]);
+              Xb[idx] = fmaf(wv.x, g.x, fmaf(wv.y, g.y, Xb[idx]));
+            });
           }
         }
       }
       for (int kc = 0; kc < K; ++kc) {
         for (int p = 0; p < 2; ++p) {
-          const C2* src = XZall + (size_t)(2 * kc + p) * P;
+          const float* Xp = X + ((size_t)4 * kc + 2 * p) * P;
           C2* dst = part_s + kc * spart_stride + (size_t)unit * 2 * Q + (size_t)p * Q;
-          for (int idx = threadIdx.x; idx < P; idx += blockDim.x) G[(idx / n) * LS + idx % n] = src[idx];
-          __syncthreads();
+          elements([&](int idx, C2& g) { g = mk2(Xp[idx], Xp[P + idx]); });
           fft_lines<n, -1>(G, n, LS, 1, tw);    // rows
           fft_lines<n, -1>(G, n, 1, LS, tw);    // columns
           // accumulated on the kept frequencies only
-          for (int q = threadIdx.x; q < Q; q += blockDim.x) {
-            const int ix = kcols[q / NQ], iy = kcols[q % NQ];
-            const C2 z = cmulc(G[ix * LS + iy], cmul(px[ix], py[iy]));
-            C2 d = dst[q];
-            d.x += z.x;
-            d.y += z.y;
-            dst[q] = d;
+          for (int e = threadIdx.x; e < Q; e += blockDim.x) {
+            const int ix = kcols[e / NQ], iy = kcols[e % NQ];
+            dst[e] = cadd(dst[e], cmulc(G[ix * LS + iy], cmul(px[ix], py[iy])));
           }
           __syncthreads();
         }
@@ -687,19 +646,19 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_vjp_smem(
   }
 }
 
-#include "i3_vjp_wl.cuh"
+#include "i3_vjp_tmem.cuh"
 
 // --------------------------------------------------------------------------
-// Final: nu = direct + I1 + I2/I4 + 2 nu_f (into w0) + sum of the I3 real
-// partials; gradient = 4 E P (nu + IFFT(H) / n^2) with H the sum of the I3
-// spectral partials.  P keeps the kept frequencies only and FFT(IFFT(H)) =
+// Final: nu = direct + I1 + I2/I4 + 2 nu_f (into w0) + R, the reduced I3 real-space
+// partials (planes [4][P], FP64); gradient = 4 E P (nu + IFFT(H) / n^2) with H the
+// reduced I3 spectral partials (k_reduce_k3).  P keeps the kept frequencies only and FFT(IFFT(H)) =
 // n^2 H, so H (stored on those frequencies) is added to FFT(nu) there.
 // One block per cell; writes grad[c][4][N][N] (FP64).
 // --------------------------------------------------------------------------
 template <int n, class T>
 __global__ void __launch_bounds__(kThreads) k_vjp_final(
-    const typename Vec2Of<T>::type* nu, const T* nuf, const typename Vec2Of<T>::type* part_r,
-    const typename Vec2Of<T>::type* part_s, int nparts, typename Vec2Of<T>::type* ws,
+    const typename Vec2Of<T>::type* nu, const T* nuf, const double* R, size_t r_stride,
+    const typename Vec2Of<T>::type* spec, size_t spec_stride, typename Vec2Of<T>::type* ws,
     const typename Vec2Of<T>::type* __restrict__ gtw, double* grad, int accumulate) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -715,27 +674,15 @@ __global__ void __launch_bounds__(kThreads) k_vjp_final(
   C2* slot = ws + (size_t)blockIdx.x * 5 * P;
   C2* V = slot;            // [2] total real-space cotangent pairs
   C2* F = slot + 2 * P;    // [2] their transforms
-  C2* H = slot + 4 * P;    // [2][Q] spectral sum on the kept frequencies
-  const C2* pr = part_r + (size_t)c * nparts * 2 * P;
-  const C2* ps = part_s + (size_t)c * nparts * 2 * Q;
+  const double* Rc = R + c * r_stride;
+  const C2* H = spec + c * spec_stride;   // [2][Q]
   for (int i = threadIdx.x; i < 2 * P; i += blockDim.x) {
-    double sx = 0, sy = 0;
-    for (int u = 0; u < nparts; ++u) {
-      const C2 a = pr[(size_t)u * 2 * P + i];
-      sx += (double)a.x; sy += (double)a.y;
-    }
+    const int e = i % P;
+    const double* Rp = Rc + (size_t)(i < P ? 0 : 2) * P + e;
     const C2 d = nu[(size_t)c * 2 * P + i];
-    double vx = (double)d.x + sx, vy = (double)d.y + sy;
+    double vx = (double)d.x + Rp[0], vy = (double)d.y + Rp[P];
     if (i < P) vx += 2.0 * (double)nuf[(size_t)c * P + i];
     V[i] = mk2((T)vx, (T)vy);
-  }
-  for (int i = threadIdx.x; i < 2 * Q; i += blockDim.x) {
-    double hx = 0, hy = 0;
-    for (int u = 0; u < nparts; ++u) {
-      const C2 b = ps[(size_t)u * 2 * Q + i];
-      hx += (double)b.x; hy += (double)b.y;
-    }
-    H[i] = mk2((T)hx, (T)hy);
   }
   __syncthreads();
   const T invP = (T)(1.0 / (double)P);
@@ -773,6 +720,22 @@ __global__ void __launch_bounds__(kThreads) k_vjp_final(
 
 }  // namespace
 
+// I3 transpose kernels per (n, T): staged in FP64 and above 128 points; in FP32 the teams with
+// tensor-memory exchanges at 32, 64 and 128 points, the element-pass shared-memory kernel at 16 and 96
+// and as variant 1 at 128.
+template <int n, class T>
+constexpr bool vjp_tmem() {
+  return std::is_same<T, float>::value && (n == 32 || n == 64 || n == 128);
+}
+template <int n, class T>
+constexpr bool vjp_smem() {
+  return std::is_same<T, float>::value && (n == 16 || n == 96 || n == 128);
+}
+template <int n, class T>
+constexpr bool vjp_staged() {
+  return !vjp_tmem<n, T>() && !vjp_smem<n, T>();
+}
+
 template <int n, class T>
 void set_vjp_smem_attributes() {
   static unsigned long long done = 0;
@@ -781,19 +744,14 @@ void set_vjp_smem_attributes() {
   cudaFuncSetAttribute(k_vjp_seed<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   cudaFuncSetAttribute(k_i1_vjp<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   cudaFuncSetAttribute(k_i24_vjp<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_i3_vjp<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   cudaFuncSetAttribute(k_vjp_final<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if constexpr (std::is_same<T, float>::value && use_i3_smem<n>())
+  if constexpr (vjp_staged<n, T>())
+    cudaFuncSetAttribute(k_i3_vjp<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)i3_sf_smem_bytes<n, T, kVjpCB>());
+  if constexpr (vjp_smem<n, T>())
     cudaFuncSetAttribute(k_i3_vjp_smem<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)i3_smem_bytes<n>());
-  if constexpr (std::is_same<T, float>::value && n == kWlN)
-    cudaFuncSetAttribute(k_i3_vjp_wl<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)i3_vjp_wl_smem_bytes());
-}
-
-// I3 transpose kernels per (n, T): the warp-local kernel (FP32, 128 points, one cotangent) is variant
-// 0 where it exists, the element-pass shared-memory kernel variant 1; other sizes have one.
-template <int n, class T>
-constexpr int i3_vjp_variant_count() {
-  return (std::is_same<T, float>::value && n == kWlN) ? 2 : 1;
+  if constexpr (vjp_tmem<n, T>())
+    cudaFuncSetAttribute(k_i3_vjp_tmem<n>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TmShape<n>::smem);
 }
 
 // Forward prep/I1/I2+I4 once (the VJP needs wfine, D^, K2, K4^), then per cotangent the seed and the
@@ -836,8 +794,10 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
     T* muK2 = (T*)vw.muK2 + k * r_stride;
     C2* mu4 = (C2*)vw.mu4 + k * c_stride;
     C2* mu3 = (C2*)vw.mu3 + k * c_stride;
+    C2* muh = (C2*)vw.muh + k * c_stride;
+    T* mupl = vw.mupl ? (T*)vw.mupl + k * 2 * c_stride : nullptr;
     k_vjp_seed<n, T><<<ncells, kThreads, sm, s>>>(lam[k], wfine, Dacc, K2acc, K4acc, nu, nuf, muD, muK2, mu4, mu3,
-                                                  ws, tb.tw);
+                                                  muh, mupl, ws, tb.tw);
     // I1 and I2/I4 transposes over (cell, angle chunk) blocks; their per-chunk cotangents go to the
     // forward's chunk-partial buffers (free once per_cell_terms has reduced them) and are summed in
     // chunk order into nu and nuf
@@ -859,31 +819,43 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
   const int nunits = ncells * t.J * vw.nmc;
   const int grid = nunits < vw.grid ? nunits : vw.grid;
   begin(KG_VJP_I3);
-  if constexpr (std::is_same<T, float>::value && use_i3_smem<n>()) {
-    bool wl = false;
-    if constexpr (n == kWlN) {
-      wl = (K == 1 && vw.i3v == 0);
-      if (wl)
-        k_i3_vjp_wl<n><<<grid, kWlThreads, i3_vjp_wl_smem_bytes(), s>>>(
-            what, wfine, (C2*)vw.mu3, (C2*)vw.part_r, (C2*)vw.part_s, ws, tb.tw, tb.psip_s, tb.phase, t.J, t.M,
-            vw.nmc, vw.mch, nunits);
+  bool done = false;
+  if constexpr (vjp_tmem<n, T>()) {
+    if (K == 1 && vw.i3v == 0) {
+      k_i3_vjp_tmem<n><<<grid, TmShape<n>::NT, TmShape<n>::smem, s>>>(
+          what, (const T*)cw.wplane, (const T*)vw.mupl, (C2*)vw.muh, (C2*)vw.part_r, (C2*)vw.part_s, ws, tb.psip_s,
+          tb.phase, t.J, t.M, vw.nmc, nunits);
+      done = true;
     }
-    if (!wl)
+  }
+  if constexpr (vjp_smem<n, T>()) {
+    if (!done)
       k_i3_vjp_smem<n><<<grid, kThreadsI3Smem, i3_smem_bytes<n>(), s>>>(
-          what, wfine, (C2*)vw.mu3, (C2*)vw.part_r, (C2*)vw.part_s, ws, tb.tw, tb.psip_s, tb.phase, t.J, t.M,
-          vw.nmc, vw.mch, nunits, K, c_stride, part_stride, spart_stride);
-  } else
-    k_i3_vjp<n, T><<<grid, kThreads, sm, s>>>(what, wfine, (C2*)vw.mu3, (C2*)vw.part_r, (C2*)vw.part_s, ws, tb.tw,
-                                              tb.psip_s, tb.phase, t.J, t.M, vw.nmc, vw.mch, nunits, K, c_stride,
-                                              part_stride, spart_stride);
+          what, wfine, (C2*)vw.mu3, (C2*)vw.muh, (C2*)vw.part_r, (C2*)vw.part_s, ws, tb.tw, tb.psip_s, tb.phase, t.J,
+          t.M, vw.nmc, nunits, K, c_stride, part_stride, spart_stride);
+    done = true;
+  }
+  if constexpr (vjp_staged<n, T>()) {
+    k_i3_vjp<n, T><<<grid, kThreads, i3_sf_smem_bytes<n, T, kVjpCB>(), s>>>(
+        what, wfine, (C2*)vw.mu3, (C2*)vw.muh, (C2*)vw.part_r, (C2*)vw.part_s, ws, tb.tw, tb.psip_s, tb.phase, t.J,
+        t.M, vw.nmc, nunits, K, c_stride, part_stride, spart_stride);
+    done = true;
+  }
+  if (!done) return cudaErrorInvalidValue;
   end();
   ++launches;
   begin(KG_VJP);
+  const int units = t.J * vw.nmc;
+  constexpr int np = 2 * n * n, nq = 2 * xi_kept<n>() * xi_kept<n>();
   for (int k = 0; k < K; ++k) {
-    k_vjp_final<n, T><<<ncells, kThreads, sm, s>>>((C2*)vw.nu + k * c_stride, (T*)vw.nuf + k * r_stride,
-                                                   (C2*)vw.part_r + k * part_stride, (C2*)vw.part_s + k * spart_stride,
-                                                   t.J * vw.nmc, ws, tb.tw, grad[k], accumulate);
-    ++launches;
+    C2* pr = (C2*)vw.part_r + k * part_stride;
+    C2* ps = (C2*)vw.part_s + k * spart_stride;
+    reduce_partials<T>(pr, cw.K3sum, ps, units, np, nq, ncells, s);
+    const double* R = cw.K3sum ? (const double*)cw.K3sum : (const double*)pr;
+    k_vjp_final<n, T><<<ncells, kThreads, sm, s>>>((C2*)vw.nu + k * c_stride, (T*)vw.nuf + k * r_stride, R,
+                                                   (cw.K3sum ? (size_t)1 : (size_t)units) * 2 * np, ps,
+                                                   (size_t)units * nq, ws, tb.tw, grad[k], accumulate);
+    launches += 2;
   }
   end();
   return cudaGetLastError();
@@ -893,15 +865,11 @@ template <int n, class T>
 int i3_vjp_blocks_per_sm() {
   set_vjp_smem_attributes<n, T>();
   int b = 0;
-  if constexpr (std::is_same<T, float>::value && n == kWlN) {
-    int b2 = 0;   // the grid serves both variants: the smaller residency of the two
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_i3_vjp_smem<n>, kThreadsI3Smem, i3_smem_bytes<n>());
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b2, k_i3_vjp_wl<n>, kWlThreads, i3_vjp_wl_smem_bytes());
-    if (b2 < b) b = b2;
-  } else if constexpr (std::is_same<T, float>::value && use_i3_smem<n>())
+  if constexpr (vjp_tmem<n, T>()) b = 1;   // a block of 512 threads with the SM's tensor memory (and variant 1: 1)
+  else if constexpr (vjp_smem<n, T>())
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_i3_vjp_smem<n>, kThreadsI3Smem, i3_smem_bytes<n>());
   else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_i3_vjp<n, T>, kThreads, smem_bytes<n, T>());
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_i3_vjp<n, T>, kThreads, i3_sf_smem_bytes<n, T, kVjpCB>());
   return b < 1 ? 1 : b;
 }
 

@@ -278,143 +278,3 @@ __global__ void __launch_bounds__(NT, MINB) k_i3_fused(const I3Jobs<float> jobs,
     __syncthreads();   // psm is reloaded by the next unit
   }
 }
-
-// --------------------------------------------------------------------------
-// Warp-local passes (padded grid of 128 points, 512 threads), used by the I3 transpose.  In the row
-// passes warp w owns rows [8 w, 8 w + 8), in the column passes warp pair g owns columns
-// [16 g, 16 g + 16): their stages synchronise with __syncwarp or a named barrier of the pair, and the
-// block synchronises only where the passes change ownership (rows -> columns, columns -> rows).  Field
-// layout: element (x, y) at x * kWlPitch + y + y / 16 (one pad word per 16 elements, row pitch
-// 146 = 2 mod 16), which keeps every stage's accesses free of bank conflicts under the lane mappings
-// below.
-// --------------------------------------------------------------------------
-constexpr int kWlN = 128, kWlThreads = 512, kWlPitch = 146;
-
-__device__ __forceinline__ int wl_addr(int x, int y) { return x * kWlPitch + y + (y >> 4); }
-
-__device__ __forceinline__ void wl_pair_sync(int g) {   // the two warps of pair g (ids 1..8)
-  asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(64) : "memory");
-}
-
-constexpr int kWlPsiPitch = kWlN + 1;   // psi'_j rows padded: the two half-warps of a column stage
-                                         // read rows 16 apart, which would share banks at pitch 128
-constexpr size_t i3_wl_smem_bytes() {    // twiddles (two orders), the skewed field, psi'_j
-  return (size_t)(2 * kWlN + kWlN * kWlPitch) * sizeof(float2) + (size_t)kWlN * kWlPsiPitch * sizeof(float);
-}
-
-// Column pass stages of warp pair g on its 16 columns (tt = thread index within the pair).
-// Stage A: tasks (column c = tt mod 16, t2 = tt / 16 + 4 i); stage B: (c, k1 = tt / 16 + 4 i).
-template <int SIGN>
-__device__ __forceinline__ void wl_cols_stage_a(float2* G, const float2* tw, int g, int tt) {
-  constexpr int A = Split<kWlN>::A, B = Split<kWlN>::B;
-  const int y = 16 * g + (tt & 15);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int t2 = (tt >> 4) + 4 * i;
-    float2 v[A];
-#pragma unroll
-    for (int k = 0; k < A; ++k) v[k] = G[wl_addr(B * k + t2, y)];
-    if (SIGN < 0) {
-      dft<A, -1>(v);
-#pragma unroll
-      for (int k = 1; k < A; ++k) v[k] = cmul(v[k], tw[t2 * A + k]);
-    } else {
-#pragma unroll
-      for (int k = 1; k < A; ++k) v[k] = cmulc(v[k], tw[t2 * A + k]);
-      dft<A, 1>(v);
-    }
-#pragma unroll
-    for (int k = 0; k < A; ++k) G[wl_addr(B * k + t2, y)] = v[k];
-  }
-}
-
-// Row pass stage B of warp w on its 8 rows: tasks (row 8 w + (lane mod 8), k1 = lane / 8 + 4 i).
-template <int SIGN>
-__device__ __forceinline__ void wl_rows_stage_b(float2* G, int w, int lane) {
-  constexpr int B = Split<kWlN>::B;
-  const int x = 8 * w + (lane & 7);
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int k1 = (lane >> 3) + 4 * i;
-    float2 b[B];
-#pragma unroll
-    for (int t = 0; t < B; ++t) b[t] = G[wl_addr(x, B * k1 + t)];
-    dft<B, SIGN>(b);
-#pragma unroll
-    for (int t = 0; t < B; ++t) G[wl_addr(x, B * k1 + t)] = b[t];
-  }
-}
-
-// The shifted pair S = S_jm(w_p) (eq. approxH-JM's spectral shift: the phase-multiplied Xi
-// coefficients of `in`, inverse 2-D transform) into S[x n + y] (natural order) on the warp-local
-// passes.  The coefficients are zero outside Xi x Xi, a quarter of the padded grid: in the permuted
-// order a stage-B line of 16 holds Xi frequencies at t = 0..3, 12..15 only, so the rows are
-// transformed first and only the four Xi rows of each warp (stage B with its first radix-2 stage
-// reduced, stage A), then every column from those rows alone (stage B reduced in the same way, stage
-// A storing S, coalesced along y).  The other rows of G are not touched.  Ends with a block barrier:
-// S is complete for every thread and G is free.
-__device__ __forceinline__ void wl_shift(float2* G, const float2* tw, const float2* twT, const float2* in,
-                                         const float2* px, const float2* py, float2* S, int w, int lane, int g,
-                                         int tt) {
-  using C2 = float2;
-  constexpr int n = kWlN, A = Split<n>::A, B = Split<n>::B;
-  static_assert(A == 8 && B == 16, "Xi pattern of the 8 x 16 split");
-  const int xr0 = 8 * w + 4 * (w & 1);   // this warp's Xi rows: x mod 16 in 0..3 or 12..15
-  {
-    const int x = xr0 + (lane & 3), k1 = lane >> 2;
-    const C2 pxx = px[x];
-    C2 b[B];
-#pragma unroll
-    for (int t = 0; t < B; ++t) {
-      if (t < 4 || t >= 12) {
-        const int y = B * k1 + t;
-        b[t] = cmul(in[x * n + y], cmul(pxx, py[y]));
-      } else {
-        b[t] = zero2<float>();
-      }
-    }
-    dft_xi<B, 1>(b);
-#pragma unroll
-    for (int t = 0; t < B; ++t) G[wl_addr(x, B * k1 + t)] = b[t];
-  }
-  __syncwarp();
-  const int t2r = lane & 15;
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int x = xr0 + (lane >> 4) + 2 * i;
-    C2 v[A];
-#pragma unroll
-    for (int k1 = 0; k1 < A; ++k1) v[k1] = G[wl_addr(x, B * k1 + t2r)];
-#pragma unroll
-    for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2r]);
-    dft<A, 1>(v);
-#pragma unroll
-    for (int t1 = 0; t1 < A; ++t1) G[wl_addr(x, B * t1 + t2r)] = v[t1];
-  }
-  __syncthreads();
-  const int y = 16 * g + (tt & 15);
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int k1 = (tt >> 4) + 4 * i;
-    C2 b[B];
-#pragma unroll
-    for (int t = 0; t < B; ++t) b[t] = (t < 4 || t >= 12) ? G[wl_addr(B * k1 + t, y)] : zero2<float>();
-    dft_xi<B, 1>(b);
-#pragma unroll
-    for (int t = 0; t < B; ++t) G[wl_addr(B * k1 + t, y)] = b[t];
-  }
-  wl_pair_sync(g);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int t2 = (tt >> 4) + 4 * i;
-    C2 v[A];
-#pragma unroll
-    for (int k = 0; k < A; ++k) v[k] = G[wl_addr(B * k + t2, y)];
-#pragma unroll
-    for (int k = 1; k < A; ++k) v[k] = cmulc(v[k], tw[t2 * A + k]);
-    dft<A, 1>(v);
-#pragma unroll
-    for (int k = 0; k < A; ++k) S[(B * k + t2) * n + y] = v[k];
-  }
-  __syncthreads();
-}

@@ -31,28 +31,29 @@
 // Shared memory holds one chunk at a time; no pass copies a chunk through it without transforming.
 #pragma once
 
-template <int n, class T, int NTH, int CB, int MINB>
-__global__ void __launch_bounds__(NTH, MINB)
-    k_i3_sf(const I3Jobs<T> jobs, typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__ gtw) {
+// The passes of one block on its scratch field G', with one chunk sm of shared memory.
+template <int n, class T, int NTH, int CB>
+struct StagedLines {
   using C2 = typename Vec2Of<T>::type;
-  constexpr int A = Split<n>::A, B = Split<n>::B, P = n * n;
-  constexpr int RC = Chunk<n, sizeof(C2), CB>::RC, CC = Chunk<n, sizeof(C2), CB>::CC, LS = Chunk<n, sizeof(C2), CB>::LS;
-  constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C2* twT = reinterpret_cast<C2*>(smem_raw);  // twT[k1 B + t2] = exp(-2 pi i t2 k1 / n) (t2-fastest lanes)
-  C2* sm = twT + n;                           // one chunk: [RC][LS] rows, or [CC][LS] lines of G'
+  static constexpr int A = Split<n>::A, B = Split<n>::B, P = n * n;
+  static constexpr int RC = Chunk<n, sizeof(C2), CB>::RC, CC = Chunk<n, sizeof(C2), CB>::CC,
+                       LS = Chunk<n, sizeof(C2), CB>::LS;
+  static constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
   static_assert(RC == CC, "row and line chunks share the buffer");
-  __shared__ int kslot[n];
-  for (int pos = threadIdx.x; pos < n; pos += NTH) twT[(pos % A) * B + pos / A] = gtw[pos];
-  build_xi_slots<n>(kslot);
-  const int tid = threadIdx.x;
-  C2* slot = ws + (size_t)blockIdx.x * 4 * P;
-  C2* Sig = slot;           // [2][P] shifted pairs s_0 + i s_1, s_2 + i s_3
-  C2* G = slot + 2 * P;     // G'[ky][x] between the passes
-  C2* V = slot + 3 * P;     // sum_b eta_b w_b U_ab of the current pair of a
+  C2* twT;           // twT[k1 B + t2] = exp(-2 pi i t2 k1 / n) (t2-fastest lanes)
+  C2* sm;            // one chunk: [RC][LS] rows, or [CC][LS] lines of G'
+  const int* kslot;  // [n] xi_slot
+  C2* G;             // G'[ky][x] between the passes
 
+  // the li-th of the n / 2 lines ky of Xi: its permuted position
+  __device__ __forceinline__ static int xi_line(int li) {
+    const int k1 = li / (B / 2), t = li % (B / 2);
+    return B * k1 + (t < B / 4 ? t : t + B / 2);
+  }
   // rows of load(idx), idx = row * n + y, into lines of G' (XI: into the Xi lines only)
-  auto rows_forward = [&](auto xi, auto load) {
+  template <bool XI, class LOAD>
+  __device__ __forceinline__ void rows_forward(LOAD load) const {
+    const int tid = threadIdx.x;
     for (int r0 = 0; r0 < n; r0 += RC) {
       for (int task = tid; task < RC * B; task += NTH) {
         const int r = task / B, t2 = task % B;
@@ -75,22 +76,23 @@ __global__ void __launch_bounds__(NTH, MINB)
         dft<B, -1>(b);
 #pragma unroll
         for (int t = 0; t < B; ++t)
-          if (!decltype(xi)::value || xi_t<B>(t)) G[(B * k1 + t) * n + r0 + r] = b[t];
+          if (!XI || xi_t<B>(t)) G[(B * k1 + t) * n + r0 + r] = b[t];
       }
       __syncthreads();
     }
-  };
+  }
   // rows of G' back to real space, handed to epi(idx, v) (XI: only the Xi lines are non-zero)
-  auto rows_inverse = [&](auto xi, auto epi) {
+  template <bool XI, class EPI>
+  __device__ __forceinline__ void rows_inverse(EPI epi) const {
+    const int tid = threadIdx.x;
     for (int r0 = 0; r0 < n; r0 += RC) {
       for (int task = tid; task < RC * A; task += NTH) {
         const int r = task % RC, k1 = task / RC;
         C2* base = sm + r * LS + B * k1;
         C2 b[B];
 #pragma unroll
-        for (int t = 0; t < B; ++t)
-          b[t] = (!decltype(xi)::value || xi_t<B>(t)) ? G[(B * k1 + t) * n + r0 + r] : zero2<T>();
-        if constexpr (decltype(xi)::value) dft_xi<B, 1>(b);
+        for (int t = 0; t < B; ++t) b[t] = (!XI || xi_t<B>(t)) ? G[(B * k1 + t) * n + r0 + r] : zero2<T>();
+        if constexpr (XI) dft_xi<B, 1>(b);
         else dft<B, 1>(b);
 #pragma unroll
         for (int t = 0; t < B; ++t) base[t] = b[t];
@@ -109,13 +111,135 @@ __global__ void __launch_bounds__(NTH, MINB)
       }
       __syncthreads();
     }
-  };
-  // the li-th of the n / 2 lines ky of Xi: its permuted position
-  auto xi_line = [&](int li) {
-    const int k1 = li / (B / 2), t = li % (B / 2);
-    return B * k1 + (t < B / 4 ? t : t + B / 2);
-  };
+  }
+  // stage A of lines in shared memory, back into G' (inverse)
+  __device__ __forceinline__ void lines_out(int nl, int c0, bool xi) const {
+    for (int task = threadIdx.x; task < nl * B; task += NTH) {
+      const int cc = task / B, t2 = task % B, ky = xi ? xi_line(c0 + cc) : c0 + cc;
+      C2 v[A];
+#pragma unroll
+      for (int k1 = 0; k1 < A; ++k1) v[k1] = sm[cc * LS + B * k1 + t2];
+#pragma unroll
+      for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2]);
+      dft<A, 1>(v);
+#pragma unroll
+      for (int t1 = 0; t1 < A; ++t1) G[ky * n + B * t1 + t2] = v[t1];
+    }
+    __syncthreads();
+  }
+  // stage A of lines of G' into shared memory (forward)
+  __device__ __forceinline__ void lines_in(int nl, int c0, bool xi) const {
+    for (int task = threadIdx.x; task < nl * B; task += NTH) {
+      const int cc = task / B, t2 = task % B, ky = xi ? xi_line(c0 + cc) : c0 + cc;
+      C2 v[A];
+#pragma unroll
+      for (int t1 = 0; t1 < A; ++t1) v[t1] = G[ky * n + B * t1 + t2];
+      dft<A, -1>(v);
+#pragma unroll
+      for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
+#pragma unroll
+      for (int k1 = 0; k1 < A; ++k1) sm[cc * LS + B * k1 + t2] = v[k1];
+    }
+    __syncthreads();
+  }
+  // Psi'_j of the field load(idx), handed to epi(idx, v)
+  template <class LOAD, class EPI>
+  __device__ __forceinline__ void convolve(const T* __restrict__ psp, LOAD load, EPI epi) const {
+    rows_forward<false>(load);
+    for (int c0 = 0; c0 < n; c0 += CC) {
+      lines_in(CC, c0, false);
+      for (int task = threadIdx.x; task < CC * A; task += NTH) {
+        const int cc = task % CC, k1 = task / CC;
+        C2* base = sm + cc * LS + B * k1;
+        C2 z[B];
+#pragma unroll
+        for (int t = 0; t < B; ++t) z[t] = base[t];
+        dft<B, -1>(z);
+        T sc[B];
+#pragma unroll
+        for (int t = 0; t < B; ++t) sc[t] = psp[(B * k1 + t) * n + c0 + cc];
+        dft_scaled<B, 1>(z, sc);
+#pragma unroll
+        for (int t = 0; t < B; ++t) base[t] = z[t];
+      }
+      __syncthreads();
+      lines_out(CC, c0, false);
+    }
+    rows_inverse<false>(epi);
+  }
+  // The shift S of the Xi coefficients `in`, handed to epi(idx, v): the Xi lines along x, then the rows
+  template <class EPI>
+  __device__ __forceinline__ void shift(const C2* in, const C2* px, const C2* py, EPI epi) const {
+    for (int c0 = 0; c0 < n / 2; c0 += CC) {
+      const int nl = (n / 2 - c0) < CC ? (n / 2 - c0) : CC;
+      for (int task = threadIdx.x; task < nl * A; task += NTH) {
+        const int cc = task % nl, k1 = task / nl, ky = xi_line(c0 + cc);
+        const C2 pyy = py[ky];
+        C2* base = sm + cc * LS + B * k1;
+        C2 b[B];
+#pragma unroll
+        for (int t = 0; t < B; ++t)
+          b[t] = xi_t<B>(t) ? cmul(in[(B * k1 + t) * n + ky], cmul(px[B * k1 + t], pyy)) : zero2<T>();
+        dft_xi<B, 1>(b);
+#pragma unroll
+        for (int t = 0; t < B; ++t) base[t] = b[t];
+      }
+      __syncthreads();
+      lines_out(nl, c0, true);
+    }
+    rows_inverse<true>(epi);
+  }
+  // The shift back S* of the field load(idx): rows, then the Xi lines along x, times the conjugate phase,
+  // added to (or, with `first`, put into) dst on the kept frequencies
+  template <class LOAD>
+  __device__ __forceinline__ void shift_back(const C2* px, const C2* py, C2* dst, bool first, LOAD load) const {
+    rows_forward<true>(load);
+    for (int c0 = 0; c0 < n / 2; c0 += CC) {
+      const int nl = (n / 2 - c0) < CC ? (n / 2 - c0) : CC;
+      lines_in(nl, c0, true);
+      for (int task = threadIdx.x; task < nl * A; task += NTH) {
+        const int cc = task % nl, k1 = task / nl, ky = xi_line(c0 + cc), sy = kslot[ky];
+        const C2* base = sm + cc * LS + B * k1;
+        C2 b[B];
+#pragma unroll
+        for (int t = 0; t < B; ++t) b[t] = base[t];
+        dft<B, -1>(b);
+        if (sy < 0) continue;
+        const C2 pyy = py[ky];
+#pragma unroll
+        for (int t = 0; t < B; ++t)
+          if (xi_t<B>(t)) {
+            const int sx = kslot[B * k1 + t];
+            if (sx >= 0) {
+              const C2 z = cmulc(b[t], cmul(px[B * k1 + t], pyy));
+              C2* o = dst + sx * NQ + sy;
+              *o = first ? z : cadd(*o, z);
+            }
+          }
+      }
+      __syncthreads();
+    }
+  }
+};
 
+template <int n, class T, int NTH, int CB, int MINB>
+__global__ void __launch_bounds__(NTH, MINB)
+    k_i3_sf(const I3Jobs<T> jobs, typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__ gtw) {
+  using C2 = typename Vec2Of<T>::type;
+  using Lines = StagedLines<n, T, NTH, CB>;
+  constexpr int A = Split<n>::A, B = Split<n>::B, P = n * n, Q = Lines::Q;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int kslot[n];
+  C2* slot = ws + (size_t)blockIdx.x * 4 * P;
+  C2* Sig = slot;           // [2][P] shifted pairs s_0 + i s_1, s_2 + i s_3
+  C2* V = slot + 3 * P;     // sum_b eta_b w_b U_ab of the current pair of a
+  Lines ln;
+  ln.twT = reinterpret_cast<C2*>(smem_raw);
+  ln.sm = ln.twT + n;
+  ln.kslot = kslot;
+  ln.G = slot + 2 * P;
+  for (int pos = threadIdx.x; pos < n; pos += NTH) ln.twT[(pos % A) * B + pos / A] = gtw[pos];
+  build_xi_slots<n>(kslot);
   for (int gunit = blockIdx.x; gunit < jobs.total; gunit += gridDim.x) {
     const I3Job<T>& jb = jobs.job[i3_job_of(jobs, gunit)];
     const int unit = gunit - jb.unit_begin;
@@ -125,7 +249,7 @@ __global__ void __launch_bounds__(NTH, MINB)
     const int c = unit / (J * nmc);
     const int j = (unit / nmc) % J;
     const int mc = unit % nmc;
-    C2* acc = jb.K3part + (size_t)unit * 2 * P;
+    T* K = reinterpret_cast<T*>(jb.K3part + (size_t)unit * 2 * P);   // [4][P]
     C2* spec = jb.K3spec + (size_t)unit * 2 * Q;
     const T* __restrict__ psp = jb.psip_s + (size_t)j * P;
     const C2* wf = jb.wfine + (size_t)c * 2 * P;
@@ -136,152 +260,42 @@ __global__ void __launch_bounds__(NTH, MINB)
       it = gr.next;
       const C2* px = phase + ((size_t)j * M + gr.m) * 2 * n;
       const C2* py = px + n;
-      // shifted pairs: the Xi lines along x, then the rows
       for (int p = 0; p < 2; ++p) {
-        const C2* in = what + ((size_t)c * 4 + p) * P;
-        for (int c0 = 0; c0 < n / 2; c0 += CC) {
-          const int nl = (n / 2 - c0) < CC ? (n / 2 - c0) : CC;
-          for (int task = tid; task < nl * A; task += NTH) {
-            const int cc = task % nl, k1 = task / nl, ky = xi_line(c0 + cc);
-            const C2 pyy = py[ky];
-            C2* base = sm + cc * LS + B * k1;
-            C2 b[B];
-#pragma unroll
-            for (int t = 0; t < B; ++t)
-              b[t] = xi_t<B>(t) ? cmul(in[(B * k1 + t) * n + ky], cmul(px[B * k1 + t], pyy)) : zero2<T>();
-            dft_xi<B, 1>(b);
-#pragma unroll
-            for (int t = 0; t < B; ++t) base[t] = b[t];
-          }
-          __syncthreads();
-          for (int task = tid; task < nl * B; task += NTH) {
-            const int cc = task / B, t2 = task % B, ky = xi_line(c0 + cc);
-            C2 v[A];
-#pragma unroll
-            for (int k1 = 0; k1 < A; ++k1) v[k1] = sm[cc * LS + B * k1 + t2];
-#pragma unroll
-            for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2]);
-            dft<A, 1>(v);
-#pragma unroll
-            for (int t1 = 0; t1 < A; ++t1) G[ky * n + B * t1 + t2] = v[t1];
-          }
-          __syncthreads();
-        }
         C2* S = Sig + (size_t)p * P;
-        rows_inverse(std::true_type{}, [&](int idx, C2 v) { S[idx] = v; });
+        ln.shift(what + ((size_t)c * 4 + p) * P, px, py, [&](int idx, C2 v) { S[idx] = v; });
       }
       for (int q = gr.q0; q < gr.q1; ++q) {
         const C2* wq = wf + (size_t)q * P;
         const C2* Sq = Sig + (size_t)q * P;
         for (int b = 0; b < 4; ++b) {
-          // U_{2q,b} + i U_{2q+1,b} = Psi'((w_2q + i w_2q+1) s_b)
+          // U_{2q,b} + i U_{2q+1,b} = Psi'((w_2q + i w_2q+1) s_b);
+          // K3_b += eta_2q s_2q Re U + eta_2q+1 s_2q+1 Im U;  V_q += eta_b w_b U (x part of q = 0 with the
+          // sign that C_0 has against C_1..C_3, see k_assemble)
           const T* Sb = reinterpret_cast<const T*>(Sig + (size_t)(b >> 1) * P) + (b & 1);
-          rows_forward(std::false_type{}, [&](int idx) { return cscale(wq[idx], Sb[2 * idx]); });
-          // ---- line pass along x: forward, psi'_j, inverse on lines c0..c0+CC of G' ----
-          for (int c0 = 0; c0 < n; c0 += CC) {
-            for (int task = tid; task < CC * B; task += NTH) {
-              const int cc = task / B, t2 = task % B;
-              C2 v[A];
-#pragma unroll
-              for (int t1 = 0; t1 < A; ++t1) v[t1] = G[(c0 + cc) * n + B * t1 + t2];
-              dft<A, -1>(v);
-#pragma unroll
-              for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
-#pragma unroll
-              for (int k1 = 0; k1 < A; ++k1) sm[cc * LS + B * k1 + t2] = v[k1];
-            }
-            __syncthreads();
-            for (int task = tid; task < CC * A; task += NTH) {
-              const int cc = task % CC, k1 = task / CC;
-              C2* base = sm + cc * LS + B * k1;
-              C2 z[B];
-#pragma unroll
-              for (int t = 0; t < B; ++t) z[t] = base[t];
-              dft<B, -1>(z);
-              T sc[B];
-#pragma unroll
-              for (int t = 0; t < B; ++t) sc[t] = psp[(B * k1 + t) * n + c0 + cc];
-              dft_scaled<B, 1>(z, sc);
-#pragma unroll
-              for (int t = 0; t < B; ++t) base[t] = z[t];
-            }
-            __syncthreads();
-            for (int task = tid; task < CC * B; task += NTH) {
-              const int cc = task / B, t2 = task % B;
-              C2 v[A];
-#pragma unroll
-              for (int k1 = 0; k1 < A; ++k1) v[k1] = sm[cc * LS + B * k1 + t2];
-#pragma unroll
-              for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2]);
-              dft<A, 1>(v);
-#pragma unroll
-              for (int t1 = 0; t1 < A; ++t1) G[(c0 + cc) * n + B * t1 + t2] = v[t1];
-            }
-            __syncthreads();
-          }
-          // ---- K3_b += eta_2q s_2q Re U + eta_2q+1 s_2q+1 Im U;  V_q += eta_b w_b U (x part of q = 0
-          // with the sign that C_0 has against C_1..C_3, see k_assemble) ----
-          T* Kb = reinterpret_cast<T*>(acc) + (size_t)b * P;
           const T* wb = reinterpret_cast<const T*>(wf + (size_t)(b >> 1) * P) + (b & 1);
+          T* Kb = K + (size_t)b * P;
           const T e0 = q == 0 ? (T)1 : (T)-1, eb = b == 0 ? (T)1 : (T)-1;
-          rows_inverse(std::false_type{}, [&](int idx, C2 v) {
-            const C2 s = Sq[idx];
-            const T k = fmaT(e0 * s.x, v.x, -s.y * v.y);
-            Kb[idx] = k_first ? k : Kb[idx] + k;
-            if (gr.pair) {
-              const T f = eb * wb[2 * idx], fx = -e0 * f;
-              if (b == 0) {
-                V[idx] = mk2(fx * v.x, f * v.y);
-              } else {
-                const C2 d = V[idx];
-                V[idx] = mk2(fmaT(fx, v.x, d.x), fmaT(f, v.y, d.y));
-              }
-            }
-          });
+          ln.convolve(
+              psp, [&](int idx) { return cscale(wq[idx], Sb[2 * idx]); },
+              [&](int idx, C2 v) {
+                const C2 s = Sq[idx];
+                const T k = fmaT(e0 * s.x, v.x, -s.y * v.y);
+                Kb[idx] = k_first ? k : Kb[idx] + k;
+                if (gr.pair) {
+                  const T f = eb * wb[2 * idx], fx = -e0 * f;
+                  if (b == 0) {
+                    V[idx] = mk2(fx * v.x, f * v.y);
+                  } else {
+                    const C2 d = V[idx];
+                    V[idx] = mk2(fmaT(fx, v.x, d.x), fmaT(f, v.y, d.y));
+                  }
+                }
+              });
         }
         k_first = false;
         if (!gr.pair) continue;
-        // ---- shifted back: rows, then the Xi lines along x, times the conjugate phase ----
-        rows_forward(std::true_type{}, [&](int idx) { return V[idx]; });
-        C2* sq = spec + (size_t)q * Q;
-        const bool first = s_first[q];
+        ln.shift_back(px, py, spec + (size_t)q * Q, s_first[q], [&](int idx) { return V[idx]; });
         s_first[q] = false;
-        for (int c0 = 0; c0 < n / 2; c0 += CC) {
-          const int nl = (n / 2 - c0) < CC ? (n / 2 - c0) : CC;
-          for (int task = tid; task < nl * B; task += NTH) {
-            const int cc = task / B, t2 = task % B, ky = xi_line(c0 + cc);
-            C2 v[A];
-#pragma unroll
-            for (int t1 = 0; t1 < A; ++t1) v[t1] = G[ky * n + B * t1 + t2];
-            dft<A, -1>(v);
-#pragma unroll
-            for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
-#pragma unroll
-            for (int k1 = 0; k1 < A; ++k1) sm[cc * LS + B * k1 + t2] = v[k1];
-          }
-          __syncthreads();
-          for (int task = tid; task < nl * A; task += NTH) {
-            const int cc = task % nl, k1 = task / nl, ky = xi_line(c0 + cc), sy = kslot[ky];
-            const C2* base = sm + cc * LS + B * k1;
-            C2 b[B];
-#pragma unroll
-            for (int t = 0; t < B; ++t) b[t] = base[t];
-            dft<B, -1>(b);
-            if (sy < 0) continue;
-            const C2 pyy = py[ky];
-#pragma unroll
-            for (int t = 0; t < B; ++t)
-              if (xi_t<B>(t)) {
-                const int sx = kslot[B * k1 + t];
-                if (sx >= 0) {
-                  const C2 z = cmulc(b[t], cmul(px[B * k1 + t], pyy));
-                  C2* o = sq + sx * NQ + sy;
-                  *o = first ? z : cadd(*o, z);
-                }
-              }
-          }
-          __syncthreads();
-        }
       }
     }
     for (int q = 0; q < 2; ++q)

@@ -235,12 +235,12 @@ __device__ __forceinline__ int tm_xi_line(int L) {
   return L < n / 4 ? L : L < n / 2 ? L + n / 2 : 0;
 }
 
-// The shifted pair S (phase-multiplied Xi coefficients `in`, inverse 2-D transform) into planes Sx,
-// Sx + P: y lines of the n / 2 lines kx of Xi, then the x lines.  Starts and ends with F free.
+// The shifted pair S (phase-multiplied Xi coefficients `in`, inverse 2-D transform) into planes Sx (times
+// sign_x), Sx + P: y lines of the n / 2 lines kx of Xi, then the x lines.  Starts and ends with F free.
 template <int n>
 __device__ __forceinline__ void tm_shift(const TmLine<n>& ln, float2* F, int L, int team, int tt,
                                          const float2* __restrict__ in, const float2* px, const float2* py,
-                                         float* Sx) {
+                                         float* Sx, float sign_x = 1.f) {
   constexpr int LS = TmShape<n>::LS, H = TmShape<n>::H, JPT = TmShape<n>::JPT, P = n * n, PER = TmXi<n>::PER;
   constexpr int TT = TmShape<n>::TEAM_THREADS, X = n / 2;
   const int kxi = tm_xi_line<n>(L);
@@ -275,7 +275,7 @@ __device__ __forceinline__ void tm_shift(const TmLine<n>& ln, float2* F, int L, 
 #pragma unroll
         for (int t1 = 0; t1 < 32; ++t1) {
           const int idx = (H * t1 + ln.h) * n + L;
-          Sx[idx] = v[t1].x;
+          Sx[idx] = sign_x * v[t1].x;
           Sx[P + idx] = v[t1].y;
         }
       }

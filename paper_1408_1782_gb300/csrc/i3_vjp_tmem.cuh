@@ -1,0 +1,214 @@
+// Transpose of the I3 (Hu-Ying, eq. approxH-JM) term's derivative in FP32 on padded grids of 32, 64
+// and 128 points, one cotangent per product: the node pairs of k_i3_vjp on the teams and
+// tensor-memory exchanges of k_i3_tmem.  Included by collision_vjp.cuh inside its anonymous namespace.
+//
+// Per pair of nodes, q and b the two convolutions U and Z run on one copy of the code.  X_q's sums
+// over b live in tensor memory; every other sum is added in memory at the thread's own points by
+// reductions (no other thread adds there, so the order is fixed): R[4][P] is the unit's real-space
+// partial, X[4][P] the team's scratch, written first by the Z convolutions of the pair's first q.
+// I3 transpose, 128 cells of N = 64, J = M = 32: 258 (node by node, transforms exchanged in
+// shared memory) -> 130.5 ms.
+#pragma once
+
+template <int n>
+__global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_vjp_tmem(
+    const float2* what, const float* wplane, const float* mupl, const float2* muh, float2* part_r, float2* part_s,
+    float2* ws, const float* __restrict__ psip_s, const float2* __restrict__ phase, int J, int M, int nmc,
+    int nunits) {
+  using C2 = float2;
+  using Sh = TmShape<n>;
+  constexpr int P = n * n, H = Sh::H;
+  constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
+  constexpr int CH = 8;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint32_t tm_slot;
+  const uint32_t tm_base = tmem_alloc<Sh::COLS>(&tm_slot);
+  const TmLine<n> ln = tm_setup<n>(smem_raw, tm_base);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, h = ln.h;
+  const int team = (w >> 2) / H * (4 / Sh::SPT) + (w & 3) / Sh::SPT;
+  const int L = 32 * ((w & 3) % Sh::SPT) + lane;
+  const int tt = L + n * h;
+  C2* F = reinterpret_cast<C2*>(smem_raw + Sh::tw_bytes + team * Sh::team_bytes);
+  float* psm = reinterpret_cast<float*>(F + n * Sh::LS);
+  const uint32_t tv = ln.ex + Sh::EX + 64 * h;                     // X_q: real parts, then imaginary parts
+  const int slot = team * gridDim.x + blockIdx.x, nslots = gridDim.x * Sh::TEAMS;
+  float* S = reinterpret_cast<float*>(ws) + (size_t)slot * 12 * P;  // [4][P] shifted components of the state
+  float* Nu = S + 4 * P;                                            // [4][P] of the cotangent
+  float* X = Nu + 4 * P;                                            // [4][P]
+  auto keep_step = [&]() {   // as in k_i3_tmem
+    if constexpr (Sh::TEAMS > 1) __syncthreads();
+  };
+  for (int g0 = 0; g0 < nunits; g0 += nslots) {
+    const bool have = g0 + slot < nunits;
+    const int unit = have ? g0 + slot : 0;
+    const int c = unit / (J * nmc);
+    const int j = (unit / nmc) % J;
+    const int mc = unit % nmc;
+    float* R = reinterpret_cast<float*>(part_r + (size_t)unit * 2 * P);   // [4][P]
+    C2* ps = part_s + (size_t)unit * 2 * Q;
+    if (have) {
+      const float* __restrict__ src = psip_s + (size_t)j * P;
+      for (int i = tt; i < P; i += Sh::TEAM_THREADS) psm[freq_of_pos<n>(i % n) * n + freq_of_pos<n>(i / n)] = src[i];
+#pragma unroll 4
+      for (int t1 = 0; t1 < 32; ++t1)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) R[(size_t)a * P + (H * t1 + h) * n + L] = 0.f;
+    }
+    const float* __restrict__ W = wplane + (size_t)c * 4 * P;
+    const float* __restrict__ Mu = mupl + (size_t)c * 4 * P;
+    int it = i3_chunk_begin(mc, nmc, M);
+    const int it1 = have ? i3_chunk_begin(mc + 1, nmc, M) : it;
+    bool s_first = true;
+    for (;;) {
+      const bool more = it < it1;
+      if constexpr (Sh::TEAMS > 1) {
+        if (!__syncthreads_or(more)) break;
+      } else {
+        if (!more) break;
+      }
+      I3Group gr = {0, 0, 0, it, false};
+      if (more) gr = i3_group_at(it, it1, M);
+      it = gr.next;
+      const C2* px = phase + ((size_t)j * M + gr.m) * 2 * n;
+      const C2* py = px + n;
+      // shifted components of the state, then of the cotangent (component 0 of mu3 is -2 pi mu_0)
+#pragma unroll 1
+      for (int f = 0; f < 4; ++f) {
+        keep_step();
+        const int p = f & 1;
+        if (more && (f < 2 || gr.pair))
+          tm_shift<n>(ln, F, L, team, tt, (f < 2 ? what + ((size_t)c * 4 + p) * P : muh + ((size_t)c * 2 + p) * P), px,
+                      py, (f < 2 ? S : Nu) + (size_t)(2 * p) * P, f == 2 ? -1.f : 1.f);
+      }
+#pragma unroll 1
+      for (int q = 0; q < 2; ++q) {
+        const bool on = q >= gr.q0 && q < gr.q1;
+        const bool first_q = q == gr.q0;
+        const float* __restrict__ Wq = W + (size_t)(2 * q) * P;
+        const float* Sq = S + (size_t)(2 * q) * P;      // rewritten every pair: plain (coherent) loads
+        const float* Nq = Nu + (size_t)(2 * q) * P;
+        const float e0 = q == 0 ? 1.f : -1.f;
+        C2 v[32];
+#pragma unroll 1
+        for (int bz = 0; bz < 8; ++bz) {
+          keep_step();
+          if (!on) continue;
+          const int b = bz >> 1;
+          const bool z = (bz & 1) != 0;
+          const float* __restrict__ wb = W + (size_t)b * P;
+          const float* __restrict__ mb = Mu + (size_t)b * P;
+          const float* Sb = S + (size_t)b * P;
+          const float eb = b == 0 ? 1.f : -1.f;
+          if (!z) {   // U = Psi'((w_2q + i w_2q+1) s_b)
+#pragma unroll
+            for (int t1 = 0; t1 < 32; ++t1) {
+              const int idx = (H * t1 + h) * n + L;
+              const float sb = Sb[idx];
+              v[t1] = mk2(Wq[idx] * sb, Wq[P + idx] * sb);
+            }
+          } else {    // Z = Psi'(mu_b (eta s)_q + eta_b w_b nu_q)
+#pragma unroll
+            for (int t1 = 0; t1 < 32; ++t1) {
+              const int idx = (H * t1 + h) * n + L;
+              const float m = mb[idx];
+              v[t1] = mk2(e0 * m * Sq[idx], -m * Sq[P + idx]);
+              if (gr.pair) {
+                const float f = eb * wb[idx];
+                v[t1] = mk2(fmaf(f, Nq[idx], v[t1].x), fmaf(f, Nq[P + idx], v[t1].y));
+              }
+            }
+          }
+          tm_convolve<n>(ln, F, psm, L, team, v);
+          if (!z) {
+            // X_q += mu_b (eta_2q Re U, eta_2q+1 Im U);  R_b += eta_b nu_q . U
+#pragma unroll
+            for (int i = 0; i < 32; i += CH) {
+              float Vx[CH], Vy[CH], m[CH], nx[CH], ny[CH];
+              if (b > 0) {
+                tmem_ld(tv + i, Vx);
+                tmem_ld(tv + 32 + i, Vy);
+              }
+#pragma unroll
+              for (int t = 0; t < CH; ++t) {
+                const int idx = (H * (i + t) + h) * n + L;
+                m[t] = mb[idx];
+                nx[t] = gr.pair ? Nq[idx] : 0.f;
+                ny[t] = gr.pair ? Nq[P + idx] : 0.f;
+              }
+              if (b > 0) {
+                tmem_wait_ld(Vx);
+                tmem_wait_ld(Vy);
+              } else {
+#pragma unroll
+                for (int t = 0; t < CH; ++t) Vx[t] = Vy[t] = 0.f;
+              }
+#pragma unroll
+              for (int t = 0; t < CH; ++t) {
+                const C2 u = v[i + t];
+                Vx[t] = fmaf(e0 * m[t], u.x, Vx[t]);
+                Vy[t] = fmaf(-m[t], u.y, Vy[t]);
+                if (gr.pair)
+                  atomicAdd(R + (size_t)b * P + (H * (i + t) + h) * n + L, eb * fmaf(nx[t], u.x, ny[t] * u.y));
+              }
+              tmem_st(tv + i, Vx);
+              tmem_st(tv + 32 + i, Vy);
+            }
+            tmem_wait_st();
+          } else {
+            // R_q += s_b Z;  X_b += w_q . Z
+            float* Rq = R + (size_t)(2 * q) * P;
+            float* Xb = X + (size_t)b * P;
+#pragma unroll
+            for (int i = 0; i < 32; i += CH) {
+              float sb[CH], wx[CH], wy[CH];
+#pragma unroll
+              for (int t = 0; t < CH; ++t) {
+                const int idx = (H * (i + t) + h) * n + L;
+                sb[t] = Sb[idx];
+                wx[t] = Wq[idx];
+                wy[t] = Wq[P + idx];
+              }
+#pragma unroll
+              for (int t = 0; t < CH; ++t) {
+                const C2 u = v[i + t];
+                const int idx = (H * (i + t) + h) * n + L;
+                atomicAdd(Rq + idx, sb[t] * u.x);
+                atomicAdd(Rq + P + idx, sb[t] * u.y);
+                const float d = fmaf(wx[t], u.x, wy[t] * u.y);
+                if (first_q) Xb[idx] = d;
+                else atomicAdd(Xb + idx, d);
+              }
+            }
+          }
+        }
+        if (!on) continue;
+        tmem_ld_c<32>(tv, tv + 32, v);
+        tmem_wait_ld_c<32>(v);
+        float* Xq = X + (size_t)(2 * q) * P;
+#pragma unroll
+        for (int t1 = 0; t1 < 32; ++t1) {
+          const int idx = (H * t1 + h) * n + L;
+          atomicAdd(Xq + idx, v[t1].x);
+          atomicAdd(Xq + P + idx, v[t1].y);
+        }
+      }
+      // X shifted back (its sums are in L2: loads that bypass L1)
+#pragma unroll 1
+      for (int p = 0; p < 2; ++p) {
+        keep_step();
+        if (!more) continue;
+        C2 v[32];
+        const float* Xp = X + (size_t)(2 * p) * P;
+#pragma unroll
+        for (int t1 = 0; t1 < 32; ++t1) {
+          const int idx = (H * t1 + h) * n + L;
+          v[t1] = mk2(__ldcg(Xp + idx), __ldcg(Xp + P + idx));
+        }
+        tm_shift_back<n>(ln, F, L, team, tt, v, px, py, ps + (size_t)p * Q, s_first);
+      }
+      s_first = false;
+    }
+    tm_team_sync<n>(team);   // psm is reloaded by the next unit
+  }
+  tmem_free<Sh::COLS>(tm_base);
+}

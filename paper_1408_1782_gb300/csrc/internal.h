@@ -145,7 +145,9 @@ struct VjpWork {
   void* muK2 = nullptr;  // [nb][n*n] (real)
   void* mu4 = nullptr;   // [nb][2][n*n] cotangent of the raw K4 pairs
   void* mu3 = nullptr;   // [nb][2][n*n] cotangent of the raw K3 pairs
-  void* part_r = nullptr;  // [nb*J*nmc][2][n*n] I3 transpose partials, real space
+  void* muh = nullptr;   // [nb][2][n*n] its Xi coefficients (component 0 with the opposite sign)
+  void* mupl = nullptr;  // [nb][4][n*n] mu3 as planes (FP32, n = 32, 64, 128 only)
+  void* part_r = nullptr;  // [nb*J*nmc][2][n*n] I3 transpose partials, real space (four planes)
   void* part_s = nullptr;  // [nb*J*nmc][2][(n/2-1)^2] I3 transpose partials, Fourier space, kept frequencies
   void* ws = nullptr;
 };

@@ -93,3 +93,31 @@ def test_fp32_with_every_team_busy(qbe, N, J, M, ncells):
         out.append(s.collide(w).cpu().numpy())
         s.close()
     assert np.abs(out[1] - out[0]).max() < TOL[1] * np.abs(out[0]).max()
+
+
+def _derivative(s, w, dw):
+    """C'(w) dw: C is cubic in w, so the five-point difference is exact for every step."""
+    f = [s.collide(np.ascontiguousarray(w + h * dw)) for h in (1.0, -1.0, 2.0, -2.0)]
+    return (8.0 * (f[0] - f[1]) - (f[2] - f[3])) / 12.0
+
+
+@pytest.mark.parametrize("N,J,M,ncells", [(8, 4, 1, 2), (8, 4, 2, 3), (16, 4, 5, 2), (16, 16, 6, 24), (32, 2, 3, 2),
+                                          (48, 2, 2, 1), (64, 2, 3, 2), (96, 2, 1, 1), (128, 2, 2, 1)])
+def test_transpose_with_node_pairs(qbe, N, J, M, ncells):
+    """(dC/dW)^T over a lone middle node, odd M, half pairs (few units) and whole pairs: the FP64 product
+    against the forward's own derivative (1e-11 of the sum of absolute products, the adjoint tests'
+    bound), the FP32-split product against the FP64 one."""
+    w = inputs.synthetic_w(N, ncells, seed=30 + N, perturb=0.05)
+    dw = 0.1 * w * inputs.random_field(w.shape, seed=31)
+    lam = inputs.random_field(w.shape, seed=32)
+    s = qbe.Solver(N, ncells, J=J, M=M)
+    g = s.collide_vjp(w, lam)
+    jv = _derivative(s, w, dw)
+    gap = abs(np.sum(lam * jv) - np.sum(g * dw)) / max(np.sum(np.abs(lam * jv)), np.sum(np.abs(g * dw)))
+    assert gap < 1e-11
+    s.close()
+    s = qbe.Solver(N, ncells, J=J, M=M, precision=1)
+    for v in range(s.vjp_i3_variant()[1]):
+        s.set_vjp_i3_variant(v)
+        assert np.abs(s.collide_vjp(w, lam) - g).max() < TOL[1] * np.abs(g).max(), v
+    s.close()
