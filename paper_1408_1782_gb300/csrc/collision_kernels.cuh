@@ -89,6 +89,12 @@ __device__ __forceinline__ void zero_fields(C2* p, int count) {
   __syncthreads();
 }
 
+template <class C2>
+__device__ __forceinline__ void zero_fields_team(C2* p, int count) {
+  for (int i = element_first(); i < count; i += element_stride()) p[i] = mk2((typename RealOf<C2>::type)0, (typename RealOf<C2>::type)0);
+  team_sync();
+}
+
 template <class T>
 __device__ __forceinline__ typename Vec2Of<T>::type zero2() {
   return mk2((T)0, (T)0);
@@ -134,7 +140,7 @@ __device__ __forceinline__ I3Group i3_group_at(int it, int it1, int M) {
 // The coarse DFT is the fine forward FFT of the zero-interleaved samples
 // (its spectrum repeats with period N), scaled by 1/N^2 and cut to Xi.
 // --------------------------------------------------------------------------
-template <int n, class T>
+template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w, typename Vec2Of<T>::type* what,
                                                    typename Vec2Of<T>::type* wfine, T* wplane,
                                                    typename Vec2Of<T>::type* ws,
@@ -145,14 +151,15 @@ __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w,
   C2* sm = tw + n;
   load_twiddles<n>(tw, gtw);
   constexpr int N = n / 2, P = n * n;
-  const int c = blockIdx.x;
+  const int cq = cluster_index(), c = cq >> 2, q = cq & 3;   // one team per cell and coefficient pair
   const double* wc = w + (size_t)c * 4 * N * N;
-  C2* G = ws + (size_t)blockIdx.x * P;
+  C2* G = ws + (size_t)cq * P;
   const T invN2 = (T)(1.0 / ((double)N * N));
-  for (int q = 0; q < 4; ++q) {
+  C2* out = what + ((size_t)c * 4 + q) * P;
+  {
     const int a = (q == 0) ? 0 : (q == 1) ? 2 : (q == 2) ? 1 : 3;
     const int b = (q == 0) ? 1 : (q == 1) ? 3 : (q == 2) ? 2 : -1;
-    row_pass<n, -1, false, 0>(
+    row_pass<n, -1, false, 0, CB>(
         sm, tw,
         [&](int ix, int iy) {
           if ((ix | iy) & 1) return zero2<T>();
@@ -160,22 +167,22 @@ __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w,
           return mk2((T)wc[(a * N + i) * N + j], b >= 0 ? (T)wc[(b * N + i) * N + j] : (T)0);
         },
         NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-    C2* out = what + ((size_t)c * 4 + q) * P;
-    col_pass<n, -1, false, 0>(
-        sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
+    col_pass<n, -1, false, 0, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
         [&](int ix, int iy, C2 v) {
           const bool keep = in_xi<n>(freq_of_pos<n>(ix)) && in_xi<n>(freq_of_pos<n>(iy));
           out[ix * n + iy] = keep ? cscale(v, invN2) : zero2<T>();
         });
   }
-  for (int p = 0; p < 2; ++p) {
-    const C2* in = what + ((size_t)c * 4 + p) * P;
+  if (q < 2) {
+    const int p = q;
+    const C2* in = out;
     C2* out = wfine + ((size_t)c * 2 + p) * P;
-    col_pass<n, 1, false, 0>(
-        sm, tw, [&](int ix, int iy) { return in[ix * n + iy]; }, NoMid(),
+    col_pass<n, 1, false, 0, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&in[ix * n + iy]); }, NoMid(),
         [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-    row_pass<n, 1, false, 0>(
-        sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
+    row_pass<n, 1, false, 0, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
         [&](int ix, int iy, C2 v) {
           out[ix * n + iy] = v;
           if (wplane) {
@@ -191,7 +198,7 @@ __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w,
 // I1 (conservative part): D^_b(sigma) = sum_j' K_j'(sigma) FFT[(2w0-1) IFFT(phi'_j' w_b^)].
 // One block per cell; pairs (w1 + i w2) and (w3).
 // --------------------------------------------------------------------------
-template <int n, class T>
+template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads) k_i1(const typename Vec2Of<T>::type* what,
                                                  const typename Vec2Of<T>::type* wfine, typename Vec2Of<T>::type* Dacc,
                                                  typename Vec2Of<T>::type* ws,
@@ -205,10 +212,10 @@ __global__ void __launch_bounds__(kThreads) k_i1(const typename Vec2Of<T>::type*
   load_twiddles<n>(tw, gtw);
   constexpr int P = n * n;
   // block (cell c, angle chunk ch): angles j' in [J ch / nch, J (ch + 1) / nch); D partial [c][ch]
-  const int c = blockIdx.x / nch, ch = blockIdx.x % nch;
-  C2* G = ws + (size_t)blockIdx.x * P;
-  C2* D = Dacc + (size_t)blockIdx.x * 2 * P;
-  zero_fields(D, 2 * P);
+  const int c = cluster_index() / nch, ch = cluster_index() % nch;
+  C2* G = ws + (size_t)cluster_index() * P;
+  C2* D = Dacc + (size_t)cluster_index() * 2 * P;
+  zero_fields_team(D, 2 * P);
   const C2* wf0 = wfine + (size_t)c * 2 * P;
   for (int jp = J * ch / nch; jp < J * (ch + 1) / nch; ++jp) {
     const T* ph = phip + (size_t)jp * P;
@@ -216,15 +223,15 @@ __global__ void __launch_bounds__(kThreads) k_i1(const typename Vec2Of<T>::type*
     for (int p = 0; p < 2; ++p) {
       const C2* in = what + ((size_t)c * 4 + 2 + p) * P;
       C2* Dp = D + (size_t)p * P;
-      col_pass<n, 1, false, 0>(
+      col_pass<n, 1, false, 0, CB>(
           sm, tw, [&](int ix, int iy) { return cscale(in[ix * n + iy], ph[ix * n + iy]); }, NoMid(),
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-      row_pass<n, 1, true, -1>(
-          sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; },
+      row_pass<n, 1, true, -1, CB>(
+          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); },
           [&](int ix, int iy, C2 v) { return cscale(v, (T)2 * wf0[ix * n + iy].x - (T)1); },
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-      col_pass<n, -1, false, 0>(
-          sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
+      col_pass<n, -1, false, 0, CB>(
+          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
           [&](int ix, int iy, C2 v) {
             const T k = K[ix * n + iy];
             const C2 d = Dp[ix * n + iy];
@@ -240,7 +247,7 @@ __global__ void __launch_bounds__(kThreads) k_i1(const typename Vec2Of<T>::type*
 //   K2  += 2 (pi/J) sum_a eta_a F_{a,j} F_{a,j+J/2}
 //   K4^ += (pi/J) [psi_j FFT((2w0-1) F_{.,j+J/2}) + psi_{j+J/2} FFT((2w0-1) F_{.,j})] / n^2
 // --------------------------------------------------------------------------
-template <int n, class T>
+template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads) k_i24(const typename Vec2Of<T>::type* what,
                                                   const typename Vec2Of<T>::type* wfine, T* K2acc,
                                                   typename Vec2Of<T>::type* K4acc, typename Vec2Of<T>::type* ws,
@@ -253,15 +260,15 @@ __global__ void __launch_bounds__(kThreads) k_i24(const typename Vec2Of<T>::type
   load_twiddles<n>(tw, gtw);
   constexpr int P = n * n;
   // block (cell c, chunk ch) of the J/2 angle pairs; K2, K4 partials [c][ch]
-  const int c = blockIdx.x / nch, ch = blockIdx.x % nch;
-  C2* slot = ws + (size_t)blockIdx.x * 5 * P;
+  const int c = cluster_index() / nch, ch = cluster_index() % nch;
+  C2* slot = ws + (size_t)cluster_index() * 5 * P;
   C2* FA = slot;            // [2][P]
   C2* FB = slot + 2 * P;    // [2][P]
   C2* G = slot + 4 * P;
-  T* K2 = K2acc + (size_t)blockIdx.x * P;
-  C2* K4 = K4acc + (size_t)blockIdx.x * 2 * P;
-  for (int i = threadIdx.x; i < P; i += blockDim.x) K2[i] = (T)0;
-  zero_fields(K4, 2 * P);
+  T* K2 = K2acc + (size_t)cluster_index() * P;
+  C2* K4 = K4acc + (size_t)cluster_index() * 2 * P;
+  for (int i = element_first(); i < P; i += element_stride()) K2[i] = (T)0;
+  zero_fields_team(K4, 2 * P);
   const C2* wf0 = wfine + (size_t)c * 2 * P;
   const T wj = (T)(kPi / J);
   const T scale = (T)(kPi / J / (double)P);
@@ -273,30 +280,30 @@ __global__ void __launch_bounds__(kThreads) k_i24(const typename Vec2Of<T>::type
       for (int h = 0; h < 2; ++h) {
         const T* ps = psi + (size_t)(h == 0 ? j : jp) * P;
         C2* F = (h == 0 ? FA : FB) + (size_t)p * P;
-        col_pass<n, 1, false, 0>(
+        col_pass<n, 1, false, 0, CB>(
             sm, tw, [&](int ix, int iy) { return cscale(in[ix * n + iy], ps[ix * n + iy]); }, NoMid(),
             [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-        row_pass<n, 1, false, 0>(
-            sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
+        row_pass<n, 1, false, 0, CB>(
+            sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
             [&](int ix, int iy, C2 v) { F[ix * n + iy] = v; });
       }
     }
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-      const C2 a0 = FA[i], a1 = FA[P + i], b0 = FB[i], b1 = FB[P + i];
+    for (int i = element_first(); i < P; i += element_stride()) {
+      const C2 a0 = ldc(&FA[i]), a1 = ldc(&FA[P + i]), b0 = ldc(&FB[i]), b1 = ldc(&FB[P + i]);
       const T s = a0.x * b0.x - a0.y * b0.y - a1.x * b1.x - a1.y * b1.y;
       K2[i] = fmaT((T)2 * wj, s, K2[i]);
     }
-    __syncthreads();
+    team_sync();
     for (int p = 0; p < 2; ++p) {
       C2* K4p = K4 + (size_t)p * P;
       for (int h = 0; h < 2; ++h) {
         const C2* F = (h == 0 ? FB : FA) + (size_t)p * P;   // psi_j pairs with F_{j+J/2}
         const T* ps = psi + (size_t)(h == 0 ? j : jp) * P;
-        row_pass<n, -1, false, 0>(
-            sm, tw, [&](int ix, int iy) { return cscale(F[ix * n + iy], (T)2 * wf0[ix * n + iy].x - (T)1); },
+        row_pass<n, -1, false, 0, CB>(
+            sm, tw, [&](int ix, int iy) { return cscale(ldc(&F[ix * n + iy]), (T)2 * wf0[ix * n + iy].x - (T)1); },
             NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-        col_pass<n, -1, false, 0>(
-            sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
+        col_pass<n, -1, false, 0, CB>(
+            sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
             [&](int ix, int iy, C2 v) {
               const T k = scale * ps[ix * n + iy];
               const C2 d = K4p[ix * n + iy];
@@ -635,29 +642,6 @@ __host__ __device__ constexpr int i3_cluster_slab() {   // complex elements of t
 template <int n>
 constexpr size_t i3_cluster_smem_bytes() {   // twiddles (two orders), the slab, psi' columns
   return (size_t)(2 * n + i3_cluster_slab<n>()) * sizeof(float2) + (size_t)n * (n / kI3Cluster) * sizeof(float);
-}
-
-__device__ __forceinline__ int cluster_rank() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return (int)r;
-}
-__device__ __forceinline__ int cluster_index() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
-  return (int)r;
-}
-__device__ __forceinline__ int cluster_count() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(r));
-  return (int)r;
-}
-// All threads of all CTAs of the cluster.  The arrive has release and the wait acquire semantics at
-// cluster scope, so global writes made before it by any thread of the cluster are visible after it
-// to every thread of the cluster; reads of another CTA's writes use ld.global.cg (L2, the point of
-// coherence) so that no stale L1 line can serve them.
-__device__ __forceinline__ void cluster_sync_global() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // The cluster kernel's launch shapes: NT threads per CTA and the accumulation mode.  MODE 0: loop a
@@ -1076,7 +1060,7 @@ void reduce_partials(typename Vec2Of<T>::type* part, double2* sum, typename Vec2
 // after a node-by-node kernel): their Fourier-space parts, added to the spectrum of C inside the projection
 // (C_0 holds -2 pi K3_0 and C_c holds +2 pi K3raw_c; the sign of component 0 is already in spec).
 // --------------------------------------------------------------------------
-template <int n, class T>
+template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>::type* wfine,
                                                        const typename Vec2Of<T>::type* Dacc, const T* K2acc,
                                                        const typename Vec2Of<T>::type* K4acc, const double2* k3,
@@ -1090,18 +1074,18 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
   C2* sm = tw + n;
   load_twiddles<n>(tw, gtw);
   constexpr int N = n / 2, P = n * n;
-  const int c = blockIdx.x;
-  C2* slot = ws + (size_t)blockIdx.x * 6 * P;
+  const int c = cluster_index();
+  C2* slot = ws + (size_t)cluster_index() * 6 * P;
   C2* B0 = slot;
   // D pairs -> slot[0], slot[1]; K4 pairs -> slot[2], slot[3] (inverse 2-D transforms)
   for (int f = 0; f < 4; ++f) {
     const C2* in = (f < 2) ? (Dacc + ((size_t)c * 2 + f) * P) : (K4acc + ((size_t)c * 2 + (f - 2)) * P);
     C2* out = slot + (size_t)f * P;
-    col_pass<n, 1, false, 0>(
+    col_pass<n, 1, false, 0, CB>(
         sm, tw, [&](int ix, int iy) { return in[ix * n + iy]; }, NoMid(),
         [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
-    row_pass<n, 1, false, 0>(
-        sm, tw, [&](int ix, int iy) { return out[ix * n + iy]; }, NoMid(),
+    row_pass<n, 1, false, 0, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&out[ix * n + iy]); }, NoMid(),
         [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
   }
   constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
@@ -1111,14 +1095,15 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
   const T* K2 = K2acc + (size_t)c * P;
   const double tp = 2.0 * kPi;
   const double* k3r = reinterpret_cast<const double*>(k3c);
-  for (int i = threadIdx.x; i < P; i += blockDim.x) {
+  for (int i = element_first(); i < P; i += element_stride()) {
     // node-by-node kernels: pairs (K3_0, K3_1), (K3_2, K3_3); kernels in pairs: four planes
     const double2 k3a = spec ? mk2(k3r[i], k3r[P + i]) : k3c[i];
     const double2 k3b = spec ? mk2(k3r[2 * P + i], k3r[3 * P + i]) : k3c[P + i];
     const double w0 = wf0[i].x, w1 = wf0[i].y, w2 = wf1[i].x, w3 = wf1[i].y;
-    const double D1 = slot[i].x, D2 = slot[i].y, D3 = slot[P + i].x;
-    const double K40 = slot[2 * P + i].x, K41 = -(double)slot[2 * P + i].y;   // eta_b applied
-    const double K42 = -(double)slot[3 * P + i].x, K43 = -(double)slot[3 * P + i].y;
+    const C2 s0 = ldc(&slot[i]), s1 = ldc(&slot[P + i]), s2 = ldc(&slot[2 * P + i]), s3 = ldc(&slot[3 * P + i]);
+    const double D1 = s0.x, D2 = s0.y, D3 = s1.x;
+    const double K40 = s2.x, K41 = -(double)s2.y;   // eta_b applied
+    const double K42 = -(double)s3.x, K43 = -(double)s3.y;
     const double K30 = k3a.x, K31 = -k3a.y, K32 = -k3b.x, K33 = -k3b.y;
     const double k2 = K2[i];
     const double C0 = tp * (k2 * (1.0 - w0) - K30 + w0 * K40 + w1 * K41 + w2 * K42 + w3 * K43);
@@ -1128,18 +1113,18 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
     B0[i] = mk2((T)C0, (T)C1);
     B0[P + i] = mk2((T)C2v, (T)C3);
   }
-  __syncthreads();
+  team_sync();
   const T invP = (T)(1.0 / (double)P);
   double* co = cout + (size_t)c * 4 * N * N;
   C2* H = slot + 2 * P;
   for (int p = 0; p < 2; ++p) {
     const C2* F = B0 + (size_t)p * P;
     const C2* Hs = spec ? spec + c * spec_stride + (size_t)p * Q : nullptr;
-    row_pass<n, -1, false, 0>(
-        sm, tw, [&](int ix, int iy) { return F[ix * n + iy]; }, NoMid(),
+    row_pass<n, -1, false, 0, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&F[ix * n + iy]); }, NoMid(),
         [&](int ix, int iy, C2 v) { H[ix * n + iy] = v; });
-    col_pass<n, -1, true, 1>(
-        sm, tw, [&](int ix, int iy) { return H[ix * n + iy]; },
+    col_pass<n, -1, true, 1, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&H[ix * n + iy]); },
         [&](int ix, int iy, C2 v) {
           const int sx = xi_slot<n>(ix), sy = xi_slot<n>(iy);
           if (sx < 0 || sy < 0) return zero2<T>();
@@ -1150,8 +1135,8 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
           return cscale(v, invP);
         },
         [&](int ix, int iy, C2 v) { H[ix * n + iy] = v; });
-    row_pass<n, 1, false, 0>(
-        sm, tw, [&](int ix, int iy) { return H[ix * n + iy]; }, NoMid(),
+    row_pass<n, 1, false, 0, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&H[ix * n + iy]); }, NoMid(),
         [&](int ix, int iy, C2 v) {
           if (((ix | iy) & 1) == 0) {
             const int i = ix >> 1, j = iy >> 1;
@@ -1164,11 +1149,57 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
 
 }  // namespace
 
+// Chunk bytes of the per-cell kernels: one block per team takes 64 KB chunks; in a team of several
+// blocks a chunk is n / 8 rows or columns, so that up to 8 blocks share a pass.
+constexpr int kCellCB = 65536;
 template <int n, class T>
-size_t smem_bytes() {
-  using C2 = typename Vec2Of<T>::type;
-  return (size_t)(n + Chunk<n, sizeof(C2)>::SMEM_ELEMS) * sizeof(C2);
+constexpr int team_cb() {
+  return n * (n / 8) * 2 * (int)sizeof(T);
 }
+template <int n, class T, int CB>
+size_t cell_smem_bytes() {
+  using C2 = typename Vec2Of<T>::type;
+  return (size_t)(n + Chunk<n, sizeof(C2), CB>::SMEM_ELEMS) * sizeof(C2);
+}
+// Blocks per team of a per-cell kernel over `teams` teams: 1, 2, 4 or 8, the most that stay within three
+// blocks per SM.  The FP64 passes of one cell keep one SM's FP64 unit (two lanes per clock) busy while
+// the others idle, the FP32 ones wait for its latency.  One cell, N = 32 FP64, per C[W]: k_prep 279 ->
+// 31 us, k_i1 390 -> 120 us, k_i24 427 -> 163 us; two steps of it 18.8 -> 14.7 ms.
+inline int cell_team(int teams) {
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  int size = 1;
+  while (size < 8 && 2LL * size * teams <= 3LL * nsm) size *= 2;
+  return size;
+}
+// Launches a per-cell kernel over `teams` teams: `one` with a block each, `several` with a cluster each.
+template <class... K, class... Args>
+cudaError_t launch_cells(void (*one)(K...), void (*several)(K...), int teams, size_t smem_one, size_t smem_several,
+                         cudaStream_t s, Args... args) {
+  const int size = cell_team(teams);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)teams * size);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = size == 1 ? smem_one : smem_several;
+  cfg.stream = s;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = size;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = size == 1 ? 0 : 1;
+  return cudaLaunchKernelEx(&cfg, size == 1 ? one : several, static_cast<K>(args)...);
+}
+#define QBE_CELLS(kernel, teams, s, ...)                                                                     \
+  launch_cells(kernel<n, T, kCellCB>, kernel<n, T, team_cb<n, T>()>, teams, cell_smem_bytes<n, T, kCellCB>(), \
+               cell_smem_bytes<n, T, team_cb<n, T>()>(), s, __VA_ARGS__)
+#define QBE_CELLS_SMEM(kernel)                                                                                 \
+  cudaFuncSetAttribute(kernel<n, T, kCellCB>, cudaFuncAttributeMaxDynamicSharedMemorySize,                   \
+                       (int)cell_smem_bytes<n, T, kCellCB>());                                                \
+  cudaFuncSetAttribute(kernel<n, T, team_cb<n, T>()>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
+                       (int)cell_smem_bytes<n, T, team_cb<n, T>()>())
 
 template <int n, class T, int CB>
 size_t i3_staged_smem_bytes() {
@@ -1269,11 +1300,10 @@ template <int n, class T>
 void set_smem_attributes() {
   static unsigned long long done = 0;
   if (!first_on_device(done)) return;
-  const int sm = (int)smem_bytes<n, T>();
-  cudaFuncSetAttribute(k_prep<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_i1<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_i24<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_assemble<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  QBE_CELLS_SMEM(k_prep);
+  QBE_CELLS_SMEM(k_i1);
+  QBE_CELLS_SMEM(k_i24);
+  QBE_CELLS_SMEM(k_assemble);
   for (int v = 0; v < i3_nvariants<n, T>(); ++v) {
     const I3Launch l = i3_variant<n, T>(v);
     cudaFuncSetAttribute(l.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.smem);
@@ -1390,16 +1420,17 @@ cudaError_t per_cell_terms(const Tables& t, CollisionWork& cw, typename Vec2Of<T
   const TabPtrs<T> tb = tab_ptrs<T>(t);
   const C2* what = (const C2*)cw.what;
   const C2* wfine = (const C2*)cw.wfine;
-  const size_t sm = smem_bytes<n, T>();
   const int nch = cw.nch < 1 ? 1 : cw.nch;
   C2* D = (C2*)(nch > 1 ? cw.Dpart : cw.Dacc);
   T* K2 = (T*)(nch > 1 ? cw.K2part : cw.K2acc);
   C2* K4 = (C2*)(nch > 1 ? cw.K4part : cw.K4acc);
   if (tm) tm->begin(KG_I1, s);
-  k_i1<n, T><<<ncells * nch, kThreads, sm, s>>>(what, wfine, D, ws, tb.tw, tb.phip, tb.Ktab, t.J, nch);
+  cudaError_t e = QBE_CELLS(k_i1, ncells * nch, s, what, wfine, D, ws, tb.tw, tb.phip, tb.Ktab, t.J, nch);
+  if (e != cudaSuccess) return e;
   if (tm) tm->end(s);
   if (tm) tm->begin(KG_I24, s);
-  k_i24<n, T><<<ncells * nch, kThreads, sm, s>>>(what, wfine, K2, K4, ws, tb.tw, tb.psi, t.J, nch);
+  e = QBE_CELLS(k_i24, ncells * nch, s, what, wfine, K2, K4, ws, tb.tw, tb.psi, t.J, nch);
+  if (e != cudaSuccess) return e;
   if (nch > 1) {
     k_reduce_chunks<T><<<(ncells * 5 * n * n + kThreads * 8 - 1) / (kThreads * 8), kThreads, 0, s>>>(
         (const T*)cw.Dpart, (const T*)cw.K2part, (const T*)cw.K4part, (T*)cw.Dacc, (T*)cw.K2acc, (T*)cw.K4acc, nch,
@@ -1423,13 +1454,13 @@ cudaError_t collide_pre_n(const Tables& t, CollisionWork& cw, const double* w, i
   C2* what = (C2*)cw.what;
   C2* wfine = (C2*)cw.wfine;
   C2* ws = (C2*)cw.ws;
-  const size_t sm = smem_bytes<n, T>();
   auto begin = [&](int g) { if (tm) tm->begin(g, s); };
   auto end = [&]() { if (tm) tm->end(s); };
   begin(KG_PREP);
-  k_prep<n, T><<<ncells, kThreads, sm, s>>>(w, what, wfine, (T*)cw.wplane, ws, tb.tw);
+  cudaError_t e = QBE_CELLS(k_prep, 4 * ncells, s, w, what, wfine, (T*)cw.wplane, ws, tb.tw);
   end();
-  cudaError_t e = per_cell_terms<n, T>(t, cw, ws, ncells, s, launches, tm);
+  if (e != cudaSuccess) return e;
+  e = per_cell_terms<n, T>(t, cw, ws, ncells, s, launches, tm);
   if (e != cudaSuccess) return e;
   ++launches;
   return cudaGetLastError();
@@ -1519,10 +1550,11 @@ cudaError_t collide_post_n(const Tables& t, CollisionWork& cw, double* c, int nc
   C2* spec = cw.i3_paired ? (C2*)cw.K3spec : nullptr;
   reduce_partials<T>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, ncells, s);
   const double2* k3 = cw.K3sum ? cw.K3sum : (const double2*)cw.K3part;
-  k_assemble<n, T><<<ncells, kThreads, smem_bytes<n, T>(), s>>>(
-      (C2*)cw.wfine, (C2*)cw.Dacc, (T*)cw.K2acc, (C2*)cw.K4acc, k3, cw.K3sum ? (size_t)np : (size_t)nparts * np, spec,
-      (size_t)nparts * nq, (C2*)cw.ws, tb.tw, c);
+  const cudaError_t e =
+      QBE_CELLS(k_assemble, ncells, s, (C2*)cw.wfine, (C2*)cw.Dacc, (T*)cw.K2acc, (C2*)cw.K4acc, k3,
+                cw.K3sum ? (size_t)np : (size_t)nparts * np, spec, (size_t)nparts * nq, (C2*)cw.ws, tb.tw, c);
   if (tm) tm->end(s);
+  if (e != cudaSuccess) return e;
   launches += 2;
   return cudaGetLastError();
 }

@@ -42,7 +42,7 @@ __device__ __forceinline__ C2 mul_i(C2 v, typename RealOf<C2>::type s) {   // v 
 // pairs), mu3[c][2] (raw K3 pairs), muh[c][2] (2 pi times the Xi coefficients of
 // the pairs mu_0 + i mu_1, mu_2 + i mu_3).
 // --------------------------------------------------------------------------
-template <int n, class T>
+template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads) k_vjp_seed(
     const double* __restrict__ lam, const typename Vec2Of<T>::type* wfine, const typename Vec2Of<T>::type* Dacc,
     const T* K2acc, const typename Vec2Of<T>::type* K4acc, typename Vec2Of<T>::type* nu, T* nuf,
@@ -55,8 +55,8 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
   C2* sm = tw + n;
   load_twiddles<n>(tw, gtw);
   constexpr int N = n / 2, P = n * n;
-  const int c = blockIdx.x;
-  C2* slot = ws + (size_t)blockIdx.x * 6 * P;
+  const int c = cluster_index();
+  C2* slot = ws + (size_t)cluster_index() * 6 * P;
   C2* MU = slot;             // [2] cotangent of C_fine pairs (0,1), (2,3)
   C2* DK = slot + 2 * P;     // [4] D pairs, K4 pairs in real space
   const double* lc = lam + (size_t)c * 4 * N * N;
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
   for (int p = 0; p < 2; ++p) {
     C2* M = MU + (size_t)p * P;
     C2* muhp = muh + ((size_t)c * 2 + p) * P;
-    row_pass<n, -1, false, 0>(
+    row_pass<n, -1, false, 0, CB>(
         sm, tw,
         [&](int ix, int iy) {
           if ((ix | iy) & 1) return zero2<T>();
@@ -72,8 +72,8 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
           return mk2((T)lc[((2 * p) * N + i) * N + j], (T)lc[((2 * p + 1) * N + i) * N + j]);
         },
         NoMid(), [&](int ix, int iy, C2 v) { M[ix * n + iy] = v; });
-    col_pass<n, -1, true, 1>(
-        sm, tw, [&](int ix, int iy) { return M[ix * n + iy]; },
+    col_pass<n, -1, true, 1, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&M[ix * n + iy]); },
         [&](int ix, int iy, C2 v) {
           const bool keep = in_xi<n>(freq_of_pos<n>(ix)) && in_xi<n>(freq_of_pos<n>(iy));
           const C2 z = keep ? cscale(v, invP) : zero2<T>();
@@ -81,18 +81,18 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
           return z;
         },
         [&](int ix, int iy, C2 v) { M[ix * n + iy] = v; });
-    row_pass<n, 1, false, 0>(
-        sm, tw, [&](int ix, int iy) { return M[ix * n + iy]; }, NoMid(),
+    row_pass<n, 1, false, 0, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&M[ix * n + iy]); }, NoMid(),
         [&](int ix, int iy, C2 v) { M[ix * n + iy] = v; });
   }
   for (int f = 0; f < 4; ++f) {
     const C2* in = (f < 2) ? (Dacc + ((size_t)c * 2 + f) * P) : (K4acc + ((size_t)c * 2 + (f - 2)) * P);
     C2* out = DK + (size_t)f * P;
-    col_pass<n, 1, false, 0>(
+    col_pass<n, 1, false, 0, CB>(
         sm, tw, [&](int ix, int iy) { return in[ix * n + iy]; }, NoMid(),
         [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
-    row_pass<n, 1, false, 0>(
-        sm, tw, [&](int ix, int iy) { return out[ix * n + iy]; }, NoMid(),
+    row_pass<n, 1, false, 0, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&out[ix * n + iy]); }, NoMid(),
         [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
   }
   const C2* wf0 = wfine + (size_t)c * 2 * P;
@@ -105,12 +105,14 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
   C2* mu4c = mu4 + (size_t)c * 2 * P;
   C2* mu3c = mu3 + (size_t)c * 2 * P;
   const double tp = 2.0 * kPi;
-  for (int i = threadIdx.x; i < P; i += blockDim.x) {
-    const double m0 = MU[i].x, m1 = MU[i].y, m2 = MU[P + i].x, m3 = MU[P + i].y;
+  for (int i = element_first(); i < P; i += element_stride()) {
+    const C2 mu01 = ldc(&MU[i]), mu23 = ldc(&MU[P + i]);
+    const C2 dk0 = ldc(&DK[i]), dk1 = ldc(&DK[P + i]), dk2 = ldc(&DK[2 * P + i]), dk3 = ldc(&DK[3 * P + i]);
+    const double m0 = mu01.x, m1 = mu01.y, m2 = mu23.x, m3 = mu23.y;
     const double w0 = wf0[i].x, w1 = wf0[i].y, w2 = wf1[i].x, w3 = wf1[i].y;
-    const double D1 = DK[i].x, D2 = DK[i].y, D3 = DK[P + i].x;
-    const double K40 = DK[2 * P + i].x, K41 = -(double)DK[2 * P + i].y;
-    const double K42 = -(double)DK[3 * P + i].x, K43 = -(double)DK[3 * P + i].y;
+    const double D1 = dk0.x, D2 = dk0.y, D3 = dk1.x;
+    const double K40 = dk2.x, K41 = -(double)dk2.y;
+    const double K42 = -(double)dk3.x, K43 = -(double)dk3.y;
     const double k2 = K2[i];
     // C0 = 2pi[K2(1-w0) - K3_0 + w0 K4_0 + w.K4];  C_c = -2 (D x w)_c + 2pi[-K2 w_c - K3_c + w0 K4_c + K4_0 w_c]
     const double g0 = tp * (m0 * (K40 - k2) + m1 * K41 + m2 * K42 + m3 * K43);
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
 // I1 transpose.  D_b = -K'(f A w_b) with A = "multiply by i phi'_j'", K' = "by i K_j'":
 //   nu_f += sum_j' (K' mu_b)(A w_b),   nu_b += -A(f K' mu_b).  One block per cell.
 // --------------------------------------------------------------------------
-template <int n, class T>
+template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads) k_i1_vjp(
     const typename Vec2Of<T>::type* what, const typename Vec2Of<T>::type* wfine,
     const typename Vec2Of<T>::type* muD, typename Vec2Of<T>::type* nu, T* nuf, typename Vec2Of<T>::type* ws,
@@ -162,18 +164,18 @@ __global__ void __launch_bounds__(kThreads) k_i1_vjp(
   constexpr int P = n * n;
   // block (cell c, angle chunk ch); with nch > 1, nu and nuf are per-(cell, chunk) partials (zeroed
   // here, completed by k_i24_vjp, summed by k_add_chunks), with nch = 1 the cell's own accumulators
-  const int c = blockIdx.x / nch, ch = blockIdx.x % nch;
-  C2* slot = ws + (size_t)blockIdx.x * 3 * P;
+  const int c = cluster_index() / nch, ch = cluster_index() % nch;
+  C2* slot = ws + (size_t)cluster_index() * 3 * P;
   C2* Aw = slot;          // A w_pair
   C2* Bm = slot + P;      // K' mu_pair
   C2* G = slot + 2 * P;
   const C2* wf0 = wfine + (size_t)c * 2 * P;
-  C2* nuc = nu + (size_t)blockIdx.x * 2 * P;
-  T* nufc = nuf + (size_t)blockIdx.x * P;
+  C2* nuc = nu + (size_t)cluster_index() * 2 * P;
+  T* nufc = nuf + (size_t)cluster_index() * P;
   if (nch > 1) {
-    zero_fields(nuc, 2 * P);
-    for (int i = threadIdx.x; i < P; i += blockDim.x) nufc[i] = (T)0;
-    __syncthreads();
+    zero_fields_team(nuc, 2 * P);
+    for (int i = element_first(); i < P; i += element_stride()) nufc[i] = (T)0;
+    team_sync();
   }
   const T invP = (T)(1.0 / (double)P);
   for (int jp = J * ch / nch; jp < J * (ch + 1) / nch; ++jp) {
@@ -183,39 +185,39 @@ __global__ void __launch_bounds__(kThreads) k_i1_vjp(
       const C2* in = what + ((size_t)c * 4 + 2 + p) * P;
       const C2* mu = muD + ((size_t)c * 2 + p) * P;
       // Aw = IFFT(i phi' w^)
-      col_pass<n, 1, false, 0>(
+      col_pass<n, 1, false, 0, CB>(
           sm, tw, [&](int ix, int iy) { return mul_i(in[ix * n + iy], ph[ix * n + iy]); }, NoMid(),
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-      row_pass<n, 1, false, 0>(
-          sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
+      row_pass<n, 1, false, 0, CB>(
+          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
           [&](int ix, int iy, C2 v) { Aw[ix * n + iy] = v; });
       // Bm = IFFT(i K FFT(mu))   (K already carries 1/n^2)
-      row_pass<n, -1, false, 0>(
+      row_pass<n, -1, false, 0, CB>(
           sm, tw, [&](int ix, int iy) { return mu[ix * n + iy]; }, NoMid(),
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-      col_pass<n, -1, true, 1>(
-          sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; },
+      col_pass<n, -1, true, 1, CB>(
+          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); },
           [&](int ix, int iy, C2 v) { return mul_i(v, K[ix * n + iy]); },
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-      row_pass<n, 1, false, 0>(
-          sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
+      row_pass<n, 1, false, 0, CB>(
+          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
           [&](int ix, int iy, C2 v) { Bm[ix * n + iy] = v; });
       // nu_f += Re.Re + Im.Im ;  then -A(f Bm) into nu (pair layout of this p)
-      row_pass<n, -1, false, 0>(
+      row_pass<n, -1, false, 0, CB>(
           sm, tw,
           [&](int ix, int iy) {
             const int i = ix * n + iy;
-            const C2 a = Aw[i], b = Bm[i];
+            const C2 a = ldc(&Aw[i]), b = ldc(&Bm[i]);
             nufc[i] += a.x * b.x + a.y * b.y;
             return cscale(b, (T)2 * wf0[i].x - (T)1);
           },
           NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-      col_pass<n, -1, true, 1>(
-          sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; },
+      col_pass<n, -1, true, 1, CB>(
+          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); },
           [&](int ix, int iy, C2 v) { return mul_i(v, -ph[ix * n + iy] * invP); },
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-      row_pass<n, 1, false, 0>(
-          sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
+      row_pass<n, 1, false, 0, CB>(
+          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
           [&](int ix, int iy, C2 v) {
             const int i = ix * n + iy;
             // pair p = 0 carries components (1, 2) -> nu pair 0 .y and nu pair 1 .x; p = 1 carries (3, -)
@@ -236,7 +238,7 @@ __global__ void __launch_bounds__(kThreads) k_i1_vjp(
 //   K4raw_b = (pi/J) sum_{j<J/2} [Psi_j(f F_{b,j'}) + Psi_j'(f F_{b,j})]
 // One block per cell.
 // --------------------------------------------------------------------------
-template <int n, class T>
+template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads) k_i24_vjp(
     const typename Vec2Of<T>::type* what, const typename Vec2Of<T>::type* wfine, const T* muK2,
     const typename Vec2Of<T>::type* mu4, typename Vec2Of<T>::type* nu, T* nuf, typename Vec2Of<T>::type* ws,
@@ -248,8 +250,8 @@ __global__ void __launch_bounds__(kThreads) k_i24_vjp(
   load_twiddles<n>(tw, gtw);
   constexpr int P = n * n;
   // block (cell c, chunk ch of the J/2 angle pairs); nu, nuf as in k_i1_vjp
-  const int c = blockIdx.x / nch, ch = blockIdx.x % nch;
-  C2* slot = ws + (size_t)blockIdx.x * 7 * P;
+  const int c = cluster_index() / nch, ch = cluster_index() % nch;
+  C2* slot = ws + (size_t)cluster_index() * 7 * P;
   C2* FA = slot;             // [2] F_{.,j}
   C2* FB = slot + 2 * P;     // [2] F_{.,j'}
   C2* PM = slot + 4 * P;     // [2] Psi(mu4) for the current direction
@@ -257,8 +259,8 @@ __global__ void __launch_bounds__(kThreads) k_i24_vjp(
   const C2* wf0 = wfine + (size_t)c * 2 * P;
   const T* mk2c = muK2 + (size_t)c * P;
   const C2* m4 = mu4 + (size_t)c * 2 * P;
-  C2* nuc = nu + (size_t)blockIdx.x * 2 * P;
-  T* nufc = nuf + (size_t)blockIdx.x * P;
+  C2* nuc = nu + (size_t)cluster_index() * 2 * P;
+  T* nufc = nuf + (size_t)cluster_index() * P;
   const T wj = (T)(kPi / J);
   const T invP = (T)(1.0 / (double)P);
   const int H = J / 2;
@@ -269,11 +271,11 @@ __global__ void __launch_bounds__(kThreads) k_i24_vjp(
       for (int h = 0; h < 2; ++h) {
         const T* ps = psi + (size_t)(h == 0 ? j : jq) * P;
         C2* F = (h == 0 ? FA : FB) + (size_t)p * P;
-        col_pass<n, 1, false, 0>(
+        col_pass<n, 1, false, 0, CB>(
             sm, tw, [&](int ix, int iy) { return cscale(in[ix * n + iy], ps[ix * n + iy]); }, NoMid(),
             [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-        row_pass<n, 1, false, 0>(
-            sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
+        row_pass<n, 1, false, 0, CB>(
+            sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
             [&](int ix, int iy, C2 v) { F[ix * n + iy] = v; });
       }
     }
@@ -289,19 +291,19 @@ __global__ void __launch_bounds__(kThreads) k_i24_vjp(
         // K2 part: nu_a += 2 (pi/J) eta_a Psi_{dir}(muK2 * F_other)
         // K4 part: PMp = Psi_{dir}(mu4_pair)
         for (int part = 0; part < 2; ++part) {
-          row_pass<n, -1, false, 0>(
+          row_pass<n, -1, false, 0, CB>(
               sm, tw,
               [&](int ix, int iy) {
                 const int i = ix * n + iy;
-                return part == 0 ? cscale(F[i], mk2c[i]) : mup[i];
+                return part == 0 ? cscale(ldc(&F[i]), mk2c[i]) : mup[i];
               },
               NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-          col_pass<n, -1, true, 1>(
-              sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; },
+          col_pass<n, -1, true, 1, CB>(
+              sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); },
               [&](int ix, int iy, C2 v) { return cscale(v, ps[ix * n + iy] * invP); },
               [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-          row_pass<n, 1, false, 0>(
-              sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
+          row_pass<n, 1, false, 0, CB>(
+              sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
               [&](int ix, int iy, C2 v) {
                 const int i = ix * n + iy;
                 if (part == 0) {
@@ -315,21 +317,21 @@ __global__ void __launch_bounds__(kThreads) k_i24_vjp(
               });
         }
         // nu_f += (pi/J) PM . F_other ; nu_b += (pi/J) Psi_other(f PM)
-        row_pass<n, -1, false, 0>(
+        row_pass<n, -1, false, 0, CB>(
             sm, tw,
             [&](int ix, int iy) {
               const int i = ix * n + iy;
-              const C2 pmv = PMp[i], fv = F[i];
+              const C2 pmv = ldc(&PMp[i]), fv = ldc(&F[i]);
               nufc[i] += wj * (pmv.x * fv.x + pmv.y * fv.y);
               return cscale(pmv, (T)2 * wf0[i].x - (T)1);
             },
             NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-        col_pass<n, -1, true, 1>(
-            sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; },
+        col_pass<n, -1, true, 1, CB>(
+            sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); },
             [&](int ix, int iy, C2 v) { return cscale(v, pq[ix * n + iy] * invP); },
             [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-        row_pass<n, 1, false, 0>(
-            sm, tw, [&](int ix, int iy) { return G[ix * n + iy]; }, NoMid(),
+        row_pass<n, 1, false, 0, CB>(
+            sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
             [&](int ix, int iy, C2 v) {
               const int i = ix * n + iy;
               C2 o = nuc[(size_t)p * P + i];
@@ -655,7 +657,7 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_vjp_smem(
 // n^2 H, so H (stored on those frequencies) is added to FFT(nu) there.
 // One block per cell; writes grad[c][4][N][N] (FP64).
 // --------------------------------------------------------------------------
-template <int n, class T>
+template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads) k_vjp_final(
     const typename Vec2Of<T>::type* nu, const T* nuf, const double* R, size_t r_stride,
     const typename Vec2Of<T>::type* spec, size_t spec_stride, typename Vec2Of<T>::type* ws,
@@ -670,13 +672,13 @@ __global__ void __launch_bounds__(kThreads) k_vjp_final(
   load_twiddles<n>(tw, gtw);
   constexpr int N = n / 2, P = n * n;
   constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
-  const int c = blockIdx.x;
-  C2* slot = ws + (size_t)blockIdx.x * 5 * P;
+  const int c = cluster_index();
+  C2* slot = ws + (size_t)cluster_index() * 5 * P;
   C2* V = slot;            // [2] total real-space cotangent pairs
   C2* F = slot + 2 * P;    // [2] their transforms
   const double* Rc = R + c * r_stride;
   const C2* H = spec + c * spec_stride;   // [2][Q]
-  for (int i = threadIdx.x; i < 2 * P; i += blockDim.x) {
+  for (int i = element_first(); i < 2 * P; i += element_stride()) {
     const int e = i % P;
     const double* Rp = Rc + (size_t)(i < P ? 0 : 2) * P + e;
     const C2 d = nu[(size_t)c * 2 * P + i];
@@ -684,18 +686,18 @@ __global__ void __launch_bounds__(kThreads) k_vjp_final(
     if (i < P) vx += 2.0 * (double)nuf[(size_t)c * P + i];
     V[i] = mk2((T)vx, (T)vy);
   }
-  __syncthreads();
+  team_sync();
   const T invP = (T)(1.0 / (double)P);
   for (int p = 0; p < 2; ++p) {
     C2* Vp = V + (size_t)p * P;
     C2* Fp = F + (size_t)p * P;
     const C2* Hp = H + (size_t)p * Q;
     // 4 E P (V + IFFT(H) / n^2)
-    row_pass<n, -1, false, 0>(
-        sm, tw, [&](int ix, int iy) { return Vp[ix * n + iy]; }, NoMid(),
+    row_pass<n, -1, false, 0, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&Vp[ix * n + iy]); }, NoMid(),
         [&](int ix, int iy, C2 v) { Fp[ix * n + iy] = v; });
-    col_pass<n, -1, true, 1>(
-        sm, tw, [&](int ix, int iy) { return Fp[ix * n + iy]; },
+    col_pass<n, -1, true, 1, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&Fp[ix * n + iy]); },
         [&](int ix, int iy, C2 v) {
           const int sx = kslot[ix], sy = kslot[iy];
           if (sx < 0 || sy < 0) return zero2<T>();
@@ -704,8 +706,8 @@ __global__ void __launch_bounds__(kThreads) k_vjp_final(
         },
         [&](int ix, int iy, C2 v) { Fp[ix * n + iy] = v; });
     double* g = grad + (size_t)c * 4 * N * N;
-    row_pass<n, 1, false, 0>(
-        sm, tw, [&](int ix, int iy) { return Fp[ix * n + iy]; }, NoMid(),
+    row_pass<n, 1, false, 0, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&Fp[ix * n + iy]); }, NoMid(),
         [&](int ix, int iy, C2 v) {
           if (((ix | iy) & 1) == 0) {
             const int i = ix >> 1, j = iy >> 1;
@@ -740,11 +742,10 @@ template <int n, class T>
 void set_vjp_smem_attributes() {
   static unsigned long long done = 0;
   if (!first_on_device(done)) return;
-  const int sm = (int)smem_bytes<n, T>();
-  cudaFuncSetAttribute(k_vjp_seed<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_i1_vjp<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_i24_vjp<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_vjp_final<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  QBE_CELLS_SMEM(k_vjp_seed);
+  QBE_CELLS_SMEM(k_i1_vjp);
+  QBE_CELLS_SMEM(k_i24_vjp);
+  QBE_CELLS_SMEM(k_vjp_final);
   if constexpr (vjp_staged<n, T>())
     cudaFuncSetAttribute(k_i3_vjp<n, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)i3_sf_smem_bytes<n, T, kVjpCB>());
@@ -771,7 +772,6 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
   T* K2acc = (T*)cw.K2acc;
   C2* K4acc = (C2*)cw.K4acc;
   C2* ws = (C2*)vw.ws;
-  const size_t sm = smem_bytes<n, T>();
   constexpr size_t P = (size_t)n * n;
   const size_t c_stride = (size_t)vw.nb * 2 * P;           // complex cotangent buffers, per cotangent
   const size_t r_stride = (size_t)vw.nb * P;               // real cotangent buffers, per cotangent
@@ -781,10 +781,11 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
   auto begin = [&](int g) { if (tm) tm->begin(g, s); };
   auto end = [&]() { if (tm) tm->end(s); };
   begin(KG_VJP);
-  k_prep<n, T><<<ncells, kThreads, sm, s>>>(w, what, wfine, (T*)cw.wplane, ws, tb.tw);
+  cudaError_t e = QBE_CELLS(k_prep, 4 * ncells, s, w, what, wfine, (T*)cw.wplane, ws, tb.tw);
+  if (e != cudaSuccess) return e;
   ++launches;
   {
-    const cudaError_t e = per_cell_terms<n, T>(t, cw, ws, ncells, s, launches, nullptr);
+    e = per_cell_terms<n, T>(t, cw, ws, ncells, s, launches, nullptr);
     if (e != cudaSuccess) return e;
   }
   for (int k = 0; k < K; ++k) {
@@ -796,18 +797,19 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
     C2* mu3 = (C2*)vw.mu3 + k * c_stride;
     C2* muh = (C2*)vw.muh + k * c_stride;
     T* mupl = vw.mupl ? (T*)vw.mupl + k * 2 * c_stride : nullptr;
-    k_vjp_seed<n, T><<<ncells, kThreads, sm, s>>>(lam[k], wfine, Dacc, K2acc, K4acc, nu, nuf, muD, muK2, mu4, mu3,
-                                                  muh, mupl, ws, tb.tw);
+    e = QBE_CELLS(k_vjp_seed, ncells, s, lam[k], wfine, Dacc, K2acc, K4acc, nu, nuf, muD, muK2, mu4, mu3, muh, mupl, ws,
+                  tb.tw);
+    if (e != cudaSuccess) return e;
     // I1 and I2/I4 transposes over (cell, angle chunk) blocks; their per-chunk cotangents go to the
     // forward's chunk-partial buffers (free once per_cell_terms has reduced them) and are summed in
     // chunk order into nu and nuf
     const int nch = cw.nch < 1 ? 1 : cw.nch;
     C2* nup = nch > 1 ? (C2*)cw.Dpart : nu;
     T* nufp = nch > 1 ? (T*)cw.K2part : nuf;
-    k_i1_vjp<n, T><<<ncells * nch, kThreads, sm, s>>>(what, wfine, muD, nup, nufp, ws, tb.tw, tb.phip, tb.Ktab, t.J,
-                                                      nch);
-    k_i24_vjp<n, T><<<ncells * nch, kThreads, sm, s>>>(what, wfine, muK2, mu4, nup, nufp, ws, tb.tw, tb.psi, t.J,
-                                                       nch);
+    e = QBE_CELLS(k_i1_vjp, ncells * nch, s, what, wfine, muD, nup, nufp, ws, tb.tw, tb.phip, tb.Ktab, t.J, nch);
+    if (e != cudaSuccess) return e;
+    e = QBE_CELLS(k_i24_vjp, ncells * nch, s, what, wfine, muK2, mu4, nup, nufp, ws, tb.tw, tb.psi, t.J, nch);
+    if (e != cudaSuccess) return e;
     launches += 3;
     if (nch > 1) {
       k_add_chunks<T><<<(ncells * 5 * n * n + kThreads * 8 - 1) / (kThreads * 8), kThreads, 0, s>>>(
@@ -852,9 +854,9 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
     C2* ps = (C2*)vw.part_s + k * spart_stride;
     reduce_partials<T>(pr, cw.K3sum, ps, units, np, nq, ncells, s);
     const double* R = cw.K3sum ? (const double*)cw.K3sum : (const double*)pr;
-    k_vjp_final<n, T><<<ncells, kThreads, sm, s>>>((C2*)vw.nu + k * c_stride, (T*)vw.nuf + k * r_stride, R,
-                                                   (cw.K3sum ? (size_t)1 : (size_t)units) * 2 * np, ps,
-                                                   (size_t)units * nq, ws, tb.tw, grad[k], accumulate);
+    e = QBE_CELLS(k_vjp_final, ncells, s, (C2*)vw.nu + k * c_stride, (T*)vw.nuf + k * r_stride, R,
+                  (cw.K3sum ? (size_t)1 : (size_t)units) * 2 * np, ps, (size_t)units * nq, ws, tb.tw, grad[k], accumulate);
+    if (e != cudaSuccess) return e;
     launches += 2;
   }
   end();

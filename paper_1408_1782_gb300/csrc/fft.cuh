@@ -41,6 +41,43 @@ __host__ __device__ __forceinline__ int pos_of_freq(int k) {
   return B * (k % A) + k / A;
 }
 
+// The team of a pass: the blocks of a cluster (a plain launch is a cluster of one).  Its blocks share
+// the chunks of every pass, and data that one block writes and another reads goes through L2 between
+// cluster barriers (release / acquire at cluster scope; the reads bypass L1: ldc).
+__device__ __forceinline__ int cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ int cluster_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ int cluster_index() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
+  return (int)r;
+}
+__device__ __forceinline__ int cluster_count() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(r));
+  return (int)r;
+}
+// All threads of all blocks of the cluster.
+__device__ __forceinline__ void cluster_sync_global() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void team_sync() {
+  if (cluster_size() > 1) cluster_sync_global();
+  else __syncthreads();
+}
+template <class C>
+__device__ __forceinline__ C ldc(const C* p) { return __ldcg(p); }
+// Element loops shared by the team: for (i = element_first(); i < count; i += element_stride()).
+__device__ __forceinline__ int element_first() { return cluster_rank() * blockDim.x + threadIdx.x; }
+__device__ __forceinline__ int element_stride() { return cluster_size() * blockDim.x; }
+
 // Real type of a complex vector type, and fused multiply-add per precision.
 template <class C2> struct RealOf;
 template <> struct RealOf<double2> { using type = double; };
@@ -407,7 +444,7 @@ template <int n, int ELEM = 16, int CB = 65536> struct Chunk {
   static constexpr int SMEM_ELEMS = (RC * LS > CC * n ? RC * LS : CC * n);
 };
 
-// Row pass over an n x n field (rows = fixed ix, transform along iy):
+// Row pass over an n x n field (rows = fixed ix, transform along iy), its chunks shared by the team:
 // for each chunk: sm[r][iy] = ld(ix, iy); [FFT DIR1]; [sm = mid(ix, iy, sm)]; [FFT DIR2]; st(ix, iy, sm).
 // DIR = 0 skips that transform; HAS_MID selects the pointwise middle step.
 template <int n, int DIR1, bool HAS_MID, int DIR2, int CB = 65536, bool XI = false, class C2, class LD, class MID,
@@ -415,7 +452,8 @@ template <int n, int DIR1, bool HAS_MID, int DIR2, int CB = 65536, bool XI = fal
 __device__ __forceinline__ void row_pass(C2* sm, const C2* tw, LD ld, MID mid, ST st) {
   constexpr int RC = Chunk<n, sizeof(C2), CB>::RC, LS = Chunk<n, sizeof(C2), CB>::LS;
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int r0 = 0; r0 < n; r0 += RC) {
+  const int ranks = cluster_size();
+  for (int r0 = cluster_rank() * RC; r0 < n; r0 += ranks * RC) {
 #pragma unroll 4
     for (int idx = tid; idx < RC * n; idx += nt) {
       const int r = idx / n, iy = idx % n;
@@ -439,6 +477,7 @@ __device__ __forceinline__ void row_pass(C2* sm, const C2* tw, LD ld, MID mid, S
     }
     __syncthreads();
   }
+  if (ranks > 1) cluster_sync_global();
 }
 
 // Column pass (transform along ix) over chunks of CC columns held as sm[ix][c].
@@ -446,7 +485,8 @@ template <int n, int DIR1, bool HAS_MID, int DIR2, int CB = 65536, class C2, cla
 __device__ __forceinline__ void col_pass(C2* sm, const C2* tw, LD ld, MID mid, ST st) {
   constexpr int CC = Chunk<n, sizeof(C2), CB>::CC;
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int c0 = 0; c0 < n; c0 += CC) {
+  const int ranks = cluster_size();
+  for (int c0 = cluster_rank() * CC; c0 < n; c0 += ranks * CC) {
 #pragma unroll 4
     for (int idx = tid; idx < CC * n; idx += nt) {
       const int ix = idx / CC, c = idx % CC;
@@ -470,6 +510,7 @@ __device__ __forceinline__ void col_pass(C2* sm, const C2* tw, LD ld, MID mid, S
     }
     __syncthreads();
   }
+  if (ranks > 1) cluster_sync_global();
 }
 
 // Column pass doing a circular convolution along ix for each column iy:
