@@ -18,7 +18,9 @@ namespace qbe {
 
 namespace {
 
-__device__ __forceinline__ double xlogx(double x) { return x > 0.0 ? x * log(x) : 0.0; }
+// 0 at x = 1 without the logarithm: 1 - lam rounds to 1 over most of the velocity box (the tails), and
+// k_entropy is bound by the FP64 instructions of its logarithms.
+__device__ __forceinline__ double xlogx(double x) { return x > 0.0 && x != 1.0 ? x * log(x) : 0.0; }
 
 // Per cell: dv^2 sum_v -[lam log lam + (1 - lam) log(1 - lam)] over both eigenvalues.
 __global__ void __launch_bounds__(256) k_entropy(const double* __restrict__ W, int N, double L, double* out) {
