@@ -181,7 +181,7 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   cw.ws_slots = nb > cw.grid_i3 ? nb : cw.grid_i3;
   cw.nch = per_cell_chunks(nb, t.J);
   size_t ws_fields = 6 * (size_t)nb;
-  if (5 * (size_t)nb * cw.nch > ws_fields) ws_fields = 5 * (size_t)nb * cw.nch;   // k_i24: 5 fields per block
+  if (5 * (size_t)nb * cw.nch > ws_fields) ws_fields = 5 * (size_t)nb * cw.nch;
   if (3 * (size_t)cw.grid_max > ws_fields) ws_fields = 3 * (size_t)cw.grid_max;
   // A requested grid is cut to this many blocks (and a launch to the resident ones, at most grid_max).
   cw.grid_cap = (int)(ws_fields / 3 < (size_t)INT_MAX ? ws_fields / 3 : INT_MAX);
@@ -189,6 +189,8 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   // which a block has (128 / n)^2
   cw.i3_fields = prec == 0 ? 4 : t.n == 64 ? 8 : t.n == 32 ? 32 : 3;
   if ((size_t)cw.i3_fields * cw.grid_max > ws_fields) ws_fields = (size_t)cw.i3_fields * cw.grid_max;
+  // k_i124: per (cell, chunk, pair) one field for I1 and three for I2/I4
+  if (8 * (size_t)nb * cw.nch > ws_fields) ws_fields = 8 * (size_t)nb * cw.nch;
   cw.ws_fields = ws_fields;
   cudaError_t e;
 #define QBE_ALLOC(ptr, bytes) \
@@ -199,9 +201,9 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   QBE_ALLOC(cw.Dacc, (size_t)nb * 2 * P * cz);
   QBE_ALLOC(cw.K2acc, (size_t)nb * P * rz);
   QBE_ALLOC(cw.K4acc, (size_t)nb * 2 * P * cz);
+  QBE_ALLOC(cw.K2part, (size_t)nb * cw.nch * 2 * P * rz);
   if (cw.nch > 1) {
     QBE_ALLOC(cw.Dpart, (size_t)nb * cw.nch * 2 * P * cz);
-    QBE_ALLOC(cw.K2part, (size_t)nb * cw.nch * P * rz);
     QBE_ALLOC(cw.K4part, (size_t)nb * cw.nch * 2 * P * cz);
   }
   QBE_ALLOC(cw.K3part, nparts * 2 * P * cz);
@@ -342,10 +344,10 @@ cudaError_t alloc_vjp_work(const Tables& t, int nb, VjpWork& vw, int prec, int k
                               : 3 + 4 * (size_t)kcap;
   size_t ws_fields = 7 * (size_t)nb;
   if (per_block * vw.grid > ws_fields) ws_fields = per_block * vw.grid;
-  // per (cell, angle chunk) block: the recomputed forward's I2/I4 kernel 5 fields, the I2/I4
+  // per (cell, angle chunk): the recomputed forward's I1 and I2/I4 teams 8 fields, the I2/I4
   // transpose 7
   const size_t nch = (size_t)per_cell_chunks(nb, t.J);
-  if (7 * (size_t)nb * nch > ws_fields) ws_fields = 7 * (size_t)nb * nch;
+  if (8 * (size_t)nb * nch > ws_fields) ws_fields = 8 * (size_t)nb * nch;
   const size_t kc = (size_t)kcap;
   const size_t cz = prec == 1 ? sizeof(float2) : sizeof(double2);
   const size_t rz = cz / 2;

@@ -178,11 +178,13 @@ __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w,
     const int p = q;
     const C2* in = out;
     C2* out = wfine + ((size_t)c * 2 + p) * P;
-    col_pass<n, 1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&in[ix * n + iy]); }, NoMid(),
+    xi_col_pass<n, CB>(
+        sm, tw, [&](int ix, int iy) { return ldc(&in[ix * n + iy]); },
         [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-    row_pass<n, 1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
+    row_pass<n, 1, false, 0, CB, true>(
+        sm, tw,
+        [&](int ix, int iy) { return xi_t<Split<n>::B>(iy % Split<n>::B) ? ldc(&G[ix * n + iy]) : zero2<T>(); },
+        NoMid(),
         [&](int ix, int iy, C2 v) {
           out[ix * n + iy] = v;
           if (wplane) {
@@ -195,40 +197,64 @@ __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w,
 }
 
 // --------------------------------------------------------------------------
-// I1 (conservative part): D^_b(sigma) = sum_j' K_j'(sigma) FFT[(2w0-1) IFFT(phi'_j' w_b^)].
-// One block per cell; pairs (w1 + i w2) and (w3).
+// The per-cell terms before I3, one team per (cell c, angle chunk ch, pair p) and kind:
+//   I1 (conservative part): D^_b(sigma) = sum_j' K_j'(sigma) FFT[(2w0-1) IFFT(phi'_j' w_b^)], pairs
+//     (w1 + i w2) and (w3); angles j' in [J ch / nch, J (ch + 1) / nch); D partial [c][ch][p]
+//   I2 and I4, over angle pairs (j, j + J/2), j in chunk ch of J/2, F_{a,j} = IFFT(psi_j w_a^) (real),
+//     pairs (0,1), (2,3):
+//     K2  += 2 (pi/J) sum_a eta_a F_{a,j} F_{a,j+J/2}                                 partial [c][ch][p]
+//     K4^ += (pi/J) [psi_j FFT((2w0-1) F_{.,j+J/2}) + psi_{j+J/2} FFT((2w0-1) F_{.,j})] / n^2
+// Teams [0, 2 nch ncells) take I1, the next as many I2/I4 (both kinds in one launch: with few cells
+// neither fills the GPU); `first` is the team of the launch's first block.  The inverse transforms skip
+// what lies outside Xi.
 // --------------------------------------------------------------------------
+template <int n, class T>
+struct CellTerms {
+  using C2 = typename Vec2Of<T>::type;
+  const C2* what;
+  const C2* wfine;
+  C2* D;          // [c][ch][2][P]
+  T* K2;          // [c][ch][2][P], cells k2_cell reals apart
+  C2* K4;         // [c][ch][2][P]
+  size_t k2_cell;
+  C2* ws1;        // one field per I1 team
+  C2* ws24;       // three fields per I2/I4 team
+  const C2* tw;
+  const T* phip;
+  const T* Ktab;
+  const T* psi;
+  int J, nch, teams1, first;
+};
+
 template <int n, class T, int CB>
-__global__ void __launch_bounds__(kThreads) k_i1(const typename Vec2Of<T>::type* what,
-                                                 const typename Vec2Of<T>::type* wfine, typename Vec2Of<T>::type* Dacc,
-                                                 typename Vec2Of<T>::type* ws,
-                                                 const typename Vec2Of<T>::type* __restrict__ gtw,
-                                                 const T* __restrict__ phip, const T* __restrict__ Ktab, int J,
-                                                 int nch) {
+__global__ void __launch_bounds__(kThreads) k_i124(const CellTerms<n, T> a) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
   C2* sm = tw + n;
-  load_twiddles<n>(tw, gtw);
-  constexpr int P = n * n;
-  // block (cell c, angle chunk ch): angles j' in [J ch / nch, J (ch + 1) / nch); D partial [c][ch]
-  const int c = cluster_index() / nch, ch = cluster_index() % nch;
-  C2* G = ws + (size_t)cluster_index() * P;
-  C2* D = Dacc + (size_t)cluster_index() * 2 * P;
-  zero_fields_team(D, 2 * P);
-  const C2* wf0 = wfine + (size_t)c * 2 * P;
-  for (int jp = J * ch / nch; jp < J * (ch + 1) / nch; ++jp) {
-    const T* ph = phip + (size_t)jp * P;
-    const T* K = Ktab + (size_t)jp * P;
-    for (int p = 0; p < 2; ++p) {
-      const C2* in = what + ((size_t)c * 4 + 2 + p) * P;
-      C2* Dp = D + (size_t)p * P;
-      col_pass<n, 1, false, 0, CB>(
-          sm, tw, [&](int ix, int iy) { return cscale(in[ix * n + iy], ph[ix * n + iy]); }, NoMid(),
+  load_twiddles<n>(tw, a.tw);
+  constexpr int P = n * n, B = Split<n>::B;
+  const int team = cluster_index() + a.first, J = a.J, nch = a.nch;
+  const bool i1 = team < a.teams1;
+  const int id = i1 ? team : team - a.teams1;
+  const int p = id & 1, cch = id >> 1, c = cch / nch, ch = cch % nch;
+  const C2* wf0 = a.wfine + (size_t)c * 2 * P;
+  auto load_xi = [&](const C2* G) {
+    return [G](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&G[ix * n + iy]) : zero2<T>(); };
+  };
+  if (i1) {
+    C2* G = a.ws1 + (size_t)id * P;
+    C2* Dp = a.D + (size_t)id * P;
+    const C2* in = a.what + ((size_t)c * 4 + 2 + p) * P;
+    zero_fields_team(Dp, P);
+    for (int jp = J * ch / nch; jp < J * (ch + 1) / nch; ++jp) {
+      const T* ph = a.phip + (size_t)jp * P;
+      const T* K = a.Ktab + (size_t)jp * P;
+      xi_col_pass<n, CB>(
+          sm, tw, [&](int ix, int iy) { return cscale(in[ix * n + iy], ph[ix * n + iy]); },
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-      row_pass<n, 1, true, -1, CB>(
-          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); },
-          [&](int ix, int iy, C2 v) { return cscale(v, (T)2 * wf0[ix * n + iy].x - (T)1); },
+      row_pass<n, 1, true, -1, CB, true>(
+          sm, tw, load_xi(G), [&](int ix, int iy, C2 v) { return cscale(v, (T)2 * wf0[ix * n + iy].x - (T)1); },
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
       col_pass<n, -1, false, 0, CB>(
           sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
@@ -238,107 +264,82 @@ __global__ void __launch_bounds__(kThreads) k_i1(const typename Vec2Of<T>::type*
             Dp[ix * n + iy] = mk2(fmaT(k, v.x, d.x), fmaT(k, v.y, d.y));
           });
     }
+    return;
   }
-}
-
-// --------------------------------------------------------------------------
-// I2 and I4: one block per cell, loop over angle pairs (j, j + J/2).
-//   F_{a,j} = IFFT(psi_j w_a^) (real), pairs (0,1), (2,3)
-//   K2  += 2 (pi/J) sum_a eta_a F_{a,j} F_{a,j+J/2}
-//   K4^ += (pi/J) [psi_j FFT((2w0-1) F_{.,j+J/2}) + psi_{j+J/2} FFT((2w0-1) F_{.,j})] / n^2
-// --------------------------------------------------------------------------
-template <int n, class T, int CB>
-__global__ void __launch_bounds__(kThreads) k_i24(const typename Vec2Of<T>::type* what,
-                                                  const typename Vec2Of<T>::type* wfine, T* K2acc,
-                                                  typename Vec2Of<T>::type* K4acc, typename Vec2Of<T>::type* ws,
-                                                  const typename Vec2Of<T>::type* __restrict__ gtw,
-                                                  const T* __restrict__ psi, int J, int nch) {
-  using C2 = typename Vec2Of<T>::type;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  C2* tw = reinterpret_cast<C2*>(smem_raw);
-  C2* sm = tw + n;
-  load_twiddles<n>(tw, gtw);
-  constexpr int P = n * n;
-  // block (cell c, chunk ch) of the J/2 angle pairs; K2, K4 partials [c][ch]
-  const int c = cluster_index() / nch, ch = cluster_index() % nch;
-  C2* slot = ws + (size_t)cluster_index() * 5 * P;
-  C2* FA = slot;            // [2][P]
-  C2* FB = slot + 2 * P;    // [2][P]
-  C2* G = slot + 4 * P;
-  T* K2 = K2acc + (size_t)cluster_index() * P;
-  C2* K4 = K4acc + (size_t)cluster_index() * 2 * P;
+  C2* FA = a.ws24 + (size_t)id * 3 * P;
+  C2* FB = FA + P;
+  C2* G = FA + 2 * P;
+  T* K2 = a.K2 + c * a.k2_cell + ((size_t)ch * 2 + p) * P;
+  C2* K4 = a.K4 + (size_t)id * P;
   for (int i = element_first(); i < P; i += element_stride()) K2[i] = (T)0;
-  zero_fields_team(K4, 2 * P);
-  const C2* wf0 = wfine + (size_t)c * 2 * P;
+  zero_fields_team(K4, P);
+  const C2* in = a.what + ((size_t)c * 4 + p) * P;
   const T wj = (T)(kPi / J);
   const T scale = (T)(kPi / J / (double)P);
+  const T e0 = p == 0 ? (T)1 : (T)-1;   // eta of component 2 p
   const int H = J / 2;
   for (int j = H * ch / nch; j < H * (ch + 1) / nch; ++j) {
     const int jp = j + J / 2;
-    for (int p = 0; p < 2; ++p) {
-      const C2* in = what + ((size_t)c * 4 + p) * P;
-      for (int h = 0; h < 2; ++h) {
-        const T* ps = psi + (size_t)(h == 0 ? j : jp) * P;
-        C2* F = (h == 0 ? FA : FB) + (size_t)p * P;
-        col_pass<n, 1, false, 0, CB>(
-            sm, tw, [&](int ix, int iy) { return cscale(in[ix * n + iy], ps[ix * n + iy]); }, NoMid(),
-            [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-        row_pass<n, 1, false, 0, CB>(
-            sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
-            [&](int ix, int iy, C2 v) { F[ix * n + iy] = v; });
-      }
+    for (int h = 0; h < 2; ++h) {
+      const T* ps = a.psi + (size_t)(h == 0 ? j : jp) * P;
+      C2* F = h == 0 ? FA : FB;
+      xi_col_pass<n, CB>(
+          sm, tw, [&](int ix, int iy) { return cscale(in[ix * n + iy], ps[ix * n + iy]); },
+          [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
+      row_pass<n, 1, false, 0, CB, true>(
+          sm, tw, load_xi(G), NoMid(), [&](int ix, int iy, C2 v) { F[ix * n + iy] = v; });
     }
     for (int i = element_first(); i < P; i += element_stride()) {
-      const C2 a0 = ldc(&FA[i]), a1 = ldc(&FA[P + i]), b0 = ldc(&FB[i]), b1 = ldc(&FB[P + i]);
-      const T s = a0.x * b0.x - a0.y * b0.y - a1.x * b1.x - a1.y * b1.y;
-      K2[i] = fmaT((T)2 * wj, s, K2[i]);
+      const C2 fa = ldc(&FA[i]), fb = ldc(&FB[i]);
+      K2[i] = fmaT((T)2 * wj, e0 * fa.x * fb.x - fa.y * fb.y, K2[i]);
     }
     team_sync();
-    for (int p = 0; p < 2; ++p) {
-      C2* K4p = K4 + (size_t)p * P;
-      for (int h = 0; h < 2; ++h) {
-        const C2* F = (h == 0 ? FB : FA) + (size_t)p * P;   // psi_j pairs with F_{j+J/2}
-        const T* ps = psi + (size_t)(h == 0 ? j : jp) * P;
-        row_pass<n, -1, false, 0, CB>(
-            sm, tw, [&](int ix, int iy) { return cscale(ldc(&F[ix * n + iy]), (T)2 * wf0[ix * n + iy].x - (T)1); },
-            NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-        col_pass<n, -1, false, 0, CB>(
-            sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
-            [&](int ix, int iy, C2 v) {
-              const T k = scale * ps[ix * n + iy];
-              const C2 d = K4p[ix * n + iy];
-              K4p[ix * n + iy] = mk2(fmaT(k, v.x, d.x), fmaT(k, v.y, d.y));
-            });
-      }
+    for (int h = 0; h < 2; ++h) {
+      const C2* F = h == 0 ? FB : FA;   // psi_j pairs with F_{j+J/2}
+      const T* ps = a.psi + (size_t)(h == 0 ? j : jp) * P;
+      row_pass<n, -1, false, 0, CB>(
+          sm, tw, [&](int ix, int iy) { return cscale(ldc(&F[ix * n + iy]), (T)2 * wf0[ix * n + iy].x - (T)1); },
+          NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
+      col_pass<n, -1, false, 0, CB>(
+          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
+          [&](int ix, int iy, C2 v) {
+            const T k = scale * ps[ix * n + iy];
+            const C2 d = K4[ix * n + iy];
+            K4[ix * n + iy] = mk2(fmaT(k, v.x, d.x), fmaT(k, v.y, d.y));
+          });
     }
   }
 }
 
-// Sum of the per-chunk partials of k_i1 (D, 2 complex fields) and k_i24 (K2 real, K4 2 complex)
-// of each cell, in chunk order: part[c][ch][...] -> acc[c][...].
+// Sums of the partials of k_i124 of each cell, in order: D and K4 (2 complex fields each) over the nch
+// chunks (skipped with one: the kernel writes the sums), K2 (real) over its 2 nch planes.
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_reduce_chunks(const T* __restrict__ Dpart, const T* __restrict__ K2part,
                                                             const T* __restrict__ K4part, T* Dacc, T* K2acc, T* K4acc,
-                                                            int nch, int ncells, size_t P) {
-  const size_t per_c = 4 * P, per_r = P;   // reals per cell: D and K4 (2 complex fields each), K2
-  const size_t total = (size_t)ncells * (2 * per_c + per_r);
+                                                            int nch, int ncells, size_t P, size_t k2_cell) {
+  const size_t per_c = nch > 1 ? 4 * P : 0;   // reals of D and of K4 per cell
+  const size_t total = (size_t)ncells * (2 * per_c + P);
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const T* src;
+    const T* p;
     T* dst;
-    size_t c, e, stride;
-    if (i < (size_t)ncells * per_c) {
-      c = i / per_c; e = i % per_c; src = Dpart; dst = Dacc; stride = per_c;
-    } else if (i < (size_t)ncells * 2 * per_c) {
-      const size_t k = i - (size_t)ncells * per_c;
-      c = k / per_c; e = k % per_c; src = K4part; dst = K4acc; stride = per_c;
+    size_t stride;
+    int planes = nch;
+    if (i < (size_t)ncells * 2 * per_c) {
+      const bool second = i >= (size_t)ncells * per_c;
+      const size_t k = second ? i - (size_t)ncells * per_c : i;
+      stride = per_c;
+      p = (second ? K4part : Dpart) + (k / per_c * nch) * per_c + k % per_c;
+      dst = (second ? K4acc : Dacc) + k;
     } else {
       const size_t k = i - (size_t)ncells * 2 * per_c;
-      c = k / per_r; e = k % per_r; src = K2part; dst = K2acc; stride = per_r;
+      stride = P;
+      planes = 2 * nch;
+      p = K2part + k / P * k2_cell + k % P;
+      dst = K2acc + k;
     }
-    const T* p = src + (c * nch) * stride + e;
     T sum = p[0];
-    for (int ch = 1; ch < nch; ++ch) sum += p[(size_t)ch * stride];
-    dst[c * stride + e] = sum;
+    for (int ch = 1; ch < planes; ++ch) sum += p[(size_t)ch * stride];
+    *dst = sum;
   }
 }
 
@@ -1301,8 +1302,7 @@ void set_smem_attributes() {
   static unsigned long long done = 0;
   if (!first_on_device(done)) return;
   QBE_CELLS_SMEM(k_prep);
-  QBE_CELLS_SMEM(k_i1);
-  QBE_CELLS_SMEM(k_i24);
+  QBE_CELLS_SMEM(k_i124);
   QBE_CELLS_SMEM(k_assemble);
   for (int v = 0; v < i3_nvariants<n, T>(); ++v) {
     const I3Launch l = i3_variant<n, T>(v);
@@ -1411,33 +1411,49 @@ const char* i3_variant_name(int v) {
   return i3_variant<n, T>(v).name;
 }
 
-// I1 and I2/I4 of ncells cells over (cell, angle chunk) blocks (cw.nch chunks per cell), then the
-// chunk partials summed into Dacc, K2acc, K4acc (skipped with one chunk: the kernels write there).
+// I1 and I2/I4 of ncells cells (k_i124), then its partials summed into Dacc, K2acc, K4acc.  One launch
+// for both kinds; two where they are timed apart, or share their scratch (the workspace without K2part
+// has six fields per cell, and keeps the K2 planes in the coefficients that only I1 reads).
 template <int n, class T>
 cudaError_t per_cell_terms(const Tables& t, CollisionWork& cw, typename Vec2Of<T>::type* ws, int ncells,
                            cudaStream_t s, long long& launches, KernelTimer* tm) {
   using C2 = typename Vec2Of<T>::type;
+  constexpr size_t P = (size_t)n * n;
   const TabPtrs<T> tb = tab_ptrs<T>(t);
-  const C2* what = (const C2*)cw.what;
-  const C2* wfine = (const C2*)cw.wfine;
   const int nch = cw.nch < 1 ? 1 : cw.nch;
-  C2* D = (C2*)(nch > 1 ? cw.Dpart : cw.Dacc);
-  T* K2 = (T*)(nch > 1 ? cw.K2part : cw.K2acc);
-  C2* K4 = (C2*)(nch > 1 ? cw.K4part : cw.K4acc);
-  if (tm) tm->begin(KG_I1, s);
-  cudaError_t e = QBE_CELLS(k_i1, ncells * nch, s, what, wfine, D, ws, tb.tw, tb.phip, tb.Ktab, t.J, nch);
+  const bool own_k2 = cw.K2part != nullptr;
+  CellTerms<n, T> a;
+  a.what = (const C2*)cw.what;
+  a.wfine = (const C2*)cw.wfine;
+  a.D = (C2*)(nch > 1 ? cw.Dpart : cw.Dacc);
+  a.K4 = (C2*)(nch > 1 ? cw.K4part : cw.K4acc);
+  a.K2 = own_k2 ? (T*)cw.K2part : (T*)((C2*)cw.what + 2 * P);
+  a.k2_cell = own_k2 ? 2 * (size_t)nch * P : 8 * P;
+  a.tw = tb.tw;
+  a.phip = tb.phip;
+  a.Ktab = tb.Ktab;
+  a.psi = tb.psi;
+  a.J = t.J;
+  a.nch = nch;
+  a.teams1 = 2 * ncells * nch;
+  a.first = 0;
+  a.ws1 = ws;
+  a.ws24 = own_k2 ? ws + a.teams1 * P : ws;
+  const bool apart = !own_k2 || (tm && tm->on);
+  if (tm && apart) tm->begin(KG_I1, s);
+  cudaError_t e = QBE_CELLS(k_i124, apart ? a.teams1 : 2 * a.teams1, s, a);
   if (e != cudaSuccess) return e;
-  if (tm) tm->end(s);
-  if (tm) tm->begin(KG_I24, s);
-  e = QBE_CELLS(k_i24, ncells * nch, s, what, wfine, K2, K4, ws, tb.tw, tb.psi, t.J, nch);
-  if (e != cudaSuccess) return e;
-  if (nch > 1) {
-    k_reduce_chunks<T><<<(ncells * 5 * n * n + kThreads * 8 - 1) / (kThreads * 8), kThreads, 0, s>>>(
-        (const T*)cw.Dpart, (const T*)cw.K2part, (const T*)cw.K4part, (T*)cw.Dacc, (T*)cw.K2acc, (T*)cw.K4acc, nch,
-        ncells, (size_t)n * n);
+  if (tm && apart) tm->end(s);
+  if (apart) {
+    a.first = a.teams1;
+    if (tm) tm->begin(KG_I24, s);
+    e = QBE_CELLS(k_i124, a.teams1, s, a);
+    if (e != cudaSuccess) return e;
     ++launches;
   }
-  if (tm) tm->end(s);
+  k_reduce_chunks<T><<<(ncells * 5 * n * n + kThreads * 8 - 1) / (kThreads * 8), kThreads, 0, s>>>(
+      (const T*)a.D, a.K2, (const T*)a.K4, (T*)cw.Dacc, (T*)cw.K2acc, (T*)cw.K4acc, nch, ncells, P, a.k2_cell);
+  if (tm && apart) tm->end(s);
   launches += 2;
   return cudaGetLastError();
 }

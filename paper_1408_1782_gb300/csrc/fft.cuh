@@ -513,6 +513,36 @@ __device__ __forceinline__ void col_pass(C2* sm, const C2* tw, LD ld, MID mid, S
   if (ranks > 1) cluster_sync_global();
 }
 
+// Inverse column pass of a spectrum that vanishes outside Xi: the n / 2 columns of Xi only, ld(ix, iy)
+// called for Xi rows only (iy, ix permuted positions).
+template <int n, int CB = 65536, class C2, class LD, class ST>
+__device__ __forceinline__ void xi_col_pass(C2* sm, const C2* tw, LD ld, ST st) {
+  constexpr int CC = Chunk<n, sizeof(C2), CB>::CC, B = Split<n>::B;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  auto column = [](int li) {
+    const int k1 = li / (B / 2), t = li % (B / 2);
+    return B * k1 + (t < B / 4 ? t : t + B / 2);
+  };
+  const int ranks = cluster_size();
+  for (int c0 = cluster_rank() * CC; c0 < n / 2; c0 += ranks * CC) {
+    const int nc = (n / 2 - c0) < CC ? (n / 2 - c0) : CC;
+#pragma unroll 4
+    for (int idx = tid; idx < nc * n; idx += nt) {
+      const int ix = idx / nc, c = idx % nc;
+      if (xi_t<B>(ix % B)) sm[ix * CC + c] = ld(ix, column(c0 + c));   // the first stage reads no other
+    }
+    __syncthreads();
+    fft_lines<n, 1, true>(sm, nc, 1, CC, tw);
+#pragma unroll 4
+    for (int idx = tid; idx < nc * n; idx += nt) {
+      const int ix = idx / nc, c = idx % nc;
+      st(ix, column(c0 + c), sm[ix * CC + c]);
+    }
+    __syncthreads();
+  }
+  if (ranks > 1) cluster_sync_global();
+}
+
 // Column pass doing a circular convolution along ix for each column iy:
 // sm[ix][c] = ld(ix, iy); forward FFT; times mul(pos_x, iy); inverse FFT; st(ix, iy, value).
 template <int n, int CB = 65536, class C2, class LD, class MUL, class ST>

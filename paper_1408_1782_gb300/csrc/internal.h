@@ -104,7 +104,7 @@ struct CollisionWork {
   void* K4acc = nullptr;     // [nb][2][n*n] spectral K4 pairs (0,1), (2,3)
   int nch = 1;               // angle chunks per cell of the I1 and I2/I4 kernels
   void* Dpart = nullptr;     // their per-chunk partials [nb][nch][...] (nch > 1 only)
-  void* K2part = nullptr;
+  void* K2part = nullptr;    // [nb][2 nch][n*n]; null: k_i124 keeps its K2 planes in `what`
   void* K4part = nullptr;
   // fine-grid K3 partial sums [nb*J*nmc]: [2][n*n] pairs (0,1), (2,3) of the node-by-node kernels, four
   // planes [4][n*n] (reals) of the kernels that take the nodes in pairs
