@@ -133,7 +133,8 @@ __device__ __forceinline__ I3Group i3_group_at(int it, int it1, int M) {
 
 // --------------------------------------------------------------------------
 // Prep: Xi coefficients of the four Pauli components (paired) and the
-// fine-grid interpolants.  One block per cell.
+// fine-grid interpolants.  One team per cell and coefficient pair.  (Outside Xi the
+// coefficients are zero and not stored: no kernel reads there.)
 //   what[c][0] = w0^ + i w1^, [1] = w2^ + i w3^, [2] = w1^ + i w2^, [3] = w3^
 //   wfine[c][0] = w0 + i w1, [1] = w2 + i w3  on the fine grid;
 //   wplane (may be null): the same four components as planes [c][4][n*n].
@@ -155,45 +156,43 @@ __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w,
   const double* wc = w + (size_t)c * 4 * N * N;
   C2* G = ws + (size_t)cq * P;
   const T invN2 = (T)(1.0 / ((double)N * N));
+  constexpr int B = Split<n>::B;
   C2* out = what + ((size_t)c * 4 + q) * P;
-  {
-    const int a = (q == 0) ? 0 : (q == 1) ? 2 : (q == 2) ? 1 : 3;
-    const int b = (q == 0) ? 1 : (q == 1) ? 3 : (q == 2) ? 2 : -1;
-    row_pass<n, -1, false, 0, CB>(
-        sm, tw,
-        [&](int ix, int iy) {
-          if ((ix | iy) & 1) return zero2<T>();
-          const int i = ix >> 1, j = iy >> 1;
-          return mk2((T)wc[(a * N + i) * N + j], b >= 0 ? (T)wc[(b * N + i) * N + j] : (T)0);
-        },
-        NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-    col_pass<n, -1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
-        [&](int ix, int iy, C2 v) {
-          const bool keep = in_xi<n>(freq_of_pos<n>(ix)) && in_xi<n>(freq_of_pos<n>(iy));
-          out[ix * n + iy] = keep ? cscale(v, invN2) : zero2<T>();
-        });
+  const int a = (q == 0) ? 0 : (q == 1) ? 2 : (q == 2) ? 1 : 3;
+  const int b = (q == 0) ? 1 : (q == 1) ? 3 : (q == 2) ? 2 : -1;
+  even_row_pass<n, -1, CB>(
+      sm, tw,
+      [&](int ix, int iy) {
+        if (iy & 1) return zero2<T>();
+        const int i = ix >> 1, j = iy >> 1;
+        return mk2((T)wc[(a * N + i) * N + j], b >= 0 ? (T)wc[(b * N + i) * N + j] : (T)0);
+      },
+      [&](int ix, int iy, C2 v) {
+        if (xi_t<B>(iy % B)) G[ix * n + iy] = v;
+      });
+  auto load = [&](int ix, int iy) { return (ix & 1) ? zero2<T>() : ldc(&G[ix * n + iy]); };
+  auto coef = [&](int ix, int iy, C2 v) {
+    const bool keep = xi_slot<n>(ix) >= 0 && xi_slot<n>(iy) >= 0;
+    const C2 z = keep ? cscale(v, invN2) : zero2<T>();
+    out[ix * n + iy] = z;
+    return z;
+  };
+  if (q >= 2) {
+    xi_col_filter<n, true, false, CB>(sm, tw, load, coef, [](int, int, C2) {});
+    return;
   }
-  if (q < 2) {
-    const int p = q;
-    const C2* in = out;
-    C2* out = wfine + ((size_t)c * 2 + p) * P;
-    xi_col_pass<n, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&in[ix * n + iy]); },
-        [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-    row_pass<n, 1, false, 0, CB, true>(
-        sm, tw,
-        [&](int ix, int iy) { return xi_t<Split<n>::B>(iy % Split<n>::B) ? ldc(&G[ix * n + iy]) : zero2<T>(); },
-        NoMid(),
-        [&](int ix, int iy, C2 v) {
-          out[ix * n + iy] = v;
-          if (wplane) {
-            T* pl = wplane + ((size_t)c * 4 + 2 * p) * P + ix * n + iy;
-            pl[0] = v.x;
-            pl[P] = v.y;
-          }
-        });
-  }
+  xi_col_filter<n, true, true, CB>(sm, tw, load, coef, [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
+  C2* fine = wfine + ((size_t)c * 2 + q) * P;
+  row_pass<n, 1, false, 0, CB, true>(
+      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&G[ix * n + iy]) : zero2<T>(); }, NoMid(),
+      [&](int ix, int iy, C2 v) {
+        fine[ix * n + iy] = v;
+        if (wplane) {
+          T* pl = wplane + ((size_t)c * 4 + 2 * q) * P + ix * n + iy;
+          pl[0] = v.x;
+          pl[P] = v.y;
+        }
+      });
 }
 
 // --------------------------------------------------------------------------
@@ -1054,19 +1053,46 @@ void reduce_partials(typename Vec2Of<T>::type* part, double2* sum, typename Vec2
   }
 }
 
+// Real-space D pairs and K4 pairs of each cell (inverse 2-D transforms), DK[c][4][P]: one team per cell
+// and pair.
+template <int n, class T, int CB>
+__global__ void __launch_bounds__(kThreads) k_dk_fields(const typename Vec2Of<T>::type* Dacc,
+                                                        const typename Vec2Of<T>::type* K4acc,
+                                                        typename Vec2Of<T>::type* DK,
+                                                        const typename Vec2Of<T>::type* __restrict__ gtw) {
+  using C2 = typename Vec2Of<T>::type;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C2* tw = reinterpret_cast<C2*>(smem_raw);
+  C2* sm = tw + n;
+  load_twiddles<n>(tw, gtw);
+  constexpr int P = n * n;
+  const int c = cluster_index() >> 2, f = cluster_index() & 3;
+  const C2* in = (f < 2) ? (Dacc + ((size_t)c * 2 + f) * P) : (K4acc + ((size_t)c * 2 + (f - 2)) * P);
+  C2* out = DK + (size_t)cluster_index() * P;
+  col_pass<n, 1, false, 0, CB>(
+      sm, tw, [&](int ix, int iy) { return in[ix * n + iy]; }, NoMid(),
+      [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
+  row_pass<n, 1, false, 0, CB>(
+      sm, tw, [&](int ix, int iy) { return ldc(&out[ix * n + iy]); }, NoMid(),
+      [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
+}
+
 // --------------------------------------------------------------------------
 // Assemble C on the fine grid from D, K2, K3, K4 (Pauli formulas of Sec. 3.1),
 // then FFT, cut to Xi (without the -N/2 line), inverse FFT and sample the
-// coarse nodes.  One block per cell.  k3: the reduced K3 of a cell (FP64), k3_stride apart; spec (null
-// after a node-by-node kernel): their Fourier-space parts, added to the spectrum of C inside the projection
-// (C_0 holds -2 pi K3_0 and C_c holds +2 pi K3raw_c; the sign of component 0 is already in spec).
+// coarse nodes.  One team per cell and pair (C_0, C_1) or (C_2, C_3); the pointwise
+// formulas are evaluated on the load of the first pass, and after it only the Xi
+// columns and the even rows are transformed.  k3: the reduced K3 of a cell (FP64),
+// k3_stride apart; spec (null after a node-by-node kernel): their Fourier-space parts,
+// added to the spectrum of C inside the projection (C_0 holds -2 pi K3_0 and C_c holds
+// +2 pi K3raw_c; the sign of component 0 is already in spec).
 // --------------------------------------------------------------------------
 template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>::type* wfine,
-                                                       const typename Vec2Of<T>::type* Dacc, const T* K2acc,
-                                                       const typename Vec2Of<T>::type* K4acc, const double2* k3,
-                                                       size_t k3_stride, const typename Vec2Of<T>::type* spec,
-                                                       size_t spec_stride, typename Vec2Of<T>::type* ws,
+                                                       const typename Vec2Of<T>::type* DK, const T* K2acc,
+                                                       const double2* k3, size_t k3_stride,
+                                                       const typename Vec2Of<T>::type* spec, size_t spec_stride,
+                                                       typename Vec2Of<T>::type* ws,
                                                        const typename Vec2Of<T>::type* __restrict__ gtw,
                                                        double* cout) {
   using C2 = typename Vec2Of<T>::type;
@@ -1074,78 +1100,69 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
   C2* tw = reinterpret_cast<C2*>(smem_raw);
   C2* sm = tw + n;
   load_twiddles<n>(tw, gtw);
-  constexpr int N = n / 2, P = n * n;
-  const int c = cluster_index();
-  C2* slot = ws + (size_t)cluster_index() * 6 * P;
-  C2* B0 = slot;
-  // D pairs -> slot[0], slot[1]; K4 pairs -> slot[2], slot[3] (inverse 2-D transforms)
-  for (int f = 0; f < 4; ++f) {
-    const C2* in = (f < 2) ? (Dacc + ((size_t)c * 2 + f) * P) : (K4acc + ((size_t)c * 2 + (f - 2)) * P);
-    C2* out = slot + (size_t)f * P;
-    col_pass<n, 1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return in[ix * n + iy]; }, NoMid(),
-        [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
-    row_pass<n, 1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&out[ix * n + iy]); }, NoMid(),
-        [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
-  }
-  constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
+  constexpr int N = n / 2, P = n * n, NQ = xi_kept<n>(), Q = NQ * NQ, B = Split<n>::B;
+  const int c = cluster_index() >> 1, p = cluster_index() & 1;
+  C2* H = ws + (size_t)cluster_index() * P;
+  const C2* dk = DK + (size_t)c * 4 * P;
   const double2* k3c = k3 + c * k3_stride;
+  const double* k3r = reinterpret_cast<const double*>(k3c);
   const C2* wf0 = wfine + (size_t)c * 2 * P;
   const C2* wf1 = wf0 + P;
   const T* K2 = K2acc + (size_t)c * P;
   const double tp = 2.0 * kPi;
-  const double* k3r = reinterpret_cast<const double*>(k3c);
-  for (int i = element_first(); i < P; i += element_stride()) {
-    // node-by-node kernels: pairs (K3_0, K3_1), (K3_2, K3_3); kernels in pairs: four planes
-    const double2 k3a = spec ? mk2(k3r[i], k3r[P + i]) : k3c[i];
-    const double2 k3b = spec ? mk2(k3r[2 * P + i], k3r[3 * P + i]) : k3c[P + i];
-    const double w0 = wf0[i].x, w1 = wf0[i].y, w2 = wf1[i].x, w3 = wf1[i].y;
-    const C2 s0 = ldc(&slot[i]), s1 = ldc(&slot[P + i]), s2 = ldc(&slot[2 * P + i]), s3 = ldc(&slot[3 * P + i]);
-    const double D1 = s0.x, D2 = s0.y, D3 = s1.x;
-    const double K40 = s2.x, K41 = -(double)s2.y;   // eta_b applied
-    const double K42 = -(double)s3.x, K43 = -(double)s3.y;
-    const double K30 = k3a.x, K31 = -k3a.y, K32 = -k3b.x, K33 = -k3b.y;
-    const double k2 = K2[i];
-    const double C0 = tp * (k2 * (1.0 - w0) - K30 + w0 * K40 + w1 * K41 + w2 * K42 + w3 * K43);
-    const double C1 = -2.0 * (D2 * w3 - D3 * w2) + tp * (-k2 * w1 - K31 + w0 * K41 + K40 * w1);
-    const double C2v = -2.0 * (D3 * w1 - D1 * w3) + tp * (-k2 * w2 - K32 + w0 * K42 + K40 * w2);
-    const double C3 = -2.0 * (D1 * w2 - D2 * w1) + tp * (-k2 * w3 - K33 + w0 * K43 + K40 * w3);
-    B0[i] = mk2((T)C0, (T)C1);
-    B0[P + i] = mk2((T)C2v, (T)C3);
-  }
-  team_sync();
   const T invP = (T)(1.0 / (double)P);
   double* co = cout + (size_t)c * 4 * N * N;
-  C2* H = slot + 2 * P;
-  for (int p = 0; p < 2; ++p) {
-    const C2* F = B0 + (size_t)p * P;
-    const C2* Hs = spec ? spec + c * spec_stride + (size_t)p * Q : nullptr;
-    row_pass<n, -1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&F[ix * n + iy]); }, NoMid(),
-        [&](int ix, int iy, C2 v) { H[ix * n + iy] = v; });
-    col_pass<n, -1, true, 1, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&H[ix * n + iy]); },
-        [&](int ix, int iy, C2 v) {
-          const int sx = xi_slot<n>(ix), sy = xi_slot<n>(iy);
-          if (sx < 0 || sy < 0) return zero2<T>();
-          if (Hs) {
-            const C2 h = Hs[sx * NQ + sy];
-            v = mk2(fmaT((T)tp, h.x, v.x), fmaT((T)tp, h.y, v.y));
-          }
-          return cscale(v, invP);
-        },
-        [&](int ix, int iy, C2 v) { H[ix * n + iy] = v; });
-    row_pass<n, 1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&H[ix * n + iy]); }, NoMid(),
-        [&](int ix, int iy, C2 v) {
-          if (((ix | iy) & 1) == 0) {
-            const int i = ix >> 1, j = iy >> 1;
-            co[((2 * p) * N + i) * N + j] = (double)v.x;
-            co[((2 * p + 1) * N + i) * N + j] = (double)v.y;
-          }
-        });
-  }
+  const C2* Hs = spec ? spec + c * spec_stride + (size_t)p * Q : nullptr;
+  row_pass<n, -1, false, 0, CB>(
+      sm, tw,
+      [&](int ix, int iy) {
+        const int i = ix * n + iy;
+        // node-by-node kernels: pairs (K3_0, K3_1), (K3_2, K3_3); kernels in pairs: four planes
+        const double2 k3p = spec ? mk2(k3r[2 * p * P + i], k3r[(2 * p + 1) * P + i]) : k3c[p * P + i];
+        const double w0 = wf0[i].x, w1 = wf0[i].y, w2 = wf1[i].x, w3 = wf1[i].y;
+        const C2 s0 = dk[i], s1 = dk[P + i], s2 = dk[2 * P + i], s3 = dk[3 * P + i];
+        const double D1 = s0.x, D2 = s0.y, D3 = s1.x;
+        const double K40 = s2.x, K41 = -(double)s2.y;   // eta_b applied
+        const double K42 = -(double)s3.x, K43 = -(double)s3.y;
+        const double k2 = K2[i];
+        if (p == 0) {
+          const double K30 = k3p.x, K31 = -k3p.y;
+          const double C0 = tp * (k2 * (1.0 - w0) - K30 + w0 * K40 + w1 * K41 + w2 * K42 + w3 * K43);
+          const double C1 = -2.0 * (D2 * w3 - D3 * w2) + tp * (-k2 * w1 - K31 + w0 * K41 + K40 * w1);
+          return mk2((T)C0, (T)C1);
+        }
+        const double K32 = -k3p.x, K33 = -k3p.y;
+        const double C2v = -2.0 * (D3 * w1 - D1 * w3) + tp * (-k2 * w2 - K32 + w0 * K42 + K40 * w2);
+        const double C3 = -2.0 * (D1 * w2 - D2 * w1) + tp * (-k2 * w3 - K33 + w0 * K43 + K40 * w3);
+        return mk2((T)C2v, (T)C3);
+      },
+      NoMid(),
+      [&](int ix, int iy, C2 v) {
+        if (xi_t<B>(iy % B)) H[ix * n + iy] = v;
+      });
+  xi_col_filter<n, true, true, CB>(
+      sm, tw, [&](int ix, int iy) { return ldc(&H[ix * n + iy]); },
+      [&](int ix, int iy, C2 v) {
+        const int sx = xi_slot<n>(ix), sy = xi_slot<n>(iy);
+        if (sx < 0 || sy < 0) return zero2<T>();
+        if (Hs) {
+          const C2 h = Hs[sx * NQ + sy];
+          v = mk2(fmaT((T)tp, h.x, v.x), fmaT((T)tp, h.y, v.y));
+        }
+        return cscale(v, invP);
+      },
+      [&](int ix, int iy, C2 v) {
+        if (!(ix & 1)) H[ix * n + iy] = v;
+      });
+  even_row_pass<n, 1, CB, true>(
+      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&H[ix * n + iy]) : zero2<T>(); },
+      [&](int ix, int iy, C2 v) {
+        if (!(iy & 1)) {
+          const int i = ix >> 1, j = iy >> 1;
+          co[((2 * p) * N + i) * N + j] = (double)v.x;
+          co[((2 * p + 1) * N + i) * N + j] = (double)v.y;
+        }
+      });
 }
 
 }  // namespace
@@ -1303,6 +1320,7 @@ void set_smem_attributes() {
   if (!first_on_device(done)) return;
   QBE_CELLS_SMEM(k_prep);
   QBE_CELLS_SMEM(k_i124);
+  QBE_CELLS_SMEM(k_dk_fields);
   QBE_CELLS_SMEM(k_assemble);
   for (int v = 0; v < i3_nvariants<n, T>(); ++v) {
     const I3Launch l = i3_variant<n, T>(v);
@@ -1566,12 +1584,15 @@ cudaError_t collide_post_n(const Tables& t, CollisionWork& cw, double* c, int nc
   C2* spec = cw.i3_paired ? (C2*)cw.K3spec : nullptr;
   reduce_partials<T>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, ncells, s);
   const double2* k3 = cw.K3sum ? cw.K3sum : (const double2*)cw.K3part;
-  const cudaError_t e =
-      QBE_CELLS(k_assemble, ncells, s, (C2*)cw.wfine, (C2*)cw.Dacc, (T*)cw.K2acc, (C2*)cw.K4acc, k3,
-                cw.K3sum ? (size_t)np : (size_t)nparts * np, spec, (size_t)nparts * nq, (C2*)cw.ws, tb.tw, c);
+  C2* DK = (C2*)cw.ws;   // [ncells][4][P], then a field per (cell, pair)
+  cudaError_t e = QBE_CELLS(k_dk_fields, 4 * ncells, s, (C2*)cw.Dacc, (C2*)cw.K4acc, DK, tb.tw);
+  if (e != cudaSuccess) return e;
+  e = QBE_CELLS(k_assemble, 2 * ncells, s, (C2*)cw.wfine, DK, (T*)cw.K2acc, k3,
+                cw.K3sum ? (size_t)np : (size_t)nparts * np, spec, (size_t)nparts * nq,
+                DK + (size_t)ncells * 4 * n * n, tb.tw, c);
   if (tm) tm->end(s);
   if (e != cudaSuccess) return e;
-  launches += 2;
+  launches += 3;
   return cudaGetLastError();
 }
 

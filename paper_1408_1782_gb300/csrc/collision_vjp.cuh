@@ -35,79 +35,80 @@ __device__ __forceinline__ C2 mul_i(C2 v, typename RealOf<C2>::type s) {   // v 
 }
 
 // --------------------------------------------------------------------------
-// Seed: mu = P(E^T lambda) on the fine grid, the forward D and K4 fields, and
-// the transpose of the pointwise Pauli assembly.  One block per cell.
-// Outputs: nu[c][2] (direct cotangent of the w pairs), nuf[c] (cotangent of
-// f = 2 w0 - 1), muD[c][2] (pairs (D1,D2),(D3,-)), muK2[c], mu4[c][2] (raw K4
-// pairs), mu3[c][2] (raw K3 pairs), muh[c][2] (2 pi times the Xi coefficients of
-// the pairs mu_0 + i mu_1, mu_2 + i mu_3).
+// mu = P(E^T lambda) on the fine grid: MU[c][2] (pairs (0,1), (2,3)) and muh[c][2], 2 pi times the Xi
+// coefficients of the pairs mu_0 + i mu_1, mu_2 + i mu_3 (outside Xi not stored).  One team per cell and
+// pair.
 // --------------------------------------------------------------------------
 template <int n, class T, int CB>
-__global__ void __launch_bounds__(kThreads) k_vjp_seed(
-    const double* __restrict__ lam, const typename Vec2Of<T>::type* wfine, const typename Vec2Of<T>::type* Dacc,
-    const T* K2acc, const typename Vec2Of<T>::type* K4acc, typename Vec2Of<T>::type* nu, T* nuf,
-    typename Vec2Of<T>::type* muD, T* muK2, typename Vec2Of<T>::type* mu4, typename Vec2Of<T>::type* mu3,
-    typename Vec2Of<T>::type* muh, T* mupl, typename Vec2Of<T>::type* ws,
-    const typename Vec2Of<T>::type* __restrict__ gtw) {
+__global__ void __launch_bounds__(kThreads) k_vjp_mu(const double* __restrict__ lam, typename Vec2Of<T>::type* MU,
+                                                     typename Vec2Of<T>::type* muh,
+                                                     const typename Vec2Of<T>::type* __restrict__ gtw) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
   C2* sm = tw + n;
   load_twiddles<n>(tw, gtw);
-  constexpr int N = n / 2, P = n * n;
-  const int c = cluster_index();
-  C2* slot = ws + (size_t)cluster_index() * 6 * P;
-  C2* MU = slot;             // [2] cotangent of C_fine pairs (0,1), (2,3)
-  C2* DK = slot + 2 * P;     // [4] D pairs, K4 pairs in real space
+  constexpr int N = n / 2, P = n * n, B = Split<n>::B;
+  const int c = cluster_index() >> 1, p = cluster_index() & 1;
+  C2* M = MU + (size_t)cluster_index() * P;
+  C2* muhp = muh + (size_t)cluster_index() * P;
   const double* lc = lam + (size_t)c * 4 * N * N;
   const T invP = (T)(1.0 / (double)P);
-  for (int p = 0; p < 2; ++p) {
-    C2* M = MU + (size_t)p * P;
-    C2* muhp = muh + ((size_t)c * 2 + p) * P;
-    row_pass<n, -1, false, 0, CB>(
-        sm, tw,
-        [&](int ix, int iy) {
-          if ((ix | iy) & 1) return zero2<T>();
-          const int i = ix >> 1, j = iy >> 1;
-          return mk2((T)lc[((2 * p) * N + i) * N + j], (T)lc[((2 * p + 1) * N + i) * N + j]);
-        },
-        NoMid(), [&](int ix, int iy, C2 v) { M[ix * n + iy] = v; });
-    col_pass<n, -1, true, 1, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&M[ix * n + iy]); },
-        [&](int ix, int iy, C2 v) {
-          const bool keep = in_xi<n>(freq_of_pos<n>(ix)) && in_xi<n>(freq_of_pos<n>(iy));
-          const C2 z = keep ? cscale(v, invP) : zero2<T>();
-          muhp[ix * n + iy] = cscale(z, (T)(2.0 * kPi));
-          return z;
-        },
-        [&](int ix, int iy, C2 v) { M[ix * n + iy] = v; });
-    row_pass<n, 1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&M[ix * n + iy]); }, NoMid(),
-        [&](int ix, int iy, C2 v) { M[ix * n + iy] = v; });
-  }
-  for (int f = 0; f < 4; ++f) {
-    const C2* in = (f < 2) ? (Dacc + ((size_t)c * 2 + f) * P) : (K4acc + ((size_t)c * 2 + (f - 2)) * P);
-    C2* out = DK + (size_t)f * P;
-    col_pass<n, 1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return in[ix * n + iy]; }, NoMid(),
-        [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
-    row_pass<n, 1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&out[ix * n + iy]); }, NoMid(),
-        [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
-  }
-  const C2* wf0 = wfine + (size_t)c * 2 * P;
-  const C2* wf1 = wf0 + P;
-  const T* K2 = K2acc + (size_t)c * P;
-  C2* nuc = nu + (size_t)c * 2 * P;
-  T* nufc = nuf + (size_t)c * P;
-  C2* muDc = muD + (size_t)c * 2 * P;
-  T* muK2c = muK2 + (size_t)c * P;
-  C2* mu4c = mu4 + (size_t)c * 2 * P;
-  C2* mu3c = mu3 + (size_t)c * 2 * P;
-  const double tp = 2.0 * kPi;
-  for (int i = element_first(); i < P; i += element_stride()) {
-    const C2 mu01 = ldc(&MU[i]), mu23 = ldc(&MU[P + i]);
-    const C2 dk0 = ldc(&DK[i]), dk1 = ldc(&DK[P + i]), dk2 = ldc(&DK[2 * P + i]), dk3 = ldc(&DK[3 * P + i]);
+  even_row_pass<n, -1, CB>(
+      sm, tw,
+      [&](int ix, int iy) {
+        if (iy & 1) return zero2<T>();
+        const int i = ix >> 1, j = iy >> 1;
+        return mk2((T)lc[((2 * p) * N + i) * N + j], (T)lc[((2 * p + 1) * N + i) * N + j]);
+      },
+      [&](int ix, int iy, C2 v) {
+        if (xi_t<B>(iy % B)) M[ix * n + iy] = v;
+      });
+  xi_col_filter<n, true, true, CB>(
+      sm, tw, [&](int ix, int iy) { return (ix & 1) ? zero2<T>() : ldc(&M[ix * n + iy]); },
+      [&](int ix, int iy, C2 v) {
+        const bool keep = xi_slot<n>(ix) >= 0 && xi_slot<n>(iy) >= 0;
+        const C2 z = keep ? cscale(v, invP) : zero2<T>();
+        muhp[ix * n + iy] = cscale(z, (T)(2.0 * kPi));
+        return z;
+      },
+      [&](int ix, int iy, C2 v) { M[ix * n + iy] = v; });
+  row_pass<n, 1, false, 0, CB, true>(
+      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&M[ix * n + iy]) : zero2<T>(); }, NoMid(),
+      [&](int ix, int iy, C2 v) { M[ix * n + iy] = v; });
+}
+
+// --------------------------------------------------------------------------
+// Seed: the transpose of the pointwise Pauli assembly, from mu (k_vjp_mu) and the forward D and K4
+// fields (k_dk_fields).  Outputs: nu[c][2] (direct cotangent of the w pairs), nuf[c] (cotangent of
+// f = 2 w0 - 1), muD[c][2] (pairs (D1,D2),(D3,-)), muK2[c], mu4[c][2] (raw K4
+// pairs), mu3[c][2] (raw K3 pairs), mupl[c][4] (may be null: mu3 as planes).
+// --------------------------------------------------------------------------
+template <int n, class T>
+__global__ void __launch_bounds__(kThreads) k_vjp_seed(
+    const typename Vec2Of<T>::type* MUall, const typename Vec2Of<T>::type* DKall,
+    const typename Vec2Of<T>::type* wfine, const T* K2acc, typename Vec2Of<T>::type* nu, T* nuf,
+    typename Vec2Of<T>::type* muD, T* muK2, typename Vec2Of<T>::type* mu4, typename Vec2Of<T>::type* mu3, T* mupl,
+    int ncells) {
+  using C2 = typename Vec2Of<T>::type;
+  constexpr int P = n * n;
+  for (size_t g = (size_t)blockIdx.x * kThreads + threadIdx.x; g < (size_t)ncells * P;
+       g += (size_t)gridDim.x * kThreads) {
+    const int c = (int)(g / P), i = (int)(g % P);
+    const C2* MU = MUall + (size_t)c * 2 * P;
+    const C2* DK = DKall + (size_t)c * 4 * P;
+    const C2* wf0 = wfine + (size_t)c * 2 * P;
+    const C2* wf1 = wf0 + P;
+    const T* K2 = K2acc + (size_t)c * P;
+    C2* nuc = nu + (size_t)c * 2 * P;
+    T* nufc = nuf + (size_t)c * P;
+    C2* muDc = muD + (size_t)c * 2 * P;
+    T* muK2c = muK2 + (size_t)c * P;
+    C2* mu4c = mu4 + (size_t)c * 2 * P;
+    C2* mu3c = mu3 + (size_t)c * 2 * P;
+    const double tp = 2.0 * kPi;
+    const C2 mu01 = MU[i], mu23 = MU[P + i];
+    const C2 dk0 = DK[i], dk1 = DK[P + i], dk2 = DK[2 * P + i], dk3 = DK[3 * P + i];
     const double m0 = mu01.x, m1 = mu01.y, m2 = mu23.x, m3 = mu23.y;
     const double w0 = wf0[i].x, w1 = wf0[i].y, w2 = wf1[i].x, w3 = wf1[i].y;
     const double D1 = dk0.x, D2 = dk0.y, D3 = dk1.x;
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(kThreads) k_i1_vjp(
   C2* tw = reinterpret_cast<C2*>(smem_raw);
   C2* sm = tw + n;
   load_twiddles<n>(tw, gtw);
-  constexpr int P = n * n;
+  constexpr int P = n * n, B = Split<n>::B;
   // block (cell c, angle chunk ch); with nch > 1, nu and nuf are per-(cell, chunk) partials (zeroed
   // here, completed by k_i24_vjp, summed by k_add_chunks), with nch = 1 the cell's own accumulators
   const int c = cluster_index() / nch, ch = cluster_index() % nch;
@@ -185,11 +186,11 @@ __global__ void __launch_bounds__(kThreads) k_i1_vjp(
       const C2* in = what + ((size_t)c * 4 + 2 + p) * P;
       const C2* mu = muD + ((size_t)c * 2 + p) * P;
       // Aw = IFFT(i phi' w^)
-      col_pass<n, 1, false, 0, CB>(
-          sm, tw, [&](int ix, int iy) { return mul_i(in[ix * n + iy], ph[ix * n + iy]); }, NoMid(),
+      xi_col_pass<n, CB>(
+          sm, tw, [&](int ix, int iy) { return mul_i(in[ix * n + iy], ph[ix * n + iy]); },
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-      row_pass<n, 1, false, 0, CB>(
-          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
+      row_pass<n, 1, false, 0, CB, true>(
+          sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&G[ix * n + iy]) : zero2<T>(); }, NoMid(),
           [&](int ix, int iy, C2 v) { Aw[ix * n + iy] = v; });
       // Bm = IFFT(i K FFT(mu))   (K already carries 1/n^2)
       row_pass<n, -1, false, 0, CB>(
@@ -248,7 +249,7 @@ __global__ void __launch_bounds__(kThreads) k_i24_vjp(
   C2* tw = reinterpret_cast<C2*>(smem_raw);
   C2* sm = tw + n;
   load_twiddles<n>(tw, gtw);
-  constexpr int P = n * n;
+  constexpr int P = n * n, B = Split<n>::B;
   // block (cell c, chunk ch of the J/2 angle pairs); nu, nuf as in k_i1_vjp
   const int c = cluster_index() / nch, ch = cluster_index() % nch;
   C2* slot = ws + (size_t)cluster_index() * 7 * P;
@@ -271,11 +272,11 @@ __global__ void __launch_bounds__(kThreads) k_i24_vjp(
       for (int h = 0; h < 2; ++h) {
         const T* ps = psi + (size_t)(h == 0 ? j : jq) * P;
         C2* F = (h == 0 ? FA : FB) + (size_t)p * P;
-        col_pass<n, 1, false, 0, CB>(
-            sm, tw, [&](int ix, int iy) { return cscale(in[ix * n + iy], ps[ix * n + iy]); }, NoMid(),
+        xi_col_pass<n, CB>(
+            sm, tw, [&](int ix, int iy) { return cscale(in[ix * n + iy], ps[ix * n + iy]); },
             [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
-        row_pass<n, 1, false, 0, CB>(
-            sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
+        row_pass<n, 1, false, 0, CB, true>(
+            sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&G[ix * n + iy]) : zero2<T>(); }, NoMid(),
             [&](int ix, int iy, C2 v) { F[ix * n + iy] = v; });
       }
     }
@@ -655,7 +656,7 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_vjp_smem(
 // partials (planes [4][P], FP64); gradient = 4 E P (nu + IFFT(H) / n^2) with H the
 // reduced I3 spectral partials (k_reduce_k3).  P keeps the kept frequencies only and FFT(IFFT(H)) =
 // n^2 H, so H (stored on those frequencies) is added to FFT(nu) there.
-// One block per cell; writes grad[c][4][N][N] (FP64).
+// One team per cell and pair; writes grad[c][4][N][N] (FP64).
 // --------------------------------------------------------------------------
 template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads) k_vjp_final(
@@ -666,58 +667,53 @@ __global__ void __launch_bounds__(kThreads) k_vjp_final(
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
   C2* sm = tw + n;
-  __shared__ int kslot[n];
-  __shared__ int kcols[n];
-  build_xi_slots<n>(kslot, kcols);
   load_twiddles<n>(tw, gtw);
-  constexpr int N = n / 2, P = n * n;
+  constexpr int N = n / 2, P = n * n, B = Split<n>::B;
   constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
-  const int c = cluster_index();
-  C2* slot = ws + (size_t)cluster_index() * 5 * P;
-  C2* V = slot;            // [2] total real-space cotangent pairs
-  C2* F = slot + 2 * P;    // [2] their transforms
-  const double* Rc = R + c * r_stride;
-  const C2* H = spec + c * spec_stride;   // [2][Q]
-  for (int i = element_first(); i < 2 * P; i += element_stride()) {
-    const int e = i % P;
-    const double* Rp = Rc + (size_t)(i < P ? 0 : 2) * P + e;
-    const C2 d = nu[(size_t)c * 2 * P + i];
-    double vx = (double)d.x + Rp[0], vy = (double)d.y + Rp[P];
-    if (i < P) vx += 2.0 * (double)nuf[(size_t)c * P + i];
-    V[i] = mk2((T)vx, (T)vy);
-  }
-  team_sync();
+  const int c = cluster_index() >> 1, p = cluster_index() & 1;
+  C2* F = ws + (size_t)cluster_index() * P;
+  const double* Rc = R + c * r_stride + (size_t)2 * p * P;
+  const C2* Hp = spec + c * spec_stride + (size_t)p * Q;
+  const C2* nup = nu + ((size_t)c * 2 + p) * P;
+  const T* nufc = nuf + (size_t)c * P;
   const T invP = (T)(1.0 / (double)P);
-  for (int p = 0; p < 2; ++p) {
-    C2* Vp = V + (size_t)p * P;
-    C2* Fp = F + (size_t)p * P;
-    const C2* Hp = H + (size_t)p * Q;
-    // 4 E P (V + IFFT(H) / n^2)
-    row_pass<n, -1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&Vp[ix * n + iy]); }, NoMid(),
-        [&](int ix, int iy, C2 v) { Fp[ix * n + iy] = v; });
-    col_pass<n, -1, true, 1, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&Fp[ix * n + iy]); },
-        [&](int ix, int iy, C2 v) {
-          const int sx = kslot[ix], sy = kslot[iy];
-          if (sx < 0 || sy < 0) return zero2<T>();
-          const C2 h = Hp[sx * NQ + sy];
-          return cscale(cadd(v, h), invP);
-        },
-        [&](int ix, int iy, C2 v) { Fp[ix * n + iy] = v; });
-    double* g = grad + (size_t)c * 4 * N * N;
-    row_pass<n, 1, false, 0, CB>(
-        sm, tw, [&](int ix, int iy) { return ldc(&Fp[ix * n + iy]); }, NoMid(),
-        [&](int ix, int iy, C2 v) {
-          if (((ix | iy) & 1) == 0) {
-            const int i = ix >> 1, j = iy >> 1;
-            double* g0 = g + ((2 * p) * N + i) * N + j;
-            double* g1 = g + ((2 * p + 1) * N + i) * N + j;
-            *g0 = (accumulate ? *g0 : 0.0) + 4.0 * (double)v.x;
-            *g1 = (accumulate ? *g1 : 0.0) + 4.0 * (double)v.y;
-          }
-        });
-  }
+  // 4 E P (V + IFFT(H) / n^2), V the total real-space cotangent of the pair
+  row_pass<n, -1, false, 0, CB>(
+      sm, tw,
+      [&](int ix, int iy) {
+        const int i = ix * n + iy;
+        const C2 d = nup[i];
+        double vx = (double)d.x + Rc[i];
+        const double vy = (double)d.y + Rc[P + i];
+        if (p == 0) vx += 2.0 * (double)nufc[i];
+        return mk2((T)vx, (T)vy);
+      },
+      NoMid(),
+      [&](int ix, int iy, C2 v) {
+        if (xi_t<B>(iy % B)) F[ix * n + iy] = v;
+      });
+  xi_col_filter<n, true, true, CB>(
+      sm, tw, [&](int ix, int iy) { return ldc(&F[ix * n + iy]); },
+      [&](int ix, int iy, C2 v) {
+        const int sx = xi_slot<n>(ix), sy = xi_slot<n>(iy);
+        if (sx < 0 || sy < 0) return zero2<T>();
+        return cscale(cadd(v, Hp[sx * NQ + sy]), invP);
+      },
+      [&](int ix, int iy, C2 v) {
+        if (!(ix & 1)) F[ix * n + iy] = v;
+      });
+  double* g = grad + (size_t)c * 4 * N * N;
+  even_row_pass<n, 1, CB, true>(
+      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&F[ix * n + iy]) : zero2<T>(); },
+      [&](int ix, int iy, C2 v) {
+        if (!(iy & 1)) {
+          const int i = ix >> 1, j = iy >> 1;
+          double* g0 = g + ((2 * p) * N + i) * N + j;
+          double* g1 = g + ((2 * p + 1) * N + i) * N + j;
+          *g0 = (accumulate ? *g0 : 0.0) + 4.0 * (double)v.x;
+          *g1 = (accumulate ? *g1 : 0.0) + 4.0 * (double)v.y;
+        }
+      });
 }
 
 }  // namespace
@@ -742,7 +738,7 @@ template <int n, class T>
 void set_vjp_smem_attributes() {
   static unsigned long long done = 0;
   if (!first_on_device(done)) return;
-  QBE_CELLS_SMEM(k_vjp_seed);
+  QBE_CELLS_SMEM(k_vjp_mu);
   QBE_CELLS_SMEM(k_i1_vjp);
   QBE_CELLS_SMEM(k_i24_vjp);
   QBE_CELLS_SMEM(k_vjp_final);
@@ -788,6 +784,10 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
     e = per_cell_terms<n, T>(t, cw, ws, ncells, s, launches, nullptr);
     if (e != cudaSuccess) return e;
   }
+  C2* DK = ws;   // [ncells][4][P] real-space D and K4 pairs of the state
+  e = QBE_CELLS(k_dk_fields, 4 * ncells, s, Dacc, K4acc, DK, tb.tw);
+  if (e != cudaSuccess) return e;
+  ++launches;
   for (int k = 0; k < K; ++k) {
     C2* nu = (C2*)vw.nu + k * c_stride;
     T* nuf = (T*)vw.nuf + k * r_stride;
@@ -797,9 +797,18 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
     C2* mu3 = (C2*)vw.mu3 + k * c_stride;
     C2* muh = (C2*)vw.muh + k * c_stride;
     T* mupl = vw.mupl ? (T*)vw.mupl + k * 2 * c_stride : nullptr;
-    e = QBE_CELLS(k_vjp_seed, ncells, s, lam[k], wfine, Dacc, K2acc, K4acc, nu, nuf, muD, muK2, mu4, mu3, muh, mupl, ws,
-                  tb.tw);
+    C2* MU = DK + (size_t)ncells * 4 * P;   // [ncells][2][P]
+    e = QBE_CELLS(k_vjp_mu, 2 * ncells, s, lam[k], MU, muh, tb.tw);
     if (e != cudaSuccess) return e;
+    if (k > 0) {   // the I1 and I2/I4 transposes of the cotangent before used the scratch
+      e = QBE_CELLS(k_dk_fields, 4 * ncells, s, Dacc, K4acc, DK, tb.tw);
+      if (e != cudaSuccess) return e;
+      ++launches;
+    }
+    const size_t seed_blocks = ((size_t)ncells * P + kThreads - 1) / kThreads;
+    k_vjp_seed<n, T><<<(unsigned)(seed_blocks < 65535 ? seed_blocks : 65535), kThreads, 0, s>>>(
+        MU, DK, wfine, K2acc, nu, nuf, muD, muK2, mu4, mu3, mupl, ncells);
+    ++launches;
     // I1 and I2/I4 transposes over (cell, angle chunk) blocks; their per-chunk cotangents go to the
     // forward's chunk-partial buffers (free once per_cell_terms has reduced them) and are summed in
     // chunk order into nu and nuf
@@ -854,7 +863,7 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
     C2* ps = (C2*)vw.part_s + k * spart_stride;
     reduce_partials<T>(pr, cw.K3sum, ps, units, np, nq, ncells, s);
     const double* R = cw.K3sum ? (const double*)cw.K3sum : (const double*)pr;
-    e = QBE_CELLS(k_vjp_final, ncells, s, (C2*)vw.nu + k * c_stride, (T*)vw.nuf + k * r_stride, R,
+    e = QBE_CELLS(k_vjp_final, 2 * ncells, s, (C2*)vw.nu + k * c_stride, (T*)vw.nuf + k * r_stride, R,
                   (cw.K3sum ? (size_t)1 : (size_t)units) * 2 * np, ps, (size_t)units * nq, ws, tb.tw, grad[k], accumulate);
     if (e != cudaSuccess) return e;
     launches += 2;

@@ -513,31 +513,75 @@ __device__ __forceinline__ void col_pass(C2* sm, const C2* tw, LD ld, MID mid, S
   if (ranks > 1) cluster_sync_global();
 }
 
-// Inverse column pass of a spectrum that vanishes outside Xi: the n / 2 columns of Xi only, ld(ix, iy)
-// called for Xi rows only (iy, ix permuted positions).
-template <int n, int CB = 65536, class C2, class LD, class ST>
-__device__ __forceinline__ void xi_col_pass(C2* sm, const C2* tw, LD ld, ST st) {
-  constexpr int CC = Chunk<n, sizeof(C2), CB>::CC, B = Split<n>::B;
+// Passes over n / 2 of the lines: the chunks are halved where a chunk is n / 8 lines (teams of up to eight
+// blocks), so that eight blocks share these passes too.
+template <int n, int CHUNK>
+__host__ __device__ constexpr int half_chunk() {
+  return (CHUNK == n / 8 && CHUNK > 1) ? CHUNK / 2 : CHUNK;
+}
+// The li-th of the n / 2 permuted positions of Xi.
+template <int n>
+__host__ __device__ __forceinline__ int xi_position(int li) {
+  constexpr int B = Split<n>::B;
+  const int k1 = li / (B / 2), t = li % (B / 2);
+  return B * k1 + (t < B / 4 ? t : t + B / 2);
+}
+
+// Column passes over the n / 2 columns iy of Xi.  FWD: forward transform of ld(ix, iy), then mid(ix, iy, v)
+// on the Xi rows (permuted positions); without FWD ld gives the spectrum and is called for Xi rows only.
+// INV: inverse transform (zero outside the Xi rows), then st(ix, iy, v) on every row.
+template <int n, bool FWD, bool INV, int CB = 65536, class C2, class LD, class MID, class ST>
+__device__ __forceinline__ void xi_col_filter(C2* sm, const C2* tw, LD ld, MID mid, ST st) {
+  constexpr int CC = half_chunk<n, Chunk<n, sizeof(C2), CB>::CC>(), B = Split<n>::B;
   const int tid = threadIdx.x, nt = blockDim.x;
-  auto column = [](int li) {
-    const int k1 = li / (B / 2), t = li % (B / 2);
-    return B * k1 + (t < B / 4 ? t : t + B / 2);
-  };
   const int ranks = cluster_size();
   for (int c0 = cluster_rank() * CC; c0 < n / 2; c0 += ranks * CC) {
     const int nc = (n / 2 - c0) < CC ? (n / 2 - c0) : CC;
 #pragma unroll 4
     for (int idx = tid; idx < nc * n; idx += nt) {
       const int ix = idx / nc, c = idx % nc;
-      if (xi_t<B>(ix % B)) sm[ix * CC + c] = ld(ix, column(c0 + c));   // the first stage reads no other
+      if (FWD || xi_t<B>(ix % B)) sm[ix * CC + c] = ld(ix, xi_position<n>(c0 + c));
     }
     __syncthreads();
-    fft_lines<n, 1, true>(sm, nc, 1, CC, tw);
+    if constexpr (FWD) {
+      fft_lines<n, -1>(sm, nc, 1, CC, tw);
 #pragma unroll 4
-    for (int idx = tid; idx < nc * n; idx += nt) {
-      const int ix = idx / nc, c = idx % nc;
-      st(ix, column(c0 + c), sm[ix * CC + c]);
+      for (int idx = tid; idx < nc * n; idx += nt) {
+        const int ix = idx / nc, c = idx % nc;
+        if (xi_t<B>(ix % B)) sm[ix * CC + c] = mid(ix, xi_position<n>(c0 + c), sm[ix * CC + c]);
+      }
+      __syncthreads();
     }
+    if constexpr (INV) {
+      fft_lines<n, 1, true>(sm, nc, 1, CC, tw);
+#pragma unroll 4
+      for (int idx = tid; idx < nc * n; idx += nt) {
+        const int ix = idx / nc, c = idx % nc;
+        st(ix, xi_position<n>(c0 + c), sm[ix * CC + c]);
+      }
+      __syncthreads();
+    }
+  }
+  if (ranks > 1) cluster_sync_global();
+}
+template <int n, int CB = 65536, class C2, class LD, class ST>
+__device__ __forceinline__ void xi_col_pass(C2* sm, const C2* tw, LD ld, ST st) {
+  xi_col_filter<n, false, true, CB>(sm, tw, ld, [](int, int, C2 v) { return v; }, st);
+}
+// Row pass over the even rows ix (the coarse nodes, or a zero-interleaved coarse field).
+template <int n, int DIR, int CB = 65536, bool XI = false, class C2, class LD, class ST>
+__device__ __forceinline__ void even_row_pass(C2* sm, const C2* tw, LD ld, ST st) {
+  constexpr int RC = half_chunk<n, Chunk<n, sizeof(C2), CB>::RC>(), LS = Chunk<n, sizeof(C2), CB>::LS;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int ranks = cluster_size();
+  for (int r0 = cluster_rank() * RC; r0 < n / 2; r0 += ranks * RC) {
+    const int nr = (n / 2 - r0) < RC ? (n / 2 - r0) : RC;
+#pragma unroll 4
+    for (int idx = tid; idx < nr * n; idx += nt) sm[idx / n * LS + idx % n] = ld(2 * (r0 + idx / n), idx % n);
+    __syncthreads();
+    fft_lines<n, DIR, XI>(sm, nr, LS, 1, tw);
+#pragma unroll 4
+    for (int idx = tid; idx < nr * n; idx += nt) st(2 * (r0 + idx / n), idx % n, sm[idx / n * LS + idx % n]);
     __syncthreads();
   }
   if (ranks > 1) cluster_sync_global();
