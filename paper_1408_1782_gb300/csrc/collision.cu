@@ -86,22 +86,62 @@ bool i3_paired(int n, int prec, int variant) {
 #undef QBE_CALL
 }
 
-double i3_chunk_cost(int begin, int end, int M, bool paired) {
-  if (!paired) return 18.0 * (end - begin);      // 2 shifts, 16 transforms of 8 convolutions
+namespace {
+// Two-dimensional transforms of a middle node, a node pair and half a pair.
+struct NodeCost {
+  double mid, pair, half;
+};
+constexpr NodeCost kForwardCost = {18, 20, 11};      // 2 shifts, 2 per convolution (8 or 4), back 2 or 1
+constexpr NodeCost kTransposeCost = {36, 38, 22};    // 2 or 4 shifts, 16 or 8 convolutions, 2 back
+
+double chunk_cost(int begin, int end, int M, const NodeCost& c) {
   double cost = 0;
   for (int it = begin; it < end;) {
     if ((M & 1) && it == M - 1) {
-      cost += 18.0;                              // the middle node
+      cost += c.mid;
       it += 1;
     } else if ((it & 1) == 0 && it + 1 < end) {
-      cost += 20.0;                              // a pair: 2 shifts, 8 convolutions, 2 back
+      cost += c.pair;
       it += 2;
     } else {
-      cost += 11.0;                              // half a pair
+      cost += c.half;
       it += 1;
     }
   }
   return cost;
+}
+
+// m-chunks per (cell, angle) for a launch that works on G units at a time, unit u on slot u mod G: `base`,
+// or up to three times as many (at least `most_at_least`, at most M) where that evens out the slots'
+// loads by more than a hundredth, within 4 GB of partials.  A unit's fixed costs (its tables loaded, its
+// partials written and reduced) count per_unit transforms.
+int even_chunks(long long cj, int G, int M, int base, int most_at_least, size_t unit_bytes, const NodeCost& c,
+                double per_unit) {
+  double best = 0;
+  int best_nmc = base;
+  const int most = 3 * base > most_at_least ? 3 * base : most_at_least;
+  for (int want = base; want <= most && want <= M; ++want) {
+    const int mch = (M + want - 1) / want, nmc = (M + mch - 1) / mch;
+    const long long units = cj * nmc;
+    if (want > base && (nmc == base || (size_t)units * unit_bytes > ((size_t)4 << 30))) continue;
+    const int g = G < units ? G : (int)units;
+    std::vector<double> load(g, 0.0), cost(nmc);
+    for (int mc = 0; mc < nmc; ++mc)
+      cost[mc] = per_unit + chunk_cost(i3_chunk_begin(mc, nmc, M), i3_chunk_begin(mc + 1, nmc, M), M, c);
+    for (long long u = 0; u < units; ++u) load[u % g] += cost[u % nmc];
+    double mx = 0;
+    for (double l : load) mx = l > mx ? l : mx;
+    if (want == base || mx < 0.99 * best) {
+      best = mx;
+      best_nmc = nmc;
+    }
+  }
+  return best_nmc;
+}
+}  // namespace
+
+double i3_chunk_cost(int begin, int end, int M, bool paired) {
+  return paired ? chunk_cost(begin, end, M, kForwardCost) : kForwardCost.mid * (end - begin);
 }
 
 // Angle chunks per cell of the I1 and I2/I4 kernels: enough (cell, chunk) blocks to fill about one
@@ -154,28 +194,9 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
     cw.nmc = (t.M + cw.mch - 1) / cw.mch;
   };
   set_chunks(nmc);
-  if (i3_paired(t.n, prec, v0)) {
-    // Up to three times as many chunks where they even out the blocks' loads (unit u goes to block
-    // u mod G) within 4 GB of partials: a unit's fixed costs (its partials written and reduced, about
-    // a fiftieth of a pair's transforms) against the last, partly filled wave.
-    const int base = cw.nmc;
-    double best = 0;
-    int best_nmc = base;
-    for (int want = base; want <= 3 * base && want <= t.M; ++want) {
-      set_chunks(want);
-      const long long units = (long long)nb * t.J * cw.nmc;
-      if (want > base && (cw.nmc == base || (size_t)units * part_bytes > ((size_t)4 << 30))) continue;
-      const int G = i3_concurrency(t.n, prec, v0, cw.grid_i3, (int)(units < INT_MAX ? units : INT_MAX));
-      std::vector<double> load(G, 0.0), cost(cw.nmc);
-      for (int mc = 0; mc < cw.nmc; ++mc)
-        cost[mc] = 0.4 + i3_chunk_cost(i3_chunk_begin(mc, cw.nmc, t.M), i3_chunk_begin(mc + 1, cw.nmc, t.M), t.M, true);
-      for (long long u = 0; u < units; ++u) load[u % G] += cost[u % cw.nmc];
-      double mx = 0;
-      for (double l : load) mx = l > mx ? l : mx;
-      if (want == base || mx < 0.99 * best) { best = mx; best_nmc = cw.nmc; }
-    }
-    set_chunks(best_nmc);
-  }
+  if (i3_paired(t.n, prec, v0))
+    set_chunks(even_chunks(cj, i3_concurrency(t.n, prec, v0, cw.grid_i3, INT_MAX), t.M, cw.nmc, 1, part_bytes,
+                           kForwardCost, 0.4));
   const size_t nparts = (size_t)nb * t.J * cw.nmc;
   cw.nparts_cap = nparts;
   cw.ws_slots = nb > cw.grid_i3 ? nb : cw.grid_i3;
@@ -337,6 +358,15 @@ cudaError_t alloc_vjp_work(const Tables& t, int nb, VjpWork& vw, int prec, int k
   if (nmc < 1) nmc = 1;
   vw.mch = (t.M + nmc - 1) / nmc;
   vw.nmc = (t.M + vw.mch - 1) / vw.mch;
+  {
+    const size_t Q1 = (size_t)(t.n / 2 - 1) * (t.n / 2 - 1);
+    // (of as many cotangents as a product can carry: the chunking, and with it the order of the sums, must
+    // not depend on how many this workspace holds)
+    const size_t unit_bytes =
+        (size_t)vjp_cotangent_group(t, prec) * 2 * (P + Q1) * (prec == 1 ? sizeof(float2) : sizeof(double2));
+    vw.nmc = even_chunks(cj, vw.grid * teams, t.M, vw.nmc, 8, unit_bytes, kTransposeCost, 1.0);
+    vw.mch = (t.M + vw.nmc - 1) / vw.nmc;
+  }
   const size_t nparts = (size_t)nb * t.J * vw.nmc;
   // per-cell kernels: 7 fields per cell; I3 transpose per block: 3 + 4 K fields (staged; the
   // shared-memory kernel one less), 6 per team

@@ -997,11 +997,15 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
 
 // --------------------------------------------------------------------------
 // Sums of the per-unit I3 partials of each cell, in FP64: the np fine-grid values (2 n^2 complex) and
-// the nq Fourier-space values (kept frequencies; nq = 0 where the launch wrote none).  A block takes
-// 256 / G points with G threads each, thread g the units u = g mod G, added in the order of g.
-// Bound by HBM (or L2, where the partials still sit there).  It was part of k_assemble, whose one
-// block per cell read a single cell's partials alone: at one cell of N = 32, J = M = 32, 1024 units,
-// 5.2 of the 5.5 ms of that kernel.
+// the nq Fourier-space values (kept frequencies; nq = 0 where the launch wrote none), 16 bytes per
+// load.  A block takes 256 / G such words with G threads each, thread g the units u = g mod G, added in
+// the order of g.  Bound by HBM (or L2, where the partials still sit there).  It was part of k_assemble,
+// whose one block per cell read a single cell's partials alone: at one cell of N = 32, J = M = 32, 1024
+// units, 5.2 of the 5.5 ms of that kernel.
+// FP32 partials are added as unevaluated sums hi + lo of two floats (the error-free addition of Knuth,
+// TwoSum; about 48 bits) and combined in FP64: converting and adding each value in FP64 bound the kernel
+// at a fifth of the memory rate (two FP64 lanes per clock), 128 cells of N = 64 1234 us
+// against 264 us.
 // sum: [ncells][np], or null (FP64): in place into the cell's first unit; the Fourier-space sums are
 // always put there.
 // --------------------------------------------------------------------------
@@ -1009,46 +1013,72 @@ template <class T, int G>
 __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* part, double2* sum,
                                                    typename Vec2Of<T>::type* spec, int nparts, int np, int nq,
                                                    int chunks) {
-  using C2 = typename Vec2Of<T>::type;
-  constexpr int PT = 256 / G;
+  using Word = typename std::conditional<sizeof(T) == 8, double2, float4>::type;
+  constexpr int PT = 256 / G, VEC = sizeof(T) == 8 ? 1 : 2;   // complex values per word
   const size_t c = blockIdx.x / chunks;
-  const int i = (blockIdx.x % chunks) * PT + threadIdx.x % PT, g = threadIdx.x / PT;
+  const int i = ((blockIdx.x % chunks) * PT + threadIdx.x % PT) * VEC, g = threadIdx.x / PT;
   const bool real_space = i < np;
-  C2* src = real_space ? part + c * nparts * np + i : spec + c * nparts * nq + (i - np);
-  const size_t stride = real_space ? np : nq;
-  double sx = 0, sy = 0;
+  Word* src = reinterpret_cast<Word*>(real_space ? part + c * nparts * np + i : spec + c * nparts * nq + (i - np));
+  const size_t stride = (size_t)(real_space ? np : nq) / VEC;
+  double s[2 * VEC] = {};
   if (i < np + nq) {
+    if constexpr (VEC == 1) {
 #pragma unroll 8
-    for (int u = g; u < nparts; u += G) {
-      const C2 v = src[(size_t)u * stride];
-      sx += (double)v.x;
-      sy += (double)v.y;
+      for (int u = g; u < nparts; u += G) {
+        const Word v = src[(size_t)u * stride];
+        s[0] += v.x;
+        s[1] += v.y;
+      }
+    } else {
+      float hi[4] = {}, lo[4] = {};
+#pragma unroll 8
+      for (int u = g; u < nparts; u += G) {
+        const Word v = src[(size_t)u * stride];
+        const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float t = __fadd_rn(hi[k], x[k]), z = __fsub_rn(t, hi[k]);
+          lo[k] = __fadd_rn(lo[k], __fadd_rn(__fsub_rn(hi[k], __fsub_rn(t, z)), __fsub_rn(x[k], z)));
+          hi[k] = t;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) s[k] = (double)hi[k] + (double)lo[k];
     }
   }
   if constexpr (G > 1) {
-    __shared__ double2 red[G][PT];
-    red[g][threadIdx.x % PT] = mk2(sx, sy);
+    __shared__ double red[G][2 * VEC][PT];
+#pragma unroll
+    for (int k = 0; k < 2 * VEC; ++k) red[g][k][threadIdx.x % PT] = s[k];
     __syncthreads();
     if (g > 0) return;
-    for (int k = 1; k < G; ++k) {
-      sx += red[k][threadIdx.x].x;
-      sy += red[k][threadIdx.x].y;
-    }
+    for (int j = 1; j < G; ++j)
+#pragma unroll
+      for (int k = 0; k < 2 * VEC; ++k) s[k] += red[j][k][threadIdx.x];
   }
   if (i >= np + nq) return;
-  if (real_space && sum) sum[c * np + i] = mk2(sx, sy);
-  else *src = mk2((T)sx, (T)sy);
+  if (real_space && sum) {
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) sum[c * np + i + k] = mk2(s[2 * k], s[2 * k + 1]);
+  } else {
+    T* o = reinterpret_cast<T*>(src);
+#pragma unroll
+    for (int k = 0; k < 2 * VEC; ++k) o[k] = (T)s[k];
+  }
 }
 
-// From 16 units per cell on, eight threads per point: short columns of loads, more of them in flight.
+// One thread per word where that gives a thousand threads per SM, eight otherwise: short columns of loads,
+// more of them in flight.
 template <class T>
 void reduce_partials(typename Vec2Of<T>::type* part, double2* sum, typename Vec2Of<T>::type* spec, int nparts, int np,
                      int nq, int ncells, cudaStream_t s) {
-  if (nparts >= 16) {
-    const int chunks = (np + nq + 31) / 32;
+  constexpr int VEC = sizeof(T) == 8 ? 1 : 2;
+  const int words = (np + nq) / VEC;
+  if (nparts >= 16 && (long long)words * ncells < 152 * 1024) {
+    const int chunks = (words + 31) / 32;
     k_reduce_k3<T, 8><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, nparts, np, nq, chunks);
   } else {
-    const int chunks = (np + nq + 255) / 256;
+    const int chunks = (words + 255) / 256;
     k_reduce_k3<T, 1><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, nparts, np, nq, chunks);
   }
 }
