@@ -391,12 +391,11 @@ template <int n, class T>
 __global__ void __launch_bounds__(kThreads, 3) k_i3_vjp(
     const typename Vec2Of<T>::type* what, const typename Vec2Of<T>::type* wfine,
     const typename Vec2Of<T>::type* mu3, const typename Vec2Of<T>::type* muh, typename Vec2Of<T>::type* part_r,
-    typename Vec2Of<T>::type* part_s, typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__ gtw,
-    const T* __restrict__ psip_s, const typename Vec2Of<T>::type* __restrict__ phase, int J, int M, int nmc,
-    int nunits, int K, size_t mu_stride, size_t part_stride, size_t spart_stride) {
+    typename Vec2Of<T>::type* part_s, typename Vec2Of<T>::type* ws, const T* __restrict__ psip_s,
+    const typename Vec2Of<T>::type* __restrict__ phase, int J, int M, int nmc, int nunits, int K, size_t mu_stride, size_t part_stride, size_t spart_stride) {
   using C2 = typename Vec2Of<T>::type;
   using Lines = StagedLines<n, T, kThreads, kVjpCB>;
-  constexpr int A = Split<n>::A, B = Split<n>::B, P = n * n, Q = Lines::Q;
+  constexpr int P = n * n, Q = Lines::Q;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int kslot[n];
   C2* slot = ws + (size_t)blockIdx.x * (3 + 4 * K) * P;
@@ -404,11 +403,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_i3_vjp(
   C2* Nu = slot + 3 * P;                           // [K][2][P] shifted pairs of the cotangents
   T* X = reinterpret_cast<T*>(slot + (3 + 2 * K) * (size_t)P);   // [K][4][P]
   Lines ln;
-  ln.twT = reinterpret_cast<C2*>(smem_raw);
-  ln.sm = ln.twT + n;
+  ln.init(reinterpret_cast<C2*>(smem_raw));
   ln.kslot = kslot;
   ln.G = slot + 2 * P;
-  for (int pos = threadIdx.x; pos < n; pos += kThreads) ln.twT[(pos % A) * B + pos / A] = gtw[pos];
   build_xi_slots<n>(kslot);
   for (int unit = blockIdx.x; unit < nunits; unit += gridDim.x) {
     const int c = unit / (J * nmc);
@@ -848,8 +845,8 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
   }
   if constexpr (vjp_staged<n, T>()) {
     k_i3_vjp<n, T><<<grid, kThreads, i3_sf_smem_bytes<n, T, kVjpCB>(), s>>>(
-        what, wfine, (C2*)vw.mu3, (C2*)vw.muh, (C2*)vw.part_r, (C2*)vw.part_s, ws, tb.tw, tb.psip_s, tb.phase, t.J,
-        t.M, vw.nmc, nunits, K, c_stride, part_stride, spart_stride);
+        what, wfine, (C2*)vw.mu3, (C2*)vw.muh, (C2*)vw.part_r, (C2*)vw.part_s, ws, tb.psip_s, tb.phase, t.J, t.M,
+        vw.nmc, nunits, K, c_stride, part_stride, spart_stride);
     done = true;
   }
   if (!done) return cudaErrorInvalidValue;

@@ -244,10 +244,9 @@ struct Dft<R, SIGN, C2, false> {
       const C2 t1 = cadd(x1, x2);
       const C2 t2 = mk2(fmaT((T)-0.5, t1.x, x0.x), fmaT((T)-0.5, t1.y, x0.y));
       const C2 d = csub(x1, x2);
-      const C2 t3 = mk2(-h3 * d.y, h3 * d.x);   // i * SIGN * sqrt(3)/2 * (x1 - x2)
-      a[k] = cadd(x0, t1);
-      a[k + Q] = cadd(t2, t3);
-      a[k + 2 * Q] = csub(t2, t3);
+      a[k] = cadd(x0, t1);   // and t2 +- i SIGN sqrt(3)/2 (x1 - x2), as FMAs
+      a[k + Q] = mk2(fmaT(-h3, d.y, t2.x), fmaT(h3, d.x, t2.y));
+      a[k + 2 * Q] = mk2(fmaT(h3, d.y, t2.x), fmaT(-h3, d.x, t2.y));
     }
   }
 };
@@ -276,6 +275,53 @@ __device__ __forceinline__ void dft_scaled(C2 (&a)[R], const typename RealOf<C2>
   DftStage<R, SIGN, 4, C2>::run(b);
 #pragma unroll
   for (int i = 0; i < R; ++i) a[i] = b[i];
+}
+
+// DFT of length R (a power of two) at shifted frequencies: the twiddle factors between the two stages of a
+// line, w^(k1 t) on input t, merged into the butterflies.  tw(S / 2 - 1 + k) is the factor of butterfly k of
+// the stage of span S (merged_twiddle).  With p = u + w x as four FMAs and u - w x = 2 u - p as two more, a
+// butterfly takes six instructions; the twiddle products of their own took R - 1 times four.
+template <int R, int S, class C2>
+struct MergedStage {
+  template <class TW>
+  __device__ __forceinline__ static void run(C2 (&b)[R], TW tw) {
+    using T = typename RealOf<C2>::type;
+#pragma unroll
+    for (int k = 0; k < S / 2; ++k) {
+      const C2 w = tw(S / 2 - 1 + k);
+#pragma unroll
+      for (int g = 0; g < R; g += S) {
+        const C2 u = b[g + k], x = b[g + k + S / 2];
+        const C2 p = mk2(fmaT(w.x, x.x, fmaT(-w.y, x.y, u.x)), fmaT(w.x, x.y, fmaT(w.y, x.x, u.y)));
+        b[g + k] = p;
+        b[g + k + S / 2] = mk2(fmaT((T)2, u.x, -p.x), fmaT((T)2, u.y, -p.y));
+      }
+    }
+    MergedStage<R, 2 * S, C2>::run(b, tw);
+  }
+};
+template <int R, class C2>
+struct MergedStage<R, 2 * R, C2> {
+  template <class TW>
+  __device__ __forceinline__ static void run(C2 (&)[R], TW) {}
+};
+template <int R, class C2, class TW>
+__device__ __forceinline__ void dft_merged(C2 (&a)[R], TW tw) {
+  constexpr int L2 = ilog2c(R);
+  C2 b[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) b[i] = a[bitrev(i, L2)];
+  MergedStage<R, 2, C2>::run(b, tw);
+#pragma unroll
+  for (int i = 0; i < R; ++i) a[i] = b[i];
+}
+// Exponent m of the factor exp(-+2 pi i m / n) that entry e = S / 2 - 1 + k of a length-R stage takes at
+// shift s, with step Q = n / R between its frequencies: (s + Q k) R / S.
+template <int R>
+__host__ __device__ constexpr int merged_exponent(int e, int s, int Q) {
+  int S = 2;
+  while (S / 2 - 1 + S / 2 <= e) S *= 2;
+  return (s + Q * (e - (S / 2 - 1))) * (R / S);
 }
 
 // Band-limited (Xi) frequencies |k| < n/4 of a line of n = A B points: in the permuted order

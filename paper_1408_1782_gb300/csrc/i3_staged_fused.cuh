@@ -40,7 +40,16 @@ struct StagedLines {
                        LS = Chunk<n, sizeof(C2), CB>::LS;
   static constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
   static_assert(RC == CC, "row and line chunks share the buffer");
-  C2* twT;           // twT[k1 B + t2] = exp(-2 pi i t2 k1 / n) (t2-fastest lanes)
+  // FP64: twiddles merged into the second stage of a line (dft_merged), forward [k1][B - 1] (a warp shares k1,
+  // and k1 = 0 has none), inverse [A - 1][t2] (t2-fastest lanes).  A 128-point line takes 2324 (forward) and
+  // 2336 instead of 2464 FP64 instructions, and the FP64 pipe is what bounds these kernels: k_i3_sf took
+  // 423.6 -> 389.4 ms (32 cells at N = 64, J = M = 32), 365.3 -> 330.5 (128 cells, N = 32), 486.7 -> 466.6
+  // (64 cells, N = 48, whose radix-12 inverse keeps its products), the transpose 415 -> 381 (16 cells, N = 64).
+  // FP32 keeps the products, [k1][t2]: a merged line alone rounds 8-13% worse (FP32, n = 16..128).
+  static constexpr bool kMergeB = sizeof(T) == 8, kMergeA = kMergeB && (A & (A - 1)) == 0;
+  static constexpr int kTwF = kMergeB ? A * (B - 1) : 0, kTwI = kMergeA ? (A - 1) * B : n;
+  C2* twF;
+  C2* twI;
   C2* sm;            // one chunk: [RC][LS] rows, or [CC][LS] lines of G'
   const int* kslot;  // [n] xi_slot
   C2* G;             // G'[ky][x] between the passes
@@ -49,6 +58,46 @@ struct StagedLines {
   __device__ __forceinline__ static int xi_line(int li) {
     const int k1 = li / (B / 2), t = li % (B / 2);
     return B * k1 + (t < B / 4 ? t : t + B / 2);
+  }
+  __device__ __forceinline__ void init(C2* smem) {
+    twF = smem;
+    twI = twF + kTwF;
+    sm = twI + kTwI;
+    for (int i = threadIdx.x; i < kTwF; i += NTH) twF[i] = root(-merged_exponent<B>(i % (B - 1), i / (B - 1), A));
+    for (int i = threadIdx.x; i < kTwI; i += NTH)
+      twI[i] = kMergeA ? root(merged_exponent<A>(i / B, i % B, B)) : root(-(i / B) * (i % B));
+  }
+  // between the stages of a forward line
+  __device__ __forceinline__ void twiddle_forward(C2 (&v)[A], int t2) const {
+    if constexpr (!kMergeB) {
+#pragma unroll
+      for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twI[k1 * B + t2]);
+    }
+  }
+  __device__ static C2 root(int m) {   // exp(2 pi i m / n)
+    double sn, cs;
+    sincospi(2.0 * (double)m / n, &sn, &cs);
+    return mk2((T)cs, (T)sn);
+  }
+  // second stage of a forward line: b[t2] -> spectrum values of k1 + A (0..B-1)
+  __device__ __forceinline__ void stage_b_forward(C2 (&b)[B], int k1) const {
+    if (!kMergeB || k1 == 0) {
+      dft<B, -1>(b);
+    } else {
+      const C2* w = twF + k1 * (B - 1);
+      dft_merged<B>(b, [&](int e) { return w[e]; });
+    }
+  }
+  // second stage of an inverse line: v[k1] -> elements B (0..A-1) + t2
+  __device__ __forceinline__ void stage_a_inverse(C2 (&v)[A], int t2) const {
+    if constexpr (kMergeA) {
+      const C2* w = twI + t2;
+      dft_merged<A>(v, [&](int e) { return w[e * B]; });
+    } else {
+#pragma unroll
+      for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twI[k1 * B + t2]);
+      dft<A, 1>(v);
+    }
   }
   // rows of load(idx), idx = row * n + y, into lines of G' (XI: into the Xi lines only)
   template <bool XI, class LOAD>
@@ -61,8 +110,7 @@ struct StagedLines {
 #pragma unroll
         for (int t1 = 0; t1 < A; ++t1) v[t1] = load((r0 + r) * n + B * t1 + t2);
         dft<A, -1>(v);
-#pragma unroll
-        for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
+        twiddle_forward(v, t2);
 #pragma unroll
         for (int k1 = 0; k1 < A; ++k1) sm[r * LS + B * k1 + t2] = v[k1];
       }
@@ -73,7 +121,7 @@ struct StagedLines {
         C2 b[B];
 #pragma unroll
         for (int t = 0; t < B; ++t) b[t] = base[t];
-        dft<B, -1>(b);
+        stage_b_forward(b, k1);
 #pragma unroll
         for (int t = 0; t < B; ++t)
           if (!XI || xi_t<B>(t)) G[(B * k1 + t) * n + r0 + r] = b[t];
@@ -103,9 +151,7 @@ struct StagedLines {
         C2 v[A];
 #pragma unroll
         for (int k1 = 0; k1 < A; ++k1) v[k1] = sm[r * LS + B * k1 + t2];
-#pragma unroll
-        for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2]);
-        dft<A, 1>(v);
+        stage_a_inverse(v, t2);
 #pragma unroll
         for (int t1 = 0; t1 < A; ++t1) epi((r0 + r) * n + B * t1 + t2, v[t1]);
       }
@@ -119,9 +165,7 @@ struct StagedLines {
       C2 v[A];
 #pragma unroll
       for (int k1 = 0; k1 < A; ++k1) v[k1] = sm[cc * LS + B * k1 + t2];
-#pragma unroll
-      for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2]);
-      dft<A, 1>(v);
+      stage_a_inverse(v, t2);
 #pragma unroll
       for (int t1 = 0; t1 < A; ++t1) G[ky * n + B * t1 + t2] = v[t1];
     }
@@ -135,8 +179,7 @@ struct StagedLines {
 #pragma unroll
       for (int t1 = 0; t1 < A; ++t1) v[t1] = G[ky * n + B * t1 + t2];
       dft<A, -1>(v);
-#pragma unroll
-      for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
+      twiddle_forward(v, t2);
 #pragma unroll
       for (int k1 = 0; k1 < A; ++k1) sm[cc * LS + B * k1 + t2] = v[k1];
     }
@@ -154,7 +197,7 @@ struct StagedLines {
         C2 z[B];
 #pragma unroll
         for (int t = 0; t < B; ++t) z[t] = base[t];
-        dft<B, -1>(z);
+        stage_b_forward(z, k1);
         T sc[B];
 #pragma unroll
         for (int t = 0; t < B; ++t) sc[t] = psp[(B * k1 + t) * n + c0 + cc];
@@ -203,7 +246,7 @@ struct StagedLines {
         C2 b[B];
 #pragma unroll
         for (int t = 0; t < B; ++t) b[t] = base[t];
-        dft<B, -1>(b);
+        stage_b_forward(b, k1);
         if (sy < 0) continue;
         const C2 pyy = py[ky];
 #pragma unroll
@@ -224,21 +267,19 @@ struct StagedLines {
 
 template <int n, class T, int NTH, int CB, int MINB>
 __global__ void __launch_bounds__(NTH, MINB)
-    k_i3_sf(const I3Jobs<T> jobs, typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__ gtw) {
+    k_i3_sf(const I3Jobs<T> jobs, typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__) {
   using C2 = typename Vec2Of<T>::type;
   using Lines = StagedLines<n, T, NTH, CB>;
-  constexpr int A = Split<n>::A, B = Split<n>::B, P = n * n, Q = Lines::Q;
+  constexpr int P = n * n, Q = Lines::Q;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int kslot[n];
   C2* slot = ws + (size_t)blockIdx.x * 4 * P;
   C2* Sig = slot;           // [2][P] shifted pairs s_0 + i s_1, s_2 + i s_3
   C2* V = slot + 3 * P;     // sum_b eta_b w_b U_ab of the current pair of a
   Lines ln;
-  ln.twT = reinterpret_cast<C2*>(smem_raw);
-  ln.sm = ln.twT + n;
+  ln.init(reinterpret_cast<C2*>(smem_raw));
   ln.kslot = kslot;
   ln.G = slot + 2 * P;
-  for (int pos = threadIdx.x; pos < n; pos += NTH) ln.twT[(pos % A) * B + pos / A] = gtw[pos];
   build_xi_slots<n>(kslot);
   for (int gunit = blockIdx.x; gunit < jobs.total; gunit += gridDim.x) {
     const I3Job<T>& jb = jobs.job[i3_job_of(jobs, gunit)];
@@ -305,6 +346,6 @@ __global__ void __launch_bounds__(NTH, MINB)
 
 template <int n, class T, int CB>
 constexpr size_t i3_sf_smem_bytes() {   // twiddles and one chunk of RC padded lines
-  using C2 = typename Vec2Of<T>::type;
-  return (size_t)(n + Chunk<n, sizeof(C2), CB>::RC * Chunk<n, sizeof(C2), CB>::LS) * sizeof(C2);
+  using L = StagedLines<n, T, 256, CB>;
+  return (size_t)(L::kTwF + L::kTwI + L::RC * L::LS) * sizeof(typename L::C2);
 }
