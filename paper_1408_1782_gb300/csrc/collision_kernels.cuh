@@ -137,7 +137,7 @@ __device__ __forceinline__ I3Group i3_group_at(int it, int it1, int M) {
 // coefficients are zero and not stored: no kernel reads there.)
 //   what[c][0] = w0^ + i w1^, [1] = w2^ + i w3^, [2] = w1^ + i w2^, [3] = w3^
 //   wfine[c][0] = w0 + i w1, [1] = w2 + i w3  on the fine grid;
-//   wplane (may be null): the same four components as planes [c][4][n*n].
+//   wplane (may be null): the same four components as planes [c][4][n*n] in thread_order.
 // The coarse DFT is the fine forward FFT of the zero-interleaved samples
 // (its spectrum repeats with period N), scaled by 1/N^2 and cut to Xi.
 // --------------------------------------------------------------------------
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w,
       [&](int ix, int iy, C2 v) {
         fine[ix * n + iy] = v;
         if (wplane) {
-          T* pl = wplane + ((size_t)c * 4 + 2 * q) * P + ix * n + iy;
+          T* pl = wplane + ((size_t)c * 4 + 2 * q) * P + thread_order(n, ix, iy);
           pl[0] = v.x;
           pl[P] = v.y;
         }
@@ -1007,12 +1007,12 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
 // at a fifth of the memory rate (two FP64 lanes per clock), 128 cells of N = 64 1234 us
 // against 264 us.
 // sum: [ncells][np], or null (FP64): in place into the cell's first unit; the Fourier-space sums are
-// always put there.
+// always put there.  order_n: padded grid size where the partials' four planes are in thread_order, else 0.
 // --------------------------------------------------------------------------
 template <class T, int G>
 __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* part, double2* sum,
                                                    typename Vec2Of<T>::type* spec, int nparts, int np, int nq,
-                                                   int chunks) {
+                                                   int chunks, int order_n) {
   using Word = typename std::conditional<sizeof(T) == 8, double2, float4>::type;
   constexpr int PT = 256 / G, VEC = sizeof(T) == 8 ? 1 : 2;   // complex values per word
   const size_t c = blockIdx.x / chunks;
@@ -1057,7 +1057,12 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
       for (int k = 0; k < 2 * VEC; ++k) s[k] += red[j][k][threadIdx.x];
   }
   if (i >= np + nq) return;
-  if (real_space && sum) {
+  if (VEC == 2 && real_space && order_n) {   // thread_order planes (FP32, sum given) into rows
+    const int n = order_n, P = n * n, H = n / 32, o = 2 * i % P, tt = o / 4 % (n * H), t1 = o / (4 * n * H) * 4;
+    double* dst = reinterpret_cast<double*>(sum + c * np) + 2 * i / P * P + tt % n;
+#pragma unroll
+    for (int k = 0; k < 2 * VEC; ++k) dst[(H * (t1 + k) + tt / n) * n] = s[k];
+  } else if (real_space && sum) {
 #pragma unroll
     for (int k = 0; k < VEC; ++k) sum[c * np + i + k] = mk2(s[2 * k], s[2 * k + 1]);
   } else {
@@ -1071,15 +1076,17 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
 // more of them in flight.
 template <class T>
 void reduce_partials(typename Vec2Of<T>::type* part, double2* sum, typename Vec2Of<T>::type* spec, int nparts, int np,
-                     int nq, int ncells, cudaStream_t s) {
+                     int nq, int ncells, int order_n, cudaStream_t s) {
   constexpr int VEC = sizeof(T) == 8 ? 1 : 2;
   const int words = (np + nq) / VEC;
   if (nparts >= 16 && (long long)words * ncells < 152 * 1024) {
     const int chunks = (words + 31) / 32;
-    k_reduce_k3<T, 8><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, nparts, np, nq, chunks);
+    k_reduce_k3<T, 8><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, nparts, np, nq, chunks,
+                                                                       order_n);
   } else {
     const int chunks = (words + 255) / 256;
-    k_reduce_k3<T, 1><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, nparts, np, nq, chunks);
+    k_reduce_k3<T, 1><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, nparts, np, nq, chunks,
+                                                                       order_n);
   }
 }
 
@@ -1293,6 +1300,12 @@ constexpr int i3_nvariants() {
   } else {
     return 4;
   }
+}
+
+// Whether a variant is k_i3_tmem, whose partials are planes in thread_order.
+template <int n, class T>
+constexpr bool i3_variant_tmem(int v) {
+  return std::is_same<T, float>::value && (n == 32 || (n == 64 && v == 0) || (n == 128 && v == 4));
 }
 
 template <int n, class T>
@@ -1576,6 +1589,7 @@ cudaError_t i3_group_n(const Tables* const* tabs, const CollisionWork* const* cw
   for (int k = 0; k < njobs; ++k) {
     if (paired && !cws[k]->K3spec) return cudaErrorInvalidValue;
     cws[k]->i3_paired = paired;
+    cws[k]->i3_thread_order = i3_variant_tmem<n, T>(v);
   }
   const I3Launch l = i3_variant<n, T>(v);
   int g = total < grid ? total : grid;
@@ -1612,7 +1626,7 @@ cudaError_t collide_post_n(const Tables& t, CollisionWork& cw, double* c, int nc
   constexpr int nq = 2 * xi_kept<n>() * xi_kept<n>();
   const int nparts = t.J * cw.nmc, nqp = cw.i3_paired ? nq : 0;
   C2* spec = cw.i3_paired ? (C2*)cw.K3spec : nullptr;
-  reduce_partials<T>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, ncells, s);
+  reduce_partials<T>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, ncells, cw.i3_thread_order ? n : 0, s);
   const double2* k3 = cw.K3sum ? cw.K3sum : (const double2*)cw.K3part;
   C2* DK = (C2*)cw.ws;   // [ncells][4][P], then a field per (cell, pair)
   cudaError_t e = QBE_CELLS(k_dk_fields, 4 * ncells, s, (C2*)cw.Dacc, (C2*)cw.K4acc, DK, tb.tw);

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kThreads) k_vjp_mu(const double* __restrict__ 
 // Seed: the transpose of the pointwise Pauli assembly, from mu (k_vjp_mu) and the forward D and K4
 // fields (k_dk_fields).  Outputs: nu[c][2] (direct cotangent of the w pairs), nuf[c] (cotangent of
 // f = 2 w0 - 1), muD[c][2] (pairs (D1,D2),(D3,-)), muK2[c], mu4[c][2] (raw K4
-// pairs), mu3[c][2] (raw K3 pairs), mupl[c][4] (may be null: mu3 as planes).
+// pairs), mu3[c][2] (raw K3 pairs), mupl[c][4] (may be null: mu3 as planes in thread_order).
 // --------------------------------------------------------------------------
 template <int n, class T>
 __global__ void __launch_bounds__(kThreads) k_vjp_seed(
@@ -137,8 +137,8 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
     // K3_b = eta_b raw_b, C_b has -2 pi K3_b
     mu3c[i] = mk2((T)(-tp * m0), (T)(tp * m1));
     mu3c[P + i] = mk2((T)(tp * m2), (T)(tp * m3));
-    if (mupl) {   // mu3 as planes
-      T* pl = mupl + (size_t)c * 4 * P + i;
+    if (mupl) {
+      T* pl = mupl + (size_t)c * 4 * P + thread_order(n, i / n, i % n);
       pl[0] = mu3c[i].x;
       pl[P] = mu3c[i].y;
       pl[2 * P] = mu3c[P + i].x;
@@ -827,9 +827,10 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
   const int nunits = ncells * t.J * vw.nmc;
   const int grid = nunits < vw.grid ? nunits : vw.grid;
   begin(KG_VJP_I3);
-  bool done = false;
+  bool done = false, tmem = false;
   if constexpr (vjp_tmem<n, T>()) {
-    if (K == 1 && vw.i3v == 0) {
+    tmem = K == 1 && vw.i3v == 0;
+    if (tmem) {
       k_i3_vjp_tmem<n><<<grid, TmShape<n>::NT, TmShape<n>::smem, s>>>(
           what, (const T*)cw.wplane, (const T*)vw.mupl, (C2*)vw.muh, (C2*)vw.part_r, (C2*)vw.part_s, ws, tb.psip_s,
           tb.phase, t.J, t.M, vw.nmc, nunits);
@@ -858,7 +859,7 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
   for (int k = 0; k < K; ++k) {
     C2* pr = (C2*)vw.part_r + k * part_stride;
     C2* ps = (C2*)vw.part_s + k * spart_stride;
-    reduce_partials<T>(pr, cw.K3sum, ps, units, np, nq, ncells, s);
+    reduce_partials<T>(pr, cw.K3sum, ps, units, np, nq, ncells, tmem ? n : 0, s);
     const double* R = cw.K3sum ? (const double*)cw.K3sum : (const double*)pr;
     e = QBE_CELLS(k_vjp_final, 2 * ncells, s, (C2*)vw.nu + k * c_stride, (T*)vw.nuf + k * r_stride, R,
                   (cw.K3sum ? (size_t)1 : (size_t)units) * 2 * np, ps, (size_t)units * nq, ws, tb.tw, grad[k], accumulate);

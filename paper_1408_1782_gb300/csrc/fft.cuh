@@ -28,6 +28,13 @@ template <> struct Split<256> { static constexpr int A = 16, B = 16; };
 template <> struct Split<96>  { static constexpr int A = 12, B = 8;  };
 template <> struct Split<192> { static constexpr int A = 12, B = 16; };
 
+// Place of point (x, y) in a plane of n = 32 H points a side laid out for k_i3_tmem's threads: thread
+// y + n h holds the elements x = H t1 + h of line y, four consecutive t1 side by side.
+__host__ __device__ __forceinline__ int thread_order(int n, int x, int y) {
+  const int H = n / 32, t1 = x / H;
+  return ((t1 / 4) * n * H + y + n * (x % H)) * 4 + t1 % 4;
+}
+
 // Frequency index (0..n-1, standard wrap) stored at permuted position pos.
 template <int n>
 __host__ __device__ __forceinline__ int freq_of_pos(int pos) {

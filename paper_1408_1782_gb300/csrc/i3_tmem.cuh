@@ -235,8 +235,15 @@ __device__ __forceinline__ int tm_xi_line(int L) {
   return L < n / 4 ? L : L < n / 2 ? L + n / 2 : 0;
 }
 
+// The calling thread's words of a plane in thread_order: elements 4 g .. 4 g + 3 are word g * TEAM_THREADS.
+__device__ __forceinline__ float4* tm_quad(float* plane, int tt) { return reinterpret_cast<float4*>(plane) + tt; }
+__device__ __forceinline__ const float4* tm_quad(const float* plane, int tt) {
+  return reinterpret_cast<const float4*>(plane) + tt;
+}
+__device__ __forceinline__ float quad_at(const float4& q, int i) { return i == 0 ? q.x : i == 1 ? q.y : i == 2 ? q.z : q.w; }
+
 // The shifted pair S (phase-multiplied Xi coefficients `in`, inverse 2-D transform) into planes Sx (times
-// sign_x), Sx + P: y lines of the n / 2 lines kx of Xi, then the x lines.  Starts and ends with F free.
+// sign_x), Sx + P, in thread_order: y lines of the n / 2 lines kx of Xi, then the x lines.  Starts and ends with F free.
 template <int n>
 __device__ __forceinline__ void tm_shift(const TmLine<n>& ln, float2* F, int L, int team, int tt,
                                          const float2* __restrict__ in, const float2* px, const float2* py,
@@ -273,10 +280,10 @@ __device__ __forceinline__ void tm_shift(const TmLine<n>& ln, float2* F, int L, 
         }
       } else {
 #pragma unroll
-        for (int t1 = 0; t1 < 32; ++t1) {
-          const int idx = (H * t1 + ln.h) * n + L;
-          Sx[idx] = sign_x * v[t1].x;
-          Sx[P + idx] = v[t1].y;
+        for (int g = 0; g < 8; ++g) {
+          const float2* z = v + 4 * g;
+          tm_quad(Sx, tt)[g * TT] = make_float4(sign_x * z[0].x, sign_x * z[1].x, sign_x * z[2].x, sign_x * z[3].x);
+          tm_quad(Sx + P, tt)[g * TT] = make_float4(z[0].y, z[1].y, z[2].y, z[3].y);
         }
       }
     }
@@ -425,7 +432,7 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_tmem(const I3Jobs<floa
                                                               const float2* __restrict__) {
   using C2 = float2;
   using Sh = TmShape<n>;
-  constexpr int P = n * n, H = Sh::H;
+  constexpr int P = n * n, H = Sh::H, TT = Sh::TEAM_THREADS;
   constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
   constexpr int CH = 8;   // points per group of the epilogue's loads (n = 128: 4 51.6, 8 50.9, 16 64.2 ms)
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -458,7 +465,7 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_tmem(const I3Jobs<floa
     const int c = unit / (J * nmc);
     const int j = (unit / nmc) % J;
     const int mc = unit % nmc;
-    float* K = reinterpret_cast<float*>(jb.K3part + (size_t)unit * 2 * P);   // [4][P]
+    float* K = reinterpret_cast<float*>(jb.K3part + (size_t)unit * 2 * P);   // [4][P], thread_order
     C2* spec = jb.K3spec + (size_t)unit * 2 * Q;
     if (have) {
       const float* __restrict__ src = jb.psip_s + (size_t)j * P;
@@ -488,23 +495,24 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_tmem(const I3Jobs<floa
 #pragma unroll 1
       for (int q = Sh::TEAMS > 1 ? 0 : gr.q0; q < (Sh::TEAMS > 1 ? 2 : gr.q1); ++q) {
         const bool on = Sh::TEAMS == 1 || (q >= gr.q0 && q < gr.q1);
-        const float* __restrict__ Wq = W + (size_t)(2 * q) * P;
-        const float* Sq = S + (size_t)(2 * q) * P;      // rewritten every pair: plain (coherent) loads
+        const float4* __restrict__ Wq = tm_quad(W + (size_t)(2 * q) * P, tt);
+        const float4* Sq = tm_quad(S + (size_t)(2 * q) * P, tt);      // rewritten every pair: plain (coherent) loads
         const float e0 = q == 0 ? 1.f : -1.f;
         C2 v[32];
 #pragma unroll 1
         for (int b = 0; b < 4; ++b) {
           keep_step();
           if (!on) continue;
-          const float* __restrict__ wb = W + (size_t)b * P;
-          const float* Sb = S + (size_t)b * P;
-          float* Kb = K + (size_t)b * P;
+          const float4* __restrict__ wb = tm_quad(W + (size_t)b * P, tt);
+          const float4* Sb = tm_quad(S + (size_t)b * P, tt);
+          float4* Kb = tm_quad(K + (size_t)b * P, tt);
           // U = Psi'((w_2q + i w_2q+1) s_b)
 #pragma unroll
-          for (int t1 = 0; t1 < 32; ++t1) {
-            const int idx = (H * t1 + h) * n + L;
-            const float sb = Sb[idx];
-            v[t1] = mk2(Wq[idx] * sb, Wq[P + idx] * sb);
+          for (int g = 0; g < 8; ++g) {
+            const float4 sb = Sb[g * TT], wx = Wq[g * TT], wy = Wq[P / 4 + g * TT];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              v[4 * g + i] = mk2(quad_at(wx, i) * quad_at(sb, i), quad_at(wy, i) * quad_at(sb, i));
           }
           tm_convolve<n>(ln, F, psm, L, team, v);
           // K3_b += eta_2q s_2q Re U + eta_2q+1 s_2q+1 Im U (no other thread adds to this point of the
@@ -518,13 +526,13 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_tmem(const I3Jobs<floa
               tmem_ld(tv + i, Vx);
               tmem_ld(tv + 32 + i, Vy);
             }
-            float sx[CH], sy[CH], wv[CH];
+            float4 sx[CH / 4], sy[CH / 4], wv[CH / 4];
 #pragma unroll
-            for (int t = 0; t < CH; ++t) {
-              const int idx = (H * (i + t) + h) * n + L;
-              sx[t] = Sq[idx];
-              sy[t] = Sq[P + idx];
-              wv[t] = wb[idx];
+            for (int g = 0; g < CH / 4; ++g) {
+              const int e = (i / 4 + g) * TT;
+              sx[g] = Sq[e];
+              sy[g] = Sq[P / 4 + e];
+              wv[g] = wb[e];
             }
             if (b > 0) {
               tmem_wait_ld(Vx);
@@ -533,16 +541,21 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_tmem(const I3Jobs<floa
 #pragma unroll
               for (int t = 0; t < CH; ++t) Vx[t] = Vy[t] = 0.f;
             }
+            float k[CH];
 #pragma unroll
             for (int t = 0; t < CH; ++t) {
               const C2 u = v[i + t];
-              const float k = fmaf(e0 * sx[t], u.x, -sy[t] * u.y);
-              float* kp = Kb + (H * (i + t) + h) * n + L;
-              if (k_first) *kp = k;
-              else atomicAdd(kp, k);
-              const float f = eb * wv[t];
+              k[t] = fmaf(e0 * quad_at(sx[t / 4], t % 4), u.x, -quad_at(sy[t / 4], t % 4) * u.y);
+              const float f = eb * quad_at(wv[t / 4], t % 4);
               Vx[t] = fmaf(-e0 * f, u.x, Vx[t]);
               Vy[t] = fmaf(f, u.y, Vy[t]);
+            }
+#pragma unroll
+            for (int g = 0; g < CH / 4; ++g) {
+              float4* kp = Kb + (i / 4 + g) * TT;
+              const float* kg = k + 4 * g;
+              if (k_first) *kp = make_float4(kg[0], kg[1], kg[2], kg[3]);
+              else red_add4(kp, kg[0], kg[1], kg[2], kg[3]);
             }
             tmem_st(tv + i, Vx);
             tmem_st(tv + 32 + i, Vy);

@@ -17,7 +17,7 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_vjp_tmem(
     int nunits) {
   using C2 = float2;
   using Sh = TmShape<n>;
-  constexpr int P = n * n, H = Sh::H;
+  constexpr int P = n * n, H = Sh::H, TT = Sh::TEAM_THREADS;
   constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
   constexpr int CH = 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -50,9 +50,7 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_vjp_tmem(
       const float* __restrict__ src = psip_s + (size_t)j * P;
       for (int i = tt; i < P; i += Sh::TEAM_THREADS) psm[freq_of_pos<n>(i % n) * n + freq_of_pos<n>(i / n)] = src[i];
 #pragma unroll 4
-      for (int t1 = 0; t1 < 32; ++t1)
-#pragma unroll
-        for (int a = 0; a < 4; ++a) R[(size_t)a * P + (H * t1 + h) * n + L] = 0.f;
+      for (int i = 0; i < 32; ++i) tm_quad(R, tt)[i * TT] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     const float* __restrict__ W = wplane + (size_t)c * 4 * P;
     const float* __restrict__ Mu = mupl + (size_t)c * 4 * P;
@@ -84,9 +82,9 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_vjp_tmem(
       for (int q = 0; q < 2; ++q) {
         const bool on = q >= gr.q0 && q < gr.q1;
         const bool first_q = q == gr.q0;
-        const float* __restrict__ Wq = W + (size_t)(2 * q) * P;
-        const float* Sq = S + (size_t)(2 * q) * P;      // rewritten every pair: plain (coherent) loads
-        const float* Nq = Nu + (size_t)(2 * q) * P;
+        const float4* __restrict__ Wq = tm_quad(W + (size_t)(2 * q) * P, tt);
+        const float4* Sq = tm_quad(S + (size_t)(2 * q) * P, tt);      // rewritten every pair: plain (coherent) loads
+        const float4* Nq = tm_quad(Nu + (size_t)(2 * q) * P, tt);
         const float e0 = q == 0 ? 1.f : -1.f;
         C2 v[32];
 #pragma unroll 1
@@ -95,45 +93,59 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_vjp_tmem(
           if (!on) continue;
           const int b = bz >> 1;
           const bool z = (bz & 1) != 0;
-          const float* __restrict__ wb = W + (size_t)b * P;
-          const float* __restrict__ mb = Mu + (size_t)b * P;
-          const float* Sb = S + (size_t)b * P;
+          const float4* __restrict__ wb = tm_quad(W + (size_t)b * P, tt);
+          const float4* __restrict__ mb = tm_quad(Mu + (size_t)b * P, tt);
+          const float4* Sb = tm_quad(S + (size_t)b * P, tt);
           const float eb = b == 0 ? 1.f : -1.f;
           if (!z) {   // U = Psi'((w_2q + i w_2q+1) s_b)
 #pragma unroll
-            for (int t1 = 0; t1 < 32; ++t1) {
-              const int idx = (H * t1 + h) * n + L;
-              const float sb = Sb[idx];
-              v[t1] = mk2(Wq[idx] * sb, Wq[P + idx] * sb);
+            for (int g = 0; g < 8; ++g) {
+              const float4 sb = Sb[g * TT], wx = Wq[g * TT], wy = Wq[P / 4 + g * TT];
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                v[4 * g + i] = mk2(quad_at(wx, i) * quad_at(sb, i), quad_at(wy, i) * quad_at(sb, i));
             }
           } else {    // Z = Psi'(mu_b (eta s)_q + eta_b w_b nu_q)
 #pragma unroll
-            for (int t1 = 0; t1 < 32; ++t1) {
-              const int idx = (H * t1 + h) * n + L;
-              const float m = mb[idx];
-              v[t1] = mk2(e0 * m * Sq[idx], -m * Sq[P + idx]);
+            for (int g = 0; g < 8; ++g) {
+              const float4 m4 = mb[g * TT], sx = Sq[g * TT], sy = Sq[P / 4 + g * TT];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const float m = quad_at(m4, i);
+                v[4 * g + i] = mk2(e0 * m * quad_at(sx, i), -m * quad_at(sy, i));
+              }
               if (gr.pair) {
-                const float f = eb * wb[idx];
-                v[t1] = mk2(fmaf(f, Nq[idx], v[t1].x), fmaf(f, Nq[P + idx], v[t1].y));
+                const float4 w4 = wb[g * TT], nx = Nq[g * TT], ny = Nq[P / 4 + g * TT];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  const float f = eb * quad_at(w4, i);
+                  C2& z = v[4 * g + i];
+                  z = mk2(fmaf(f, quad_at(nx, i), z.x), fmaf(f, quad_at(ny, i), z.y));
+                }
               }
             }
           }
           tm_convolve<n>(ln, F, psm, L, team, v);
           if (!z) {
             // X_q += mu_b (eta_2q Re U, eta_2q+1 Im U);  R_b += eta_b nu_q . U
+            float4* Rb = tm_quad(R + (size_t)b * P, tt);
 #pragma unroll
             for (int i = 0; i < 32; i += CH) {
-              float Vx[CH], Vy[CH], m[CH], nx[CH], ny[CH];
+              float Vx[CH], Vy[CH];
               if (b > 0) {
                 tmem_ld(tv + i, Vx);
                 tmem_ld(tv + 32 + i, Vy);
               }
+              float4 m[CH / 4], nx[CH / 4], ny[CH / 4];
 #pragma unroll
-              for (int t = 0; t < CH; ++t) {
-                const int idx = (H * (i + t) + h) * n + L;
-                m[t] = mb[idx];
-                nx[t] = gr.pair ? Nq[idx] : 0.f;
-                ny[t] = gr.pair ? Nq[P + idx] : 0.f;
+              for (int g = 0; g < CH / 4; ++g) {
+                const int e = (i / 4 + g) * TT;
+                m[g] = mb[e];
+                nx[g] = ny[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (gr.pair) {
+                  nx[g] = Nq[e];
+                  ny[g] = Nq[P / 4 + e];
+                }
               }
               if (b > 0) {
                 tmem_wait_ld(Vx);
@@ -142,13 +154,19 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_vjp_tmem(
 #pragma unroll
                 for (int t = 0; t < CH; ++t) Vx[t] = Vy[t] = 0.f;
               }
+              float r[CH];
 #pragma unroll
               for (int t = 0; t < CH; ++t) {
                 const C2 u = v[i + t];
-                Vx[t] = fmaf(e0 * m[t], u.x, Vx[t]);
-                Vy[t] = fmaf(-m[t], u.y, Vy[t]);
-                if (gr.pair)
-                  atomicAdd(R + (size_t)b * P + (H * (i + t) + h) * n + L, eb * fmaf(nx[t], u.x, ny[t] * u.y));
+                const float mt = quad_at(m[t / 4], t % 4);
+                Vx[t] = fmaf(e0 * mt, u.x, Vx[t]);
+                Vy[t] = fmaf(-mt, u.y, Vy[t]);
+                r[t] = eb * fmaf(quad_at(nx[t / 4], t % 4), u.x, quad_at(ny[t / 4], t % 4) * u.y);
+              }
+              if (gr.pair) {
+#pragma unroll
+                for (int g = 0; g < CH / 4; ++g)
+                  red_add4(Rb + (i / 4 + g) * TT, r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
               }
               tmem_st(tv + i, Vx);
               tmem_st(tv + 32 + i, Vy);
@@ -156,40 +174,32 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_vjp_tmem(
             tmem_wait_st();
           } else {
             // R_q += s_b Z;  X_b += w_q . Z
-            float* Rq = R + (size_t)(2 * q) * P;
-            float* Xb = X + (size_t)b * P;
+            float4* Rq = tm_quad(R + (size_t)(2 * q) * P, tt);
+            float4* Xb = tm_quad(X + (size_t)b * P, tt);
 #pragma unroll
-            for (int i = 0; i < 32; i += CH) {
-              float sb[CH], wx[CH], wy[CH];
+            for (int g = 0; g < 8; ++g) {
+              const float4 sb = Sb[g * TT], wx = Wq[g * TT], wy = Wq[P / 4 + g * TT];
+              float d[4];
 #pragma unroll
-              for (int t = 0; t < CH; ++t) {
-                const int idx = (H * (i + t) + h) * n + L;
-                sb[t] = Sb[idx];
-                wx[t] = Wq[idx];
-                wy[t] = Wq[P + idx];
-              }
-#pragma unroll
-              for (int t = 0; t < CH; ++t) {
-                const C2 u = v[i + t];
-                const int idx = (H * (i + t) + h) * n + L;
-                atomicAdd(Rq + idx, sb[t] * u.x);
-                atomicAdd(Rq + P + idx, sb[t] * u.y);
-                const float d = fmaf(wx[t], u.x, wy[t] * u.y);
-                if (first_q) Xb[idx] = d;
-                else atomicAdd(Xb + idx, d);
-              }
+              for (int i = 0; i < 4; ++i)
+                d[i] = fmaf(quad_at(wx, i), v[4 * g + i].x, quad_at(wy, i) * v[4 * g + i].y);
+              const C2* u = v + 4 * g;
+              red_add4(Rq + g * TT, sb.x * u[0].x, sb.y * u[1].x, sb.z * u[2].x, sb.w * u[3].x);
+              red_add4(Rq + P / 4 + g * TT, sb.x * u[0].y, sb.y * u[1].y, sb.z * u[2].y, sb.w * u[3].y);
+              if (first_q) Xb[g * TT] = make_float4(d[0], d[1], d[2], d[3]);
+              else red_add4(Xb + g * TT, d[0], d[1], d[2], d[3]);
             }
           }
         }
         if (!on) continue;
         tmem_ld_c<32>(tv, tv + 32, v);
         tmem_wait_ld_c<32>(v);
-        float* Xq = X + (size_t)(2 * q) * P;
+        float4* Xq = tm_quad(X + (size_t)(2 * q) * P, tt);
 #pragma unroll
-        for (int t1 = 0; t1 < 32; ++t1) {
-          const int idx = (H * t1 + h) * n + L;
-          atomicAdd(Xq + idx, v[t1].x);
-          atomicAdd(Xq + P + idx, v[t1].y);
+        for (int g = 0; g < 8; ++g) {
+          const C2* z = v + 4 * g;
+          red_add4(Xq + g * TT, z[0].x, z[1].x, z[2].x, z[3].x);
+          red_add4(Xq + P / 4 + g * TT, z[0].y, z[1].y, z[2].y, z[3].y);
         }
       }
       // X shifted back (its sums are in L2: loads that bypass L1)
@@ -198,11 +208,12 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_vjp_tmem(
         keep_step();
         if (!more) continue;
         C2 v[32];
-        const float* Xp = X + (size_t)(2 * p) * P;
+        const float4* Xp = tm_quad(X + (size_t)(2 * p) * P, tt);
 #pragma unroll
-        for (int t1 = 0; t1 < 32; ++t1) {
-          const int idx = (H * t1 + h) * n + L;
-          v[t1] = mk2(__ldcg(Xp + idx), __ldcg(Xp + P + idx));
+        for (int g = 0; g < 8; ++g) {
+          const float4 x = __ldcg(Xp + g * TT), y = __ldcg(Xp + P / 4 + g * TT);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) v[4 * g + i] = mk2(quad_at(x, i), quad_at(y, i));
         }
         tm_shift_back<n>(ln, F, L, team, tt, v, px, py, ps + (size_t)p * Q, s_first);
       }

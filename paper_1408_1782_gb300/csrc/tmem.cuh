@@ -83,6 +83,12 @@ __device__ __forceinline__ void tmem_st(uint32_t a, const float (&v)[CNT]) {
   for (int i = 0; i < CNT; i += 4) tmem_st4(a + i, v + i);
 }
 
+// Adds four floats in memory (16-byte aligned), nothing returned.
+__device__ __forceinline__ void red_add4(float4* p, float a, float b, float c, float d) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
+               : "memory");
+}
+
 // Eight consecutive columns from / to registers named one by one.
 __device__ __forceinline__ void tmem_ld8(uint32_t a, float& v0, float& v1, float& v2, float& v3, float& v4, float& v5,
                                          float& v6, float& v7) {
