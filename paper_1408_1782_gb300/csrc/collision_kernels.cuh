@@ -624,7 +624,9 @@ template <> struct FusedShapes<128> {   // variant 4: k_i3_tmem
 // every global access: 4 CTAs x 1024 threads 239.9 ms; 8 CTAs x 512 threads (two CTAs of
 // different clusters per SM) 255.4 ms; the staged k_i3 294.5 ms.  With the line stages reading
 // and writing the transposed field directly: 219.1 ms (1024 threads, mode 0 below), 192.4 ms
-// (512 threads, mode 1 node by node), 132.4 ms (mode 1, nodes in pairs).
+// (512 threads, mode 1 node by node), 132.4 ms (mode 1, nodes in pairs, the sums over a in registers).
+// Those took 64 of a thread's 128 registers; in tensor memory they leave room for both of its tasks' loads at
+// a time: 14 cells 58.0 -> 42.7 ms, N = 96, 32 cells 70.8 -> 62.6 ms.
 constexpr int kI3Cluster = 4;             // CTAs per cluster
 constexpr int kThreadsI3Cluster = 1024;   // threads per CTA of mode 0
 
@@ -647,8 +649,8 @@ constexpr size_t i3_cluster_smem_bytes() {   // twiddles (two orders), the slab,
 // The cluster kernel's launch shapes: NT threads per CTA and the accumulation mode.  MODE 0: loop a
 // (outer), p (inner), each convolution's last stage adds eta_a S_a T into the unit's partial sum in
 // global memory (read-modify-write per convolution).  MODE 1: loop p (outer), a (inner), the last
-// stage accumulates over a in registers (each thread owns the same points in every convolution) and
-// the partial sum is written once per (m, p); NT = R B / 2, so that every thread owns two row tasks.
+// stage accumulates over a in tensor memory (each thread owns the same points in every convolution);
+// NT = R B / 2, so that every thread owns two row tasks.
 template <int n>
 constexpr int i3_cluster_threads(int mode) {
   return mode == 0 ? kThreadsI3Cluster : (n / kI3Cluster) * Split<n>::B / 2;
@@ -665,7 +667,7 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
   constexpr int TA = (R * B + NT - 1) / NT;          // row tasks (r, t2) per thread in an A stage
   constexpr int TB = (R * A + NT - 1) / NT;          // tasks (r, k1) per thread in a B stage
   constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
-  static_assert(MODE == 0 || R * B == 2 * NT, "register accumulation: two row tasks per thread");
+  static_assert(MODE == 0 || R * B == 2 * NT, "accumulation at the thread's own points: two row tasks per thread");
   static_assert(n % kI3Cluster == 0 && (n / 2) % kI3Cluster == 0, "cluster split");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
@@ -685,6 +687,12 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
   }
   for (int pos = threadIdx.x; pos < n; pos += NT) twT[(pos % A) * B + pos / A] = gtw[pos];
   load_twiddles<n>(tw, gtw);
+  __shared__ uint32_t tm_slot;
+  uint32_t tm_base = 0, tv = 0;                      // MODE 1: V_q, per row task A real, A imaginary parts
+  if constexpr (MODE == 1) {
+    tm_base = tmem_alloc<tmem_columns(NT, 2 * TA * A)>(&tm_slot);
+    tv = tmem_mine<2 * TA * A>(tm_base);
+  }
   const int tid = threadIdx.x;
   const int rank = cluster_rank();
   const int r0 = rank * R;                           // this CTA's first row / column
@@ -696,28 +704,53 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
   // transform's permuted order): the row passes reach it from stage B (lanes = consecutive rows of
   // this CTA) and the line pass from stage A (contiguous in x), so every global access is inside a
   // line stage and coalesced.
+  // Each stage loads both of a thread's tasks before it transforms the first: the loads' latency is what
+  // bounds the kernel.
+  auto a_task = [&](int i, int& r, int& t2) {        // row task i of the thread
+    const int task = tid + i * NT;
+    r = task / B;
+    t2 = task % B;
+    return TA * NT == R * B || task < R * B;
+  };
+  auto b_task = [&](int i, int& r, int& k1) {
+    const int task = tid + i * NT;
+    r = task % R;
+    k1 = task / R;
+    return TB * NT == R * A || task < R * A;
+  };
+  // lines of v through stage A into F
+  auto stage_a_forward = [&](C2 (&v)[A], int r, int t2) {
+    dft<A, -1>(v);
+#pragma unroll
+    for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
+#pragma unroll
+    for (int k1 = 0; k1 < A; ++k1) F[r * LS + B * k1 + t2] = v[k1];
+  };
+  auto stage_a_inverse = [&](C2 (&v)[A], int r, int t2) {
+#pragma unroll
+    for (int k1 = 0; k1 < A; ++k1) v[k1] = F[r * LS + B * k1 + t2];
+#pragma unroll
+    for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2]);
+    dft<A, 1>(v);
+  };
   auto convolve = [&](auto load, auto epi) {
+    int r, t2, k1;
+    {
+      C2 v[TA][A];
 #pragma unroll
-    for (int i = 0; i < TA; ++i) {                   // forward rows: stage A loads the product
-      const int task = tid + i * NT;
-      if (TA * NT == R * B || task < R * B) {
-        const int r = task / B, t2 = task % B;
-        C2 v[A];
+      for (int i = 0; i < TA; ++i)                   // forward rows: stage A loads the product
+        if (a_task(i, r, t2)) {
 #pragma unroll
-        for (int t1 = 0; t1 < A; ++t1) v[t1] = load(r * n + B * t1 + t2);
-        dft<A, -1>(v);
+          for (int t1 = 0; t1 < A; ++t1) v[i][t1] = load(r * n + B * t1 + t2);
+        }
 #pragma unroll
-        for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
-#pragma unroll
-        for (int k1 = 0; k1 < A; ++k1) F[r * LS + B * k1 + t2] = v[k1];
-      }
+      for (int i = 0; i < TA; ++i)
+        if (a_task(i, r, t2)) stage_a_forward(v[i], r, t2);
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < TB; ++i) {
-      const int task = tid + i * NT;
-      if (TB * NT == R * A || task < R * A) {
-        const int r = task % R, k1 = task / R;
+    for (int i = 0; i < TB; ++i)
+      if (b_task(i, r, k1)) {
         C2 b[B];
 #pragma unroll
         for (int t = 0; t < B; ++t) b[t] = F[r * LS + B * k1 + t];
@@ -725,89 +758,66 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
 #pragma unroll
         for (int t = 0; t < B; ++t) Gs[(size_t)(B * k1 + t) * n + r0 + r] = b[t];
       }
-    }
     cluster_sync_global();                           // all rows transformed
     // psi' convolution along x on this CTA's lines ky in [r0, r0 + R)
+    {
+      C2 v[TA][A];
 #pragma unroll
-    for (int i = 0; i < TA; ++i) {
-      const int task = tid + i * NT;
-      if (TA * NT == R * B || task < R * B) {
-        const int cc = task / B, t2 = task % B;
-        C2 v[A];
+      for (int i = 0; i < TA; ++i)
+        if (a_task(i, r, t2)) {
 #pragma unroll
-        for (int t1 = 0; t1 < A; ++t1) v[t1] = __ldcg(&Gs[(size_t)(r0 + cc) * n + B * t1 + t2]);
-        dft<A, -1>(v);
+          for (int t1 = 0; t1 < A; ++t1) v[i][t1] = __ldcg(&Gs[(size_t)(r0 + r) * n + B * t1 + t2]);
+        }
 #pragma unroll
-        for (int k1 = 1; k1 < A; ++k1) v[k1] = cmul(v[k1], twT[k1 * B + t2]);
-#pragma unroll
-        for (int k1 = 0; k1 < A; ++k1) F[cc * LS + B * k1 + t2] = v[k1];
-      }
+      for (int i = 0; i < TA; ++i)
+        if (a_task(i, r, t2)) stage_a_forward(v[i], r, t2);
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < TB; ++i) {
-      const int task = tid + i * NT;
-      if (TB * NT == R * A || task < R * A) {
-        const int cc = task % R, k1 = task / R;
+    for (int i = 0; i < TB; ++i)
+      if (b_task(i, r, k1)) {
         C2 b[B];
 #pragma unroll
-        for (int t = 0; t < B; ++t) b[t] = F[cc * LS + B * k1 + t];
+        for (int t = 0; t < B; ++t) b[t] = F[r * LS + B * k1 + t];
         dft<B, -1>(b);
         float sc[B];
 #pragma unroll
-        for (int t = 0; t < B; ++t) sc[t] = psl[(B * k1 + t) * R + cc];
+        for (int t = 0; t < B; ++t) sc[t] = psl[(B * k1 + t) * R + r];
         dft_scaled<B, 1>(b, sc);
-#pragma unroll
-        for (int t = 0; t < B; ++t) F[cc * LS + B * k1 + t] = b[t];
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < TA; ++i) {
-      const int task = tid + i * NT;
-      if (TA * NT == R * B || task < R * B) {
-        const int cc = task / B, t2 = task % B;
-        C2 v[A];
-#pragma unroll
-        for (int k1 = 0; k1 < A; ++k1) v[k1] = F[cc * LS + B * k1 + t2];
-#pragma unroll
-        for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2]);
-        dft<A, 1>(v);
-#pragma unroll
-        for (int t1 = 0; t1 < A; ++t1) Gs[(size_t)(r0 + cc) * n + B * t1 + t2] = v[t1];
-      }
-    }
-    cluster_sync_global();                           // all lines convolved
-    // inverse rows on this CTA's rows: stage B loads, stage A hands its results to the epilogue
-#pragma unroll
-    for (int i = 0; i < TB; ++i) {
-      const int task = tid + i * NT;
-      if (TB * NT == R * A || task < R * A) {
-        const int r = task % R, k1 = task / R;
-        C2 b[B];
-#pragma unroll
-        for (int t = 0; t < B; ++t) b[t] = __ldcg(&Gs[(size_t)(B * k1 + t) * n + r0 + r]);
-        dft<B, 1>(b);
 #pragma unroll
         for (int t = 0; t < B; ++t) F[r * LS + B * k1 + t] = b[t];
       }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < TA; ++i)
+      if (a_task(i, r, t2)) {
+        C2 v[A];
+        stage_a_inverse(v, r, t2);
+#pragma unroll
+        for (int t1 = 0; t1 < A; ++t1) Gs[(size_t)(r0 + r) * n + B * t1 + t2] = v[t1];
+      }
+    cluster_sync_global();                           // all lines convolved
+    // inverse rows on this CTA's rows: stage B loads, the epilogue takes stage A
+    {
+      C2 b[TB][B];
+#pragma unroll
+      for (int i = 0; i < TB; ++i)
+        if (b_task(i, r, k1)) {
+#pragma unroll
+          for (int t = 0; t < B; ++t) b[i][t] = __ldcg(&Gs[(size_t)(B * k1 + t) * n + r0 + r]);
+        }
+#pragma unroll
+      for (int i = 0; i < TB; ++i)
+        if (b_task(i, r, k1)) {
+          dft<B, 1>(b[i]);
+#pragma unroll
+          for (int t = 0; t < B; ++t) F[r * LS + B * k1 + t] = b[i][t];
+        }
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < TA; ++i) {
-      const int task = tid + i * NT;
-      if (TA * NT == R * B || task < R * B) {
-        const int r = task / B, t2 = task % B;
-        C2 v[A];
-#pragma unroll
-        for (int k1 = 0; k1 < A; ++k1) v[k1] = F[r * LS + B * k1 + t2];
-#pragma unroll
-        for (int k1 = 1; k1 < A; ++k1) v[k1] = cmulc(v[k1], twT[k1 * B + t2]);
-        dft<A, 1>(v);
-#pragma unroll
-        for (int t1 = 0; t1 < A; ++t1) epi(i, t1, r * n + B * t1 + t2, v[t1]);
-      }
-    }
+    for (int i = 0; i < TA; ++i)
+      if (a_task(i, r, t2)) epi(i, r, t2);
     __syncthreads();
   };
   for (int gunit = cluster_index(); gunit < jobs.total; gunit += cluster_count()) {
@@ -888,10 +898,16 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
             const C2* Sp = Sig + (size_t)p * P + (size_t)r0 * n;
             C2* accp = acc + (size_t)p * P + (size_t)r0 * n;
             convolve([&](int idx) { return cscale(Sp[idx], wa[2 * idx]); },
-                     [&](int, int, int idx, C2 v) {
-                       const float f = eta * Sa[2 * idx];
-                       const C2 d = accp[idx];
-                       accp[idx] = mk2(fmaT(f, v.x, d.x), fmaT(f, v.y, d.y));
+                     [&](int, int r, int t2) {
+                       C2 v[A];
+                       stage_a_inverse(v, r, t2);
+#pragma unroll
+                       for (int t1 = 0; t1 < A; ++t1) {
+                         const int idx = r * n + B * t1 + t2;
+                         const float f = eta * Sa[2 * idx];
+                         const C2 d = accp[idx];
+                         accp[idx] = mk2(fmaT(f, v[t1].x, d.x), fmaT(f, v[t1].y, d.y));
+                       }
                      });
           }
         }
@@ -902,21 +918,46 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
           const C2* wq = wf + (size_t)q * P + (size_t)r0 * n;
           const C2* Sq = Sig + (size_t)q * P + (size_t)r0 * n;
           const float e0 = q == 0 ? 1.f : -1.f;
-          C2 V[TA][A];
           for (int b = 0; b < 4; ++b) {
             const float* Sb = reinterpret_cast<const float*>(Sig + (size_t)(b >> 1) * P + (size_t)r0 * n) + (b & 1);
             const float* wb = reinterpret_cast<const float*>(wf + (size_t)(b >> 1) * P + (size_t)r0 * n) + (b & 1);
             float* Kb = reinterpret_cast<float*>(acc) + (size_t)b * P + (size_t)r0 * n;
             const float eb = b == 0 ? 1.f : -1.f;
             convolve([&](int idx) { return cscale(wq[idx], Sb[2 * idx]); },
-                     [&](int i, int t1, int idx, C2 v) {
-                       const C2 s = Sq[idx];
-                       const float k = fmaT(e0 * s.x, v.x, -s.y * v.y);
-                       if (k_first) Kb[idx] = k;
-                       else atomicAdd(Kb + idx, k);  // no other thread adds to this point
-                       const float f = eb * wb[2 * idx], fx = -e0 * f;
-                       if (b == 0) V[i][t1] = mk2(fx * v.x, f * v.y);
-                       else V[i][t1] = mk2(fmaT(fx, v.x, V[i][t1].x), fmaT(f, v.y, V[i][t1].y));
+                     [&](int i, int r, int t2) {
+                       C2 s[A], v[A];
+                       float wv[A];
+#pragma unroll
+                       for (int t1 = 0; t1 < A; ++t1) {
+                         const int idx = r * n + B * t1 + t2;
+                         s[t1] = Sq[idx];
+                         wv[t1] = wb[2 * idx];
+                       }
+                       stage_a_inverse(v, r, t2);
+                       const uint32_t tvi = tv + 2 * A * i;
+#pragma unroll
+                       for (int g = 0; g < A; g += 4) {
+                         float Vx[4] = {}, Vy[4] = {};
+                         if (b > 0) {
+                           tmem_ld(tvi + g, Vx);
+                           tmem_ld(tvi + A + g, Vy);
+                           tmem_wait_ld(Vx);
+                           tmem_wait_ld(Vy);
+                         }
+#pragma unroll
+                         for (int t = 0; t < 4; ++t) {
+                           const int t1 = g + t, idx = r * n + B * t1 + t2;
+                           const float k = fmaT(e0 * s[t1].x, v[t1].x, -s[t1].y * v[t1].y);
+                           if (k_first) Kb[idx] = k;
+                           else atomicAdd(Kb + idx, k);  // no other thread adds to this point
+                           const float f = eb * wv[t1];
+                           Vx[t] = fmaT(-e0 * f, v[t1].x, Vx[t]);
+                           Vy[t] = fmaT(f, v[t1].y, Vy[t]);
+                         }
+                         tmem_st(tvi + g, Vx);
+                         tmem_st(tvi + A + g, Vy);
+                       }
+                       tmem_wait_st();               // loaded again after the next convolution
                      });
           }
           k_first = false;
@@ -925,11 +966,15 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
 #pragma unroll
           for (int i = 0; i < TA; ++i) {
             const int task = tid + i * NT, r = task / B, t2 = task % B;
-            dft<A, -1>(V[i]);
+            float Vx[A], Vy[A];
+            tmem_ld(tv + 2 * A * i, Vx);
+            tmem_ld(tv + 2 * A * i + A, Vy);
+            tmem_wait_ld(Vx);
+            tmem_wait_ld(Vy);
+            C2 v[A];
 #pragma unroll
-            for (int k1 = 1; k1 < A; ++k1) V[i][k1] = cmul(V[i][k1], twT[k1 * B + t2]);
-#pragma unroll
-            for (int k1 = 0; k1 < A; ++k1) F[r * LS + B * k1 + t2] = V[i][k1];
+            for (int t1 = 0; t1 < A; ++t1) v[t1] = mk2(Vx[t1], Vy[t1]);
+            stage_a_forward(v, r, t2);
           }
           __syncthreads();
 #pragma unroll
@@ -993,6 +1038,7 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
       }
     }
   }
+  if constexpr (MODE == 1) tmem_free<tmem_columns(NT, 2 * TA * A)>(tm_base);
 }
 
 // --------------------------------------------------------------------------
@@ -1315,8 +1361,8 @@ I3Launch i3_variant(int v) {
     constexpr int NT1 = i3_cluster_threads<n>(1);
     if (v == 1)
       l = {(const void*)k_i3_cluster<n, NT1, 1>, NT1, i3_cluster_smem_bytes<n>(), true,
-           n == 256 ? "node pairs, cluster of 4 CTAs x 512 threads, register accumulation"
-                    : "node pairs, cluster of 4 CTAs x 384 threads, register accumulation"};
+           n == 256 ? "node pairs, cluster of 4 CTAs x 512 threads, sums in tensor memory"
+                    : "node pairs, cluster of 4 CTAs x 384 threads, sums in tensor memory"};
     else
       l = {(const void*)k_i3_cluster<n, kThreadsI3Cluster, 0>, kThreadsI3Cluster, i3_cluster_smem_bytes<n>(), true,
            "cluster of 4 CTAs x 1024 threads"};
