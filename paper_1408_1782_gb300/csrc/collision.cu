@@ -218,7 +218,7 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   if ((e = cudaMalloc((void**)&(ptr), (bytes))) != cudaSuccess) { free_collision_work(cw); return e; }
   QBE_ALLOC(cw.what, (size_t)nb * 4 * P * cz);
   QBE_ALLOC(cw.wfine, (size_t)nb * 2 * P * cz);
-  if (prec == 1 && (t.n == 32 || t.n == 64 || t.n == 128)) QBE_ALLOC(cw.wplane, (size_t)nb * 4 * P * rz);
+  if (prec == 1 && t.n != 16 && t.n != 96) QBE_ALLOC(cw.wplane, (size_t)nb * 4 * P * rz);
   QBE_ALLOC(cw.Dacc, (size_t)nb * 2 * P * cz);
   QBE_ALLOC(cw.K2acc, (size_t)nb * P * rz);
   QBE_ALLOC(cw.K4acc, (size_t)nb * 2 * P * cz);

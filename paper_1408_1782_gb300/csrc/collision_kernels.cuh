@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w,
       [&](int ix, int iy, C2 v) {
         fine[ix * n + iy] = v;
         if (wplane) {
-          T* pl = wplane + ((size_t)c * 4 + 2 * q) * P + thread_order(n, ix, iy);
+          T* pl = wplane + ((size_t)c * 4 + 2 * q) * P + thread_order<n>(ix, iy);
           pl[0] = v.x;
           pl[P] = v.y;
         }
@@ -666,6 +666,7 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
   constexpr int A = Split<n>::A, B = Split<n>::B;
   constexpr int TA = (R * B + NT - 1) / NT;          // row tasks (r, t2) per thread in an A stage
   constexpr int TB = (R * A + NT - 1) / NT;          // tasks (r, k1) per thread in a B stage
+  constexpr int W4 = TA * A / 4;                     // MODE 1: words of a thread in a plane of R rows
   constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
   static_assert(MODE == 0 || R * B == 2 * NT, "accumulation at the thread's own points: two row tasks per thread");
   static_assert(n % kI3Cluster == 0 && (n / 2) % kI3Cluster == 0, "cluster split");
@@ -739,10 +740,7 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
       C2 v[TA][A];
 #pragma unroll
       for (int i = 0; i < TA; ++i)                   // forward rows: stage A loads the product
-        if (a_task(i, r, t2)) {
-#pragma unroll
-          for (int t1 = 0; t1 < A; ++t1) v[i][t1] = load(r * n + B * t1 + t2);
-        }
+        if (a_task(i, r, t2)) load(i, r, t2, v[i]);
 #pragma unroll
       for (int i = 0; i < TA; ++i)
         if (a_task(i, r, t2)) stage_a_forward(v[i], r, t2);
@@ -841,7 +839,8 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
     #pragma unroll 1
     for (int idx = tid; idx < n * R; idx += NT) psl[idx] = psp[(idx / R) * n + r0 + idx % R];
     __syncthreads();
-    const C2* wf = jb.wfine + (size_t)c * 2 * P;
+    const C2* wf = jb.wfine + (size_t)c * 2 * P;     // MODE 0
+    const float* __restrict__ wp = jb.wplane + (size_t)c * 4 * P + (size_t)r0 * n;   // MODE 1: this block's rows
     const int it1 = i3_chunk_begin(mc + 1, nmc, M);
     C2* spec = jb.K3spec + (size_t)unit * 2 * Q;     // MODE 1
     bool k_first = true, s_first0 = true, s_first1 = true;
@@ -875,15 +874,26 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
       for (int p = 0; p < 2; ++p) {
         C2* S = Sig + (size_t)p * P + (size_t)r0 * n;
         #pragma unroll 1
-        #pragma unroll 1
-      for (int idx = tid; idx < R * n; idx += NT) {
+        for (int idx = tid; idx < R * n; idx += NT) {
           const int r = idx / n, iy = idx % n;
           F[r * LS + iy] = xmask[iy] ? __ldcg(&S[idx]) : zero2<float>();
         }
         __syncthreads();
         fft_lines<n, 1, true>(F, R, LS, 1, tw);
-        #pragma unroll 1
-        for (int idx = tid; idx < R * n; idx += NT) S[idx] = F[(idx / n) * LS + idx % n];
+        if constexpr (MODE == 0) {
+          #pragma unroll 1
+          for (int idx = tid; idx < R * n; idx += NT) S[idx] = F[(idx / n) * LS + idx % n];
+        } else {                                     // the rows' two planes, in thread_order
+          float4* S4 = reinterpret_cast<float4*>(S) + tid;
+#pragma unroll 2
+          for (int w = 0; w < W4; ++w) {
+            const int task = tid + w / (A / 4) * NT;
+            const C2* f = F + task / B * LS + task % B + B * (w % (A / 4) * 4);
+            const C2 z0 = f[0], z1 = f[B], z2 = f[2 * B], z3 = f[3 * B];
+            S4[w * NT] = make_float4(z0.x, z1.x, z2.x, z3.x);
+            S4[(W4 + w) * NT] = make_float4(z0.y, z1.y, z2.y, z3.y);
+          }
+        }
         __syncthreads();
       }
       // from here on this CTA reads only its own rows of the shifted fields
@@ -897,7 +907,13 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
           for (int p = 0; p < 2; ++p) {
             const C2* Sp = Sig + (size_t)p * P + (size_t)r0 * n;
             C2* accp = acc + (size_t)p * P + (size_t)r0 * n;
-            convolve([&](int idx) { return cscale(Sp[idx], wa[2 * idx]); },
+            convolve([&](int, int r, int t2, C2 (&v)[A]) {
+#pragma unroll
+                       for (int t1 = 0; t1 < A; ++t1) {
+                         const int idx = r * n + B * t1 + t2;
+                         v[t1] = cscale(Sp[idx], wa[2 * idx]);
+                       }
+                     },
                      [&](int, int r, int t2) {
                        C2 v[A];
                        stage_a_inverse(v, r, t2);
@@ -915,47 +931,60 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
         const int xl0 = rank * XC;                   // this CTA's share of the n / 2 lines ky of Xi
         auto xi_line = [&](int cc) { return xcols[xl0 + cc]; };
         for (int q = gr.q0; q < gr.q1; ++q) {
-          const C2* wq = wf + (size_t)q * P + (size_t)r0 * n;
-          const C2* Sq = Sig + (size_t)q * P + (size_t)r0 * n;
+          // this thread's words of the rows' planes
+          const float4* wq = reinterpret_cast<const float4*>(wp + (size_t)(2 * q) * P) + tid;
+          const float4* Sq = reinterpret_cast<const float4*>(Sig + (size_t)q * P + (size_t)r0 * n) + tid;
           const float e0 = q == 0 ? 1.f : -1.f;
           for (int b = 0; b < 4; ++b) {
-            const float* Sb = reinterpret_cast<const float*>(Sig + (size_t)(b >> 1) * P + (size_t)r0 * n) + (b & 1);
-            const float* wb = reinterpret_cast<const float*>(wf + (size_t)(b >> 1) * P + (size_t)r0 * n) + (b & 1);
-            float* Kb = reinterpret_cast<float*>(acc) + (size_t)b * P + (size_t)r0 * n;
+            const float4* Sb =
+                reinterpret_cast<const float4*>(Sig + (size_t)(b >> 1) * P + (size_t)r0 * n) + (b & 1) * W4 * NT + tid;
+            const float4* wb = reinterpret_cast<const float4*>(wp + (size_t)b * P) + tid;
+            float4* Kb = reinterpret_cast<float4*>(reinterpret_cast<float*>(acc) + (size_t)b * P + (size_t)r0 * n) + tid;
             const float eb = b == 0 ? 1.f : -1.f;
-            convolve([&](int idx) { return cscale(wq[idx], Sb[2 * idx]); },
-                     [&](int i, int r, int t2) {
-                       C2 s[A], v[A];
-                       float wv[A];
+            convolve([&](int i, int, int, C2 (&v)[A]) {
 #pragma unroll
-                       for (int t1 = 0; t1 < A; ++t1) {
-                         const int idx = r * n + B * t1 + t2;
-                         s[t1] = Sq[idx];
-                         wv[t1] = wb[2 * idx];
+                       for (int g = 0; g < A / 4; ++g) {
+                         const int w = (i * (A / 4) + g) * NT;
+                         const float4 sb = Sb[w], wx = wq[w], wy = wq[P / 4 + w];
+#pragma unroll
+                         for (int t = 0; t < 4; ++t)
+                           v[4 * g + t] = mk2(quad_at(wx, t) * quad_at(sb, t), quad_at(wy, t) * quad_at(sb, t));
                        }
+                     },
+                     [&](int i, int r, int t2) {
+                       float4 sx[A / 4], sy[A / 4], wv[A / 4];
+#pragma unroll
+                       for (int g = 0; g < A / 4; ++g) {
+                         const int w = (i * (A / 4) + g) * NT;
+                         sx[g] = Sq[w];
+                         sy[g] = Sq[W4 * NT + w];
+                         wv[g] = wb[w];
+                       }
+                       C2 v[A];
                        stage_a_inverse(v, r, t2);
                        const uint32_t tvi = tv + 2 * A * i;
 #pragma unroll
-                       for (int g = 0; g < A; g += 4) {
-                         float Vx[4] = {}, Vy[4] = {};
+                       for (int g = 0; g < A / 4; ++g) {
+                         float Vx[4] = {}, Vy[4] = {}, k[4];
                          if (b > 0) {
-                           tmem_ld(tvi + g, Vx);
-                           tmem_ld(tvi + A + g, Vy);
+                           tmem_ld(tvi + 4 * g, Vx);
+                           tmem_ld(tvi + A + 4 * g, Vy);
                            tmem_wait_ld(Vx);
                            tmem_wait_ld(Vy);
                          }
 #pragma unroll
                          for (int t = 0; t < 4; ++t) {
-                           const int t1 = g + t, idx = r * n + B * t1 + t2;
-                           const float k = fmaT(e0 * s[t1].x, v[t1].x, -s[t1].y * v[t1].y);
-                           if (k_first) Kb[idx] = k;
-                           else atomicAdd(Kb + idx, k);  // no other thread adds to this point
-                           const float f = eb * wv[t1];
-                           Vx[t] = fmaT(-e0 * f, v[t1].x, Vx[t]);
-                           Vy[t] = fmaT(f, v[t1].y, Vy[t]);
+                           const C2 u = v[4 * g + t];
+                           k[t] = fmaT(e0 * quad_at(sx[g], t), u.x, -quad_at(sy[g], t) * u.y);
+                           const float f = eb * quad_at(wv[g], t);
+                           Vx[t] = fmaT(-e0 * f, u.x, Vx[t]);
+                           Vy[t] = fmaT(f, u.y, Vy[t]);
                          }
-                         tmem_st(tvi + g, Vx);
-                         tmem_st(tvi + A + g, Vy);
+                         float4* kp = Kb + (i * (A / 4) + g) * NT;   // no other thread adds to these points
+                         if (k_first) *kp = make_float4(k[0], k[1], k[2], k[3]);
+                         else red_add4(kp, k[0], k[1], k[2], k[3]);
+                         tmem_st(tvi + 4 * g, Vx);
+                         tmem_st(tvi + A + 4 * g, Vy);
                        }
                        tmem_wait_st();               // loaded again after the next convolution
                      });
@@ -1104,10 +1133,11 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
   }
   if (i >= np + nq) return;
   if (VEC == 2 && real_space && order_n) {   // thread_order planes (FP32, sum given) into rows
-    const int n = order_n, P = n * n, H = n / 32, o = 2 * i % P, tt = o / 4 % (n * H), t1 = o / (4 * n * H) * 4;
-    double* dst = reinterpret_cast<double*>(sum + c * np) + 2 * i / P * P + tt % n;
+    const int P = order_n * order_n;
+    const ThreadWord w = thread_word(order_n, 2 * i % P / 4);
+    double* dst = reinterpret_cast<double*>(sum + c * np) + 2 * i / P * P + w.first;
 #pragma unroll
-    for (int k = 0; k < 2 * VEC; ++k) dst[(H * (t1 + k) + tt / n) * n] = s[k];
+    for (int k = 0; k < 2 * VEC; ++k) dst[w.step * k] = s[k];
   } else if (real_space && sum) {
 #pragma unroll
     for (int k = 0; k < VEC; ++k) sum[c * np + i + k] = mk2(s[2 * k], s[2 * k + 1]);
@@ -1348,10 +1378,11 @@ constexpr int i3_nvariants() {
   }
 }
 
-// Whether a variant is k_i3_tmem, whose partials are planes in thread_order.
+// Whether a variant's partials are planes in thread_order (k_i3_tmem, k_i3_cluster in pairs).
 template <int n, class T>
-constexpr bool i3_variant_tmem(int v) {
-  return std::is_same<T, float>::value && (n == 32 || (n == 64 && v == 0) || (n == 128 && v == 4));
+constexpr bool i3_variant_thread_order(int v) {
+  return std::is_same<T, float>::value &&
+         (n == 32 || (n == 64 && v == 0) || (n == 128 && v == 4) || (use_i3_cluster<n>() && v == 1));
 }
 
 template <int n, class T>
@@ -1635,7 +1666,7 @@ cudaError_t i3_group_n(const Tables* const* tabs, const CollisionWork* const* cw
   for (int k = 0; k < njobs; ++k) {
     if (paired && !cws[k]->K3spec) return cudaErrorInvalidValue;
     cws[k]->i3_paired = paired;
-    cws[k]->i3_thread_order = i3_variant_tmem<n, T>(v);
+    cws[k]->i3_thread_order = i3_variant_thread_order<n, T>(v);
   }
   const I3Launch l = i3_variant<n, T>(v);
   int g = total < grid ? total : grid;

@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
     mu3c[i] = mk2((T)(-tp * m0), (T)(tp * m1));
     mu3c[P + i] = mk2((T)(tp * m2), (T)(tp * m3));
     if (mupl) {
-      T* pl = mupl + (size_t)c * 4 * P + thread_order(n, i / n, i % n);
+      T* pl = mupl + (size_t)c * 4 * P + thread_order<n>(i / n, i % n);
       pl[0] = mu3c[i].x;
       pl[P] = mu3c[i].y;
       pl[2 * P] = mu3c[P + i].x;

@@ -28,11 +28,36 @@ template <> struct Split<256> { static constexpr int A = 16, B = 16; };
 template <> struct Split<96>  { static constexpr int A = 12, B = 8;  };
 template <> struct Split<192> { static constexpr int A = 12, B = 16; };
 
-// Place of point (x, y) in a plane of n = 32 H points a side laid out for k_i3_tmem's threads: thread
-// y + n h holds the elements x = H t1 + h of line y, four consecutive t1 side by side.
-__host__ __device__ __forceinline__ int thread_order(int n, int x, int y) {
-  const int H = n / 32, t1 = x / H;
-  return ((t1 / 4) * n * H + y + n * (x % H)) * 4 + t1 % 4;
+// Planes whose points only their own thread reads are stored in the thread order of the FP32 I3 kernel of
+// their size: 16-byte words of four elements of a thread, consecutive threads side by side.
+//   n = 32 H <= 128 (k_i3_tmem): thread y + n h holds the elements x = H t1 + h of line y;
+//   n > 128 (k_i3_cluster): block x / R of four holds R rows; thread t of its NT = R B / 2 holds, in each of
+//   its two tasks r B + t2 = t + i NT, the elements y = B t1 + t2 of row r.
+// Words of a plane: the point x n + y of the first element and the step to the next three.
+struct ThreadWord {
+  int first, step;
+};
+__host__ __device__ __forceinline__ ThreadWord thread_word(int n, int word) {
+  if (n <= 128) {
+    const int H = n / 32, t = word % (n * H);
+    return {(H * (word / (n * H) * 4) + t / n) * n + t % n, H * n};
+  }
+  const int B = 16, A4 = n / B / 4, R = n / 4, NT = R * B / 2;
+  const int block = word / (R * n / 4), w = word % (R * n / 4), ig = w / NT, task = w % NT + ig / A4 * NT;
+  return {(block * R + task / B) * n + B * (ig % A4 * 4) + task % B, B};
+}
+// Place of point (x, y).
+template <int n>
+__host__ __device__ __forceinline__ int thread_order(int x, int y) {
+  if constexpr (n <= 128) {
+    constexpr int H = n < 32 ? 1 : n / 32;
+    const int t1 = x / H;
+    return ((t1 / 4) * n * H + y + n * (x % H)) * 4 + t1 % 4;
+  } else {
+    constexpr int A = Split<n>::A, B = Split<n>::B, R = n / 4, NT = R * B / 2;
+    const int task = x % R * B + y % B, t1 = y / B;
+    return x / R * R * n + ((task / NT * (A / 4) + t1 / 4) * NT + task % NT) * 4 + t1 % 4;
+  }
 }
 
 // Frequency index (0..n-1, standard wrap) stored at permuted position pos.

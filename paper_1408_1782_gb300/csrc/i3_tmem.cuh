@@ -240,7 +240,6 @@ __device__ __forceinline__ float4* tm_quad(float* plane, int tt) { return reinte
 __device__ __forceinline__ const float4* tm_quad(const float* plane, int tt) {
   return reinterpret_cast<const float4*>(plane) + tt;
 }
-__device__ __forceinline__ float quad_at(const float4& q, int i) { return i == 0 ? q.x : i == 1 ? q.y : i == 2 ? q.z : q.w; }
 
 // The shifted pair S (phase-multiplied Xi coefficients `in`, inverse 2-D transform) into planes Sx (times
 // sign_x), Sx + P, in thread_order: y lines of the n / 2 lines kx of Xi, then the x lines.  Starts and ends with F free.

@@ -116,7 +116,7 @@ struct CollisionWork {
   // whether the last I3 launch over this workspace took the nodes in pairs (its post-processing
   // then adds K3spec); a batch launches its first member's variant for the whole group
   mutable bool i3_paired = false;
-  mutable bool i3_thread_order = false;  // ... whose partials are planes in thread_order (k_i3_tmem)
+  mutable bool i3_thread_order = false;  // ... whose partials are planes in thread_order (k_i3_tmem, k_i3_cluster in pairs)
   void* ws = nullptr;        // per-CTA scratch
   size_t ws_fields = 0;      // complex n*n fields of scratch
   int i3_fields = 3;         // of which an I3 block (or cluster) uses this many

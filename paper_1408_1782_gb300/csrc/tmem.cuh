@@ -83,6 +83,7 @@ __device__ __forceinline__ void tmem_st(uint32_t a, const float (&v)[CNT]) {
   for (int i = 0; i < CNT; i += 4) tmem_st4(a + i, v + i);
 }
 
+__device__ __forceinline__ float quad_at(const float4& q, int i) { return i == 0 ? q.x : i == 1 ? q.y : i == 2 ? q.z : q.w; }
 // Adds four floats in memory (16-byte aligned), nothing returned.
 __device__ __forceinline__ void red_add4(float4* p, float a, float b, float c, float d) {
   asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
