@@ -326,11 +326,12 @@ int qbe_arith_issue_rates(int device, void* stream, double* rates);
  *     stores fused into the line stages and the radial nodes taken in pairs +-rho_m, which share
  *     their convolutions (256 threads, 64 KB or 128 threads, 32 KB).  FP32-split form, 2N = 64, 96, 128: the fused
  *     shared-memory kernel in three thread/accumulation shapes, or the kernel
- *     whose element passes go through shared memory; the kernel with node pairs
- *     and tensor-memory exchanges as variant 0 (2N = 64, in place of the first
- *     shape) or 4 (2N = 128), and as the only one at 2N = 32; 2N = 16: the
+ *     whose element passes go through shared memory; with node pairs the kernel
+ *     with tensor-memory exchanges as variant 0 (2N = 64, in place of the first
+ *     shape) or 4 (2N = 128), and as the only one at 2N = 32, and the kernel of two
+ *     teams per block as variant 4 at 2N = 96; 2N = 16: the
  *     element-pass kernel; 2N = 192, 256: the cluster kernel with 1024 threads per CTA, or
- *     with two row tasks per thread, node pairs and register accumulation;
+ *     with two row tasks per thread, node pairs and sums in tensor memory;
  *   - the persistent grid (blocks; at most the variant's residency);
  *   - the number of m-chunks per (cell, angle) work unit.
  * qbe_i3_shape reports the current shape and the number of variants
@@ -353,9 +354,8 @@ int qbe_autotune(qbe_handle* h, double* best_ms);
 
 /* Kernel variant of the transpose of the I3 term in the collision product
  * (qbe_collide_vjp, and the reverse sweeps of qbe_step_vjp).  FP32-split form
- * at 2N = 128: variant 0 (the default) runs the convolutions on warp-local
- * passes with the sums into XZ held in registers (one cotangent per product),
- * variant 1 the kernel whose element passes go through shared memory; every
+ * at 2N = 128: variant 0 (the default) is the kernel with tensor-memory
+ * exchanges (one cotangent per product), variant 1 the kernel whose element passes go through shared memory; every
  * other grid and precision has one variant.  The variants agree to rounding.
  * qbe_vjp_i3_variant reports the current variant and the count (either
  * pointer may be NULL); qbe_set_vjp_i3_variant sets it (-1: the default;

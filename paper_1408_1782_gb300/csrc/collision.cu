@@ -208,7 +208,7 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   cw.grid_cap = (int)(ws_fields / 3 < (size_t)INT_MAX ? ws_fields / 3 : INT_MAX);
   // fields per block of the kernels that take the nodes in pairs: four in FP64; in FP32 two per team, of
   // which a block has (128 / n)^2
-  cw.i3_fields = prec == 0 ? 4 : t.n == 64 ? 8 : t.n == 32 ? 32 : 3;
+  cw.i3_fields = prec == 0 ? 4 : t.n == 64 ? 8 : t.n == 32 ? 32 : t.n == 96 ? 4 : 3;
   if ((size_t)cw.i3_fields * cw.grid_max > ws_fields) ws_fields = (size_t)cw.i3_fields * cw.grid_max;
   // k_i124: per (cell, chunk, pair) one field for I1 and three for I2/I4
   if (8 * (size_t)nb * cw.nch > ws_fields) ws_fields = 8 * (size_t)nb * cw.nch;
@@ -218,7 +218,7 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   if ((e = cudaMalloc((void**)&(ptr), (bytes))) != cudaSuccess) { free_collision_work(cw); return e; }
   QBE_ALLOC(cw.what, (size_t)nb * 4 * P * cz);
   QBE_ALLOC(cw.wfine, (size_t)nb * 2 * P * cz);
-  if (prec == 1 && t.n != 16 && t.n != 96) QBE_ALLOC(cw.wplane, (size_t)nb * 4 * P * rz);
+  if (prec == 1 && t.n != 16) QBE_ALLOC(cw.wplane, (size_t)nb * 4 * P * rz);
   QBE_ALLOC(cw.Dacc, (size_t)nb * 2 * P * cz);
   QBE_ALLOC(cw.K2acc, (size_t)nb * P * rz);
   QBE_ALLOC(cw.K4acc, (size_t)nb * 2 * P * cz);

@@ -30,7 +30,9 @@ template <> struct Split<192> { static constexpr int A = 12, B = 16; };
 
 // Planes whose points only their own thread reads are stored in the thread order of the FP32 I3 kernel of
 // their size: 16-byte words of four elements of a thread, consecutive threads side by side.
-//   n = 32 H <= 128 (k_i3_tmem): thread y + n h holds the elements x = H t1 + h of line y;
+//   n = 96 (k_i3_lines): thread t of 384 holds, in task i = 0, 1, the elements y = 8 t1 + t2 of line x, where
+//   96 t2 + x = t + 384 i;
+//   n = 32, 64, 128 = 32 H (k_i3_tmem): thread y + n h holds the elements x = H t1 + h of line y;
 //   n > 128 (k_i3_cluster): block x / R of four holds R rows; thread t of its NT = R B / 2 holds, in each of
 //   its two tasks r B + t2 = t + i NT, the elements y = B t1 + t2 of row r.
 // Words of a plane: the point x n + y of the first element and the step to the next three.
@@ -38,6 +40,10 @@ struct ThreadWord {
   int first, step;
 };
 __host__ __device__ __forceinline__ ThreadWord thread_word(int n, int word) {
+  if (n == 96) {
+    const int ig = word / 384, task = word % 384 + ig / 3 * 384;
+    return {task % n * n + 8 * (ig % 3 * 4) + task / n, 8};
+  }
   if (n <= 128) {
     const int H = n / 32, t = word % (n * H);
     return {(H * (word / (n * H) * 4) + t / n) * n + t % n, H * n};
@@ -49,7 +55,10 @@ __host__ __device__ __forceinline__ ThreadWord thread_word(int n, int word) {
 // Place of point (x, y).
 template <int n>
 __host__ __device__ __forceinline__ int thread_order(int x, int y) {
-  if constexpr (n <= 128) {
+  if constexpr (n == 96) {
+    const int task = y % 8 * n + x, t1 = y / 8;
+    return ((task / 384 * 3 + t1 / 4) * 384 + task % 384) * 4 + t1 % 4;
+  } else if constexpr (n <= 128) {
     constexpr int H = n < 32 ? 1 : n / 32;
     const int t1 = x / H;
     return ((t1 / 4) * n * H + y + n * (x % H)) * 4 + t1 % 4;

@@ -95,6 +95,12 @@ def test_fp32_with_every_team_busy(qbe, N, J, M, ncells):
     assert np.abs(out[1] - out[0]).max() < TOL[1] * np.abs(out[0]).max()
 
 
+@pytest.mark.parametrize("N,J,M,ncells", [(48, 32, 8, 8), (48, 2, 9, 40), (96, 4, 3, 4)])
+def test_fp32_grids_with_a_factor_of_three_every_team_busy(qbe, N, J, M, ncells):
+    """The same for the two teams per block of N = 48 and the clusters of N = 96 (odd M: a middle node)."""
+    test_fp32_with_every_team_busy(qbe, N, J, M, ncells)
+
+
 def _derivative(s, w, dw):
     """C'(w) dw: C is cubic in w, so the five-point difference is exact for every step."""
     f = [s.collide(np.ascontiguousarray(w + h * dw)) for h in (1.0, -1.0, 2.0, -2.0)]
