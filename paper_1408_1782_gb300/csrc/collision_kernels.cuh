@@ -591,11 +591,11 @@ __host__ __device__ constexpr bool use_i3_fused() {
   return n == 64 || n == 96 || n == 128;
 }
 // Its launch shapes per size: (threads, blocks per SM, accumulation mode of k_i3_fused), and the
-// default variant (I3 launch, J = M = 32, on a GB300).  N = 16, 256 cells: 5.1 ms for k_i3_tmem.  N = 32,
-// 128 cells: 13.2 ms for k_i3_tmem (variant 0; 28.6 ms for the fused kernel with register accumulation that
+// default variant (I3 launch, J = M = 32, on a GB300).  N = 16, 256 cells: 5.0 ms for k_i3_tmem.  N = 32,
+// 128 cells: 12.5 ms for k_i3_tmem (variant 0; 28.6 ms for the fused kernel with register accumulation that
 // it replaces), 38.8 and 52.3 for shapes 1 and 2, 19.6 for k_i3_smem.  N = 48, 64 cells: 14.3 for k_i3_lines
 // (variant 4), 25.2 for k_i3_smem (38.5 node by node), 38.8, 40.4, 53.2 for the fused shapes.  N = 64,
-// 128 cells: 49.0 for k_i3_tmem (variant 4; 88.6 for the warp-local kernel, node by node, that it
+// 128 cells: 47.6 for k_i3_tmem (variant 4; 88.6 for the warp-local kernel, node by node, that it
 // replaces), 101.1, 116.4, 114.5 for shapes 0 to 2, 83.1 for k_i3_smem.
 template <int n> struct FusedShapes;
 template <> struct FusedShapes<64> {   // variant 0: k_i3_tmem

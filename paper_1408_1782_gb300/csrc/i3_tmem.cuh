@@ -333,11 +333,15 @@ __device__ __forceinline__ void tm_shift_back(const TmLine<n>& ln, float2* F, in
   tm_team_sync<n>(team);
 }
 
+struct TmNothing {
+  __device__ void operator()() const {}
+};
 // One Psi'_j convolution of the field v (natural order, element H t1 + h of x line L = iy), in place.
 // Starts with F free of unread values of other threads; so it ends.
-template <int n>
+// pre() runs before the last line stage (one team per block: loads whose latency that stage covers).
+template <int n, class PRE = TmNothing>
 __device__ __forceinline__ void tm_convolve(const TmLine<n>& ln, float2* F, const float* psm, int L, int team,
-                                            float2 (&v)[32]) {
+                                            float2 (&v)[32], PRE pre = PRE()) {
   constexpr int LS = TmShape<n>::LS, H = TmShape<n>::H, JPT = TmShape<n>::JPT;
   auto to_lines_of_y = [&]() {
 #pragma unroll
@@ -373,6 +377,7 @@ __device__ __forceinline__ void tm_convolve(const TmLine<n>& ln, float2* F, cons
     to_lines_of_x();
 #pragma unroll
     for (int j = 0; j < JPT; ++j) tm_inv_b(ln, j, v + H * j);
+    pre();
     tm_inv_a(ln, v);
   } else {
     // one copy of the code each way: several teams share the instruction cache
@@ -433,7 +438,7 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_tmem(const I3Jobs<floa
   using Sh = TmShape<n>;
   constexpr int P = n * n, H = Sh::H, TT = Sh::TEAM_THREADS;
   constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
-  constexpr int CH = 8;   // points per group of the epilogue's loads (n = 128: 4 51.6, 8 50.9, 16 64.2 ms)
+  constexpr int D = 1;    // words fetched ahead (n = 128: 1 47.6, 2 48.1, 3 49.0 ms; groups of two fetched at once 49.0)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint32_t tm_slot;
   const uint32_t tm_base = tmem_alloc<Sh::COLS>(&tm_slot);
@@ -513,51 +518,48 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_tmem(const I3Jobs<floa
             for (int i = 0; i < 4; ++i)
               v[4 * g + i] = mk2(quad_at(wx, i) * quad_at(sb, i), quad_at(wy, i) * quad_at(sb, i));
           }
-          tm_convolve<n>(ln, F, psm, L, team, v);
+          // the epilogue's operands, D words of each plane ahead
+          float4 op[D][3];
+          auto fetch = [&](int g) {
+            op[g % D][0] = Sq[g * TT];
+            op[g % D][1] = Sq[P / 4 + g * TT];
+            op[g % D][2] = wb[g * TT];
+          };
+          tm_convolve<n>(ln, F, psm, L, team, v, [&]() {
+#pragma unroll
+            for (int g = 0; g < D; ++g) fetch(g);
+          });
+          if constexpr (Sh::TEAMS > 1) {
+#pragma unroll
+            for (int g = 0; g < D; ++g) fetch(g);
+          }
           // K3_b += eta_2q s_2q Re U + eta_2q+1 s_2q+1 Im U (no other thread adds to this point of the
           // unit's partial: a reduction in memory instead of a load and a store);  V_q += eta_b w_b U
           // (x part of q = 0 with the sign that C_0 has against C_1..C_3, see k_assemble)
           const float eb = b == 0 ? 1.f : -1.f;
 #pragma unroll
-          for (int i = 0; i < 32; i += CH) {
-            float Vx[CH], Vy[CH];
+          for (int g = 0; g < 8; ++g) {
+            float Vx[4] = {}, Vy[4] = {}, k[4];
             if (b > 0) {
-              tmem_ld(tv + i, Vx);
-              tmem_ld(tv + 32 + i, Vy);
-            }
-            float4 sx[CH / 4], sy[CH / 4], wv[CH / 4];
-#pragma unroll
-            for (int g = 0; g < CH / 4; ++g) {
-              const int e = (i / 4 + g) * TT;
-              sx[g] = Sq[e];
-              sy[g] = Sq[P / 4 + e];
-              wv[g] = wb[e];
-            }
-            if (b > 0) {
+              tmem_ld(tv + 4 * g, Vx);
+              tmem_ld(tv + 32 + 4 * g, Vy);
               tmem_wait_ld(Vx);
               tmem_wait_ld(Vy);
-            } else {
-#pragma unroll
-              for (int t = 0; t < CH; ++t) Vx[t] = Vy[t] = 0.f;
             }
-            float k[CH];
+            const float4 sx = op[g % D][0], sy = op[g % D][1], wv = op[g % D][2];
+            if (g + D < 8) fetch(g + D);
 #pragma unroll
-            for (int t = 0; t < CH; ++t) {
-              const C2 u = v[i + t];
-              k[t] = fmaf(e0 * quad_at(sx[t / 4], t % 4), u.x, -quad_at(sy[t / 4], t % 4) * u.y);
-              const float f = eb * quad_at(wv[t / 4], t % 4);
+            for (int t = 0; t < 4; ++t) {
+              const C2 u = v[4 * g + t];
+              k[t] = fmaf(e0 * quad_at(sx, t), u.x, -quad_at(sy, t) * u.y);
+              const float f = eb * quad_at(wv, t);
               Vx[t] = fmaf(-e0 * f, u.x, Vx[t]);
               Vy[t] = fmaf(f, u.y, Vy[t]);
             }
-#pragma unroll
-            for (int g = 0; g < CH / 4; ++g) {
-              float4* kp = Kb + (i / 4 + g) * TT;
-              const float* kg = k + 4 * g;
-              if (k_first) *kp = make_float4(kg[0], kg[1], kg[2], kg[3]);
-              else red_add4(kp, kg[0], kg[1], kg[2], kg[3]);
-            }
-            tmem_st(tv + i, Vx);
-            tmem_st(tv + 32 + i, Vy);
+            if (k_first) Kb[g * TT] = make_float4(k[0], k[1], k[2], k[3]);
+            else red_add4(Kb + g * TT, k[0], k[1], k[2], k[3]);
+            tmem_st(tv + 4 * g, Vx);
+            tmem_st(tv + 32 + 4 * g, Vy);
           }
           tmem_wait_st();   // V_q is loaded again after the next convolution
         }

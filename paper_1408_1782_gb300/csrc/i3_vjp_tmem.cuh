@@ -6,8 +6,8 @@
 // over b live in tensor memory; every other sum is added in memory at the thread's own points by
 // reductions (no other thread adds there, so the order is fixed): R[4][P] is the unit's real-space
 // partial, X[4][P] the team's scratch, written first by the Z convolutions of the pair's first q.
-// I3 transpose, 128 cells of N = 64, J = M = 32: 258 (node by node, transforms exchanged in
-// shared memory) -> 130.5 ms.
+// I3 transpose, 24 cells of N = 64, J = M = 32: 48 (node by node, transforms exchanged in shared memory)
+// -> 24.0 ms.
 #pragma once
 
 template <int n>
@@ -19,7 +19,6 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_vjp_tmem(
   using Sh = TmShape<n>;
   constexpr int P = n * n, H = Sh::H, TT = Sh::TEAM_THREADS;
   constexpr int NQ = xi_kept<n>(), Q = NQ * NQ;
-  constexpr int CH = 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint32_t tm_slot;
   const uint32_t tm_base = tmem_alloc<Sh::COLS>(&tm_slot);
@@ -125,51 +124,44 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_vjp_tmem(
               }
             }
           }
-          tm_convolve<n>(ln, F, psm, L, team, v);
+          // the epilogue's operands: mu_b, nu_q or s_b, w_q; the first words before the last stage
+          const float4 *o0 = z ? Sb : mb, *o1 = z ? Wq : Nq;
+          const bool two = z || gr.pair;
+          float4 op[3] = {};
+          auto fetch = [&](int g) {
+            op[0] = o0[g * TT];
+            if (two) {
+              op[1] = o1[g * TT];
+              op[2] = o1[P / 4 + g * TT];
+            }
+          };
+          tm_convolve<n>(ln, F, psm, L, team, v, [&]() { fetch(0); });
+          if constexpr (Sh::TEAMS > 1) fetch(0);
           if (!z) {
             // X_q += mu_b (eta_2q Re U, eta_2q+1 Im U);  R_b += eta_b nu_q . U
             float4* Rb = tm_quad(R + (size_t)b * P, tt);
 #pragma unroll
-            for (int i = 0; i < 32; i += CH) {
-              float Vx[CH], Vy[CH];
+            for (int g = 0; g < 8; ++g) {
+              float Vx[4] = {}, Vy[4] = {}, r[4];
               if (b > 0) {
-                tmem_ld(tv + i, Vx);
-                tmem_ld(tv + 32 + i, Vy);
-              }
-              float4 m[CH / 4], nx[CH / 4], ny[CH / 4];
-#pragma unroll
-              for (int g = 0; g < CH / 4; ++g) {
-                const int e = (i / 4 + g) * TT;
-                m[g] = mb[e];
-                nx[g] = ny[g] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (gr.pair) {
-                  nx[g] = Nq[e];
-                  ny[g] = Nq[P / 4 + e];
-                }
-              }
-              if (b > 0) {
+                tmem_ld(tv + 4 * g, Vx);
+                tmem_ld(tv + 32 + 4 * g, Vy);
                 tmem_wait_ld(Vx);
                 tmem_wait_ld(Vy);
-              } else {
-#pragma unroll
-                for (int t = 0; t < CH; ++t) Vx[t] = Vy[t] = 0.f;
               }
-              float r[CH];
+              const float4 m4 = op[0], nx = op[1], ny = op[2];
+              if (g < 7) fetch(g + 1);
 #pragma unroll
-              for (int t = 0; t < CH; ++t) {
-                const C2 u = v[i + t];
-                const float mt = quad_at(m[t / 4], t % 4);
-                Vx[t] = fmaf(e0 * mt, u.x, Vx[t]);
-                Vy[t] = fmaf(-mt, u.y, Vy[t]);
-                r[t] = eb * fmaf(quad_at(nx[t / 4], t % 4), u.x, quad_at(ny[t / 4], t % 4) * u.y);
+              for (int t = 0; t < 4; ++t) {
+                const C2 u = v[4 * g + t];
+                const float m = quad_at(m4, t);
+                Vx[t] = fmaf(e0 * m, u.x, Vx[t]);
+                Vy[t] = fmaf(-m, u.y, Vy[t]);
+                r[t] = eb * fmaf(quad_at(nx, t), u.x, quad_at(ny, t) * u.y);
               }
-              if (gr.pair) {
-#pragma unroll
-                for (int g = 0; g < CH / 4; ++g)
-                  red_add4(Rb + (i / 4 + g) * TT, r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
-              }
-              tmem_st(tv + i, Vx);
-              tmem_st(tv + 32 + i, Vy);
+              if (gr.pair) red_add4(Rb + g * TT, r[0], r[1], r[2], r[3]);
+              tmem_st(tv + 4 * g, Vx);
+              tmem_st(tv + 32 + 4 * g, Vy);
             }
             tmem_wait_st();
           } else {
@@ -178,7 +170,8 @@ __global__ void __launch_bounds__(TmShape<n>::NT, 1) k_i3_vjp_tmem(
             float4* Xb = tm_quad(X + (size_t)b * P, tt);
 #pragma unroll
             for (int g = 0; g < 8; ++g) {
-              const float4 sb = Sb[g * TT], wx = Wq[g * TT], wy = Wq[P / 4 + g * TT];
+              const float4 sb = op[0], wx = op[1], wy = op[2];
+              if (g < 7) fetch(g + 1);
               float d[4];
 #pragma unroll
               for (int i = 0; i < 4; ++i)
