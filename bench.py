@@ -51,11 +51,11 @@ SM_COUNT = 152
 FP64_FMA_PER_CLK_PER_SM = 2          # GB300: measured 2.00 DFMA lanes/clk/SM (bench.py --mode peaks)
 FP32_FMA_PER_CLK_PER_SM = 128        # measured 122 FFMA lanes/clk/SM (the same run)
 # DRAM bytes (read + write) per (cell, j, m) unit of the default I3 kernel from one ncu capture of a
-# slice (8 cells at N = 64: k_i3_sf in FP64, k_i3_wl in FP32; 4 cells at N = 128: k_i3_cluster in its
-# register-accumulating shape), scaled by units; absent for sizes with no capture of the current kernel.
-I3_DRAM_BYTES_PER_UNIT = {(64, 0): 113.013e9 / 8192, (64, 1): 3.090e9 / 8192, (128, 1): 15.160e9 / 4096}
-# The same for the default I3 transpose kernel (8 cells at N = 64: k_i3_vjp_wl, one cotangent).
-I3_VJP_DRAM_BYTES_PER_UNIT = {(64, 1): 5.463e9 / 8192}
+# slice (8 cells at N = 64: k_i3_sf in FP64, k_i3_tmem in FP32; 4 cells at N = 128: k_i3_cluster in
+# pairs), scaled by units; absent for sizes with no capture of the current kernel.
+I3_DRAM_BYTES_PER_UNIT = {(64, 0): 67.753e9 / 8192, (64, 1): 2.491e9 / 8192, (128, 1): 8.028e9 / 4096}
+# The same for the default I3 transpose kernel (8 cells at N = 64: k_i3_vjp_tmem, one cotangent).
+I3_VJP_DRAM_BYTES_PER_UNIT = {(64, 1): 13.343e9 / 8192}
 
 
 def workload(name="plain_fp64_n64", precision=None):
@@ -67,13 +67,20 @@ def workload(name="plain_fp64_n64", precision=None):
     return wl
 
 
-def i3_flops_per_unit(N):
-    """Algorithmic FLOPs of one (cell, j, m) unit of the I3 (Hu-Ying) term, FFT convention:
-    36 real 2-D transforms of P = (2N)^2 points at 2.5 P log2 P each (4 shifts, 16 forward,
-    16 inverse) plus 67 P pointwise flops (16 products, 16 psi' scalings of complex spectra,
-    16 multiply-adds, the shift phases)."""
+def i3_flops_per_unit(N, paired=True):
+    """Algorithmic FLOPs of one (cell, j, m) unit of the I3 (Hu-Ying) term, FFT convention: real 2-D
+    transforms of P = (2N)^2 points at 2.5 P log2 P each.  Two radial nodes +-rho share their
+    convolutions: 40 of them a pair (4 shifts, 16 forward, 16 inverse, 4 back) plus 103 P pointwise
+    flops (products, psi' scalings, two sums per convolution, phases), half of that per node.  The
+    kernels that take each node by itself: 36 real transforms and 67 P."""
     P = (2 * N) ** 2
-    return 90.0 * P * math.log2(P) + 67.0 * P
+    return (50.0 * P * math.log2(P) + 51.5 * P) if paired else (90.0 * P * math.log2(P) + 67.0 * P)
+
+
+def i3_shape_paired(shape):
+    """Whether the launch shape reported by the library takes the radial nodes in pairs."""
+    name = shape["name"]
+    return "node pairs" in name or "fused loads and stores" in name
 
 
 # ---------------------------------------------------------------------------
@@ -328,7 +335,7 @@ def run_ours(args):
     # roofline of the dominant kernel (I3, Hu-Ying term): FP64 ALU bound
     i3 = groups["i3"]
     avg_i3_s = i3["ms"] * 1e-3 / max(i3["launches"], 1)
-    flops_per_launch = Nx * wl["J"] * wl["M"] * i3_flops_per_unit(N)
+    flops_per_launch = Nx * wl["J"] * wl["M"] * i3_flops_per_unit(N, i3_shape_paired(s.i3_shape()))
     achieved = flops_per_launch / avg_i3_s / 1e12
     sm_max = measured_sm_max()
     lanes = FP64_FMA_PER_CLK_PER_SM if prec == 0 else FP32_FMA_PER_CLK_PER_SM
@@ -489,7 +496,7 @@ def measure_forms(args, wl, W0, s64, fp64_ms_per_step, local):
     sm_max = measured_sm_max()
     peak32 = SM_COUNT * FP32_FMA_PER_CLK_PER_SM * 2 * sm_max * 1e6 / 1e12
     avg_i3 = i3_ms * 1e-3 / max(i3_n, 1)
-    achieved = Nx * wl["J"] * wl["M"] * i3_flops_per_unit(N) / avg_i3 / 1e12
+    achieved = Nx * wl["J"] * wl["M"] * i3_flops_per_unit(N, i3_shape_paired(s.i3_shape())) / avg_i3 / 1e12
     fp32 = {
         "form": "FP32-split: collision transforms and products in FP32; input, output, partial-sum reduction, "
                 "transport, RK2 and moments in FP64",
@@ -706,7 +713,7 @@ def run_collide_only(args, wl, local):
     torch.cuda.synchronize()
     t_ms = e0.elapsed_time(e1)
     i3_ms, i3_n = s.kernel_time("i3")
-    flops = cells * wl["J"] * wl["M"] * i3_flops_per_unit(N)
+    flops = cells * wl["J"] * wl["M"] * i3_flops_per_unit(N, i3_shape_paired(s.i3_shape()))
     line = {"mode": "collide", "metric": "C[W] cell·k-pts/s", "value": args.steps * cells * N * N / (t_ms * 1e-3),
             "unit": "cell·k-pts/s", "cells": cells, "steps": args.steps, "warmup": args.warmup,
             "ms_per_eval": t_ms / args.steps, "i3_ms_per_launch": i3_ms / max(i3_n, 1),
@@ -720,14 +727,11 @@ def run_collide_only(args, wl, local):
 
 def i3_vjp_flops_per_unit(N, K=1):
     """Algorithmic FLOPs of one (cell, j, m) unit of the I3 transpose kernel carrying K cotangents,
-    same convention as i3_flops_per_unit.  Per cotangent: 72 real 2-D transforms (4 for the two
-    shifts, 64 for the 16 convolutions of complex pairs, 4 for the two forward transforms of the
-    shifted-back sums) at 2.5 P log2 P each, plus 228 P pointwise flops (shift phases, 16 scalings,
-    16 psi' products, the three pointwise sums per component, the conjugate phases and spectral
-    accumulation).  K cotangents at one state share the shifts and the 8 convolutions of the state
-    (36 real transforms), so the launch does 36 + 36 K of them."""
+    same convention as i3_flops_per_unit.  A pair of nodes +-rho: 36 + 40 K real 2-D transforms (4 for
+    the state's shifts and 32 for its 8 convolutions; per cotangent 4 for its shifts, 32 for 8
+    convolutions, 4 back) and 38 P + 208 P K pointwise flops; half of that per node."""
     P = (2 * N) ** 2
-    return 2.5 * P * math.log2(P) * (36.0 + 36.0 * K) + 228.0 * P * K
+    return 2.5 * P * math.log2(P) * (18.0 + 20.0 * K) + P * (19.0 + 104.0 * K)
 
 
 def vjp_cotangent_group(prec, N, ncot):
@@ -864,7 +868,8 @@ def measure_adjoint(wl, local, H, every, steps, warmup, cpu_baseline=True, clock
     conf = config_dict(wl, 1)
     vjp_kernel = "k_i3_vjp"                            # the staged form (FP64; FP32 above 128 points)
     if prec == 1 and 2 * N <= 128:
-        vjp_kernel = "k_i3_vjp_wl" if (2 * N == 128 and kgrp == 1 and vjp_variant == 0) else "k_i3_vjp_smem"
+        vjp_kernel = ("k_i3_vjp_tmem" if 2 * N in (32, 64) or (2 * N == 128 and vjp_variant == 0)
+                      else "k_i3_vjp_smem")
     how = ("full tape: every intermediate state kept" if tape == "full"
            else f"checkpoint every {every}, segments recomputed")
     conf.update({"horizon_steps": H, "tape": tape, "checkpoint_every": every if tape != "full" else None,

@@ -330,9 +330,9 @@ cudaError_t collide_vjp(const Tables& t, CollisionWork& cw, VjpWork& vw, const d
 // per single launch against 1297 ms for two).  The FP32 shared-memory kernels run their transforms on
 // chip: the element-pass kernel is bound by its global accumulators, and every further cotangent adds
 // three fields of them per block, which pushes the working set out of L2 (two cotangents: 685 ms
-// against 2 x 333 ms, L2 hit rate 85 % -> 68 %); the warp-local kernel (128 points) holds one
-// cotangent's shifted-back sums in registers, which leave no room for a second.  Both take one
-// cotangent at a time.
+// against 2 x 333 ms, L2 hit rate 85 % -> 68 %); the tensor-memory kernel holds one
+// cotangent's shifted-back sums there, which leave no room for a second.  Both take one cotangent at a
+// time.
 int vjp_cotangent_group(const Tables& t, int prec) { return (prec == 1 && t.n <= 128) ? 1 : kMaxCotangents; }
 
 int vjp_i3_variants(int n, int prec) { return (prec == 1 && n == 128) ? 2 : 1; }

@@ -1299,7 +1299,7 @@ size_t cell_smem_bytes() {
 // Blocks per team of a per-cell kernel over `teams` teams: 1, 2, 4 or 8, the most that stay within three
 // blocks per SM.  The FP64 passes of one cell keep one SM's FP64 unit (two lanes per clock) busy while
 // the others idle, the FP32 ones wait for its latency.  One cell, N = 32 FP64, per C[W]: k_prep 279 ->
-// 31 us, k_i1 390 -> 120 us, k_i24 427 -> 163 us; two steps of it 18.8 -> 14.7 ms.
+// 31 us, I1 and I2/I4 817 -> 283 us; two steps of it 18.8 -> 14.7 ms.
 inline int cell_team(int teams) {
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
