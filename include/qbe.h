@@ -329,7 +329,7 @@ int qbe_arith_issue_rates(int device, void* stream, double* rates);
  *     whose element passes go through shared memory; with node pairs the kernel
  *     with tensor-memory exchanges as variant 0 (2N = 64, in place of the first
  *     shape) or 4 (2N = 128), and as the only one at 2N = 32, and the kernel of two
- *     teams per block as variant 4 at 2N = 96; 2N = 16: the
+ *     teams per block as variant 3 (2N = 96, in place of the element passes); 2N = 16: the
  *     element-pass kernel; 2N = 192, 256: the cluster kernel with 1024 threads per CTA, or
  *     with two row tasks per thread, node pairs and sums in tensor memory;
  *   - the persistent grid (blocks; at most the variant's residency);

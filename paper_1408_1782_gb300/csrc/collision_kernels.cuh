@@ -594,15 +594,15 @@ __host__ __device__ constexpr bool use_i3_fused() {
 // default variant (I3 launch, J = M = 32, on a GB300).  N = 16, 256 cells: 5.0 ms for k_i3_tmem.  N = 32,
 // 128 cells: 12.5 ms for k_i3_tmem (variant 0; 28.6 ms for the fused kernel with register accumulation that
 // it replaces), 38.8 and 52.3 for shapes 1 and 2, 19.6 for k_i3_smem.  N = 48, 64 cells: 14.3 for k_i3_lines
-// (variant 4), 25.2 for k_i3_smem (38.5 node by node), 38.8, 40.4, 53.2 for the fused shapes.  N = 64,
+// (variant 3; 25.2 for k_i3_smem, which it replaces, 38.5 node by node), 38.8, 40.4, 53.2 for the fused shapes.  N = 64,
 // 128 cells: 47.6 for k_i3_tmem (variant 4; 88.6 for the warp-local kernel, node by node, that it
 // replaces), 101.1, 116.4, 114.5 for shapes 0 to 2, 83.1 for k_i3_smem.
 template <int n> struct FusedShapes;
 template <> struct FusedShapes<64> {   // variant 0: k_i3_tmem
   static constexpr int T0 = 0, B0 = 0, M0 = 1, T1 = 512, B1 = 2, M1 = 2, T2 = 256, B2 = 4, M2 = 2, DEFAULT = 0;
 };
-template <> struct FusedShapes<96> {   // variant 4: k_i3_lines
-  static constexpr int T0 = 768, B0 = 1, M0 = 0, T1 = 768, B1 = 1, M1 = 2, T2 = 384, B2 = 2, M2 = 2, DEFAULT = 4;
+template <> struct FusedShapes<96> {   // variant 3: k_i3_lines
+  static constexpr int T0 = 768, B0 = 1, M0 = 0, T1 = 768, B1 = 1, M1 = 2, T2 = 384, B2 = 2, M2 = 2, DEFAULT = 3;
 };
 template <> struct FusedShapes<128> {   // variant 4: k_i3_tmem
   static constexpr int T0 = 512, B0 = 1, M0 = 1, T1 = 1024, B1 = 1, M1 = 2, T2 = 1024, B2 = 1, M2 = 0, DEFAULT = 4;
@@ -1349,8 +1349,8 @@ size_t i3_staged_smem_bytes() {
 //     3: (128, 32 KB, 6).  Variant 0 also serves the allocation-free entry point, whose static array
 //     has no room for the pairs' Fourier-space partials at the sizes it accepts.
 //   FP32, n = 64, 96, 128: 0, 1, 2: the fused shared-memory kernel in the FusedShapes<n> shapes
-//     (0 at n = 64: k_i3_tmem), 3: k_i3_smem (1024 threads, element passes through shared memory), 4:
-//     k_i3_lines (n = 96), k_i3_tmem (n = 128)
+//     (0 at n = 64: k_i3_tmem), 3: k_i3_smem (1024 threads, element passes through shared memory; at
+//     n = 96 k_i3_lines), 4 (n = 128): k_i3_tmem
 //   FP32, n = 32: k_i3_tmem;  n = 16: k_i3_smem;  FP32, n > 128: the cluster kernel, 0: 1024 threads per CTA with a
 //     partial-sum update per convolution, 1: two row tasks per thread, node pairs, sums in tensor memory.
 struct I3Launch {
@@ -1375,7 +1375,7 @@ template <int n, class T>
 constexpr int i3_nvariants() {
   if constexpr (std::is_same<T, float>::value) {
     if constexpr (use_i3_cluster<n>()) return 2;
-    else if constexpr (use_i3_fused<n>()) return n == 64 ? 4 : 5;   // 96, 128 points: + k_i3_lines, k_i3_tmem
+    else if constexpr (use_i3_fused<n>()) return n == 128 ? 5 : 4;   // 128 points: + k_i3_tmem
     else return 1;
   } else {
     return 4;
@@ -1386,7 +1386,7 @@ constexpr int i3_nvariants() {
 template <int n, class T>
 constexpr bool i3_variant_thread_order(int v) {
   return std::is_same<T, float>::value &&
-         (n == 32 || (n == 64 && v == 0) || ((n == 96 || n == 128) && v == 4) || (use_i3_cluster<n>() && v == 1));
+         (n == 32 || (n == 64 && v == 0) || (n == 96 && v == 3) || (n == 128 && v == 4) || (use_i3_cluster<n>() && v == 1));
 }
 
 template <int n, class T>
@@ -1412,15 +1412,14 @@ I3Launch i3_variant(int v) {
       l = {(const void*)k_i3_fused<n, S::T1, S::B1, S::M1>, S::T1, i3_fused_smem_bytes<n>(), false, names[S::M1]};
     else if (v == 2)
       l = {(const void*)k_i3_fused<n, S::T2, S::B2, S::M2>, S::T2, i3_fused_smem_bytes<n>(), false, names[S::M2]};
-    else
+    else if constexpr (n == 96) {
+      using L = LineShape<n>;
+      l = {(const void*)k_i3_lines<n>, L::NT, L::smem, false, "node pairs, shared-memory, two teams of 384 threads per block",
+           L::TEAMS};
+    } else
       l = {(const void*)k_i3_smem<n>, kThreadsI3Smem, i3_smem_bytes<n>(), false, "node pairs, shared-memory, 1024 threads"};
     if constexpr (n == 128) {
       if (v == 4) l = i3_tmem_launch<n>();
-    } else if constexpr (n == 96) {
-      using L = LineShape<n>;
-      if (v == 4)
-        l = {(const void*)k_i3_lines<n>, L::NT, L::smem, false, "node pairs, shared-memory, two teams of 384 threads per block",
-             L::TEAMS};
     }
   } else if constexpr (std::is_same<T, float>::value && n == 32) {
     l = i3_tmem_launch<n>();
@@ -1549,7 +1548,7 @@ template <int n, class T>
 bool i3_variant_paired(int v) {
   if constexpr (std::is_same<T, double>::value) return v >= 2;
   else if constexpr (n > 128) return v == 1;
-  else return n <= 32 || v == 3 || v == (n == 64 ? 0 : 4);
+  else return n <= 32 || v == 3 || v == (n == 128 ? 4 : n == 64 ? 0 : 3);
 }
 
 template <int n, class T>
