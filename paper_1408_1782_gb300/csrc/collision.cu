@@ -171,7 +171,7 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
     if (b > bps_max) bps_max = b;
   }
   cw.prec = prec;
-  cw.nb = nb;
+  cw.nb = cw.order_nb = nb;
   cw.i3_variant = v0;
   cw.grid_i3 = nsm * bps;
   cw.grid_max = nsm * bps_max;

@@ -1153,13 +1153,15 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
 }
 
 // One thread per word where that gives a thousand threads per SM, eight otherwise: short columns of loads,
-// more of them in flight.
+// more of them in flight.  The order of a sum depends on it, so the line goes by the cells nb that the
+// workspace holds (the allocation-free entry, which has none of its own: one), as the chunks do: one handle
+// gives a cell the same bits in a call of one cell and of all.
 template <class T>
 void reduce_partials(typename Vec2Of<T>::type* part, double2* sum, typename Vec2Of<T>::type* spec, int nparts, int np,
-                     int nq, int ncells, int order_n, cudaStream_t s) {
+                     int nq, int nb, int ncells, int order_n, cudaStream_t s) {
   constexpr int VEC = sizeof(T) == 8 ? 1 : 2;
   const int words = (np + nq) / VEC;
-  if (nparts >= 16 && (long long)words * ncells < 152 * 1024) {
+  if (nparts >= 16 && (long long)words * nb < 152 * 1024) {
     const int chunks = (words + 31) / 32;
     k_reduce_k3<T, 8><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, nparts, np, nq, chunks,
                                                                        order_n);
@@ -1711,7 +1713,7 @@ cudaError_t collide_post_n(const Tables& t, CollisionWork& cw, double* c, int nc
   constexpr int nq = 2 * xi_kept<n>() * xi_kept<n>();
   const int nparts = t.J * cw.nmc, nqp = cw.i3_paired ? nq : 0;
   C2* spec = cw.i3_paired ? (C2*)cw.K3spec : nullptr;
-  reduce_partials<T>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, ncells, cw.i3_thread_order ? n : 0, s);
+  reduce_partials<T>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, cw.order_nb, ncells, cw.i3_thread_order ? n : 0, s);
   const double2* k3 = cw.K3sum ? cw.K3sum : (const double2*)cw.K3part;
   C2* DK = (C2*)cw.ws;   // [ncells][4][P], then a field per (cell, pair)
   cudaError_t e = QBE_CELLS(k_dk_fields, 4 * ncells, s, (C2*)cw.Dacc, (C2*)cw.K4acc, DK, tb.tw);

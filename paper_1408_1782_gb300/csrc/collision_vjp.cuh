@@ -859,7 +859,7 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
   for (int k = 0; k < K; ++k) {
     C2* pr = (C2*)vw.part_r + k * part_stride;
     C2* ps = (C2*)vw.part_s + k * spart_stride;
-    reduce_partials<T>(pr, cw.K3sum, ps, units, np, nq, ncells, tmem ? n : 0, s);
+    reduce_partials<T>(pr, cw.K3sum, ps, units, np, nq, vw.nb, ncells, tmem ? n : 0, s);
     const double* R = cw.K3sum ? (const double*)cw.K3sum : (const double*)pr;
     e = QBE_CELLS(k_vjp_final, 2 * ncells, s, (C2*)vw.nu + k * c_stride, (T*)vw.nuf + k * r_stride, R,
                   (cw.K3sum ? (size_t)1 : (size_t)units) * 2 * np, ps, (size_t)units * nq, ws, tb.tw, grad[k], accumulate);

@@ -89,6 +89,7 @@ struct I3Jobs {
 struct CollisionWork {
   int prec = 0;        // 0: FP64 transforms, 1: FP32 transforms (FP32-split form)
   int nb = 0;          // cells per batch
+  int order_nb = 1;    // cells by which the order of the partials' sums is chosen: not those of a call (reduce_partials)
   int nmc = 1;         // m-chunks per (cell, j) unit of the I3 kernel
   int mch = 1;         // m values per chunk (the largest)
   int grid_i3 = 0;     // persistent grid of the I3 kernel
