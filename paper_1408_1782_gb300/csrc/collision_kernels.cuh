@@ -310,6 +310,12 @@ __global__ void __launch_bounds__(kThreads) k_i124(const CellTerms<n, T> a) {
   }
 }
 
+// Blocks of a grid-stride kernel over `count` elements (counted in 64 bits: a call may hold millions of cells).
+inline unsigned element_blocks(size_t count) {
+  const size_t b = (count + kThreads - 1) / kThreads, most = 152 * 32;
+  return (unsigned)(b < most ? b : most);
+}
+
 // Sums of the partials of k_i124 of each cell, in order: D and K4 (2 complex fields each) over the nch
 // chunks (skipped with one: the kernel writes the sums), K2 (real) over its 2 nch planes.
 template <class T>
@@ -1599,7 +1605,7 @@ cudaError_t per_cell_terms(const Tables& t, CollisionWork& cw, typename Vec2Of<T
     if (e != cudaSuccess) return e;
     ++launches;
   }
-  k_reduce_chunks<T><<<(ncells * 5 * n * n + kThreads * 8 - 1) / (kThreads * 8), kThreads, 0, s>>>(
+  k_reduce_chunks<T><<<element_blocks((size_t)ncells * (nch > 1 ? 9 : 1) * P), kThreads, 0, s>>>(
       (const T*)a.D, a.K2, (const T*)a.K4, (T*)cw.Dacc, (T*)cw.K2acc, (T*)cw.K4acc, nch, ncells, P, a.k2_cell);
   if (tm && apart) tm->end(s);
   launches += 2;

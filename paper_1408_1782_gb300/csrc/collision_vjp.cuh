@@ -818,8 +818,8 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
     if (e != cudaSuccess) return e;
     launches += 3;
     if (nch > 1) {
-      k_add_chunks<T><<<(ncells * 5 * n * n + kThreads * 8 - 1) / (kThreads * 8), kThreads, 0, s>>>(
-          (const T*)nup, (const T*)nufp, (T*)nu, nuf, nch, ncells, (size_t)n * n);
+      k_add_chunks<T><<<element_blocks((size_t)ncells * 5 * P), kThreads, 0, s>>>(
+          (const T*)nup, (const T*)nufp, (T*)nu, nuf, nch, ncells, P);
       ++launches;
     }
   }
