@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w,
       [&](int ix, int iy, C2 v) {
         if (xi_t<B>(iy % B)) G[ix * n + iy] = v;
       });
-  auto load = [&](int ix, int iy) { return (ix & 1) ? zero2<T>() : ldc(&G[ix * n + iy]); };
+  auto load = [&](int ix, int iy) { return (ix & 1) ? zero2<T>() : ldc<n, CB>(&G[ix * n + iy]); };
   auto coef = [&](int ix, int iy, C2 v) {
     const bool keep = xi_slot<n>(ix) >= 0 && xi_slot<n>(iy) >= 0;
     const C2 z = keep ? cscale(v, invN2) : zero2<T>();
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w,
   xi_col_filter<n, true, true, CB>(sm, tw, load, coef, [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
   C2* fine = wfine + ((size_t)c * 2 + q) * P;
   row_pass<n, 1, false, 0, CB, true>(
-      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&G[ix * n + iy]) : zero2<T>(); }, NoMid(),
+      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc<n, CB>(&G[ix * n + iy]) : zero2<T>(); }, NoMid(),
       [&](int ix, int iy, C2 v) {
         fine[ix * n + iy] = v;
         if (wplane) {
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kThreads) k_i124(const CellTerms<n, T> a) {
   const int p = id & 1, cch = id >> 1, c = cch / nch, ch = cch % nch;
   const C2* wf0 = a.wfine + (size_t)c * 2 * P;
   auto load_xi = [&](const C2* G) {
-    return [G](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&G[ix * n + iy]) : zero2<T>(); };
+    return [G](int ix, int iy) { return xi_t<B>(iy % B) ? ldc<n, CB>(&G[ix * n + iy]) : zero2<T>(); };
   };
   if (i1) {
     C2* G = a.ws1 + (size_t)id * P;
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kThreads) k_i124(const CellTerms<n, T> a) {
           sm, tw, load_xi(G), [&](int ix, int iy, C2 v) { return cscale(v, (T)2 * wf0[ix * n + iy].x - (T)1); },
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
       col_pass<n, -1, false, 0, CB>(
-          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
+          sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&G[ix * n + iy]); }, NoMid(),
           [&](int ix, int iy, C2 v) {
             const T k = K[ix * n + iy];
             const C2 d = Dp[ix * n + iy];
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kThreads) k_i124(const CellTerms<n, T> a) {
           sm, tw, load_xi(G), NoMid(), [&](int ix, int iy, C2 v) { F[ix * n + iy] = v; });
     }
     for (int i = element_first(); i < P; i += element_stride()) {
-      const C2 fa = ldc(&FA[i]), fb = ldc(&FB[i]);
+      const C2 fa = ldc<n, CB>(&FA[i]), fb = ldc<n, CB>(&FB[i]);
       K2[i] = fmaT((T)2 * wj, e0 * fa.x * fb.x - fa.y * fb.y, K2[i]);
     }
     team_sync();
@@ -297,10 +297,10 @@ __global__ void __launch_bounds__(kThreads) k_i124(const CellTerms<n, T> a) {
       const C2* F = h == 0 ? FB : FA;   // psi_j pairs with F_{j+J/2}
       const T* ps = a.psi + (size_t)(h == 0 ? j : jp) * P;
       row_pass<n, -1, false, 0, CB>(
-          sm, tw, [&](int ix, int iy) { return cscale(ldc(&F[ix * n + iy]), (T)2 * wf0[ix * n + iy].x - (T)1); },
+          sm, tw, [&](int ix, int iy) { return cscale(ldc<n, CB>(&F[ix * n + iy]), (T)2 * wf0[ix * n + iy].x - (T)1); },
           NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
       col_pass<n, -1, false, 0, CB>(
-          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
+          sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&G[ix * n + iy]); }, NoMid(),
           [&](int ix, int iy, C2 v) {
             const T k = scale * ps[ix * n + iy];
             const C2 d = K4[ix * n + iy];
@@ -1198,7 +1198,7 @@ __global__ void __launch_bounds__(kThreads) k_dk_fields(const typename Vec2Of<T>
       sm, tw, [&](int ix, int iy) { return in[ix * n + iy]; }, NoMid(),
       [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
   row_pass<n, 1, false, 0, CB>(
-      sm, tw, [&](int ix, int iy) { return ldc(&out[ix * n + iy]); }, NoMid(),
+      sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&out[ix * n + iy]); }, NoMid(),
       [&](int ix, int iy, C2 v) { out[ix * n + iy] = v; });
 }
 
@@ -1266,7 +1266,7 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
         if (xi_t<B>(iy % B)) H[ix * n + iy] = v;
       });
   xi_col_filter<n, true, true, CB>(
-      sm, tw, [&](int ix, int iy) { return ldc(&H[ix * n + iy]); },
+      sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&H[ix * n + iy]); },
       [&](int ix, int iy, C2 v) {
         const int sx = xi_slot<n>(ix), sy = xi_slot<n>(iy);
         if (sx < 0 || sy < 0) return zero2<T>();
@@ -1280,7 +1280,7 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
         if (!(ix & 1)) H[ix * n + iy] = v;
       });
   even_row_pass<n, 1, CB, true>(
-      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&H[ix * n + iy]) : zero2<T>(); },
+      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc<n, CB>(&H[ix * n + iy]) : zero2<T>(); },
       [&](int ix, int iy, C2 v) {
         if (!(iy & 1)) {
           const int i = ix >> 1, j = iy >> 1;
@@ -1292,13 +1292,6 @@ __global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>:
 
 }  // namespace
 
-// Chunk bytes of the per-cell kernels: one block per team takes 64 KB chunks; in a team of several
-// blocks a chunk is n / 8 rows or columns, so that up to 8 blocks share a pass.
-constexpr int kCellCB = 65536;
-template <int n, class T>
-constexpr int team_cb() {
-  return n * (n / 8) * 2 * (int)sizeof(T);
-}
 template <int n, class T, int CB>
 size_t cell_smem_bytes() {
   using C2 = typename Vec2Of<T>::type;
@@ -1336,13 +1329,13 @@ cudaError_t launch_cells(void (*one)(K...), void (*several)(K...), int teams, si
   return cudaLaunchKernelEx(&cfg, size == 1 ? one : several, static_cast<K>(args)...);
 }
 #define QBE_CELLS(kernel, teams, s, ...)                                                                     \
-  launch_cells(kernel<n, T, kCellCB>, kernel<n, T, team_cb<n, T>()>, teams, cell_smem_bytes<n, T, kCellCB>(), \
-               cell_smem_bytes<n, T, team_cb<n, T>()>(), s, __VA_ARGS__)
+  launch_cells(kernel<n, T, kCellCB>, kernel<n, T, team_cb<n, typename Vec2Of<T>::type>()>, teams, cell_smem_bytes<n, T, kCellCB>(), \
+               cell_smem_bytes<n, T, team_cb<n, typename Vec2Of<T>::type>()>(), s, __VA_ARGS__)
 #define QBE_CELLS_SMEM(kernel)                                                                                 \
   cudaFuncSetAttribute(kernel<n, T, kCellCB>, cudaFuncAttributeMaxDynamicSharedMemorySize,                   \
                        (int)cell_smem_bytes<n, T, kCellCB>());                                                \
-  cudaFuncSetAttribute(kernel<n, T, team_cb<n, T>()>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
-                       (int)cell_smem_bytes<n, T, team_cb<n, T>()>())
+  cudaFuncSetAttribute(kernel<n, T, team_cb<n, typename Vec2Of<T>::type>()>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
+                       (int)cell_smem_bytes<n, T, team_cb<n, typename Vec2Of<T>::type>()>())
 
 template <int n, class T, int CB>
 size_t i3_staged_smem_bytes() {

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kThreads) k_vjp_mu(const double* __restrict__ 
         if (xi_t<B>(iy % B)) M[ix * n + iy] = v;
       });
   xi_col_filter<n, true, true, CB>(
-      sm, tw, [&](int ix, int iy) { return (ix & 1) ? zero2<T>() : ldc(&M[ix * n + iy]); },
+      sm, tw, [&](int ix, int iy) { return (ix & 1) ? zero2<T>() : ldc<n, CB>(&M[ix * n + iy]); },
       [&](int ix, int iy, C2 v) {
         const bool keep = xi_slot<n>(ix) >= 0 && xi_slot<n>(iy) >= 0;
         const C2 z = keep ? cscale(v, invP) : zero2<T>();
@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(kThreads) k_vjp_mu(const double* __restrict__ 
       },
       [&](int ix, int iy, C2 v) { M[ix * n + iy] = v; });
   row_pass<n, 1, false, 0, CB, true>(
-      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&M[ix * n + iy]) : zero2<T>(); }, NoMid(),
+      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc<n, CB>(&M[ix * n + iy]) : zero2<T>(); }, NoMid(),
       [&](int ix, int iy, C2 v) { M[ix * n + iy] = v; });
 }
 
@@ -190,35 +190,35 @@ __global__ void __launch_bounds__(kThreads) k_i1_vjp(
           sm, tw, [&](int ix, int iy) { return mul_i(in[ix * n + iy], ph[ix * n + iy]); },
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
       row_pass<n, 1, false, 0, CB, true>(
-          sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&G[ix * n + iy]) : zero2<T>(); }, NoMid(),
+          sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc<n, CB>(&G[ix * n + iy]) : zero2<T>(); }, NoMid(),
           [&](int ix, int iy, C2 v) { Aw[ix * n + iy] = v; });
       // Bm = IFFT(i K FFT(mu))   (K already carries 1/n^2)
       row_pass<n, -1, false, 0, CB>(
           sm, tw, [&](int ix, int iy) { return mu[ix * n + iy]; }, NoMid(),
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
       col_pass<n, -1, true, 1, CB>(
-          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); },
+          sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&G[ix * n + iy]); },
           [&](int ix, int iy, C2 v) { return mul_i(v, K[ix * n + iy]); },
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
       row_pass<n, 1, false, 0, CB>(
-          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
+          sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&G[ix * n + iy]); }, NoMid(),
           [&](int ix, int iy, C2 v) { Bm[ix * n + iy] = v; });
       // nu_f += Re.Re + Im.Im ;  then -A(f Bm) into nu (pair layout of this p)
       row_pass<n, -1, false, 0, CB>(
           sm, tw,
           [&](int ix, int iy) {
             const int i = ix * n + iy;
-            const C2 a = ldc(&Aw[i]), b = ldc(&Bm[i]);
+            const C2 a = ldc<n, CB>(&Aw[i]), b = ldc<n, CB>(&Bm[i]);
             nufc[i] += a.x * b.x + a.y * b.y;
             return cscale(b, (T)2 * wf0[i].x - (T)1);
           },
           NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
       col_pass<n, -1, true, 1, CB>(
-          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); },
+          sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&G[ix * n + iy]); },
           [&](int ix, int iy, C2 v) { return mul_i(v, -ph[ix * n + iy] * invP); },
           [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
       row_pass<n, 1, false, 0, CB>(
-          sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
+          sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&G[ix * n + iy]); }, NoMid(),
           [&](int ix, int iy, C2 v) {
             const int i = ix * n + iy;
             // pair p = 0 carries components (1, 2) -> nu pair 0 .y and nu pair 1 .x; p = 1 carries (3, -)
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kThreads) k_i24_vjp(
             sm, tw, [&](int ix, int iy) { return cscale(in[ix * n + iy], ps[ix * n + iy]); },
             [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
         row_pass<n, 1, false, 0, CB, true>(
-            sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&G[ix * n + iy]) : zero2<T>(); }, NoMid(),
+            sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc<n, CB>(&G[ix * n + iy]) : zero2<T>(); }, NoMid(),
             [&](int ix, int iy, C2 v) { F[ix * n + iy] = v; });
       }
     }
@@ -296,15 +296,15 @@ __global__ void __launch_bounds__(kThreads) k_i24_vjp(
               sm, tw,
               [&](int ix, int iy) {
                 const int i = ix * n + iy;
-                return part == 0 ? cscale(ldc(&F[i]), mk2c[i]) : mup[i];
+                return part == 0 ? cscale(ldc<n, CB>(&F[i]), mk2c[i]) : mup[i];
               },
               NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
           col_pass<n, -1, true, 1, CB>(
-              sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); },
+              sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&G[ix * n + iy]); },
               [&](int ix, int iy, C2 v) { return cscale(v, ps[ix * n + iy] * invP); },
               [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
           row_pass<n, 1, false, 0, CB>(
-              sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
+              sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&G[ix * n + iy]); }, NoMid(),
               [&](int ix, int iy, C2 v) {
                 const int i = ix * n + iy;
                 if (part == 0) {
@@ -322,17 +322,17 @@ __global__ void __launch_bounds__(kThreads) k_i24_vjp(
             sm, tw,
             [&](int ix, int iy) {
               const int i = ix * n + iy;
-              const C2 pmv = ldc(&PMp[i]), fv = ldc(&F[i]);
+              const C2 pmv = ldc<n, CB>(&PMp[i]), fv = ldc<n, CB>(&F[i]);
               nufc[i] += wj * (pmv.x * fv.x + pmv.y * fv.y);
               return cscale(pmv, (T)2 * wf0[i].x - (T)1);
             },
             NoMid(), [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
         col_pass<n, -1, true, 1, CB>(
-            sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); },
+            sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&G[ix * n + iy]); },
             [&](int ix, int iy, C2 v) { return cscale(v, pq[ix * n + iy] * invP); },
             [&](int ix, int iy, C2 v) { G[ix * n + iy] = v; });
         row_pass<n, 1, false, 0, CB>(
-            sm, tw, [&](int ix, int iy) { return ldc(&G[ix * n + iy]); }, NoMid(),
+            sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&G[ix * n + iy]); }, NoMid(),
             [&](int ix, int iy, C2 v) {
               const int i = ix * n + iy;
               C2 o = nuc[(size_t)p * P + i];
@@ -690,7 +690,7 @@ __global__ void __launch_bounds__(kThreads) k_vjp_final(
         if (xi_t<B>(iy % B)) F[ix * n + iy] = v;
       });
   xi_col_filter<n, true, true, CB>(
-      sm, tw, [&](int ix, int iy) { return ldc(&F[ix * n + iy]); },
+      sm, tw, [&](int ix, int iy) { return ldc<n, CB>(&F[ix * n + iy]); },
       [&](int ix, int iy, C2 v) {
         const int sx = xi_slot<n>(ix), sy = xi_slot<n>(iy);
         if (sx < 0 || sy < 0) return zero2<T>();
@@ -701,7 +701,7 @@ __global__ void __launch_bounds__(kThreads) k_vjp_final(
       });
   double* g = grad + (size_t)c * 4 * N * N;
   even_row_pass<n, 1, CB, true>(
-      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc(&F[ix * n + iy]) : zero2<T>(); },
+      sm, tw, [&](int ix, int iy) { return xi_t<B>(iy % B) ? ldc<n, CB>(&F[ix * n + iy]) : zero2<T>(); },
       [&](int ix, int iy, C2 v) {
         if (!(iy & 1)) {
           const int i = ix >> 1, j = iy >> 1;

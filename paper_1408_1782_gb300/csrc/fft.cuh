@@ -84,7 +84,7 @@ __host__ __device__ __forceinline__ int pos_of_freq(int k) {
 
 // The team of a pass: the blocks of a cluster (a plain launch is a cluster of one).  Its blocks share
 // the chunks of every pass, and data that one block writes and another reads goes through L2 between
-// cluster barriers (release / acquire at cluster scope; the reads bypass L1: ldc).
+// cluster barriers (release / acquire at cluster scope; the reads of teams of several blocks bypass L1: ldc).
 __device__ __forceinline__ int cluster_rank() {
   unsigned r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -113,8 +113,39 @@ __device__ __forceinline__ void team_sync() {
   if (cluster_size() > 1) cluster_sync_global();
   else __syncthreads();
 }
-template <class C>
-__device__ __forceinline__ C ldc(const C* p) { return __ldcg(p); }
+// Chunk bytes of the per-cell kernels: one block per team takes 64 KB chunks; in a team of several
+// blocks a chunk is n / 8 rows or columns, so that up to 8 blocks share a pass.
+constexpr int kCellCB = 65536;
+template <int n, class C>
+__host__ __device__ constexpr int team_cb() {
+  return n * (n / 8) * (int)sizeof(C);
+}
+// Whether a kernel of these chunks is launched with one block per team only: it needs no rank, no cluster
+// barrier, and reads its own writes through L1 (up to n = 64; larger fields only evict what L1 holds).  At
+// small n a pass is little more than its latency, and the ranks read and L1 bypassed in every pass took up to
+// a third of a kernel: FP32, 100 blocks, n = 16 k_i1_vjp 29.1 -> 21.2 us, k_i24_vjp 38.6 -> 26.9; n = 32
+// k_i24_vjp 58.4 -> 46.4; FP64, n = 16 128.4 -> 116.6.
+template <int n, class C, int CB>
+__host__ __device__ constexpr bool lone_block() {
+  return CB == kCellCB && team_cb<n, C>() != kCellCB;
+}
+// Load of what the team has written.
+template <int n, int CB, class C>
+__device__ __forceinline__ C ldc(const C* p) {
+  if constexpr (lone_block<n, C, CB>() && n <= 64) return *p;
+  else return __ldcg(p);
+}
+// Rank and size of the team that shares the chunks of a pass.
+template <int n, class C, int CB>
+__device__ __forceinline__ int pass_rank() {
+  if constexpr (lone_block<n, C, CB>()) return 0;
+  else return cluster_rank();
+}
+template <int n, class C, int CB>
+__device__ __forceinline__ int pass_ranks() {
+  if constexpr (lone_block<n, C, CB>()) return 1;
+  else return cluster_size();
+}
 // Element loops shared by the team: for (i = element_first(); i < count; i += element_stride()).
 __device__ __forceinline__ int element_first() { return cluster_rank() * blockDim.x + threadIdx.x; }
 __device__ __forceinline__ int element_stride() { return cluster_size() * blockDim.x; }
@@ -539,8 +570,8 @@ template <int n, int DIR1, bool HAS_MID, int DIR2, int CB = 65536, bool XI = fal
 __device__ __forceinline__ void row_pass(C2* sm, const C2* tw, LD ld, MID mid, ST st) {
   constexpr int RC = Chunk<n, sizeof(C2), CB>::RC, LS = Chunk<n, sizeof(C2), CB>::LS;
   const int tid = threadIdx.x, nt = blockDim.x;
-  const int ranks = cluster_size();
-  for (int r0 = cluster_rank() * RC; r0 < n; r0 += ranks * RC) {
+  const int ranks = pass_ranks<n, C2, CB>();
+  for (int r0 = pass_rank<n, C2, CB>() * RC; r0 < n; r0 += ranks * RC) {
 #pragma unroll 4
     for (int idx = tid; idx < RC * n; idx += nt) {
       const int r = idx / n, iy = idx % n;
@@ -572,8 +603,8 @@ template <int n, int DIR1, bool HAS_MID, int DIR2, int CB = 65536, class C2, cla
 __device__ __forceinline__ void col_pass(C2* sm, const C2* tw, LD ld, MID mid, ST st) {
   constexpr int CC = Chunk<n, sizeof(C2), CB>::CC;
   const int tid = threadIdx.x, nt = blockDim.x;
-  const int ranks = cluster_size();
-  for (int c0 = cluster_rank() * CC; c0 < n; c0 += ranks * CC) {
+  const int ranks = pass_ranks<n, C2, CB>();
+  for (int c0 = pass_rank<n, C2, CB>() * CC; c0 < n; c0 += ranks * CC) {
 #pragma unroll 4
     for (int idx = tid; idx < CC * n; idx += nt) {
       const int ix = idx / CC, c = idx % CC;
@@ -621,8 +652,8 @@ template <int n, bool FWD, bool INV, int CB = 65536, class C2, class LD, class M
 __device__ __forceinline__ void xi_col_filter(C2* sm, const C2* tw, LD ld, MID mid, ST st) {
   constexpr int CC = half_chunk<n, Chunk<n, sizeof(C2), CB>::CC>(), B = Split<n>::B;
   const int tid = threadIdx.x, nt = blockDim.x;
-  const int ranks = cluster_size();
-  for (int c0 = cluster_rank() * CC; c0 < n / 2; c0 += ranks * CC) {
+  const int ranks = pass_ranks<n, C2, CB>();
+  for (int c0 = pass_rank<n, C2, CB>() * CC; c0 < n / 2; c0 += ranks * CC) {
     const int nc = (n / 2 - c0) < CC ? (n / 2 - c0) : CC;
 #pragma unroll 4
     for (int idx = tid; idx < nc * n; idx += nt) {
@@ -660,8 +691,8 @@ template <int n, int DIR, int CB = 65536, bool XI = false, class C2, class LD, c
 __device__ __forceinline__ void even_row_pass(C2* sm, const C2* tw, LD ld, ST st) {
   constexpr int RC = half_chunk<n, Chunk<n, sizeof(C2), CB>::RC>(), LS = Chunk<n, sizeof(C2), CB>::LS;
   const int tid = threadIdx.x, nt = blockDim.x;
-  const int ranks = cluster_size();
-  for (int r0 = cluster_rank() * RC; r0 < n / 2; r0 += ranks * RC) {
+  const int ranks = pass_ranks<n, C2, CB>();
+  for (int r0 = pass_rank<n, C2, CB>() * RC; r0 < n / 2; r0 += ranks * RC) {
     const int nr = (n / 2 - r0) < RC ? (n / 2 - r0) : RC;
 #pragma unroll 4
     for (int idx = tid; idx < nr * n; idx += nt) sm[idx / n * LS + idx % n] = ld(2 * (r0 + idx / n), idx % n);
