@@ -1298,22 +1298,34 @@ size_t cell_smem_bytes() {
   return (size_t)(n + Chunk<n, sizeof(C2), CB>::SMEM_ELEMS) * sizeof(C2);
 }
 // Blocks per team of a per-cell kernel over `teams` teams: 1, 2, 4 or 8, the most that stay within three
-// blocks per SM.  The FP64 passes of one cell keep one SM's FP64 unit (two lanes per clock) busy while
-// the others idle, the FP32 ones wait for its latency.  One cell, N = 32 FP64, per C[W]: k_prep 279 ->
-// 31 us, I1 and I2/I4 817 -> 283 us; two steps of it 18.8 -> 14.7 ms.
-inline int cell_team(int teams) {
+// blocks per SM, or one where that is fewer than `least`.  The FP64 passes of one cell keep one SM's FP64 unit
+// (two lanes per clock) busy while the others idle, the FP32 ones wait for its latency.  One cell, N = 32 FP64,
+// per C[W]: k_prep 279 -> 31 us, I1 and I2/I4 817 -> 283 us; two steps of it 18.8 -> 14.7 ms.
+inline int cell_team(int teams, int least) {
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   int size = 1;
   while (size < 8 && 2LL * size * teams <= 3LL * nsm) size *= 2;
-  return size;
+  return size < least ? 1 : size;
+}
+// The smallest team worth its cluster barriers.  A team's chunk is n / 8 lines, so a block of a team of s runs
+// 8 / s chunks per pass, one after the other, where a block alone runs one or two larger ones.  Measured (ncu,
+// one / two / four / eight blocks, us; 50, 100 and 200 teams take 8, 4 and 2): n = 16 k_i24_vjp, FP32, 50:
+// 28/165/99/67; n = 32, FP32, 50: 46/161/100/72, FP64, 50: 293/757/400/225, 100: 292/766/409/445; n = 64, FP32,
+// 100: 159/266/162/219, 200: 199/289/348/326, FP64, 200: 2353/1875/1883/1942; n = 96, FP32, 200:
+// 632/543/536/503.  k_assemble (ASSEMBLE) gains earlier in FP32, by its formulas in FP64: n = 32, 50: 16/22/16/12;
+// n = 64, 200: 96/71/62/58.
+template <int n, class T, bool ASSEMBLE>
+constexpr int least_team() {
+  constexpr bool fp32 = std::is_same<T, float>::value && !ASSEMBLE;
+  return n == 16 ? 16 : n == 32 ? (fp32 ? 16 : 8) : n == 64 ? (fp32 ? 4 : 2) : 2;
 }
 // Launches a per-cell kernel over `teams` teams: `one` with a block each, `several` with a cluster each.
 template <class... K, class... Args>
-cudaError_t launch_cells(void (*one)(K...), void (*several)(K...), int teams, size_t smem_one, size_t smem_several,
-                         cudaStream_t s, Args... args) {
-  const int size = cell_team(teams);
+cudaError_t launch_cells(void (*one)(K...), void (*several)(K...), int least, int teams, size_t smem_one,
+                         size_t smem_several, cudaStream_t s, Args... args) {
+  const int size = cell_team(teams, least);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)teams * size);
   cfg.blockDim = dim3(kThreads);
@@ -1328,14 +1340,16 @@ cudaError_t launch_cells(void (*one)(K...), void (*several)(K...), int teams, si
   cfg.numAttrs = size == 1 ? 0 : 1;
   return cudaLaunchKernelEx(&cfg, size == 1 ? one : several, static_cast<K>(args)...);
 }
-#define QBE_CELLS(kernel, teams, s, ...)                                                                     \
-  launch_cells(kernel<n, T, kCellCB>, kernel<n, T, team_cb<n, typename Vec2Of<T>::type>()>, teams, cell_smem_bytes<n, T, kCellCB>(), \
-               cell_smem_bytes<n, T, team_cb<n, typename Vec2Of<T>::type>()>(), s, __VA_ARGS__)
-#define QBE_CELLS_SMEM(kernel)                                                                                 \
-  cudaFuncSetAttribute(kernel<n, T, kCellCB>, cudaFuncAttributeMaxDynamicSharedMemorySize,                   \
-                       (int)cell_smem_bytes<n, T, kCellCB>());                                                \
-  cudaFuncSetAttribute(kernel<n, T, team_cb<n, typename Vec2Of<T>::type>()>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
-                       (int)cell_smem_bytes<n, T, team_cb<n, typename Vec2Of<T>::type>()>())
+#define QBE_TEAM_CB team_cb<n, typename Vec2Of<T>::type>()
+#define QBE_CELLS_OF(assemble, kernel, teams, s, ...)                                                       \
+  launch_cells(kernel<n, T, kCellCB>, kernel<n, T, QBE_TEAM_CB>, least_team<n, T, assemble>(), teams,       \
+               cell_smem_bytes<n, T, kCellCB>(), cell_smem_bytes<n, T, QBE_TEAM_CB>(), s, __VA_ARGS__)
+#define QBE_CELLS(kernel, teams, s, ...) QBE_CELLS_OF(false, kernel, teams, s, __VA_ARGS__)
+#define QBE_CELLS_SMEM(kernel)                                                                              \
+  cudaFuncSetAttribute(kernel<n, T, kCellCB>, cudaFuncAttributeMaxDynamicSharedMemorySize,                  \
+                       (int)cell_smem_bytes<n, T, kCellCB>());                                              \
+  cudaFuncSetAttribute(kernel<n, T, QBE_TEAM_CB>, cudaFuncAttributeMaxDynamicSharedMemorySize,              \
+                       (int)cell_smem_bytes<n, T, QBE_TEAM_CB>())
 
 template <int n, class T, int CB>
 size_t i3_staged_smem_bytes() {
@@ -1717,7 +1731,7 @@ cudaError_t collide_post_n(const Tables& t, CollisionWork& cw, double* c, int nc
   C2* DK = (C2*)cw.ws;   // [ncells][4][P], then a field per (cell, pair)
   cudaError_t e = QBE_CELLS(k_dk_fields, 4 * ncells, s, (C2*)cw.Dacc, (C2*)cw.K4acc, DK, tb.tw);
   if (e != cudaSuccess) return e;
-  e = QBE_CELLS(k_assemble, 2 * ncells, s, (C2*)cw.wfine, DK, (T*)cw.K2acc, k3,
+  e = QBE_CELLS_OF(true, k_assemble, 2 * ncells, s, (C2*)cw.wfine, DK, (T*)cw.K2acc, k3,
                 cw.K3sum ? (size_t)np : (size_t)nparts * np, spec, (size_t)nparts * nq,
                 DK + (size_t)ncells * 4 * n * n, tb.tw, c);
   if (tm) tm->end(s);
