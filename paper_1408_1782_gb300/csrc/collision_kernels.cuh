@@ -142,10 +142,9 @@ __device__ __forceinline__ I3Group i3_group_at(int it, int it1, int M) {
 // (its spectrum repeats with period N), scaled by 1/N^2 and cut to Xi.
 // --------------------------------------------------------------------------
 template <int n, class T, int CB>
-__global__ void __launch_bounds__(kThreads) k_prep(const double* __restrict__ w, typename Vec2Of<T>::type* what,
-                                                   typename Vec2Of<T>::type* wfine, T* wplane,
-                                                   typename Vec2Of<T>::type* ws,
-                                                   const typename Vec2Of<T>::type* __restrict__ gtw) {
+__global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
+    k_prep(const double* __restrict__ w, typename Vec2Of<T>::type* what, typename Vec2Of<T>::type* wfine, T* wplane,
+           typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__ gtw) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
@@ -226,7 +225,8 @@ struct CellTerms {
 };
 
 template <int n, class T, int CB>
-__global__ void __launch_bounds__(kThreads) k_i124(const CellTerms<n, T> a) {
+__global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
+    k_i124(const CellTerms<n, T> a) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
@@ -1181,10 +1181,9 @@ void reduce_partials(typename Vec2Of<T>::type* part, double2* sum, typename Vec2
 // Real-space D pairs and K4 pairs of each cell (inverse 2-D transforms), DK[c][4][P]: one team per cell
 // and pair.
 template <int n, class T, int CB>
-__global__ void __launch_bounds__(kThreads) k_dk_fields(const typename Vec2Of<T>::type* Dacc,
-                                                        const typename Vec2Of<T>::type* K4acc,
-                                                        typename Vec2Of<T>::type* DK,
-                                                        const typename Vec2Of<T>::type* __restrict__ gtw) {
+__global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
+    k_dk_fields(const typename Vec2Of<T>::type* Dacc, const typename Vec2Of<T>::type* K4acc,
+                typename Vec2Of<T>::type* DK, const typename Vec2Of<T>::type* __restrict__ gtw) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
@@ -1213,13 +1212,10 @@ __global__ void __launch_bounds__(kThreads) k_dk_fields(const typename Vec2Of<T>
 // +2 pi K3raw_c; the sign of component 0 is already in spec).
 // --------------------------------------------------------------------------
 template <int n, class T, int CB>
-__global__ void __launch_bounds__(kThreads) k_assemble(const typename Vec2Of<T>::type* wfine,
-                                                       const typename Vec2Of<T>::type* DK, const T* K2acc,
-                                                       const double2* k3, size_t k3_stride,
-                                                       const typename Vec2Of<T>::type* spec, size_t spec_stride,
-                                                       typename Vec2Of<T>::type* ws,
-                                                       const typename Vec2Of<T>::type* __restrict__ gtw,
-                                                       double* cout) {
+__global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
+    k_assemble(const typename Vec2Of<T>::type* wfine, const typename Vec2Of<T>::type* DK, const T* K2acc,
+               const double2* k3, size_t k3_stride, const typename Vec2Of<T>::type* spec, size_t spec_stride,
+               typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__ gtw, double* cout) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);

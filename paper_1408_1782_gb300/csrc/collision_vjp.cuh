@@ -40,9 +40,9 @@ __device__ __forceinline__ C2 mul_i(C2 v, typename RealOf<C2>::type s) {   // v 
 // pair.
 // --------------------------------------------------------------------------
 template <int n, class T, int CB>
-__global__ void __launch_bounds__(kThreads) k_vjp_mu(const double* __restrict__ lam, typename Vec2Of<T>::type* MU,
-                                                     typename Vec2Of<T>::type* muh,
-                                                     const typename Vec2Of<T>::type* __restrict__ gtw) {
+__global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
+    k_vjp_mu(const double* __restrict__ lam, typename Vec2Of<T>::type* MU, typename Vec2Of<T>::type* muh,
+             const typename Vec2Of<T>::type* __restrict__ gtw) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
@@ -152,11 +152,11 @@ __global__ void __launch_bounds__(kThreads) k_vjp_seed(
 //   nu_f += sum_j' (K' mu_b)(A w_b),   nu_b += -A(f K' mu_b).  One block per cell.
 // --------------------------------------------------------------------------
 template <int n, class T, int CB>
-__global__ void __launch_bounds__(kThreads) k_i1_vjp(
-    const typename Vec2Of<T>::type* what, const typename Vec2Of<T>::type* wfine,
-    const typename Vec2Of<T>::type* muD, typename Vec2Of<T>::type* nu, T* nuf, typename Vec2Of<T>::type* ws,
-    const typename Vec2Of<T>::type* __restrict__ gtw, const T* __restrict__ phip, const T* __restrict__ Ktab,
-    int J, int nch) {
+__global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
+    k_i1_vjp(const typename Vec2Of<T>::type* what, const typename Vec2Of<T>::type* wfine,
+             const typename Vec2Of<T>::type* muD, typename Vec2Of<T>::type* nu, T* nuf, typename Vec2Of<T>::type* ws,
+             const typename Vec2Of<T>::type* __restrict__ gtw, const T* __restrict__ phip,
+             const T* __restrict__ Ktab, int J, int nch) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
@@ -240,10 +240,11 @@ __global__ void __launch_bounds__(kThreads) k_i1_vjp(
 // One block per cell.
 // --------------------------------------------------------------------------
 template <int n, class T, int CB>
-__global__ void __launch_bounds__(kThreads) k_i24_vjp(
-    const typename Vec2Of<T>::type* what, const typename Vec2Of<T>::type* wfine, const T* muK2,
-    const typename Vec2Of<T>::type* mu4, typename Vec2Of<T>::type* nu, T* nuf, typename Vec2Of<T>::type* ws,
-    const typename Vec2Of<T>::type* __restrict__ gtw, const T* __restrict__ psi, int J, int nch) {
+__global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
+    k_i24_vjp(const typename Vec2Of<T>::type* what, const typename Vec2Of<T>::type* wfine, const T* muK2,
+              const typename Vec2Of<T>::type* mu4, typename Vec2Of<T>::type* nu, T* nuf,
+              typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__ gtw,
+              const T* __restrict__ psi, int J, int nch) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);
@@ -656,10 +657,10 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_vjp_smem(
 // One team per cell and pair; writes grad[c][4][N][N] (FP64).
 // --------------------------------------------------------------------------
 template <int n, class T, int CB>
-__global__ void __launch_bounds__(kThreads) k_vjp_final(
-    const typename Vec2Of<T>::type* nu, const T* nuf, const double* R, size_t r_stride,
-    const typename Vec2Of<T>::type* spec, size_t spec_stride, typename Vec2Of<T>::type* ws,
-    const typename Vec2Of<T>::type* __restrict__ gtw, double* grad, int accumulate) {
+__global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
+    k_vjp_final(const typename Vec2Of<T>::type* nu, const T* nuf, const double* R, size_t r_stride,
+                const typename Vec2Of<T>::type* spec, size_t spec_stride, typename Vec2Of<T>::type* ws,
+                const typename Vec2Of<T>::type* __restrict__ gtw, double* grad, int accumulate) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* tw = reinterpret_cast<C2*>(smem_raw);

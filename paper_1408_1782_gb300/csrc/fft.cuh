@@ -562,6 +562,16 @@ template <int n, int ELEM = 16, int CB = 65536> struct Chunk {
   static constexpr int SMEM_ELEMS = (RC * LS > CC * n ? RC * LS : CC * n);
 };
 
+// Resident blocks that a kernel of lone blocks is compiled for at up to 64 points, at most what its chunk
+// leaves of shared memory: free to unroll the passes of known chunks, the compiler went to twice the registers
+// (k_i1_vjp at n = 16, FP64, 400 blocks: 48 -> 128 registers, 369 -> 526 us).  0: its own choice.
+template <int n, class T, int CB>
+__host__ __device__ constexpr int cell_min_blocks() {
+  using C2 = typename Vec2Of<T>::type;
+  if (!lone_block<n, C2, CB>() || n > 64) return 0;
+  return 4 * (n + Chunk<n, sizeof(C2), CB>::SMEM_ELEMS) * sizeof(C2) <= 220 * 1024 ? 4 : 3;
+}
+
 // Row pass over an n x n field (rows = fixed ix, transform along iy), its chunks shared by the team:
 // for each chunk: sm[r][iy] = ld(ix, iy); [FFT DIR1]; [sm = mid(ix, iy, sm)]; [FFT DIR2]; st(ix, iy, sm).
 // DIR = 0 skips that transform; HAS_MID selects the pointwise middle step.
