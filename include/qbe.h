@@ -51,7 +51,8 @@ extern "C" {
  * [-L, L]^2; R truncation radius of the collision integrals (B_R).
  * precision: 0 = plain FP64; 1 = FP32-split form (the collision operator's
  * transforms, products and per-unit accumulations in FP32; its input, output
- * and the reduction of its per-unit partial sums, the transport with its
+ * and the reduction of its per-unit partial sums (to FP64 sums, FP32 values
+ * added no less accurately than in FP64), the transport with its
  * boundary projections, the RK2 accumulation and the moments in FP64).  The
  * paper's values are L = 12, R = 7.5, J = M = 32. */
 typedef struct qbe_grid {

@@ -230,6 +230,7 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   QBE_ALLOC(cw.K3part, nparts * 2 * P * cz);
   if (any_paired) QBE_ALLOC(cw.K3spec, nparts * 2 * Q * cz);
   if (prec == 1) QBE_ALLOC(cw.K3sum, (size_t)nb * 2 * P * sizeof(double2));
+  if (prec == 1) QBE_ALLOC(cw.K3ssum, (size_t)nb * 2 * Q * sizeof(double2));
   QBE_ALLOC(cw.ws, ws_fields * P * cz);
   QBE_ALLOC(cw.cbuf, (size_t)nb * 4 * N * N * sizeof(double));
   QBE_ALLOC(cw.wbuf, (size_t)nb * 4 * N * N * sizeof(double));
@@ -240,7 +241,7 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
 void free_collision_work(CollisionWork& cw) {
   cudaFree(cw.what); cudaFree(cw.wfine); cudaFree(cw.wplane); cudaFree(cw.Dacc); cudaFree(cw.K2acc); cudaFree(cw.K4acc);
   cudaFree(cw.Dpart); cudaFree(cw.K2part); cudaFree(cw.K4part);
-  cudaFree(cw.K3part); cudaFree(cw.K3spec); cudaFree(cw.K3sum); cudaFree(cw.ws); cudaFree(cw.cbuf); cudaFree(cw.wbuf);
+  cudaFree(cw.K3part); cudaFree(cw.K3spec); cudaFree(cw.K3sum); cudaFree(cw.K3ssum); cudaFree(cw.ws); cudaFree(cw.cbuf); cudaFree(cw.wbuf);
   cw = CollisionWork();
 }
 

@@ -28,8 +28,11 @@
 //
 // Precision: every kernel is a template on the real type T of its transforms,
 // products and per-unit accumulations (double: the plain FP64 form; float: the
-// FP32-split form).  The state W comes in and C[W] goes out in FP64, and the
-// reduction of the per-unit K3 partial sums is done in FP64 in both forms.
+// FP32-split form).  The state W comes in and C[W] goes out in FP64.  The per-unit
+// K3 partial sums are reduced to FP64 sums in both forms (the FP32 values no less
+// accurately than by FP64 additions, float_sum.cuh); they are rounded to T once, the
+// real-space ones with the rest of C on the grid, the Fourier-space ones with the
+// spectrum of C that they are added to.
 #pragma once
 
 #include <cmath>
@@ -37,6 +40,7 @@
 #include <type_traits>
 
 #include "fft.cuh"
+#include "float_sum.cuh"
 #include "internal.h"
 #include "tmem.cuh"
 
@@ -1087,17 +1091,16 @@ __global__ void __cluster_dims__(kI3Cluster, 1, 1) __launch_bounds__(NT, 1)
 // the order of g.  Bound by HBM (or L2, where the partials still sit there).  It was part of k_assemble,
 // whose one block per cell read a single cell's partials alone: at one cell of N = 32, J = M = 32, 1024
 // units, 5.2 of the 5.5 ms of that kernel.
-// FP32 partials are added as unevaluated sums hi + lo of two floats (the error-free addition of Knuth,
-// TwoSum; about 48 bits) and combined in FP64: converting and adding each value in FP64 bound the kernel
-// at a fifth of the memory rate (two FP64 lanes per clock), 128 cells of N = 64 1234 us
-// against 264 us.
-// sum: [ncells][np], or null (FP64): in place into the cell's first unit; the Fourier-space sums are
-// always put there.  order_n: padded grid size where the partials' four planes are in thread_order, else 0.
+// FP32 partials are added as unevaluated sums of three floats, runs of 64 of them in FP64 (FloatSum):
+// converting and adding each value in FP64 bound the kernel at a fifth of the memory rate (two FP64 lanes
+// per clock), 128 cells of N = 64 1234 us against 248 us.
+// sum: [ncells][np] and spec_sum: [ncells][nq] (FP32), or null (FP64): in place into the cell's first unit.
+// order_n: padded grid size where the partials' four planes are in thread_order, else 0.
 // --------------------------------------------------------------------------
 template <class T, int G>
 __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* part, double2* sum,
-                                                   typename Vec2Of<T>::type* spec, int nparts, int np, int nq,
-                                                   int chunks, int order_n) {
+                                                   typename Vec2Of<T>::type* spec, double2* spec_sum, int nparts,
+                                                   int np, int nq, int chunks, int order_n) {
   using Word = typename std::conditional<sizeof(T) == 8, double2, float4>::type;
   constexpr int PT = 256 / G, VEC = sizeof(T) == 8 ? 1 : 2;   // complex values per word
   const size_t c = blockIdx.x / chunks;
@@ -1115,20 +1118,20 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
         s[1] += v.y;
       }
     } else {
-      float hi[4] = {}, lo[4] = {};
+      for (int u0 = g; u0 < nparts; u0 += G * FloatSum::kRun) {
+        const int u1 = min(nparts, u0 + G * FloatSum::kRun);
+        FloatSum a[4];
 #pragma unroll 8
-      for (int u = g; u < nparts; u += G) {
-        const Word v = src[(size_t)u * stride];
-        const float x[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float t = __fadd_rn(hi[k], x[k]), z = __fsub_rn(t, hi[k]);
-          lo[k] = __fadd_rn(lo[k], __fadd_rn(__fsub_rn(hi[k], __fsub_rn(t, z)), __fsub_rn(x[k], z)));
-          hi[k] = t;
+        for (int u = u0; u < u1; u += G) {
+          const Word v = src[(size_t)u * stride];
+          a[0].add(v.x);
+          a[1].add(v.y);
+          a[2].add(v.z);
+          a[3].add(v.w);
         }
-      }
 #pragma unroll
-      for (int k = 0; k < 4; ++k) s[k] = (double)hi[k] + (double)lo[k];
+        for (int k = 0; k < 4; ++k) s[k] += a[k].value();
+      }
     }
   }
   if constexpr (G > 1) {
@@ -1148,9 +1151,10 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
     double* dst = reinterpret_cast<double*>(sum + c * np) + 2 * i / P * P + w.first;
 #pragma unroll
     for (int k = 0; k < 2 * VEC; ++k) dst[w.step * k] = s[k];
-  } else if (real_space && sum) {
+  } else if (VEC == 2) {
+    double2* o = real_space ? sum + c * np + i : spec_sum + c * nq + (i - np);
 #pragma unroll
-    for (int k = 0; k < VEC; ++k) sum[c * np + i + k] = mk2(s[2 * k], s[2 * k + 1]);
+    for (int k = 0; k < VEC; ++k) o[k] = mk2(s[2 * k], s[2 * k + 1]);
   } else {
     T* o = reinterpret_cast<T*>(src);
 #pragma unroll
@@ -1163,18 +1167,18 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
 // workspace holds (the allocation-free entry, which has none of its own: one), as the chunks do: one handle
 // gives a cell the same bits in a call of one cell and of all.
 template <class T>
-void reduce_partials(typename Vec2Of<T>::type* part, double2* sum, typename Vec2Of<T>::type* spec, int nparts, int np,
-                     int nq, int nb, int ncells, int order_n, cudaStream_t s) {
+void reduce_partials(typename Vec2Of<T>::type* part, double2* sum, typename Vec2Of<T>::type* spec,
+                     double2* spec_sum, int nparts, int np, int nq, int nb, int ncells, int order_n, cudaStream_t s) {
   constexpr int VEC = sizeof(T) == 8 ? 1 : 2;
   const int words = (np + nq) / VEC;
   if (nparts >= 16 && (long long)words * nb < 152 * 1024) {
     const int chunks = (words + 31) / 32;
-    k_reduce_k3<T, 8><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, nparts, np, nq, chunks,
-                                                                       order_n);
+    k_reduce_k3<T, 8><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, spec_sum, nparts, np, nq,
+                                                                chunks, order_n);
   } else {
     const int chunks = (words + 255) / 256;
-    k_reduce_k3<T, 1><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, nparts, np, nq, chunks,
-                                                                       order_n);
+    k_reduce_k3<T, 1><<<(unsigned)chunks * ncells, 256, 0, s>>>(part, sum, spec, spec_sum, nparts, np, nq,
+                                                                chunks, order_n);
   }
 }
 
@@ -1207,14 +1211,14 @@ __global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
 // coarse nodes.  One team per cell and pair (C_0, C_1) or (C_2, C_3); the pointwise
 // formulas are evaluated on the load of the first pass, and after it only the Xi
 // columns and the even rows are transformed.  k3: the reduced K3 of a cell (FP64),
-// k3_stride apart; spec (null after a node-by-node kernel): their Fourier-space parts,
+// k3_stride apart; spec (null after a node-by-node kernel): their Fourier-space parts (FP64),
 // added to the spectrum of C inside the projection (C_0 holds -2 pi K3_0 and C_c holds
 // +2 pi K3raw_c; the sign of component 0 is already in spec).
 // --------------------------------------------------------------------------
 template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
     k_assemble(const typename Vec2Of<T>::type* wfine, const typename Vec2Of<T>::type* DK, const T* K2acc,
-               const double2* k3, size_t k3_stride, const typename Vec2Of<T>::type* spec, size_t spec_stride,
+               const double2* k3, size_t k3_stride, const double2* spec, size_t spec_stride,
                typename Vec2Of<T>::type* ws, const typename Vec2Of<T>::type* __restrict__ gtw, double* cout) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1233,7 +1237,7 @@ __global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
   const double tp = 2.0 * kPi;
   const T invP = (T)(1.0 / (double)P);
   double* co = cout + (size_t)c * 4 * N * N;
-  const C2* Hs = spec ? spec + c * spec_stride + (size_t)p * Q : nullptr;
+  const double2* Hs = spec ? spec + c * spec_stride + (size_t)p * Q : nullptr;
   row_pass<n, -1, false, 0, CB>(
       sm, tw,
       [&](int ix, int iy) {
@@ -1267,8 +1271,8 @@ __global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
         const int sx = xi_slot<n>(ix), sy = xi_slot<n>(iy);
         if (sx < 0 || sy < 0) return zero2<T>();
         if (Hs) {
-          const C2 h = Hs[sx * NQ + sy];
-          v = mk2(fmaT((T)tp, h.x, v.x), fmaT((T)tp, h.y, v.y));
+          const double2 h = Hs[sx * NQ + sy];
+          v = mk2((T)fma(tp, h.x, (double)v.x), (T)fma(tp, h.y, (double)v.y));
         }
         return cscale(v, invP);
       },
@@ -1721,14 +1725,16 @@ cudaError_t collide_post_n(const Tables& t, CollisionWork& cw, double* c, int nc
   constexpr int np = 2 * n * n;
   constexpr int nq = 2 * xi_kept<n>() * xi_kept<n>();
   const int nparts = t.J * cw.nmc, nqp = cw.i3_paired ? nq : 0;
-  C2* spec = cw.i3_paired ? (C2*)cw.K3spec : nullptr;
-  reduce_partials<T>((C2*)cw.K3part, cw.K3sum, spec, nparts, np, nqp, cw.order_nb, ncells, cw.i3_thread_order ? n : 0, s);
+  C2* part_s = cw.i3_paired ? (C2*)cw.K3spec : nullptr;
+  reduce_partials<T>((C2*)cw.K3part, cw.K3sum, part_s, cw.K3ssum, nparts, np, nqp, cw.order_nb, ncells,
+                     cw.i3_thread_order ? n : 0, s);
+  const double2* spec = !cw.i3_paired ? nullptr : cw.K3ssum ? cw.K3ssum : (const double2*)cw.K3spec;
   const double2* k3 = cw.K3sum ? cw.K3sum : (const double2*)cw.K3part;
   C2* DK = (C2*)cw.ws;   // [ncells][4][P], then a field per (cell, pair)
   cudaError_t e = QBE_CELLS(k_dk_fields, 4 * ncells, s, (C2*)cw.Dacc, (C2*)cw.K4acc, DK, tb.tw);
   if (e != cudaSuccess) return e;
   e = QBE_CELLS_OF(true, k_assemble, 2 * ncells, s, (C2*)cw.wfine, DK, (T*)cw.K2acc, k3,
-                cw.K3sum ? (size_t)np : (size_t)nparts * np, spec, (size_t)nparts * nq,
+                cw.K3sum ? (size_t)np : (size_t)nparts * np, spec, cw.K3ssum ? (size_t)nq : (size_t)nparts * nq,
                 DK + (size_t)ncells * 4 * n * n, tb.tw, c);
   if (tm) tm->end(s);
   if (e != cudaSuccess) return e;

@@ -659,7 +659,7 @@ __global__ void __launch_bounds__(kThreadsI3Smem, 1) k_i3_vjp_smem(
 template <int n, class T, int CB>
 __global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
     k_vjp_final(const typename Vec2Of<T>::type* nu, const T* nuf, const double* R, size_t r_stride,
-                const typename Vec2Of<T>::type* spec, size_t spec_stride, typename Vec2Of<T>::type* ws,
+                const double2* spec, size_t spec_stride, typename Vec2Of<T>::type* ws,
                 const typename Vec2Of<T>::type* __restrict__ gtw, double* grad, int accumulate) {
   using C2 = typename Vec2Of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -671,7 +671,7 @@ __global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
   const int c = cluster_index() >> 1, p = cluster_index() & 1;
   C2* F = ws + (size_t)cluster_index() * P;
   const double* Rc = R + c * r_stride + (size_t)2 * p * P;
-  const C2* Hp = spec + c * spec_stride + (size_t)p * Q;
+  const double2* Hp = spec + c * spec_stride + (size_t)p * Q;
   const C2* nup = nu + ((size_t)c * 2 + p) * P;
   const T* nufc = nuf + (size_t)c * P;
   const T invP = (T)(1.0 / (double)P);
@@ -695,7 +695,8 @@ __global__ void __launch_bounds__(kThreads, (cell_min_blocks<n, T, CB>()))
       [&](int ix, int iy, C2 v) {
         const int sx = xi_slot<n>(ix), sy = xi_slot<n>(iy);
         if (sx < 0 || sy < 0) return zero2<T>();
-        return cscale(cadd(v, Hp[sx * NQ + sy]), invP);
+        const double2 h = Hp[sx * NQ + sy];
+        return cscale(mk2((T)((double)v.x + h.x), (T)((double)v.y + h.y)), invP);
       },
       [&](int ix, int iy, C2 v) {
         if (!(ix & 1)) F[ix * n + iy] = v;
@@ -860,10 +861,12 @@ cudaError_t collide_vjp_n(const Tables& t, CollisionWork& cw, VjpWork& vw, const
   for (int k = 0; k < K; ++k) {
     C2* pr = (C2*)vw.part_r + k * part_stride;
     C2* ps = (C2*)vw.part_s + k * spart_stride;
-    reduce_partials<T>(pr, cw.K3sum, ps, units, np, nq, vw.nb, ncells, tmem ? n : 0, s);
+    reduce_partials<T>(pr, cw.K3sum, ps, cw.K3ssum, units, np, nq, vw.nb, ncells, tmem ? n : 0, s);
     const double* R = cw.K3sum ? (const double*)cw.K3sum : (const double*)pr;
+    const double2* H = cw.K3ssum ? cw.K3ssum : (const double2*)ps;
     e = QBE_CELLS(k_vjp_final, 2 * ncells, s, (C2*)vw.nu + k * c_stride, (T*)vw.nuf + k * r_stride, R,
-                  (cw.K3sum ? (size_t)1 : (size_t)units) * 2 * np, ps, (size_t)units * nq, ws, tb.tw, grad[k], accumulate);
+                  (cw.K3sum ? (size_t)1 : (size_t)units) * 2 * np, H, (cw.K3ssum ? (size_t)1 : (size_t)units) * nq, ws,
+                  tb.tw, grad[k], accumulate);
     if (e != cudaSuccess) return e;
     launches += 2;
   }

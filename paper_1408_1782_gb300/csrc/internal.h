@@ -114,6 +114,7 @@ struct CollisionWork {
   // [nb*J*nmc][2][(n/2-1)^2]; null: the workspace serves the node-by-node kernels only
   void* K3spec = nullptr;
   double2* K3sum = nullptr;  // [nb][2][n*n] reduced K3 in the same order (FP32 form; FP64 reduces in place)
+  double2* K3ssum = nullptr; // [nb][2][(n/2-1)^2] reduced K3spec (the same)
   // whether the last I3 launch over this workspace took the nodes in pairs (its post-processing
   // then adds K3spec); a batch launches its first member's variant for the whole group
   mutable bool i3_paired = false;
