@@ -199,6 +199,29 @@ __host__ __device__ constexpr double cos32(int k) {
                              : k == 6 ? c6 : c7);
 }
 __host__ __device__ constexpr double sin32(int k) { return cos32(k - 8); }
+// FP32 constants c = cos(2 pi k / 32) and r = tan(2 pi k / 32) of the cosine-factored butterflies of radix 32
+// (the I3 kernels with tensor-memory exchanges), for 0 < k < 16, k != 8: of the floats within two units in the
+// last place the pair whose turn c + i c r is nearest to length 1 (plus a twentieth of its error in angle).
+// Rounded each by itself they shorten a line's low frequencies by up to 3e-8 a stage, the same in every
+// convolution, so that the errors add up over the nodes; two stages of radix 8 and 16 average over more
+// constants.  Error of C[W] at N = 16, 32, 64 (J = M = 16, six states): 5.2, 5.8, 6.4e-7 -> 5.0, 5.8, 6.0e-7
+// (node by node 4.8, 5.5, 5.7e-7).  Not taken: such pairs in every radix (N = 64 6.8e-7: what I3 and the other
+// terms have in common cancels in C), radix 32 as 4 x 8 (5.6e-7 at N = 32, the same at 64, 2.7 and 6 % slower at
+// N = 64 and 16).
+struct Turn {
+  float c, r;
+};
+__host__ __device__ constexpr Turn turn32(int k) {
+  const int m = k > 8 ? 16 - k : k;
+  const Turn t = m == 1 ? Turn{0x1.f6297cp-1f, 0x1.975f62p-3f}
+               : m == 2 ? Turn{0x1.d906bcp-1f, 0x1.a8279ep-2f}
+               : m == 3 ? Turn{0x1.a9b662p-1f, 0x1.561b84p-1f}
+               : m == 4 ? Turn{0x1.6a09e8p-1f, 0x1.fffffcp-1f}
+               : m == 5 ? Turn{0x1.1c73b4p-1f, 0x1.7f218ep+0f}
+               : m == 6 ? Turn{0x1.87de2ep-2f, 0x1.3504f0p+1f}
+                        : Turn{0x1.8f8b84p-3f, 0x1.41bfeep+2f};
+  return k > 8 ? Turn{-t.c, -t.r} : t;
+}
 
 // x * exp(SIGN * 2 pi i k / R) for R <= 32, k a compile-time constant after unrolling.
 template <int R, int SIGN, class C2>
@@ -240,8 +263,8 @@ struct DftStage {
           b[g + k] = cadd(u, t);
           b[g + k + S / 2] = csub(u, t);
         } else {
-          const T c = (T)cos32(k32);
-          const T r = (T)((SIGN * sin32(k32)) / cos32(k32));
+          const T c = sizeof(T) == 4 && R == 32 ? (T)turn32(k32).c : (T)cos32(k32);
+          const T r = sizeof(T) == 4 && R == 32 ? (T)(SIGN * turn32(k32).r) : (T)((SIGN * sin32(k32)) / cos32(k32));
           const T qx = fmaT(-r, x.y, x.x);
           const T qy = fmaT(r, x.x, x.y);
           b[g + k] = mk2(fmaT(c, qx, u.x), fmaT(c, qy, u.y));
