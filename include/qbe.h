@@ -85,6 +85,13 @@ typedef struct qbe_handle qbe_handle;
 /* Create a solver for grid g on device g->device.  Allocates the state, the
  * kernel tables (G and H quadratures of eqs. approxG, approxH-J, approxH-JM)
  * and the collision workspace.  *out receives the handle (NULL on failure).
+ * The workspace is mostly partial sums of the I3 term: per cell, angle and
+ * chunk of the radial nodes 4 (2N)^2 + 4 (N-1)^2 values of the form's
+ * precision, in as many chunks as fill the GPU about eight times, and more
+ * (up to 1.5 GB, 4 GB in all) where that evens out its load.  Where the
+ * device's free memory does not hold it, it is made for fewer chunks, then
+ * for half, a quarter and so on of the cells: calls evaluate C[W] for so many
+ * at a time, with the same results to rounding.
  * Errors: QBE_ERR_ARG (bad sizes, odd J, N unsupported), QBE_ERR_ALLOC,
  * QBE_ERR_CUDA. */
 int qbe_create(const qbe_grid* g, qbe_handle** out);
@@ -161,16 +168,18 @@ int qbe_moments(qbe_handle* h, double* rho, double* mom, double* energy, int on_
 /* grad = (dC/dW at w)^T lam for ncells independent cells: w, lam, grad
  * [ncells][4][N][N] (grad may alias lam).  Does not touch the solver state.
  * The first call allocates the product's workspace (about twice the
- * collision workspace).  Errors: QBE_ERR_ARG, QBE_ERR_ALLOC, QBE_ERR_CUDA. */
+ * collision workspace; where memory is short, smaller in the same way).
+ * Errors: QBE_ERR_ARG, QBE_ERR_ALLOC, QBE_ERR_CUDA. */
 int qbe_collide_vjp(qbe_handle* h, const double* w, const double* lam, double* grad, int ncells, int on_device);
 
 /* ncot products at the same state at once: grad[k] = (dC/dW at w)^T lam[k],
  * k < ncot, with lam, grad [ncot][ncells][4][N][N] and w [ncells][4][N][N],
  * all DEVICE memory (on_device must be 1).  The products are evaluated in
  * groups that share the state's transforms (for the I3 term, the Psi'
- * convolutions of the state: 8 of the 16 per (j, m) and product); groups
- * are as in qbe_step_vjp_n;
- * each result equals qbe_collide_vjp's bit for bit.  Grows the workspace to
+ * convolutions of the state: 8 of the 16 per angle, pair of nodes and
+ * product); groups are as in qbe_step_vjp_n;
+ * each result equals qbe_collide_vjp's bit for bit (where the memory holds
+ * the whole workspace).  Grows the workspace to
  * the group size on first use.  Errors: QBE_ERR_ARG (ncot < 1, ncells < 1,
  * null pointers, on_device != 1), QBE_ERR_ALLOC, QBE_ERR_CUDA. */
 int qbe_collide_vjp_n(qbe_handle* h, int ncot, const double* w, const double* lam, double* grad, int ncells,

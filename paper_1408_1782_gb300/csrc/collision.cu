@@ -1,6 +1,7 @@
 // Size dispatch and workspace allocation of the collision operator; the
 // kernels are instantiated per fine-grid size in collision_n*.cu.
 #include <climits>
+#include <utility>
 #include <vector>
 
 #include "internal.h"
@@ -113,8 +114,8 @@ double chunk_cost(int begin, int end, int M, const NodeCost& c) {
 
 // m-chunks per (cell, angle) for a launch that works on G units at a time, unit u on slot u mod G: `base`,
 // or up to three times as many (at least `most_at_least`, at most M) where that evens out the slots'
-// loads by more than a hundredth, within 4 GB of partials.  A unit's fixed costs (its tables loaded, its
-// partials written and reduced) count per_unit transforms.
+// loads by more than a hundredth, within 4 GB of partials and 1.5 GB more than `base` takes.  A unit's fixed
+// costs (its tables loaded, its partials written and reduced) count per_unit transforms.
 int even_chunks(long long cj, int G, int M, int base, int most_at_least, size_t unit_bytes, const NodeCost& c,
                 double per_unit) {
   double best = 0;
@@ -123,7 +124,8 @@ int even_chunks(long long cj, int G, int M, int base, int most_at_least, size_t 
   for (int want = base; want <= most && want <= M; ++want) {
     const int mch = (M + want - 1) / want, nmc = (M + mch - 1) / mch;
     const long long units = cj * nmc;
-    if (want > base && (nmc == base || (size_t)units * unit_bytes > ((size_t)4 << 30))) continue;
+    const size_t bytes = (size_t)units * unit_bytes, more = (size_t)(units - cj * base) * unit_bytes;
+    if (want > base && (nmc == base || bytes > ((size_t)4 << 30) || more > ((size_t)3 << 29))) continue;
     const int g = G < units ? G : (int)units;
     std::vector<double> load(g, 0.0), cost(nmc);
     for (int mc = 0; mc < nmc; ++mc)
@@ -138,6 +140,28 @@ int even_chunks(long long cj, int G, int M, int base, int most_at_least, size_t 
   }
   return best_nmc;
 }
+
+// Buffers in one device allocation, each on a 256-byte boundary: creating a handle is a single cudaMalloc per
+// workspace, and one that does not fit leaves nothing behind.
+struct Carve {
+  std::vector<std::pair<void**, size_t>> parts;
+  size_t total = 0;
+  template <class T>
+  void add(T*& p, size_t bytes) {
+    parts.push_back({(void**)&p, total});
+    total += (bytes + 255) & ~(size_t)255;
+  }
+  cudaError_t take(void*& mem) const {
+    const cudaError_t e = cudaMalloc(&mem, total);
+    if (e != cudaSuccess) {
+      mem = nullptr;
+      cudaGetLastError();   // the caller may try a smaller one
+      return e;
+    }
+    for (const auto& p : parts) *p.first = (unsigned char*)mem + p.second;
+    return cudaSuccess;
+  }
+};
 }  // namespace
 
 double i3_chunk_cost(int begin, int end, int M, bool paired) {
@@ -156,7 +180,7 @@ int per_cell_chunks(int nb, int J) {
   return nch < 1 ? 1 : nch;
 }
 
-cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int prec) {
+cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int prec, int most_chunks) {
   const size_t P = (size_t)t.n * t.n;
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
@@ -181,6 +205,7 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   if (slots < cw.grid_i3) slots = cw.grid_i3;
   const long long cj = (long long)nb * t.J, want_nmc = (8LL * slots + cj - 1) / cj;
   int nmc = (int)(want_nmc < t.M ? want_nmc : t.M);
+  if (most_chunks > 0 && nmc > most_chunks) nmc = most_chunks;
   if (nmc < 1) nmc = 1;
   if (nmc > t.M) nmc = t.M;
   const size_t N = t.N, Q = (N - 1) * (N - 1);
@@ -194,7 +219,7 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
     cw.nmc = (t.M + cw.mch - 1) / cw.mch;
   };
   set_chunks(nmc);
-  if (i3_paired(t.n, prec, v0))
+  if (most_chunks == 0 && i3_paired(t.n, prec, v0))
     set_chunks(even_chunks(cj, i3_concurrency(t.n, prec, v0, cw.grid_i3, INT_MAX), t.M, cw.nmc, 1, part_bytes,
                            kForwardCost, 0.4));
   const size_t nparts = (size_t)nb * t.J * cw.nmc;
@@ -213,35 +238,32 @@ cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int
   // k_i124: per (cell, chunk, pair) one field for I1 and three for I2/I4
   if (8 * (size_t)nb * cw.nch > ws_fields) ws_fields = 8 * (size_t)nb * cw.nch;
   cw.ws_fields = ws_fields;
-  cudaError_t e;
-#define QBE_ALLOC(ptr, bytes) \
-  if ((e = cudaMalloc((void**)&(ptr), (bytes))) != cudaSuccess) { free_collision_work(cw); return e; }
-  QBE_ALLOC(cw.what, (size_t)nb * 4 * P * cz);
-  QBE_ALLOC(cw.wfine, (size_t)nb * 2 * P * cz);
-  if (prec == 1 && t.n != 16) QBE_ALLOC(cw.wplane, (size_t)nb * 4 * P * rz);
-  QBE_ALLOC(cw.Dacc, (size_t)nb * 2 * P * cz);
-  QBE_ALLOC(cw.K2acc, (size_t)nb * P * rz);
-  QBE_ALLOC(cw.K4acc, (size_t)nb * 2 * P * cz);
-  QBE_ALLOC(cw.K2part, (size_t)nb * cw.nch * 2 * P * rz);
+  Carve mem;
+  mem.add(cw.what, (size_t)nb * 4 * P * cz);
+  mem.add(cw.wfine, (size_t)nb * 2 * P * cz);
+  if (prec == 1 && t.n != 16) mem.add(cw.wplane, (size_t)nb * 4 * P * rz);
+  mem.add(cw.Dacc, (size_t)nb * 2 * P * cz);
+  mem.add(cw.K2acc, (size_t)nb * P * rz);
+  mem.add(cw.K4acc, (size_t)nb * 2 * P * cz);
+  mem.add(cw.K2part, (size_t)nb * cw.nch * 2 * P * rz);
   if (cw.nch > 1) {
-    QBE_ALLOC(cw.Dpart, (size_t)nb * cw.nch * 2 * P * cz);
-    QBE_ALLOC(cw.K4part, (size_t)nb * cw.nch * 2 * P * cz);
+    mem.add(cw.Dpart, (size_t)nb * cw.nch * 2 * P * cz);
+    mem.add(cw.K4part, (size_t)nb * cw.nch * 2 * P * cz);
   }
-  QBE_ALLOC(cw.K3part, nparts * 2 * P * cz);
-  if (any_paired) QBE_ALLOC(cw.K3spec, nparts * 2 * Q * cz);
-  if (prec == 1) QBE_ALLOC(cw.K3sum, (size_t)nb * 2 * P * sizeof(double2));
-  if (prec == 1) QBE_ALLOC(cw.K3ssum, (size_t)nb * 2 * Q * sizeof(double2));
-  QBE_ALLOC(cw.ws, ws_fields * P * cz);
-  QBE_ALLOC(cw.cbuf, (size_t)nb * 4 * N * N * sizeof(double));
-  QBE_ALLOC(cw.wbuf, (size_t)nb * 4 * N * N * sizeof(double));
-#undef QBE_ALLOC
-  return cudaSuccess;
+  mem.add(cw.K3part, nparts * 2 * P * cz);
+  if (any_paired) mem.add(cw.K3spec, nparts * 2 * Q * cz);
+  if (prec == 1) mem.add(cw.K3sum, (size_t)nb * 2 * P * sizeof(double2));
+  if (prec == 1) mem.add(cw.K3ssum, (size_t)nb * 2 * Q * sizeof(double2));
+  mem.add(cw.ws, ws_fields * P * cz);
+  mem.add(cw.cbuf, (size_t)nb * 4 * N * N * sizeof(double));
+  mem.add(cw.wbuf, (size_t)nb * 4 * N * N * sizeof(double));
+  const cudaError_t e = mem.take(cw.mem);
+  if (e != cudaSuccess) cw = CollisionWork();
+  return e;
 }
 
 void free_collision_work(CollisionWork& cw) {
-  cudaFree(cw.what); cudaFree(cw.wfine); cudaFree(cw.wplane); cudaFree(cw.Dacc); cudaFree(cw.K2acc); cudaFree(cw.K4acc);
-  cudaFree(cw.Dpart); cudaFree(cw.K2part); cudaFree(cw.K4part);
-  cudaFree(cw.K3part); cudaFree(cw.K3spec); cudaFree(cw.K3sum); cudaFree(cw.K3ssum); cudaFree(cw.ws); cudaFree(cw.cbuf); cudaFree(cw.wbuf);
+  cudaFree(cw.mem);
   cw = CollisionWork();
 }
 
@@ -338,7 +360,7 @@ int vjp_cotangent_group(const Tables& t, int prec) { return (prec == 1 && t.n <=
 
 int vjp_i3_variants(int n, int prec) { return (prec == 1 && n == 128) ? 2 : 1; }
 
-cudaError_t alloc_vjp_work(const Tables& t, int nb, VjpWork& vw, int prec, int kcap) {
+cudaError_t alloc_vjp_work(const Tables& t, int nb, VjpWork& vw, int prec, int kcap, int most_chunks) {
   const size_t P = (size_t)t.n * t.n;
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
@@ -356,10 +378,11 @@ cudaError_t alloc_vjp_work(const Tables& t, int nb, VjpWork& vw, int prec, int k
   // about 4 waves of (cell, j, m-chunk) units
   const long long cj = (long long)nb * t.J, want_nmc = (4LL * vw.grid * teams + cj - 1) / cj;
   int nmc = (int)(want_nmc < t.M ? want_nmc : t.M);
+  if (most_chunks > 0 && nmc > most_chunks) nmc = most_chunks;
   if (nmc < 1) nmc = 1;
   vw.mch = (t.M + nmc - 1) / nmc;
   vw.nmc = (t.M + vw.mch - 1) / vw.mch;
-  {
+  if (most_chunks == 0) {
     const size_t Q1 = (size_t)(t.n / 2 - 1) * (t.n / 2 - 1);
     // (of as many cotangents as a product can carry: the chunking, and with it the order of the sums, must
     // not depend on how many this workspace holds)
@@ -382,29 +405,26 @@ cudaError_t alloc_vjp_work(const Tables& t, int nb, VjpWork& vw, int prec, int k
   const size_t kc = (size_t)kcap;
   const size_t cz = prec == 1 ? sizeof(float2) : sizeof(double2);
   const size_t rz = cz / 2;
-  cudaError_t e;
-#define QBE_ALLOC(ptr, bytes) \
-  if ((e = cudaMalloc((void**)&(ptr), (bytes))) != cudaSuccess) { free_vjp_work(vw); return e; }
-  QBE_ALLOC(vw.nu, kc * nb * 2 * P * cz);
-  QBE_ALLOC(vw.nuf, kc * nb * P * rz);
-  QBE_ALLOC(vw.muD, kc * nb * 2 * P * cz);
-  QBE_ALLOC(vw.muK2, kc * nb * P * rz);
-  QBE_ALLOC(vw.mu4, kc * nb * 2 * P * cz);
-  QBE_ALLOC(vw.mu3, kc * nb * 2 * P * cz);
-  QBE_ALLOC(vw.muh, kc * nb * 2 * P * cz);
-  if (tm) QBE_ALLOC(vw.mupl, kc * nb * 4 * P * rz);
-  QBE_ALLOC(vw.part_r, kc * nparts * 2 * P * cz);
+  Carve mem;
+  mem.add(vw.nu, kc * nb * 2 * P * cz);
+  mem.add(vw.nuf, kc * nb * P * rz);
+  mem.add(vw.muD, kc * nb * 2 * P * cz);
+  mem.add(vw.muK2, kc * nb * P * rz);
+  mem.add(vw.mu4, kc * nb * 2 * P * cz);
+  mem.add(vw.mu3, kc * nb * 2 * P * cz);
+  mem.add(vw.muh, kc * nb * 2 * P * cz);
+  if (tm) mem.add(vw.mupl, kc * nb * 4 * P * rz);
+  mem.add(vw.part_r, kc * nparts * 2 * P * cz);
   const size_t Q = (size_t)(t.n / 2 - 1) * (t.n / 2 - 1);   // kept frequencies (Fourier-space partials)
-  QBE_ALLOC(vw.part_s, kc * nparts * 2 * Q * cz);
-  QBE_ALLOC(vw.ws, ws_fields * P * cz);
-#undef QBE_ALLOC
-  return cudaSuccess;
+  mem.add(vw.part_s, kc * nparts * 2 * Q * cz);
+  mem.add(vw.ws, ws_fields * P * cz);
+  const cudaError_t e = mem.take(vw.mem);
+  if (e != cudaSuccess) vw = VjpWork();
+  return e;
 }
 
 void free_vjp_work(VjpWork& vw) {
-  cudaFree(vw.nu); cudaFree(vw.nuf); cudaFree(vw.muD); cudaFree(vw.muK2); cudaFree(vw.mu4); cudaFree(vw.mu3);
-  cudaFree(vw.muh); cudaFree(vw.mupl);
-  cudaFree(vw.part_r); cudaFree(vw.part_s); cudaFree(vw.ws);
+  cudaFree(vw.mem);
   vw = VjpWork();
 }
 

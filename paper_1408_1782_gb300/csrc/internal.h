@@ -87,6 +87,7 @@ struct I3Jobs {
 
 // Per-evaluation buffers of the collision operator for a batch of nb cells.
 struct CollisionWork {
+  void* mem = nullptr; // the device allocation that holds the buffers below
   int prec = 0;        // 0: FP64 transforms, 1: FP32 transforms (FP32-split form)
   int nb = 0;          // cells per batch
   int order_nb = 1;    // cells by which the order of the partials' sums is chosen: not those of a call (reduce_partials)
@@ -135,6 +136,7 @@ struct CollisionWork {
 // copies of the shape given, one per cotangent.
 constexpr int kMaxCotangents = 4;
 struct VjpWork {
+  void* mem = nullptr;   // the device allocation that holds the buffers below
   int prec = 0;
   int nb = 0;
   int kcap = 1;          // cotangents one product can carry
@@ -230,7 +232,8 @@ void fermi_dirac_pauli(const qbe_fd& fd, int N, double L, std::vector<double>& o
 // Collision operator on a batch (collision.cu).  w, c: device [nb][4][N][N].
 cudaError_t collide_batch(const Tables& t, CollisionWork& cw, const double* w, double* c, int ncells,
                           cudaStream_t s, long long& launches, KernelTimer* tm);
-cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int prec = 0);
+// One allocation.  most_chunks: 0, or the most m-chunks, without those that only even out the launch's load.
+cudaError_t alloc_collision_work(const Tables& t, int nb, CollisionWork& cw, int prec = 0, int most_chunks = 0);
 template <int n, class T>
 cudaError_t collide_batch_n(const Tables& t, CollisionWork& cw, const double* w, double* c, int ncells, cudaStream_t s,
                             long long& launches, KernelTimer* tm);
@@ -284,7 +287,7 @@ void free_collision_work(CollisionWork& cw);
 cudaError_t collide_vjp(const Tables& t, CollisionWork& cw, VjpWork& vw, const double* w, const double* const* lam,
                         double* const* grad, int K, int ncells, int accumulate, cudaStream_t s, long long& launches,
                         KernelTimer* tm);
-cudaError_t alloc_vjp_work(const Tables& t, int nb, VjpWork& vw, int prec = 0, int kcap = 1);
+cudaError_t alloc_vjp_work(const Tables& t, int nb, VjpWork& vw, int prec = 0, int kcap = 1, int most_chunks = 0);
 // How many cotangents one product should carry for this grid and precision form (1 .. kMaxCotangents).
 int vjp_cotangent_group(const Tables& t, int prec);
 // I3 transpose kernel variants for a padded grid and precision (0: the default, the fastest measured).

@@ -171,6 +171,20 @@ int do_step(qbe_handle* h, double dt, double* snaps = nullptr) {
   return r;
 }
 
+// The workspace take(nb, most_chunks) for all `cells` cells at a time (most_chunks 0: as it likes).  Where the
+// device's memory does not hold it: with fewer and fewer m-chunks of the M nodes, whose partials are most of it,
+// then for a half, a quarter and so on of the cells.
+template <class TAKE>
+cudaError_t take_cells(int cells, int M, TAKE take) {
+  cudaError_t e = take(cells, 0);
+  for (int k = M; k >= 1 && e == cudaErrorMemoryAllocation; k /= 2) e = take(cells, k);
+  for (int nb = cells; nb > 1 && e == cudaErrorMemoryAllocation;) {
+    nb = (nb + 1) / 2;
+    e = take(nb, 1);
+  }
+  return e;
+}
+
 // Adjoint workspace for products carrying up to kneed cotangents at once (grown on demand).
 int ensure_vjp(qbe_handle* h, int kneed = 1) {
   if (h->vw_ready && h->vw.kcap >= kneed) return QBE_OK;
@@ -182,22 +196,25 @@ int ensure_vjp(qbe_handle* h, int kneed = 1) {
     h->lbuf = nullptr;
     h->vw_ready = false;
   }
-  cudaError_t e = alloc_vjp_work(h->tab, h->cw.nb, h->vw, h->g.precision, kneed);
-  if (e == cudaSuccess)
-    e = cudaMalloc((void**)&h->lbuf, (size_t)h->cw.nb * 4 * h->g.N * h->g.N * sizeof(double));
-  if (e != cudaSuccess) {
-    free_vjp_work(h->vw);
-    cudaFree(h->lbuf);
-    h->lbuf = nullptr;
-    return fail(h, QBE_ERR_ALLOC, std::string("adjoint workspace: ") + cudaGetErrorString(e));
-  }
+  const cudaError_t e = take_cells(h->cw.nb, h->tab.M, [&](int nb, int most) {
+    cudaError_t r = alloc_vjp_work(h->tab, nb, h->vw, h->g.precision, kneed, most);
+    if (r != cudaSuccess) return r;
+    r = cudaMalloc((void**)&h->lbuf, (size_t)nb * 4 * h->g.N * h->g.N * sizeof(double));
+    if (r != cudaSuccess) {
+      cudaGetLastError();
+      h->lbuf = nullptr;
+      free_vjp_work(h->vw);
+    }
+    return r;
+  });
+  if (e != cudaSuccess) return fail(h, QBE_ERR_ALLOC, std::string("adjoint workspace: ") + cudaGetErrorString(e));
   h->vw.i3v = h->vjp_i3v;
   h->vw_ready = true;
   return QBE_OK;
 }
 
 // grad[k] (+)= (dC/dW)^T lam[k] at the state w for K <= kMaxCotangents cotangents (device
-// [ncells][4][N][N] each), in batches of cw.nb cells; the K products share the state's transforms.
+// [ncells][4][N][N] each), in batches of vw.nb cells; the K products share the state's transforms.
 int do_collide_vjp_dev(qbe_handle* h, const double* w, const double* const* lam, double* const* grad, int K,
                        int ncells, int accumulate) {
   int r = ensure_vjp(h, K);
@@ -205,8 +222,8 @@ int do_collide_vjp_dev(qbe_handle* h, const double* w, const double* const* lam,
   const size_t per = (size_t)4 * h->g.N * h->g.N;
   const double* lk[kMaxCotangents];
   double* gk[kMaxCotangents];
-  for (int c0 = 0; c0 < ncells; c0 += h->cw.nb) {
-    const int nc = (ncells - c0) < h->cw.nb ? (ncells - c0) : h->cw.nb;
+  for (int c0 = 0; c0 < ncells; c0 += h->vw.nb) {
+    const int nc = (ncells - c0) < h->vw.nb ? (ncells - c0) : h->vw.nb;
     for (int k = 0; k < K; ++k) {
       lk[k] = lam[k] + (size_t)c0 * per;
       gk[k] = grad[k] + (size_t)c0 * per;
@@ -292,11 +309,6 @@ int qbe_create(const qbe_grid* g, qbe_handle** out) {
     qbe_destroy(h);
     return QBE_ERR_ALLOC;
   }
-  // collision batch: all cells of the state (one evaluation per RK stage)
-  if (alloc_collision_work(h->tab, g->Nx, h->cw, g->precision) != cudaSuccess) {
-    qbe_destroy(h);
-    return QBE_ERR_ALLOC;
-  }
   const size_t se = state_elems(h) * sizeof(double);
   const size_t wall = (size_t)4 * g->N * g->N * sizeof(double);
   if (cudaMalloc(&h->W, se) != cudaSuccess || cudaMalloc(&h->Wa, se) != cudaSuccess ||
@@ -305,6 +317,14 @@ int qbe_create(const qbe_grid* g, qbe_handle** out) {
       cudaMalloc(&h->mom, (size_t)g->Nx * 7 * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&h->fbar, 2 * sizeof(double)) != cudaSuccess || cudaMalloc(&h->phiL, wall) != cudaSuccess ||
       cudaMalloc(&h->phiR, wall) != cudaSuccess) {
+    qbe_destroy(h);
+    return QBE_ERR_ALLOC;
+  }
+  // collision batch: all cells of the state (one evaluation per RK stage), or as many as fit; last, so that it
+  // takes what memory the rest leaves
+  if (take_cells(g->Nx, g->M, [&](int nb, int most) {
+        return alloc_collision_work(h->tab, nb, h->cw, g->precision, most);
+      }) != cudaSuccess) {
     qbe_destroy(h);
     return QBE_ERR_ALLOC;
   }
@@ -579,8 +599,8 @@ int qbe_collide_vjp(qbe_handle* h, const double* w, const double* lam, double* g
   int r = ensure_vjp(h);
   if (r) return r;
   const size_t per = (size_t)4 * h->g.N * h->g.N;
-  for (int c0 = 0; c0 < ncells; c0 += h->cw.nb) {
-    const int nc = (ncells - c0) < h->cw.nb ? (ncells - c0) : h->cw.nb;
+  for (int c0 = 0; c0 < ncells; c0 += h->vw.nb) {
+    const int nc = (ncells - c0) < h->vw.nb ? (ncells - c0) : h->vw.nb;
     const size_t bytes = (size_t)nc * per * sizeof(double);
     cudaError_t e = cudaMemcpyAsync(h->cw.wbuf, w + (size_t)c0 * per, bytes, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess)
@@ -1064,20 +1084,32 @@ int batch_capture_step(qbe_batch* b, double dt, cudaStream_t origin) {
       }
   };
   const std::vector<std::vector<size_t>> groups = i3_groups(b);
+  // A simulation whose workspace holds a part of its cells runs its collisions whole, on its own branch.
+  auto in_parts = [](const qbe_handle* h) { return h->cw.nb < h->g.Nx; };
+  auto pre = [&](qbe_handle* h, const double* w) -> int {
+    if (in_parts(h)) return QBE_OK;
+    return collide_pre(h->tab, h->cw, w, h->g.Nx, h->stream, h->launches) == cudaSuccess ? QBE_OK : QBE_ERR_CUDA;
+  };
+  auto post = [&](qbe_handle* h, const double* w) -> int {   // C[w] in Cb
+    if (in_parts(h)) return do_collide_dev(h, w, h->Cb, h->g.Nx);
+    return collide_post(h->tab, h->cw, h->Cb, h->g.Nx, h->stream, h->launches) == cudaSuccess ? QBE_OK : QBE_ERR_CUDA;
+  };
   auto i3_all = [&](long long& launches) {
     for (auto& g : groups) {
       std::vector<const Tables*> tabs;
       std::vector<const CollisionWork*> cws;
       std::vector<int> nc;
       for (size_t i : g) {
+        if (in_parts(b->sims[i])) continue;
         tabs.push_back(&b->sims[i]->tab);
         cws.push_back(&b->sims[i]->cw);
         nc.push_back(b->sims[i]->g.Nx);
       }
-      const CollisionWork& c0 = b->sims[g[0]]->cw;
+      if (nc.empty()) continue;
+      const CollisionWork& c0 = *cws[0];
       const int cap = (int)(c0.ws_fields / c0.i3_fields);            // blocks the first simulation's scratch can hold
       const int grid = c0.grid_i3 < cap ? c0.grid_i3 : cap;   // the group's (tuned) persistent grid
-      cudaError_t e = i3_group(tabs.data(), cws.data(), nc.data(), (int)g.size(), c0.ws, grid, origin, launches);
+      cudaError_t e = i3_group(tabs.data(), cws.data(), nc.data(), (int)nc.size(), c0.ws, grid, origin, launches);
       if (e != cudaSuccess) return QBE_ERR_CUDA;
     }
     return QBE_OK;
@@ -1098,7 +1130,7 @@ int batch_capture_step(qbe_batch* b, double dt, cudaStream_t origin) {
   for (size_t i = 0; i < ns && !r; ++i) {
     qbe_handle* h = b->sims[i];
     r = do_advect(h, 0.5 * dt);
-    if (!r && collide_pre(h->tab, h->cw, h->W, h->g.Nx, h->stream, h->launches) != cudaSuccess) r = QBE_ERR_CUDA;
+    if (!r) r = pre(h, h->W);
   }
   join();
   if (!r) r = i3_all(launches);
@@ -1107,10 +1139,10 @@ int batch_capture_step(qbe_batch* b, double dt, cudaStream_t origin) {
   for (size_t i = 0; i < ns && !r; ++i) {
     qbe_handle* h = b->sims[i];
     const int Nx = h->g.Nx, N = h->g.N;
-    if (collide_post(h->tab, h->cw, h->Cb, Nx, h->stream, h->launches) != cudaSuccess ||
-        rk_stage1(h->W, h->Cb, h->B, dt, h->F0, h->Wa, Nx, N, h->stream, h->launches, nullptr) != cudaSuccess ||
-        collide_pre(h->tab, h->cw, h->Wa, Nx, h->stream, h->launches) != cudaSuccess)
+    r = post(h, h->W);
+    if (!r && rk_stage1(h->W, h->Cb, h->B, dt, h->F0, h->Wa, Nx, N, h->stream, h->launches, nullptr) != cudaSuccess)
       r = QBE_ERR_CUDA;
+    if (!r) r = pre(h, h->Wa);
   }
   join();
   if (!r) r = i3_all(launches);
@@ -1119,9 +1151,9 @@ int batch_capture_step(qbe_batch* b, double dt, cudaStream_t origin) {
   for (size_t i = 0; i < ns && !r; ++i) {
     qbe_handle* h = b->sims[i];
     const int Nx = h->g.Nx, N = h->g.N;
-    if (collide_post(h->tab, h->cw, h->Cb, Nx, h->stream, h->launches) != cudaSuccess ||
-        rk_stage2(h->W, h->F0, h->Cb, h->Wa, h->B, dt, h->W, Nx, N, h->stream, h->launches, nullptr) !=
-            cudaSuccess)
+    r = post(h, h->Wa);
+    if (!r &&
+        rk_stage2(h->W, h->F0, h->Cb, h->Wa, h->B, dt, h->W, Nx, N, h->stream, h->launches, nullptr) != cudaSuccess)
       r = QBE_ERR_CUDA;
     if (!r) r = do_advect(h, 0.5 * dt);   // even number of state-buffer swaps over the step: ends in h->W
   }
