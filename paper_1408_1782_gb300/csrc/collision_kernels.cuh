@@ -1109,6 +1109,7 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
   Word* src = reinterpret_cast<Word*>(real_space ? part + c * nparts * np + i : spec + c * nparts * nq + (i - np));
   const size_t stride = (size_t)(real_space ? np : nq) / VEC;
   double s[2 * VEC] = {};
+  FloatSum a[VEC == 2 ? 4 : 1];   // FP32: the thread's last run
   if (i < np + nq) {
     if constexpr (VEC == 1) {
 #pragma unroll 8
@@ -1120,7 +1121,13 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
     } else {
       for (int u0 = g; u0 < nparts; u0 += G * FloatSum::kRun) {
         const int u1 = min(nparts, u0 + G * FloatSum::kRun);
-        FloatSum a[4];
+        if (u0 > g) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            s[k] += a[k].value();
+            a[k] = FloatSum();
+          }
+        }
 #pragma unroll 8
         for (int u = u0; u < u1; u += G) {
           const Word v = src[(size_t)u * stride];
@@ -1129,12 +1136,47 @@ __global__ void __launch_bounds__(256) k_reduce_k3(typename Vec2Of<T>::type* par
           a[2].add(v.z);
           a[3].add(v.w);
         }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) s[k] += a[k].value();
       }
     }
   }
-  if constexpr (G > 1) {
+  if constexpr (VEC == 2) {
+    // Few values a thread (G > 1): their sums are merged as floats, FP64 additions (24 a thread) would be most of
+    // the work.
+    const bool merged = G > 1 && nparts <= FloatSum::kMerged;
+    if constexpr (G > 1) {
+      __shared__ double red[G][2 * VEC][PT + PT / 2];   // doubles, or three floats a value
+      float* fl = &reinterpret_cast<float*>(red)[threadIdx.x % PT];
+      auto at = [&](int part, int j, int k) -> float& { return fl[((part * G + j) * 4 + k) * PT]; };
+      if (merged) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          at(0, g, k) = a[k].hi;
+          at(1, g, k) = a[k].mid;
+          at(2, g, k) = a[k].lo;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) red[g][k][threadIdx.x % PT] = s[k] + a[k].value();
+      }
+      __syncthreads();
+      if (g > 0) return;
+      if (merged) {
+        for (int j = 1; j < G; ++j)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) a[k].merge(at(0, j, k), at(1, j, k), at(2, j, k));
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s[k] = red[0][k][threadIdx.x];
+        for (int j = 1; j < G; ++j)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) s[k] += red[j][k][threadIdx.x];
+      }
+    }
+    if (G == 1 || merged) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) s[k] = nparts > G * FloatSum::kRun ? s[k] + a[k].value() : a[k].value();
+    }
+  } else if constexpr (G > 1) {
     __shared__ double red[G][2 * VEC][PT];
 #pragma unroll
     for (int k = 0; k < 2 * VEC; ++k) red[g][k][threadIdx.x % PT] = s[k];

@@ -16,6 +16,12 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 SOURCE = """
 #include "float_sum.cuh"
+extern "C" double merged_sum(const float* x, int n, int groups) {   // value u in group u mod groups
+  qbe::FloatSum a[8];
+  for (int u = 0; u < n; ++u) a[u % groups].add(x[u]);
+  for (int g = 1; g < groups; ++g) a[0].merge(a[g].hi, a[g].mid, a[g].lo);
+  return a[0].value();
+}
 extern "C" double run_sum(const float* x, int n) {
   double s = 0.0;
   for (int u0 = 0; u0 < n; u0 += qbe::FloatSum::kRun) {
@@ -38,10 +44,15 @@ def run_sum(tmp_path_factory):
     with open(src, "w") as f:
         f.write(SOURCE)
     subprocess.run([gxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, src, "-o", so], check=True)
-    fn = ctypes.CDLL(so).run_sum
-    fn.restype = ctypes.c_double
-    fn.argtypes = [ctypes.c_void_p, ctypes.c_int]
-    return lambda x: fn(x.ctypes.data, len(x))
+    lib = ctypes.CDLL(so)
+    for fn, n in ((lib.run_sum, 1), (lib.merged_sum, 2)):
+        fn.restype = ctypes.c_double
+        fn.argtypes = [ctypes.c_void_p] + [ctypes.c_int] * n
+
+    def call(x, groups=0):
+        return lib.merged_sum(x.ctypes.data, len(x), groups) if groups else lib.run_sum(x.ctypes.data, len(x))
+
+    return call
 
 
 @pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 256, 1024, 4096])
@@ -63,6 +74,17 @@ def test_no_less_accurate_than_fp64(run_sum, n, spread):
     assert worst <= max(fp64, 2.0 ** -53)
 
 
+@pytest.mark.parametrize("n", [1, 16, 100, 256])
+@pytest.mark.parametrize("spread", [0, 12, 30])
+def test_merged_sums_no_less_accurate_than_fp64(run_sum, n, spread):
+    rng = np.random.default_rng(n + spread)
+    for _ in range(50):
+        x = (rng.standard_normal(n) * np.exp(rng.uniform(-spread, 0, n))).astype(np.float32)
+        exact = math.fsum(x.astype(float).tolist())
+        size = float(np.abs(x.astype(float)).sum())
+        assert abs(run_sum(x, 8) - exact) <= ((2 * n * 2.0 ** -24) ** 3 + 3 * 2.0 ** -53) * size
+
+
 def test_infinities_and_nan(run_sum):
     x = np.ones(70, np.float32)
     x[3] = np.inf
@@ -72,3 +94,7 @@ def test_infinities_and_nan(run_sum):
     x[:] = 1.0
     x[69] = np.nan
     assert math.isnan(run_sum(x))
+    x[69] = -np.inf
+    assert run_sum(x, 8) == -math.inf
+    x[3] = np.inf
+    assert math.isnan(run_sum(x, 8))
