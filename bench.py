@@ -359,7 +359,7 @@ def run_ours(args):
     # k_rk1 / k_rk2 (one timing group, per-kernel averages): 16 and 20 FP64 operations per velocity;
     # 16 and 20 words of traffic per velocity (k_rk1: W, C in, F0, W1 out; k_rk2: W, F0, C1, W1 in, W out).
     for gname, label, bytes_per_launch, ops_per_launch in (
-            ("transport", "k_advect", 2 * sb, 6 * 4 * nvel),
+            ("transport", "k_advect", 2 * sb, 17 * nvel),     # 4.25 a value: 4, and 2 to start a run of 8 cells
             ("rk", "k_rk1+k_rk2 (per kernel)", (16 + 20) / 2 * 8 * nvel, (16 + 20) / 2 * nvel)):
         ms, cnt = groups[gname]["ms"], groups[gname]["launches"]
         if cnt and ms > 0:

@@ -347,14 +347,12 @@ cudaError_t collide_vjp(const Tables& t, CollisionWork& cw, VjpWork& vw, const d
   return cudaErrorInvalidValue;
 }
 
-// Cotangents one collision product should carry.  The staged transpose kernels (FP64, and FP32 on
-// grids above 128 points) are bound by their transforms, so sharing the state's Psi' convolutions saves
-// about a quarter of the work per product at two cotangents (measured: FP64, N = 64, 16 cells, 847 ms
-// per single launch against 1297 ms for two).  The FP32 shared-memory kernels run their transforms on
-// chip: the element-pass kernel is bound by its global accumulators, and every further cotangent adds
-// three fields of them per block, which pushes the working set out of L2 (two cotangents: 685 ms
-// against 2 x 333 ms, L2 hit rate 85 % -> 68 %); the tensor-memory kernel holds one
-// cotangent's shifted-back sums there, which leave no room for a second.  Both take one cotangent at a
+// Cotangents one collision product should carry.  The staged transpose kernels (FP64, and FP32 on grids above
+// 128 points) are bound by their transforms, so sharing the state's U convolutions saves work: I3 transpose,
+// FP64, N = 64, 16 cells, J = M = 32, 381 ms for one, 598 for two, 1032 for four; FP32, N = 128, 196 and 347 ms.
+// The FP32 shared-memory kernel is bound by its sums in global memory, whose working set leaves L2 further with
+// every cotangent (16 cells of N = 48: 12.7 ms for one, 28.2 for two; N = 64, variant 1: 27.4 and 57.3); the
+// tensor-memory kernel (15.9 ms there) holds one cotangent's sums, with no room for a second.  Both take one at a
 // time.
 int vjp_cotangent_group(const Tables& t, int prec) { return (prec == 1 && t.n <= 128) ? 1 : kMaxCotangents; }
 

@@ -92,7 +92,7 @@ struct CollisionWork {
   int nb = 0;          // cells per batch
   int order_nb = 1;    // cells by which the order of the partials' sums is chosen: not those of a call (reduce_partials)
   int nmc = 1;         // m-chunks per (cell, j) unit of the I3 kernel
-  int mch = 1;         // m values per chunk (the largest)
+  int mch = 1;         // the rounding that gives nmc = ceil(M / mch); the chunks' bounds are i3_chunk_begin's
   int grid_i3 = 0;     // persistent grid of the I3 kernel
   int grid_max = 0;    // its occupancy limit (SMs x resident blocks, the largest over the variants)
   int i3_variant = 0;  // launch variant of the I3 kernel (i3_variants)
@@ -100,7 +100,7 @@ struct CollisionWork {
   // buffers of the transform precision (complex = double2 or float2)
   void* what = nullptr;      // [nb][4][n*n] spectral pairs (w0+iw1, w2+iw3, w1+iw2, w3)
   void* wfine = nullptr;     // [nb][2][n*n] fine-grid fields (w0+iw1, w2+iw3)
-  void* wplane = nullptr;    // [nb][4][n*n] the same as planes (FP32, n = 32, 64, 128 only)
+  void* wplane = nullptr;    // [nb][4][n*n] the same as planes (FP32, every size but n = 16)
   void* Dacc = nullptr;      // [nb][2][n*n] spectral D (pairs (1,2), (3,-))
   void* K2acc = nullptr;     // [nb][n*n] (real)
   void* K4acc = nullptr;     // [nb][2][n*n] spectral K4 pairs (0,1), (2,3)
@@ -119,7 +119,7 @@ struct CollisionWork {
   // whether the last I3 launch over this workspace took the nodes in pairs (its post-processing
   // then adds K3spec); a batch launches its first member's variant for the whole group
   mutable bool i3_paired = false;
-  mutable bool i3_thread_order = false;  // ... whose partials are planes in thread_order (k_i3_tmem, k_i3_cluster in pairs)
+  mutable bool i3_thread_order = false;  // ... whose partials are planes in thread_order (k_i3_tmem, k_i3_lines, k_i3_cluster in pairs)
   void* ws = nullptr;        // per-CTA scratch
   size_t ws_fields = 0;      // complex n*n fields of scratch
   int i3_fields = 3;         // of which an I3 block (or cluster) uses this many

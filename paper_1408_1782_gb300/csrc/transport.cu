@@ -112,8 +112,9 @@ AdvectCoefs make_advect_coefs(int N, double dv, double kt) {
 // A thread walks its run downwind: the difference q3 - q2 and the second slope of one cell are the
 // first ones of the next, so a value costs one load, one difference, one subtraction and two FMAs in
 // FP64 (limiter on the integer pipe) instead of four loads and three differences; the loads of the run
-// are in flight together.  The bound is FP64 issue.  N = 64, 128 cells: 46 us at R = 1, 33 us
-// at R = 8; N = 128, 256 cells 325 and 208 us.
+// are in flight together.  Bound by the FP64 pipe: at N = 64, 128 cells it is busy 78 % of the time that an
+// SM has a block, and 67 % of the launch, whose 1.7 waves leave a tail.  N = 64, 128 cells: 46 us at R = 1,
+// 33 us at R = 8; N = 128, 256 cells 325 and 208 us.
 template <int R>
 __global__ void __launch_bounds__(256) k_advect(const double* __restrict__ W, double* __restrict__ Wout, int Nx,
                                                 int N, const __grid_constant__ AdvectCoefs cf, Ghost g) {
